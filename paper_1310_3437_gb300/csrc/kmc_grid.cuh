@@ -27,59 +27,71 @@ namespace kmc {
 
 __device__ __forceinline__ float f_up(double x) { return __double2float_ru(x); }
 
+// The builder runs on one warp per simulation between the push and the next step's
+// count, so its latency is in every step: what takes it is the length of the chain of
+// dependent operations, and on this part a binary64 division or square root is a chain
+// of about 560 or 595 cycles and a 64-bit integer division of 440 (a binary32 one: 35).
+// Hence: the cell counts and the cost estimates in binary32 (only the speed depends on
+// the choice; the margins of the cell width cover the rounding, see plan_cells), square
+// roots as upper bounds from the rounded-up binary32 root, per-axis values on a lane
+// each, and every parameter read before the first use of any.  One simulation: 35 -> 7 us
+// at 4096 particles, 47 -> 12 us at 2^20.
 struct CellPlan {
   int nc[3];
-  double m;
+  float m;
   uint32_t col_shift, col_tz, nkeys;
   bool ok;
 };
 
+// an upper bound of sqrt(x) for x >= 0, within 2^-19 of it
+__device__ __forceinline__ double sqrt_up(float x) {
+  return (double)__fsqrt_ru(x) * (1.0 + 0x1p-20);
+}
+
 // cells for search radius h (before the stencil split); key space capped by max_keys.
 // Along x the radius is split into K * kxm cells (kxm = 2: narrow cells along the rows
-// of the row search), along y and z into K.
-__device__ inline CellPlan plan_cells(const double ext[3], double h, int K, uint64_t max_keys,
+// of the row search), along y and z into K.  In binary32: the quotient is within 4 u32
+// of the exact one, so a cell is at least h (1 + m) (1 - 5 u32) / Ka wide, and the
+// binary32 cell assignment needs 8 u32 nmax of the margin m >= 1e-4 + 16 u32 nmax.
+__device__ inline CellPlan plan_cells(const float ext[3], float h, int K, uint64_t max_keys,
                                       int kxm = 1) {
-  const double u32 = 0x1p-24;
   CellPlan p;
   p.ok = false;
-  p.m = 0.0;
+  p.m = 0.0f;
   p.col_shift = 0;
   p.col_tz = 1;
   p.nkeys = 1;
   p.nc[0] = p.nc[1] = p.nc[2] = 1;
   for (int attempt = 0; attempt < 64; ++attempt) {
     // margin for binary32 cell assignment: index error <= 4 u32 n per particle
-    double nmax = 0.0;
-    for (int a = 0; a < 3; ++a) {
-      double q = ext[a] * (a == 0 ? K * kxm : K) / h;
-      nmax = q > nmax ? q : nmax;
-    }
-    if (nmax > 65535.0) nmax = 65535.0;
-    p.m = 1e-4 + 16.0 * u32 * nmax;
+    const float ih = 1.0f / h;
+    const float q0 = ext[0] * (float)(K * kxm) * ih, q1 = ext[1] * (float)K * ih,
+                q2 = ext[2] * (float)K * ih;
+    const float nmax = fminf(fmaxf(q0, fmaxf(q1, q2)), 65535.0f);
+    p.m = 1e-4f + 16.0f * 0x1p-24f * nmax;
+    const float shrink = 1.0f / (1.0f + p.m);
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
       const int Ka = a == 0 ? K * kxm : K;
-      const double wt = h * (1.0 + p.m) / Ka;  // target cell width
-      double q = floor(ext[a] / wt);
-      int c = q > 65535.0 ? 65535 : (int)q;
+      const float q = (a == 0 ? q0 : a == 1 ? q1 : q2) * shrink;
+      int c = q > 65535.0f ? 65535 : (int)q;  // q >= 0: the conversion is the floor
       if (c < 2 * Ka + 1) c = 1;
       p.nc[a] = c;
     }
     // key space of the tiled column order: T x T Morton tiles, T = 2^t <= 8
     const uint32_t ny = (uint32_t)p.nc[1], nz = (uint32_t)p.nc[2];
     const uint32_t small = ny < nz ? ny : nz;
-    uint32_t t = 0;
-    while (t < 3 && (1u << (t + 1)) <= small) ++t;
-    const uint64_t T = 1ull << t;
-    const uint64_t ty = (ny + T - 1) / T, tz = (nz + T - 1) / T;
-    const uint64_t nkeys = ty * tz * T * T * (uint64_t)p.nc[0];
+    const uint32_t t = small >= 8u ? 3u : small >= 4u ? 2u : small >= 2u ? 1u : 0u;
+    const uint32_t ty = (ny + (1u << t) - 1u) >> t, tz = (nz + (1u << t) - 1u) >> t;
+    const uint64_t nkeys = ((uint64_t)(ty * tz) << (2 * t)) * (uint64_t)p.nc[0];
     if (nkeys <= max_keys) {
       p.col_shift = t;
-      p.col_tz = (uint32_t)tz;
+      p.col_tz = tz;
       p.nkeys = (uint32_t)nkeys;
       p.ok = true;
       return p;
     }
-    h *= 1.25;  // coarsen until the key space fits
+    h *= 1.25f;  // coarsen until the key space fits
   }
   return p;
 }
@@ -92,243 +104,253 @@ __device__ inline CellPlan plan_cells(const double ext[3], double h, int K, uint
 // times the rate, the same cost); a fast particle costs its reach-trimmed stencil
 // (about 1.4 times the sphere of radius R_f, at about 2 tests' time per test) plus 15
 // per (y, z) column it walks.
-__device__ inline double slow_cost(double n, double rho) { return n * (5.0 * rho + 6.0); }
+__device__ inline float slow_cost(float n, float rho) { return n * (5.0f * rho + 6.0f); }
 // The binary64 path has no row search (thread per particle or warp per cell, whole
 // stencil, binary64 pre-tests): its cost is the half stencil's pair tests, inflated
 // when cells hold fewer particles than a warp's lanes can use; a fast particle costs
 // its whole stencil at 3 units per test.
-__device__ inline double slow_cost_f64(double n, double rho, int K) {
-  const double st = (2 * K + 1.0) * (2 * K + 1.0) * (2 * K + 1.0) * 0.5;
-  const double eff = rho < 16.0 ? sqrt(16.0 / (rho > 0.25 ? rho : 0.25)) : 1.0;
+__device__ inline float slow_cost_f64(float n, float rho, int K) {
+  const float st = (2 * K + 1.0f) * (2 * K + 1.0f) * (2 * K + 1.0f) * 0.5f;
+  const float eff = rho < 16.0f ? sqrtf(16.0f / fmaxf(rho, 0.25f)) : 1.0f;
   return n * st * rho * eff;
 }
-__device__ inline double fast_cost(double nfast, double rho, double rf_cells, double ncol) {
-  const double tests = rho * 1.4 * 4.18879 * rf_cells * rf_cells * rf_cells;
-  return nfast * (2.0 * tests + 15.0 * ncol);
+__device__ inline float fast_cost(float nfast, float rho, float rf_cells, float ncol) {
+  const float tests = rho * 1.4f * 4.18879f * rf_cells * rf_cells * rf_cells;
+  return nfast * (2.0f * tests + 15.0f * ncol);
 }
 
 // Trial thresholds of the speed split, fractions of the bound V of max |v| (squares
-// rounded down), with their particle counts cleared for the next count.
-__device__ inline void set_split_thresholds(SimDev& s, float vmax2_bound) {
-  const double V = sqrt((double)vmax2_bound) * (1.0 + 0x1p-20);
-  for (int t = 0; t < kSplitTrials; ++t) {
-    const double f = (double)split_frac(t);
-    s.d.split_thr[t] = __double2float_rd(f * V * f * V);
-    s.d.split_cnt[t] = 0;
-  }
+// rounded down), with their particle counts cleared for the next count: lane t the
+// threshold t.
+__device__ inline void set_split_thresholds(SimDev& s, float vmax2_bound, uint32_t lane) {
+  if (lane >= (uint32_t)kSplitTrials) return;
+  const double fV = (double)split_frac((int)lane) * sqrt_up(vmax2_bound);
+  s.d.split_thr[lane] = __double2float_rd(fV * fV);
+  s.d.split_cnt[lane] = 0;
 }
 
 // Called by all 32 lanes of a warp: lane t < kSplitTrials estimates the cost of
-// trial threshold t, lane 0 chooses and writes the grid (the others only read).
+// trial threshold t, all lanes choose alike, lanes 0..2 take one axis each and lane 0
+// writes the rest of the grid.
 __device__ inline void compute_grid(SimDev& s, float vmax2_bound, uint64_t step, uint32_t lane) {
-  Grid& g = s.d.grid;
+  constexpr uint32_t kAll = 0xFFFFFFFFu;
   const double u32 = 0x1p-24, u64 = 0x1p-53;
-  const int K = s.K;
-  const double scale = s.cell_scale > 1.0 ? s.cell_scale : 1.0;
-  const double V = sqrt((double)vmax2_bound) * (1.0 + 0x1p-20);  // upper bound of max |v|
-  const double Rfull = s.d0 + 2.0 * V * s.dt;
-  double ext[3];
-  for (int a = 0; a < 3; ++a) {
-    ext[a] = s.box[a];
-    if (a == 0 && s.bc[0] == KMC_REFLECT) {
-      // upper x wall at the start of this step (particles are below it)
-      double X = s.piston_x0 - s.piston_u * ((double)step * s.dt);
-      ext[0] = X > 0.0 ? X : s.box[0];
-    }
+  // ---- parameters, all loads in flight together --------------------------------
+  const int K = s.K, search_kernel = s.search_kernel, split_ok = s.split_ok;
+  const uint32_t n = s.n, cell_cap = s.cell_cap;
+  const bool fp32 = s.precision == KMC_GUARDED_FP32;
+  const double d0 = s.d0, dt = s.dt, d0sq = s.d0sq, cell_scale = s.cell_scale;
+  const float min_occ = (float)s.split_min_occ;
+  const double box0 = s.box[0], box1 = s.box[1], box2 = s.box[2];
+  const int bc0 = s.bc[0], bc1 = s.bc[1], bc2 = s.bc[2];
+  const double x0 = s.piston_x0, up = s.piston_u;
+  const bool can_split = split_ok && s.d.have_counts;
+  const uint32_t my_trial = lane < (uint32_t)kSplitTrials ? lane : 0u;
+  const float my_thr = s.d.split_thr[my_trial];
+  const float my_nfast = (float)s.d.split_cnt[my_trial];
+
+  const double scale = cell_scale > 1.0 ? cell_scale : 1.0;
+  const double V = sqrt_up(vmax2_bound);  // upper bound of max |v|
+  const double Rfull = d0 + 2.0 * V * dt;
+  double ext0 = box0;
+  if (bc0 == KMC_REFLECT) {
+    // upper x wall at the start of this step (particles are below it)
+    const double X = x0 - up * ((double)step * dt);
+    ext0 = X > 0.0 ? X : box0;
   }
+  const float extf[3] = {(float)ext0, (float)box1, (float)box2};
+  const bool per[3] = {bc0 == KMC_PERIODIC, bc1 == KMC_PERIODIC, bc2 == KMC_PERIODIC};
+  const float Rf = f_up(Rfull);
 
   // ---- split threshold: estimated pair-test cost of each trial (one lane each) --
-  const bool can_split = s.split_ok && s.d.have_counts;
   bool my_feasible = false;
-  double my_cost = 0.0;
+  float my_cost = 0.0f;
   if (lane < (uint32_t)kSplitTrials) {
     const int t = (int)lane;
-    bool feasible_t = false;
-    double cost_t = 0.0;
     do {
     if (t > 0 && !can_split) break;
     // trial thresholds were set from the previous step's bound; the slow cell must
     // cover the threshold actually used for classification (a binary32 square)
-    const float sq = t == 0 ? 0.0f : s.d.split_thr[t];
-    const double S1 = t == 0 ? V : sqrt((double)sq);
+    const double S1 = t == 0 ? V : sqrt_up(my_thr);
     if (t > 0 && !(S1 < V)) break;
-    const double hs = (s.d0 + 2.0 * S1 * s.dt) * scale;
-    CellPlan p = plan_cells(ext, hs, K, (uint64_t)s.cell_cap / (t == 0 ? 1 : 2));
+    const float hs = f_up((d0 + 2.0 * S1 * dt) * scale);
+    const CellPlan p = plan_cells(extf, hs, K, (uint64_t)cell_cap / (t == 0 ? 1 : 2));
     if (!p.ok) break;
-    const double cells = (double)p.nc[0] * p.nc[1] * p.nc[2];
-    const double rho = (double)s.n / cells;
-    const bool f64 = s.precision == KMC_FP64;
+    const float rho = (float)n / ((float)p.nc[0] * (float)p.nc[1] * (float)p.nc[2]);
     if (t == 0) {
-      cost_t = f64 ? slow_cost_f64((double)s.n, rho, K) : slow_cost((double)s.n, rho);
-      feasible_t = true;
+      my_cost = fp32 ? slow_cost((float)n, rho) : slow_cost_f64((float)n, rho, K);
+      my_feasible = true;
       break;
     }
-    if (s.split_ok == 1 && rho < s.split_min_occ) break;
+    if (split_ok == 1 && rho < min_occ) break;
     // fast stencil: c cells on each side per split axis; periodic axes must hold it,
     // and no axis may be a one-cell periodic axis (no minimum-image test there)
-    const double nfast = (double)s.d.split_cnt[t];
-    double ncol = 1.0, wmin = 0.0, fast_cells = 1.0;
+    float ncol = 1.0f, iwmax = 0.0f, fast_cells = 1.0f;
     bool fits = true;
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
       if (p.nc[a] == 1) {
-        if (s.bc[a] == KMC_PERIODIC) fits = false;
+        if (per[a]) fits = false;
         continue;
       }
-      const double w = ext[a] / p.nc[a];
-      wmin = wmin == 0.0 || w < wmin ? w : wmin;
-      int c = (int)ceil(Rfull * (1.0 + p.m) / w);
+      const float iw = (float)p.nc[a] / extf[a];
+      iwmax = fmaxf(iwmax, iw);
+      // the final grid below rounds this count up in the same way
+      int c = (int)ceilf(Rf * (1.0f + p.m) * iw * (1.0f + 1e-6f));
       if (c < K) c = K;
-      if (s.bc[a] == KMC_PERIODIC && p.nc[a] < 2 * c + 2) fits = false;
-      if (a > 0) ncol *= (2.0 * c + 1.0);
-      fast_cells *= (2.0 * c + 1.0);
+      if (per[a] && p.nc[a] < 2 * c + 2) fits = false;
+      if (a > 0) ncol *= (2.0f * c + 1.0f);
+      fast_cells *= (2.0f * c + 1.0f);
     }
     if (!fits) break;
     // a fast particle's reach, its speed taken just above the threshold
-    const double rf = s.d0 + (1.15 * S1 + V) * s.dt;
-    const double rf_cells = wmin > 0.0 ? rf / wmin : 1.0;
-    cost_t = f64 ? slow_cost_f64((double)s.n - nfast, rho, K) + nfast * fast_cells * rho * 3.0
-                 : slow_cost((double)s.n - nfast, rho) + fast_cost(nfast, rho, rf_cells, ncol);
-    feasible_t = true;
+    const float rf = (float)(d0 + (1.15 * S1 + V) * dt);
+    const float rf_cells = iwmax > 0.0f ? rf * iwmax : 1.0f;
+    my_cost = fp32 ? slow_cost((float)n - my_nfast, rho) + fast_cost(my_nfast, rho, rf_cells, ncol)
+                   : slow_cost_f64((float)n - my_nfast, rho, K) + my_nfast * fast_cells * rho * 3.0f;
+    my_feasible = true;
     } while (false);
-    my_feasible = feasible_t;
-    my_cost = cost_t;
   }
-  bool feasible[kSplitTrials];
-  double cost[kSplitTrials];
-  for (int t = 0; t < kSplitTrials; ++t) {
-    feasible[t] = __shfl_sync(0xFFFFFFFFu, my_feasible ? 1 : 0, t) != 0;
-    cost[t] = __shfl_sync(0xFFFFFFFFu, my_cost, t);
-  }
-  if (lane != 0) return;  // lane 0 chooses the threshold and writes the grid
+  const uint32_t fmask = __ballot_sync(kAll, my_feasible);
   int best = 0;
-  if (s.split_ok == 2) {
+  if (split_ok == 2) {
     // forced: cycle through the feasible trial thresholds step by step
     const int want = (int)(step % (uint64_t)(kSplitTrials - 1));
     for (int d = 0; d < kSplitTrials - 1; ++d) {
       const int t = 1 + (want + d) % (kSplitTrials - 1);
-      if (feasible[t]) { best = t; break; }
+      if ((fmask >> t) & 1u) { best = t; break; }
     }
   } else {
-    for (int t = 1; t < kSplitTrials; ++t)
-      if (feasible[t] && cost[t] < 0.9 * cost[best]) best = t;
+    float cost = __shfl_sync(kAll, my_cost, 0);
+#pragma unroll
+    for (int t = 1; t < kSplitTrials; ++t) {
+      const float ct = __shfl_sync(kAll, my_cost, t);
+      if (((fmask >> t) & 1u) && ct < 0.9f * cost) { best = t; cost = ct; }
+    }
   }
-  const float s1sq = best > 0 ? s.d.split_thr[best] : 0.0f;
   const bool split = best > 0;
-  const double S1 = split ? sqrt((double)s1sq) : V;
-  g.split = split ? 1u : 0u;
-  g.split_t = best;
-  g.s1sq = s1sq;
+  const float thr = __shfl_sync(kAll, my_thr, best);
+  const float s1sq = split ? thr : 0.0f;
+  const double S1 = split ? sqrt_up(s1sq) : V;
   // trial thresholds for the next step (counted by the push of this step)
-  set_split_thresholds(s, vmax2_bound);
+  set_split_thresholds(s, vmax2_bound, lane);
 
-  CellPlan p = plan_cells(ext, (s.d0 + 2.0 * S1 * s.dt) * scale, K,
-                          (uint64_t)s.cell_cap / (split ? 2 : 1));
-  {
-    // search kernel for the slow population: warp per cell when cells are well
-    // filled; the binary32 warp-per-cell search handles no one-cell periodic axis
-    // (the row search does)
-    const double cells = (double)p.nc[0] * p.nc[1] * p.nc[2];
-    const double occ = (double)s.n / cells;
-    bool cp = false;
-    for (int a = 0; a < 3; ++a) cp = cp || (p.nc[a] == 1 && s.bc[a] == KMC_PERIODIC);
-    int mode = s.search_kernel;
-    const bool fp32 = s.precision == KMC_GUARDED_FP32;
-    if (mode == 0) {
-      if (fp32) mode = occ >= 16.0 ? KMC_SEARCH_CELL : KMC_SEARCH_ROW;
-      else mode = occ >= 4.0 ? KMC_SEARCH_CELL : KMC_SEARCH_PARTICLE;
-    }
-    if (mode == KMC_SEARCH_ROW && !fp32) mode = KMC_SEARCH_CELL;
-    if (mode == KMC_SEARCH_CELL && cp && fp32) mode = KMC_SEARCH_ROW;
-    g.mode = mode;
-    g.kx = K;
-    if (mode == KMC_SEARCH_ROW && p.nc[0] > 1) {
-      // rows of half-width cells: each particle's row is trimmed to its reach in
-      // half-cell steps (the grid is otherwise the same)
-      const CellPlan q = plan_cells(ext, (s.d0 + 2.0 * S1 * s.dt) * scale, K,
-                                    (uint64_t)s.cell_cap / (split ? 2 : 1), 2);
-      if (q.ok && q.nc[0] > 1 && q.nc[1] == p.nc[1] && q.nc[2] == p.nc[2]) {
-        p = q;
-        g.kx = 2 * K;
-      }
+  const float hs = f_up((d0 + 2.0 * S1 * dt) * scale);
+  const uint64_t max_keys = (uint64_t)cell_cap / (split ? 2 : 1);
+  CellPlan p = plan_cells(extf, hs, K, max_keys);
+  // search kernel for the slow population: warp per cell when cells are well
+  // filled; the binary32 warp-per-cell search handles no one-cell periodic axis
+  // (the row search does)
+  const float occ = (float)n / ((float)p.nc[0] * (float)p.nc[1] * (float)p.nc[2]);
+  bool cp = false;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) cp = cp || (p.nc[a] == 1 && per[a]);
+  int mode = search_kernel;
+  if (mode == 0) {
+    if (fp32) mode = occ >= 16.0f ? KMC_SEARCH_CELL : KMC_SEARCH_ROW;
+    else mode = occ >= 4.0f ? KMC_SEARCH_CELL : KMC_SEARCH_PARTICLE;
+  }
+  if (mode == KMC_SEARCH_ROW && !fp32) mode = KMC_SEARCH_CELL;
+  if (mode == KMC_SEARCH_CELL && cp && fp32) mode = KMC_SEARCH_ROW;
+  int kx = K;
+  if (mode == KMC_SEARCH_ROW && p.nc[0] > 1) {
+    // rows of half-width cells: each particle's row is trimmed to its reach in
+    // half-cell steps (the grid is otherwise the same)
+    const CellPlan q = plan_cells(extf, hs, K, max_keys, 2);
+    if (q.ok && q.nc[0] > 1 && q.nc[1] == p.nc[1] && q.nc[2] == p.nc[2]) {
+      p = q;
+      kx = 2 * K;
     }
   }
-  if (!p.ok) s.d.status |= ST_CELL_OVERFLOW;
-  const int* nc = p.nc;
-  const double m = p.m;
-  g.col_shift = p.col_shift;
-  g.col_tz = p.col_tz;
-  g.nkeys = p.nkeys;
-  g.K = K;
-  int cfast[3] = {0, 0, 0};
-  for (int a = 0; a < 3; ++a) {
-    if (!split || nc[a] == 1) continue;
-    const int Ka = a == 0 ? g.kx : K;
-    const double w = ext[a] / nc[a];
-    int c = (int)ceil(Rfull * (1.0 + m) / w);
-    if (c < Ka) c = Ka;
-    cfast[a] = c;
-  }
-  for (int a = 0; a < 3; ++a) g.cfast[a] = cfast[a];
-  for (int a = 0; a < 3; ++a) {
-    g.nc[a] = nc[a];
-    g.w[a] = nc[a] == 1 ? ext[a] : ext[a] / nc[a];
-    g.wf[a] = (float)g.w[a];
-    g.inv_wf[a] = nc[a] == 1 ? 0.0f : (float)((double)nc[a] / ext[a]);
-  }
+  const double m = (double)p.m;
 
-  // ---- binary64 sphere pre-test: R > c0 + c1 B  =>  not a candidate ----------
-  // Exactly, |r|^2 |v|^2 = (r.v)^2 + |r x v|^2, so |r|^2 = t*^2 |v|^2 + d_min^2 <
-  // dt^2 |v|^2 + d0^2 for a candidate; with the roundings of the test this holds
-  // with a relative slack below 30 u64, far inside the 2^-40 used here.
-  g.c0 = s.d0sq * (1.0 + 0x1p-40) * (1.0 + 0x1p-50);
-  g.c1 = s.dt * s.dt * (1.0 + 0x1p-40) * (1.0 + 0x1p-50);
-
-  // ---- binary32 pre-tests ------------------------------------------------------
-  // The binary32 mirror holds box coordinates and velocities, each rounded once.
-  // Error of the binary32 separation against the binary64 one, per component:
+  // ---- per axis (lanes 0..2; the other lanes repeat lane 2) ---------------------
+  // Error of the binary32 separation against the binary64 one, per component (the
+  // binary32 mirror holds box coordinates and velocities, each rounded once):
   //   multi-cell axis: both coordinates (u32 L each), a periodic image shifts one
   //     side by the rounded box length (u32 L) and that sum is rounded (u32 L); the
   //     difference itself rounds with u32 |r|: 4 u32 L + u32 rb, plus 8 u64 L for the
   //     binary64 separation's own rounding;
   //   one-cell axis (minimum image in binary32): u32 * 6.1 * extent + 8 u64 L.
   // Velocity difference: 4.1 u32 V.  Component bounds: |r_k| <= rb_k, |v_k| <= 2V.
-  double er = 0.0, rn2 = 0.0, rbmax = 0.0;
-  for (int a = 0; a < 3; ++a) {
-    const double L = s.box[a] > ext[a] ? s.box[a] : ext[a];
-    const int Ka = a == 0 ? g.kx : K;
-    const int Ke = cfast[a] > Ka ? cfast[a] : Ka;
-    double e, rb;
-    if (nc[a] == 1) {
-      e = 6.1 * u32 * L + 8.0 * u64 * L;
-      rb = s.bc[a] == KMC_PERIODIC ? 0.5 * L * (1.0 + 8.0 * u32) + 2.0 * e : L;
-    } else {
-      rb = (Ke + 1.0 + 2.0 * m) * g.w[a];
-      e = u32 * (4.0 * L + rb) * (1.0 + 1e-3) + 8.0 * u64 * L;
-    }
-    er = e > er ? e : er;
-    rbmax = rb > rbmax ? rb : rbmax;
-    rn2 += rb * rb;
-    g.Lf[a] = (float)s.box[a];
-    g.halfLf[a] = (float)(0.5 * s.box[a]);
-    g.tief[a] = f_up(4.0 * e);
+  const int ax = lane < 2u ? (int)lane : 2;
+  const int my_nc = ax == 0 ? p.nc[0] : ax == 1 ? p.nc[1] : p.nc[2];
+  const double my_ext = ax == 0 ? ext0 : ax == 1 ? box1 : box2;
+  const double my_box = ax == 0 ? box0 : ax == 1 ? box1 : box2;
+  const bool my_per = ax == 0 ? per[0] : ax == 1 ? per[1] : per[2];
+  const int Ka = ax == 0 ? kx : K;
+  const double my_w = my_nc == 1 ? my_ext : my_ext / (double)my_nc;
+  const float my_iw = (float)my_nc / (float)my_ext;
+  int my_cfast = 0;
+  if (split && my_nc != 1) {
+    // at least Rfull (1 + m) / w cells: the product is within 4 u32 of it
+    my_cfast = (int)ceilf(Rf * (1.0f + p.m) * my_iw * (1.0f + 1e-6f));
+    if (my_cfast < Ka) my_cfast = Ka;
   }
+  const double L = my_box > my_ext ? my_box : my_ext;
+  const int Ke = my_cfast > Ka ? my_cfast : Ka;
+  double my_e, my_rb;
+  if (my_nc == 1) {
+    my_e = 6.1 * u32 * L + 8.0 * u64 * L;
+    my_rb = my_per ? 0.5 * L * (1.0 + 8.0 * u32) + 2.0 * my_e : L;
+  } else {
+    my_rb = (Ke + 1.0 + 2.0 * m) * my_w;
+    my_e = u32 * (4.0 * L + my_rb) * (1.0 + 1e-3) + 8.0 * u64 * L;
+  }
+  Grid& g = s.d.grid;
+  if (lane < 3u) {
+    g.nc[lane] = my_nc;
+    g.cfast[lane] = my_cfast;
+    g.w[lane] = my_w;
+    g.wf[lane] = (float)my_w;
+    g.inv_wf[lane] = my_nc == 1 ? 0.0f : my_iw;
+    g.Lf[lane] = (float)my_box;
+    g.halfLf[lane] = (float)(0.5 * my_box);
+    g.tief[lane] = f_up(4.0 * my_e);
+  }
+  const double e0 = __shfl_sync(kAll, my_e, 0), e1 = __shfl_sync(kAll, my_e, 1),
+               e2 = __shfl_sync(kAll, my_e, 2);
+  const double b0 = __shfl_sync(kAll, my_rb, 0), b1 = __shfl_sync(kAll, my_rb, 1),
+               b2 = __shfl_sync(kAll, my_rb, 2);
+  const double L0 = __shfl_sync(kAll, L, 0), L1 = __shfl_sync(kAll, L, 1),
+               L2 = __shfl_sync(kAll, L, 2);
+  if (lane != 0) return;  // lane 0 writes the rest
+  if (!p.ok) s.d.status |= ST_CELL_OVERFLOW;
+  g.split = split ? 1u : 0u;
+  g.split_t = best;
+  g.s1sq = s1sq;
+  g.mode = mode;
+  g.kx = kx;
+  g.col_shift = p.col_shift;
+  g.col_tz = p.col_tz;
+  g.nkeys = p.nkeys;
+  g.K = K;
+
+  // ---- binary64 sphere pre-test: R > c0 + c1 B  =>  not a candidate ----------
+  // Exactly, |r|^2 |v|^2 = (r.v)^2 + |r x v|^2, so |r|^2 = t*^2 |v|^2 + d_min^2 <
+  // dt^2 |v|^2 + d0^2 for a candidate; with the roundings of the test this holds
+  // with a relative slack below 30 u64, far inside the 2^-40 used here.
+  const double dt2 = dt * dt;
+  g.c0 = d0sq * ((1.0 + 0x1p-40) * (1.0 + 0x1p-50));
+  g.c1 = dt2 * ((1.0 + 0x1p-40) * (1.0 + 0x1p-50));
+
+  // ---- binary32 pre-tests ------------------------------------------------------
+  const double er = fmax(e0, fmax(e1, e2)), rbmax = fmax(b0, fmax(b1, b2));
+  const double Lmax = fmax(L0, fmax(L1, L2));
   {
     // row trimming: a slow-slow candidate has |r| < d0 + (|v_i| + |v_j|) dt <= d0 + 2 S1 dt
-    double Lmax = 0.0;
-    for (int a = 0; a < 3; ++a) {
-      const double L = s.box[a] > ext[a] ? s.box[a] : ext[a];
-      Lmax = L > Lmax ? L : Lmax;
-    }
-    const double reach = (s.d0 + 2.0 * S1 * s.dt) * (1.0 + 1e-6);
+    const double S1dt = S1 * dt;
+    const double reach = (d0 + 2.0 * S1dt) * (1.0 + 1e-6);
     g.row_r2 = f_up(reach * reach * (1.0 + 1e-6));
     // per particle: (i, j) with j slow has |r| < d0 + (|v_i| + |v_j|) dt <= d0 + S1 dt + |v_i| dt
-    g.row_a = f_up((s.d0 + S1 * s.dt) * (1.0 + 1e-6));
-    g.row_b = f_up(s.dt * (1.0 + 1e-6));
-    g.fast_a = f_up((s.d0 + V * s.dt) * (1.0 + 1e-6));
+    g.row_a = f_up((d0 + S1dt) * (1.0 + 1e-6));
+    g.row_b = f_up(dt * (1.0 + 1e-6));
+    g.fast_a = f_up((d0 + V * dt) * (1.0 + 1e-6));
     g.row_eps = f_up(16.0 * u32 * Lmax);
     g.row_pad = f_up(4.0 * u32 * Lmax);
   }
-  const double rn = sqrt(rn2) * (1.0 + 1e-6);
+  const double rn = sqrt_up(f_up((b0 * b0 + b1 * b1) + b2 * b2)) * (1.0 + 1e-6);
+  const double V2 = V * V, rnV2 = rn * 2.0 * V;
   const double ev = 4.1 * u32 * V;
   const double g3 = 3.0 * u32 / (1.0 - 3.0 * u32);
   const double g3d = 3.0 * u64 / (1.0 - 3.0 * u64);
@@ -337,28 +359,25 @@ __device__ inline void compute_grid(SimDev& s, float vmax2_bound, uint64_t step,
   const double rel40 = 1.0 + 0x1p-40;
   const double s3 = 1.7320508075688772 * (1.0 + 1e-15);
   const double bslack = 7.0 * ev * V + 3.0 * ev * ev;  // |v|^2 - |v~|^2 slack, absolute
-  const double dt = s.dt, d0sq = s.d0sq;
   // sphere test
-  const double c0 = (rel40 * (d0sq + dt * dt * bslack) + 2.0 * s3 * er * rn) * (1.0 + g3);
-  const double c1 = dt * dt * rel40 * (1.0 + g3) / (1.0 - g3);
+  const double c0 = (rel40 * (d0sq + dt2 * bslack) + 2.0 * s3 * er * rn) * (1.0 + g3);
   g.s_c0 = f_up(c0 * up2);
-  g.s_c1 = f_up(c1 * up2);
+  g.s_c1 = f_up(dt2 * (rel40 * (1.0 + g3) / (1.0 - g3) * up2));
   // approach test (t* >= 0): |A~ - A64| <= a_g
-  const double Ga = (s3 * (ev * rn + 2.0 * V * er) + g3 * rn * 2.0 * V * 1.01 + g3d * rn * 2.0 * V) *
-                    (1.0 + 1e-3);
+  const double Ga = (s3 * (ev * rn + 2.0 * V * er) + rnV2 * (g3 * 1.01 + g3d)) * (1.0 + 1e-3);
   g.a_g = f_up(Ga);
   // time test (t* < dt): X~ = A~ - dt B~ > t_g  =>  A64 >= dt B64
-  const double Ex = u32 * (rn * 2.0 * V * 1.01 + 2.0 * dt * 4.0 * V * V * 1.02);
-  const double Gt = (Ex + Ga + dt * (8.1 * V * V * g3 + bslack)) * (1.0 + 1e-3);
+  const double Ex = u32 * (rnV2 * 1.01 + dt * V2 * 8.16);
+  const double Gt = (Ex + Ga + dt * (8.1 * g3 * V2 + bslack)) * (1.0 + 1e-3);
   g.t_g = f_up(Gt);
   g.dtf = (float)dt;
   // distance test (d_min < d0): |w~| >= w_e + d0 sqrt(B_up)  =>  W64 >= d0^2 B64
-  const double ew = (2.0 * (rbmax * ev + 2.0 * V * er) * 1.001 + g2 * 2.0 * rbmax * 2.0 * V * 1.01) +
-                    2.0 * (2.0 * u64) * rbmax * 2.0 * V;
+  const double ew = 2.0 * (rbmax * ev + 2.0 * V * er) * 1.001 + rbmax * V * (4.04 * g2 + 8.0 * u64);
   g.w_e = f_up(s3 * ew * up4);
   g.b_rel = f_up((1.0 / (1.0 - g3)) * (1.0 + g3d) * up2);
-  g.b_abs = f_up(bslack * (1.0 + g3d) * up2);
-  g.d0up = f_up(s.d0 * rel40 / sqrt(1.0 - g3d) * up4 * (1.0 + 4.0 * u32));
+  g.b_abs = f_up(bslack * ((1.0 + g3d) * up2));
+  // 1 / sqrt(1 - g3d) <= 1 + g3d
+  g.d0up = f_up(d0 * (rel40 * (1.0 + g3d) * up4 * (1.0 + 4.0 * u32)));
   g.w_rel = f_up((1.0 + g3) * up4);
 }
 

@@ -238,59 +238,74 @@ __device__ void reset_step_counters(SimDev& s) {
   s.d.vmax2_acc = 0;
 }
 
-__device__ void set_prof_due(SimDev& s) {
-  s.d.prof_due = (s.profile_bins > 0 && s.profile_every > 0 &&
-                  (s.d.step + 1) % (uint64_t)s.profile_every == 0) ? 1u : 0u;
+// x % m; the 64-bit remainder (440 cycles of dependent operations) only past 2^32
+__device__ __forceinline__ uint32_t mod_u32(uint64_t x, uint32_t m) {
+  return (x >> 32) == 0 ? (uint32_t)x % m : (uint32_t)(x % (uint64_t)m);
 }
 
-// one warp per simulation: lane 0 keeps the books, the warp builds the next grid
+// does the step that starts now (absolute index `step`) end with a profile?
+__device__ __forceinline__ uint32_t prof_due_at(const SimDev& s, uint64_t step) {
+  return (s.profile_bins > 0 && s.profile_every > 0 &&
+          mod_u32(step + 1, (uint32_t)s.profile_every) == 0) ? 1u : 0u;
+}
+
+// clears the slot of the profile that the step will write (the warp's lanes together)
+__device__ __forceinline__ void clear_profile(SimDev& s, uint32_t count, uint32_t lane) {
+  long long* out = s.prof_acc + (size_t)(count % s.prof_cap) * s.profile_bins * kProfQ;
+  for (int i = (int)lane; i < s.profile_bins * kProfQ; i += 32) out[i] = 0;
+}
+
+// One warp per simulation: lane 0 keeps the books, the warp builds the next grid.  The
+// kernel is one chain of dependent operations, so everything the record needs is read
+// before the first store (the compiler may not move a load of the descriptor across one).
 __global__ void k_finalize(Batch B) {
   const uint32_t lane = threadIdx.x & 31u;
   const int nwarps = (int)(gridDim.x * blockDim.x / 32u);
   for (int k = (int)((blockIdx.x * blockDim.x + threadIdx.x) / 32u); k < B.nsims; k += nwarps) {
     SimDev& s = *B.sims[k];
     if (!sim_active(s)) continue;
+    const uint64_t step = s.d.step, hist_count = s.d.hist_count, steps_left = s.d.steps_left;
+    const uint32_t hist_cap = s.hist_cap, was_due = s.d.prof_due, prof_cap = s.prof_cap;
+    const uint32_t n_raw = s.d.n_raw, parity = s.d.parity;
+    const uint32_t prof_count = s.d.prof_count + was_due;  // snapshots, this step's included
+    const float vmax2 = __uint_as_float(s.d.vmax2_acc);
+    const uint32_t due = prof_due_at(s, step + 1);
     if (lane == 0) {
       kmc_step_counts rec;
-      rec.step = s.d.step;
+      rec.step = step;
       uint32_t coll = 0;
       for (int r = 0; r < 4; ++r) {
         rec.round_pairs[r] = s.d.round_pairs[r];
-        coll += s.d.round_pairs[r];
+        coll += rec.round_pairs[r];
       }
       rec.collisions = coll;
       rec.edges = s.d.n_edges;
-      rec.survivors = s.d.n_raw;
+      rec.survivors = n_raw;
       rec.cells = s.d.grid.nkeys;
       rec.pair_tests = s.d.pair_tests;
       rec.fast_tests = s.d.fast_tests;
       rec.absorbed = s.d.n_absorbed;
-      rec.live = live_count(s) - s.d.n_absorbed;  // this step's grid, before the next one
-      s.hist[s.d.hist_count % s.hist_cap] = rec;
-      s.d.hist_count += 1;
-      if (s.d.prof_due) {
-        s.prof_step[s.d.prof_count % s.prof_cap] = s.d.step;
-        s.d.prof_count += 1;
+      rec.live = live_count(s) - rec.absorbed;  // this step's grid, before the next one
+      const uint32_t have = s.split_ok ? 1u : 0u;
+      s.hist[mod_u32(hist_count, hist_cap)] = rec;
+      s.d.hist_count = hist_count + 1;
+      if (was_due) {
+        s.prof_step[(prof_count - 1u) % prof_cap] = step;
+        s.d.prof_count = prof_count;
       }
-      s.d.last_raw = s.d.n_raw;
-      s.d.have_counts = s.split_ok ? 1u : 0u;
-      s.d.parity ^= 1u;
-      s.d.step += 1;
-      s.d.steps_left -= 1;
-      s.d.vmax2 = __uint_as_float(s.d.vmax2_acc);
+      s.d.last_raw = n_raw;
+      s.d.have_counts = have;
+      s.d.parity = parity ^ 1u;
+      s.d.step = step + 1;
+      s.d.steps_left = steps_left - 1;
+      s.d.vmax2 = vmax2;
+      s.d.prof_due = due;
     }
     __syncwarp();
-    compute_grid(s, s.d.vmax2, s.d.step, lane);
+    compute_grid(s, vmax2, step + 1, lane);
     __syncwarp();
-    if (lane == 0) {
-      reset_step_counters(s);
-      set_prof_due(s);
-    }
-    __syncwarp();
-    if (s.d.prof_due) {
-      long long* out = s.prof_acc + (size_t)(s.d.prof_count % s.prof_cap) * s.profile_bins * kProfQ;
-      for (int i = (int)lane; i < s.profile_bins * kProfQ; i += 32) out[i] = 0;
-    }
+    if (lane == 0) reset_step_counters(s);
+    if (due) clear_profile(s, prof_count, lane);
     __syncwarp();
   }
 }
@@ -312,10 +327,13 @@ __global__ void __launch_bounds__(kTile) k_vmax(Batch B) {
 
 // the trial thresholds of the speed split from the state's bound of max |v|^2
 __global__ void k_init_thresholds(Batch B) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < B.nsims; k += gridDim.x * blockDim.x) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const int nwarps = (int)(gridDim.x * blockDim.x / 32u);
+  for (int k = (int)((blockIdx.x * blockDim.x + threadIdx.x) / 32u); k < B.nsims; k += nwarps) {
     SimDev& s = *B.sims[k];
-    s.d.vmax2 = __uint_as_float(s.d.vmax2_acc);
-    set_split_thresholds(s, s.d.vmax2);
+    const float v2 = __uint_as_float(s.d.vmax2_acc);
+    if (lane == 0) s.d.vmax2 = v2;
+    set_split_thresholds(s, v2, lane);
   }
 }
 
@@ -357,15 +375,12 @@ __global__ void k_init_grid(Batch B) {
     __syncwarp();
     compute_grid(s, s.d.vmax2, s.d.step, lane);
     __syncwarp();
+    const uint32_t due = prof_due_at(s, s.d.step);
     if (lane == 0) {
       reset_step_counters(s);
-      set_prof_due(s);
+      s.d.prof_due = due;
     }
-    __syncwarp();
-    if (s.d.prof_due && s.prof_acc) {
-      long long* out = s.prof_acc + (size_t)(s.d.prof_count % s.prof_cap) * s.profile_bins * kProfQ;
-      for (int i = (int)lane; i < s.profile_bins * kProfQ; i += 32) out[i] = 0;
-    }
+    if (due && s.prof_acc) clear_profile(s, s.d.prof_count, lane);
     __syncwarp();
   }
 }
@@ -378,7 +393,7 @@ int launch_init_grid(const LaunchPlan& L, cudaStream_t st) {
   k_zero_vmax<<<1, 256, 0, st>>>(L.b);
   if (L.absorb) k_vmax<true><<<L.ptiles, kTile, 0, st>>>(L.b);
   else k_vmax<false><<<L.ptiles, kTile, 0, st>>>(L.b);
-  k_init_thresholds<<<(L.b.nsims + 255) / 256, 256, 0, st>>>(L.b);
+  k_init_thresholds<<<(L.b.nsims + 7) / 8, 256, 0, st>>>(L.b);
   if (L.absorb) k_split_count<true><<<L.ptiles, kTile, 0, st>>>(L.b);
   else k_split_count<false><<<L.ptiles, kTile, 0, st>>>(L.b);
   k_init_grid<<<(L.b.nsims + 7) / 8, 256, 0, st>>>(L.b);
