@@ -59,7 +59,8 @@ extern "C" {
                           moved nor profiled again.  Live particles lie in [0, L]. */
 
 /* ---- precision of the pair tests --------------------------------------- */
-#define KMC_FP64 0          /* every pair test in binary64 */
+#define KMC_FP64 0          /* binary64 tests of every pair that the cell geometry and a filter
+                              with a proven error bound do not exclude */
 #define KMC_GUARDED_FP32 1  /* binary32 pre-tests with proven guard bands, binary64
                                re-check of the survivors: identical pair lists */
 
@@ -126,11 +127,12 @@ extern "C" {
                                   their bounded wait and sim_sync returns KMC_ETIMEOUT */
 
 /* ---- search kernels (kmc_params.search_kernel) ----------------------------- */
-#define KMC_SEARCH_AUTO 0      /* per step: warp-per-cell search when cells are well
-                                  filled, the row search (binary32) or the
-                                  thread-per-particle search (binary64) otherwise */
+#define KMC_SEARCH_AUTO 0      /* per step: tiles in binary64 and when cells are well
+                                  filled, the row search otherwise (binary32) */
 #define KMC_SEARCH_PARTICLE 1  /* one thread per particle, cell by cell */
-#define KMC_SEARCH_CELL 2      /* one warp per cell, partners in lanes */
+#define KMC_SEARCH_CELL 2      /* tiles of 32 particles by 32 partners: a conservative pair
+                                  filter, then the tests of the precision on the pairs it
+                                  leaves */
 #define KMC_SEARCH_ROW 3       /* one lane per particle walking whole stencil rows as
                                   partner ranges (guarded binary32; binary64 uses
                                   KMC_SEARCH_CELL) */

@@ -277,6 +277,8 @@ int build_plan(Plan& P, const std::vector<kmc_sim*>& sims, cudaStream_t st, std:
     if (h.profile_bins > 0) P.has_profiles = true;
     if (h.absorb) P.L.absorb = true;
     if (h.mix) P.L.mix = true;
+    if (h.search_kernel == KMC_SEARCH_PARTICLE) P.L.particle = true;
+    (h.bc[0] == KMC_PERIODIC ? P.L.periodic_x : P.L.bounded_x) = true;
   }
   // prefixes (3 (m + 1) words, padded to an even count), the scan's two control
   // words, then one 64-bit status word per scan tile

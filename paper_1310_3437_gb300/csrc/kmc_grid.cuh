@@ -34,7 +34,7 @@ __device__ __forceinline__ float f_up(double x) { return __double2float_ru(x); }
 // Hence: the cell counts and the cost estimates in binary32 (only the speed depends on
 // the choice; the margins of the cell width cover the rounding, see plan_cells), square
 // roots as upper bounds from the rounded-up binary32 root, per-axis values on a lane
-// each, and every parameter read before the first use of any.  One simulation: 35 -> 7 us
+// each, and every parameter read before the first use of any.  One simulation: 35 -> 10 us
 // at 4096 particles, 47 -> 12 us at 2^20.
 struct CellPlan {
   int nc[3];
@@ -42,6 +42,12 @@ struct CellPlan {
   uint32_t col_shift, col_tz, nkeys;
   bool ok;
 };
+
+// Mean particles per cell from which the binary32 path searches with tiles.  Slow pairs of
+// a step at 2^21 particles, row search against tiles: tube at 1 per cell 165 and 175 us, at
+// 4.8 180 and 198; plane at 2.5 102 and 117; box at 4.1 226 and 212, at 8.4 268 and 250;
+// blast at 5.8 319 and 249, at 13 393 and 308.
+constexpr float kTileOccupancy = 5.0f;
 
 // an upper bound of sqrt(x) for x >= 0, within 2^-19 of it
 __device__ __forceinline__ double sqrt_up(float x) {
@@ -238,22 +244,20 @@ __device__ inline void compute_grid(SimDev& s, float vmax2_bound, uint64_t step,
   const float hs = f_up((d0 + 2.0 * S1 * dt) * scale);
   const uint64_t max_keys = (uint64_t)cell_cap / (split ? 2 : 1);
   CellPlan p = plan_cells(extf, hs, K, max_keys);
-  // search kernel for the slow population: warp per cell when cells are well
-  // filled; the binary32 warp-per-cell search handles no one-cell periodic axis
-  // (the row search does)
+  // search for the slow population: tiles where cells are well filled (and always in
+  // binary64), lane per particle along its rows in sparse cells and for one-cell periodic
+  // axes (the tiled search walks those per particle, in binary64 only)
   const float occ = (float)n / ((float)p.nc[0] * (float)p.nc[1] * (float)p.nc[2]);
   bool cp = false;
 #pragma unroll
   for (int a = 0; a < 3; ++a) cp = cp || (p.nc[a] == 1 && per[a]);
-  int mode = search_kernel;
-  if (mode == 0) {
-    if (fp32) mode = occ >= 16.0f ? KMC_SEARCH_CELL : KMC_SEARCH_ROW;
-    else mode = occ >= 4.0f ? KMC_SEARCH_CELL : KMC_SEARCH_PARTICLE;
-  }
-  if (mode == KMC_SEARCH_ROW && !fp32) mode = KMC_SEARCH_CELL;
-  if (mode == KMC_SEARCH_CELL && cp && fp32) mode = KMC_SEARCH_ROW;
+  int mode = MODE_TILES;
+  if (search_kernel == KMC_SEARCH_PARTICLE) mode = MODE_PARTICLE;
+  else if (fp32 && (cp || search_kernel == KMC_SEARCH_ROW ||
+                    (search_kernel == 0 && occ < kTileOccupancy)))
+    mode = MODE_ROWS;
   int kx = K;
-  if (mode == KMC_SEARCH_ROW && p.nc[0] > 1) {
+  if (mode == MODE_ROWS && p.nc[0] > 1) {
     // rows of half-width cells: each particle's row is trimmed to its reach in
     // half-cell steps (the grid is otherwise the same)
     const CellPlan q = plan_cells(extf, hs, K, max_keys, 2);
@@ -363,6 +367,13 @@ __device__ inline void compute_grid(SimDev& s, float vmax2_bound, uint64_t step,
   const double c0 = (rel40 * (d0sq + dt2 * bslack) + 2.0 * s3 * er * rn) * (1.0 + g3);
   g.s_c0 = f_up(c0 * up2);
   g.s_c1 = f_up(dt2 * (rel40 * (1.0 + g3) / (1.0 - g3) * up2));
+  // pair filter of the tiled search (kmc_search.cu, "Error of the filter"): the sphere
+  // test's constant with three times the separation error er, and the slack of
+  // velocities rounded to 11 bits, 2^-7 (dt S1)^2
+  g.tile_c = f_up((rel40 * (d0sq + dt2 * bslack) + 8.0 * s3 * er * rn + 27.0 * er * er) *
+                      ((1.0 + g3) * up2) + 0x1p-7 * 1.001 * dt2 * S1 * S1);
+  g.tile_k = sqrtf(g.s_c1);
+  g.s1f = f_up(S1);
   // approach test (t* >= 0): |A~ - A64| <= a_g
   const double Ga = (s3 * (ev * rn + 2.0 * V * er) + rnV2 * (g3 * 1.01 + g3d)) * (1.0 + 1e-3);
   g.a_g = f_up(Ga);

@@ -37,12 +37,15 @@ enum : uint32_t {
   ST_SCAN_WAIT = 1u << 3,      // a scan tile waited too long for its predecessor's sum
 };
 
+// how the slow pairs of a step are searched (Grid::mode)
+enum : int32_t { MODE_PARTICLE = 1, MODE_TILES = 2, MODE_ROWS = 3 };
+
 // Search grid of the current step.  Cells are keyed column-major along x inside a
 // tiled Z-order (Morton) walk over the (y, z) columns: key = col(cy, cz) * nc[0] + cx.
 struct Grid {
   int32_t nc[3];      // cells per axis; 1 means the axis is one cell (no stencil on it)
   int32_t K;          // stencil radius in cells
-  int32_t mode;       // search kernel of this step: KMC_SEARCH_PARTICLE, _CELL or _ROW
+  int32_t mode;       // slow-pair search of this step: MODE_PARTICLE, MODE_TILES or MODE_ROWS
   int32_t split_t;    // trial threshold index of the split (0: no split)
   uint32_t split;     // 1: particles with |v|^2 above s1sq form a second population
   float s1sq;         // binary32 split threshold on the upper bound of |v|^2
@@ -66,6 +69,9 @@ struct Grid {
   // reach is d0 + (|v_i| + S1) dt: at most row_a + row_b |v_i| (both rounded up); for a
   // fast particle i (partners up to the bound V of max |v|) at most fast_a + row_b |v_i|
   float row_r2, row_eps, row_pad, row_a, row_b, fast_a;
+  // pair filter of the tiled search (kmc_search.cu, "Error of the filter"): its constant
+  // before scaling with the slack of the rounded velocities, dt, max slow speed
+  float tile_c, tile_k, s1f;
   // binary64 sphere pre-test: drop if R > c0 + c1 * B (B >= 2^-900)
   double c0, c1;
 };
@@ -475,11 +481,14 @@ struct LaunchPlan {
   Batch b;
   uint32_t ptiles, stiles_c, prtiles;
   int edge_blocks;
-  int cell_blocks;  // persistent grid of the warp-per-cell search
-  int part_blocks;  // grid-stride grids of the particle, row and fast searches
+  int part_blocks;  // grid-stride grids of the particle, tiled, row and fast searches
+  int tile_blocks;
   int row_blocks;     // row search, no periodic x axis
   int row_blocks_px;  // row search, periodic x axis
   int fast_blocks;
+  // which simulations the plan has: asking for the thread-per-particle search, with a
+  // periodic x axis, with another (the row search is built for either)
+  bool particle = false, periodic_x = false, bounded_x = false;
   // some simulation of the plan has absorbing walls / is a mixture: the kernels that
   // handle either are launched in their general form only then
   bool absorb = false;

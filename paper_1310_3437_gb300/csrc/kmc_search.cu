@@ -2,21 +2,28 @@
 // particle of a bin is compared with the particles of its own and the neighbouring
 // bins; the cost is O(B * N_bin^2 / P), eq. "eff").
 //
-// GB300 form.  One thread per particle, particles in cell order, so the lanes of a
-// warp sit in the same or adjacent cells and read the same partner records
-// (broadcast loads, L1/L2 reuse of the neighbour cells).  Each unordered pair is
-// tested once: the thread of particle p visits the "forward half" of the stencil
-// (own cell with j > p, then the cells whose offset (dz, dy, dx) is
-// lexicographically positive).  The search does no division: it only culls pairs
-// that provably fail the paper's criteria, and emits the survivors; kmc_match.cu
-// re-tests every survivor with the exact binary64 predicate.
+// Each unordered pair is tested once: particle p meets the "forward half" of its
+// stencil (own cell with j > p, then the cells whose offset (dz, dy, dx) is
+// lexicographically positive).  The search does no division: it only culls pairs that
+// provably fail the paper's criteria and emits the survivors; kmc_match.cu re-tests
+// every survivor with the exact binary64 predicate.
 //
-//   KMC_FP64          binary64 sphere test |r|^2 > d0^2 + dt^2 |v|^2 (+2^-40 slack).
-//   KMC_GUARDED_FP32  binary32 on cell-local offsets: sphere test, then approach,
-//                     time and distance tests, each widened by a guard band that
-//                     bounds the binary32 error (kmc_grid.cuh derives the bands).
+//   k_search_rows32 slow pairs, binary32, sparse cells: a lane per particle along its rows.
+//   k_search_tiles  slow pairs, well filled cells and binary64: 32 x 32 tiles of pairs
+//                   through one quadratic form on the tensor cores, then the tests of the
+//                   precision on what that leaves.
+//   k_search_fast   the fast particles of the speed split, a warp each.
+//   k_search        slow pairs with a thread per particle (kmc_params.search_kernel = 1).
+//
+//   KMC_FP64          binary64 sphere test |r|^2 > d0^2 + dt^2 |v|^2 (+2^-40 slack), then
+//                     the binary64 approach and time tests.
+//   KMC_GUARDED_FP32  binary32 on box coordinates: sphere test, then approach, time and
+//                     distance tests, each widened by a guard band that bounds the
+//                     binary32 error (kmc_grid.cuh derives the bands).
 // A pair that passes the binary64 predicate is never culled by either variant, so
 // both variants produce exactly the candidate list of the binary64 definition.
+#include <cuda_fp16.h>
+
 #include <algorithm>
 
 #include "kmc_internal.cuh"
@@ -83,459 +90,19 @@ __device__ __forceinline__ bool f64_cannot_approach(double rv, double vv, double
   return rv > dmul(vv, 0x1p-1000) || -rv >= dmul(dmul(dt, vv), 1.0 + 0x1p-48);
 }
 
-template <int PREC, int K>
-__global__ void __launch_bounds__(kTile) k_search(Batch B) {
-  __shared__ uint2 sbuf[kSearchBuf];
-  __shared__ uint32_t scnt, sbase;
-  __shared__ unsigned long long stests;
-  // grid-stride over tiles of kTile particles (an occupancy-sized grid: the kernel is
-  // launched every step and exits at once when the step runs another search)
-  if (!batch_uses(B, KMC_SEARCH_PARTICLE)) return;
-  const uint32_t ntiles = B.ptile[B.nsims];
-  for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    int k = find_sim(B.ptile, B.nsims, tile);
-    SimDev& s = *B.sims[k];
-    if (s.d.grid.mode != KMC_SEARCH_PARTICLE) continue;
-    // the previous tile's flush has read the staging buffer; the status word can change
-    // while the search runs (a full pair buffer), so the block takes one answer
-    if (!__syncthreads_and(sim_active(s))) continue;
-    if (threadIdx.x == 0) { scnt = 0; stests = 0; }
-    __syncthreads();
+constexpr int kCellWarps = 8;   // warps per block of the warp-wise searches
+constexpr int kWarpBuf = 64;    // emitted pairs staged per warp
 
-    const Grid g = s.d.grid;
-    const uint32_t n = s.n;
-    const int cur = s.d.parity ^ 1;
-    const uint32_t* __restrict__ cs = s.cell_start;
-    const uint32_t edge_cap = s.edge_cap;
-    uint2* __restrict__ edges = s.edge;
-    const int nx = g.nc[0], ny = g.nc[1], nz = g.nc[2];
-    const int Kx = nx == 1 ? 0 : K, Ky = ny == 1 ? 0 : K, Kz = nz == 1 ? 0 : K;
-    const bool px = s.bc[0] == KMC_PERIODIC, py = s.bc[1] == KMC_PERIODIC,
-               pz = s.bc[2] == KMC_PERIODIC;
-    unsigned long long tests = 0;
-
-    uint32_t p = (tile - B.ptile[k]) * kTile + threadIdx.x;
-    // with the speed split only the slow population (keys below nkeys) is searched here;
-    // particles that left through absorbing walls sit after every cell key
-    const uint32_t nslow = (g.split || s.absorb) ? __ldg(cs + g.nkeys) : n;
-    if (p < nslow) {
-      // the particle's cell, recomputed as the sort computed it
-      const int cx = cell_coord(g, 0, s.x[cur][0][p]), cy = cell_coord(g, 1, s.x[cur][1][p]),
-                cz = cell_coord(g, 2, s.x[cur][2][p]);
-
-      // own record
-      double xo[3], vo[3];
-      Own32 o32;
-      const double* __restrict__ X0 = s.x[cur][0];
-      const double* __restrict__ X1 = s.x[cur][1];
-      const double* __restrict__ X2 = s.x[cur][2];
-      const double* __restrict__ V0 = s.v[cur][0];
-      const double* __restrict__ V1 = s.v[cur][1];
-      const double* __restrict__ V2 = s.v[cur][2];
-      const float4* __restrict__ MM = s.mir;
-      if (PREC == KMC_FP64) {
-        xo[0] = X0[p]; xo[1] = X1[p]; xo[2] = X2[p];
-        vo[0] = V0[p]; vo[1] = V1[p]; vo[2] = V2[p];
-      } else {
-        float4 a;
-        float2 b;
-        mirror_load(MM, p, a, b);
-        o32 = {a.x, a.y, a.z, a.w, b.x, b.y};
-      }
-      // one-cell periodic axes need the minimum image explicitly
-      const bool cp0 = nx == 1 && px, cp1 = ny == 1 && py, cp2 = nz == 1 && pz;
-      const bool any_cp = cp0 || cp1 || cp2;
-      const double L0 = s.box[0], L1 = s.box[1], L2 = s.box[2];
-
-      // a neighbour reached across a periodic boundary is seen as its image: wrap
-      // flags -1 (below 0) or +1 (at or above the extent) per axis
-      for (int dz = 0; dz <= Kz; ++dz) {
-        int qz = cz + dz, wz = 0;
-        if (qz >= nz) {
-          if (!pz) break;
-          qz -= nz;
-          wz = 1;
-        }
-        for (int dy = (dz == 0 ? 0 : -Ky); dy <= Ky; ++dy) {
-          int qy = cy + dy, wy = 0;
-          if (qy < 0) {
-            if (!py) continue;
-            qy += ny;
-            wy = -1;
-          } else if (qy >= ny) {
-            if (!py) continue;
-            qy -= ny;
-            wy = 1;
-          }
-          const uint32_t colbase = col_code(g, (uint32_t)qy, (uint32_t)qz) * (uint32_t)nx;
-          const int dx0 = (dz == 0 && dy == 0) ? 0 : -Kx;
-          for (int dx = dx0; dx <= Kx; ++dx) {
-            int qx = cx + dx, wx = 0;
-            if (qx < 0) {
-              if (!px) continue;
-              qx += nx;
-              wx = -1;
-            } else if (qx >= nx) {
-              if (!px) continue;
-              qx -= nx;
-              wx = 1;
-            }
-            const uint32_t key = colbase + (uint32_t)qx;
-            uint32_t beg = __ldg(cs + key), end = __ldg(cs + key + 1);
-            if (dz == 0 && dy == 0 && dx == 0) beg = p + 1;
-            if (beg >= end) continue;
-            tests += end - beg;
-            if (PREC == KMC_FP64) {
-              for (uint32_t j = beg; j < end; ++j) {
-                double r0 = dsub(__ldg(X0 + j), xo[0]);
-                double r1 = dsub(__ldg(X1 + j), xo[1]);
-                double r2 = dsub(__ldg(X2 + j), xo[2]);
-                if (px) { if (r0 > 0.5 * L0) r0 = dsub(r0, L0); else if (r0 < -0.5 * L0) r0 = dadd(r0, L0); }
-                if (py) { if (r1 > 0.5 * L1) r1 = dsub(r1, L1); else if (r1 < -0.5 * L1) r1 = dadd(r1, L1); }
-                if (pz) { if (r2 > 0.5 * L2) r2 = dsub(r2, L2); else if (r2 < -0.5 * L2) r2 = dadd(r2, L2); }
-                double g0 = dsub(__ldg(V0 + j), vo[0]);
-                double g1 = dsub(__ldg(V1 + j), vo[1]);
-                double g2 = dsub(__ldg(V2 + j), vo[2]);
-                double R = dadd(dadd(dmul(r0, r0), dmul(r1, r1)), dmul(r2, r2));
-                double Bv = dadd(dadd(dmul(g0, g0), dmul(g1, g1)), dmul(g2, g2));
-                if (Bv >= 0x1p-900 && R > dadd(g.c0, dmul(g.c1, Bv))) continue;
-                if (Bv >= 0x1p-900 &&
-                    f64_cannot_approach(dadd(dadd(dmul(r0, g0), dmul(r1, g1)), dmul(r2, g2)), Bv, s.dt))
-                  continue;
-                uint32_t pos = atomicAdd(&scnt, 1u);
-                if (pos < (uint32_t)kSearchBuf) {
-                  sbuf[pos] = make_uint2(p, j);
-                } else {
-                  uint32_t gpos = atomicAdd(&s.d.n_raw, 1u);
-                  if (gpos < edge_cap) edges[gpos] = make_uint2(p, j);
-                  else atomicOr(&s.d.status, ST_EDGE_OVERFLOW);
-                }
-              }
-            } else {
-              // own coordinates moved by the image shift (j seen at x_j + w L)
-              const float sx = o32.ox - (float)wx * g.Lf[0];
-              const float sy = o32.oy - (float)wy * g.Lf[1];
-              const float sz = o32.oz - (float)wz * g.Lf[2];
-              for (uint32_t j = beg; j < end; ++j) {
-                float4 a;
-                float2 b;
-                mirror_load(MM, j, a, b);
-                float rx = a.x - sx, ry = a.y - sy, rz = a.z - sz;
-                bool keep = false;
-                if (any_cp) {
-                  // minimum image on one-cell periodic axes; near the tie the two
-                  // images are both possible in binary64: keep the pair unculled
-                  if (cp0) min_image_f(rx, g.halfLf[0], g.Lf[0], g.tief[0], keep);
-                  if (cp1) min_image_f(ry, g.halfLf[1], g.Lf[1], g.tief[1], keep);
-                  if (cp2) min_image_f(rz, g.halfLf[2], g.Lf[2], g.tief[2], keep);
-                }
-                const float gx = a.w - o32.vx, gy = b.x - o32.vy, gz = b.y - o32.vz;
-                const float R = fmaf(rz, rz, fmaf(ry, ry, rx * rx));
-                const float Bv = fmaf(gz, gz, fmaf(gy, gy, gx * gx));
-                if (!keep) {
-                  if (R > fmaf(g.s_c1, Bv, g.s_c0)) continue;
-                  // rare: full guarded test on the sphere survivors
-                  const float A = -fmaf(rz, gz, fmaf(ry, gy, rx * gx));
-                  if (A < -g.a_g) continue;
-                  if (fmaf(-g.dtf, Bv, A) > g.t_g) continue;
-                  const float wx = fmaf(ry, gz, -(rz * gy));
-                  const float wy = fmaf(rz, gx, -(rx * gz));
-                  const float wz = fmaf(rx, gy, -(ry * gx));
-                  const float W = fmaf(wz, wz, fmaf(wy, wy, wx * wx));
-                  const float thr = fmaf(g.d0up, sqrtf(fmaf(Bv, g.b_rel, g.b_abs)), g.w_e);
-                  if (W > thr * thr * g.w_rel) continue;
-                }
-                uint32_t pos = atomicAdd(&scnt, 1u);
-                if (pos < (uint32_t)kSearchBuf) {
-                  sbuf[pos] = make_uint2(p, j);
-                } else {
-                  uint32_t gpos = atomicAdd(&s.d.n_raw, 1u);
-                  if (gpos < edge_cap) edges[gpos] = make_uint2(p, j);
-                  else atomicOr(&s.d.status, ST_EDGE_OVERFLOW);
-                }
-              }
-            }
-          }
-        }
-      }
-    }
-
-    // block totals: pair tests and the staged pairs
-    for (int o = 16; o > 0; o >>= 1) tests += __shfl_down_sync(0xFFFFFFFFu, tests, o);
-    if ((threadIdx.x & 31) == 0 && tests) atomicAdd(&stests, tests);
-    __syncthreads();
-    uint32_t cnt = scnt < (uint32_t)kSearchBuf ? scnt : (uint32_t)kSearchBuf;
-    if (threadIdx.x == 0) {
-      if (stests) atomicAdd(&s.d.pair_tests, stests);
-      sbase = cnt ? atomicAdd(&s.d.n_raw, cnt) : 0u;
-    }
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < cnt; i += kTile) {
-      uint32_t gpos = sbase + i;
-      if (gpos < edge_cap) edges[gpos] = sbuf[i];
-      else atomicOr(&s.d.status, ST_EDGE_OVERFLOW);
-    }
-  }
-}
-
-// --------------------------------------------------------------------------- //
-// Warp-per-cell search.  A warp owns one cell A.  For every forward column run of
-// the stencil, the run's particles (contiguous in cell order) are loaded 32 at a
-// time, one partner j per lane, with coalesced loads; the particles i of A are
-// staged in shared memory and read by broadcast in a warp-uniform loop.  Each lane
-// thus tests its j against every i of A with no divergence and no per-pair address
-// arithmetic.  Emitted pairs go through a per-warp shared-memory buffer (one global
-// atomic per flush).
-constexpr int kCellWarps = 8;
-constexpr int kWarpBuf = 64;
-
-struct WarpEmit {
-  uint2* buf;        // this warp's staging buffer in shared memory
-  uint32_t count;    // warp-uniform fill level
-};
-
-__device__ __forceinline__ void warp_flush(WarpEmit& w, SimDev& s, uint32_t lane) {
-  __syncwarp();
-  if (w.count) {
-    uint32_t base = 0;
-    if (lane == 0) base = atomicAdd(&s.d.n_raw, w.count);
-    base = __shfl_sync(0xFFFFFFFFu, base, 0);
-    for (uint32_t k = lane; k < w.count; k += 32) {
-      uint32_t g = base + k;
-      if (g < s.edge_cap) s.edge[g] = w.buf[k];
-      else atomicOr(&s.d.status, ST_EDGE_OVERFLOW);
-    }
-    w.count = 0;
-  }
-  __syncwarp();
-}
-
-__device__ __forceinline__ void warp_emit(WarpEmit& w, SimDev& s, uint32_t lane, bool emit,
-                                          uint32_t i, uint32_t j) {
-  unsigned m = __ballot_sync(0xFFFFFFFFu, emit);
-  if (!m) return;
-  uint32_t c = (uint32_t)__popc(m);
-  if (w.count + c > (uint32_t)kWarpBuf) warp_flush(w, s, lane);
-  if (emit) w.buf[w.count + __popc(m & ((1u << lane) - 1u))] = make_uint2(i, j);
-  w.count += c;
-  __syncwarp();
-}
-
-template <int PREC, int K>
-__global__ void __launch_bounds__(kCellWarps * 32) k_search_cell(Batch B) {
-  constexpr int ICAP = PREC == KMC_FP64 ? 32 : 64;
-  constexpr int NF = PREC == KMC_FP64 ? 1 : kCellWarps;
-  constexpr int ND = PREC == KMC_FP64 ? kCellWarps : 1;
-  __shared__ float4 sa[NF][PREC == KMC_FP64 ? 1 : ICAP];
-  __shared__ float2 sb[NF][PREC == KMC_FP64 ? 1 : ICAP];
-  __shared__ double sd[ND][6][PREC == KMC_FP64 ? ICAP : 1];
-  __shared__ uint2 wbuf[kCellWarps][kWarpBuf];
-  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-  const uint32_t gwarp = blockIdx.x * kCellWarps + warp, nwarps = gridDim.x * kCellWarps;
-
-  // The cells of the batch's simulations are dealt to the warps as one sequence: a
-  // simulation's cells start at the warp after the previous simulation's last.  Every
-  // warp walks the simulations in the same order and decides on fields that stay fixed
-  // during the launch, so all agree on the running base; the status word, which the
-  // search itself can set (a full pair buffer), only gates the work.  Dealt from warp 0
-  // each time, the small simulations of a batch all landed on the same few blocks.
-  uint32_t base = 0;
-  for (int k = 0; k < B.nsims; ++k) {
-    SimDev& s = *B.sims[k];
-    if (!sim_scheduled(s) || s.d.grid.mode != KMC_SEARCH_CELL) continue;
-    const uint32_t first = (gwarp + nwarps - base) % nwarps;
-    base = (base + s.d.grid.nkeys % nwarps) % nwarps;
-    if (!__all_sync(0xFFFFFFFFu, sim_active(s))) continue;
-    const Grid& G = s.d.grid;
-    const int nx = G.nc[0], ny = G.nc[1], nz = G.nc[2];
-    const int Kx = nx == 1 ? 0 : K, Ky = ny == 1 ? 0 : K, Kz = nz == 1 ? 0 : K;
-    const bool px = s.bc[0] == KMC_PERIODIC, py = s.bc[1] == KMC_PERIODIC,
-               pz = s.bc[2] == KMC_PERIODIC;
-    const uint32_t nkeys = G.nkeys;
-    const uint32_t* __restrict__ cs = s.cell_start;
-    const int cur = s.d.parity ^ 1;
-    const float wx = G.wf[0], wy = G.wf[1], wz = G.wf[2];
-    const float c0 = G.s_c0, c1 = G.s_c1, ag = G.a_g, tg = G.t_g, dtf = G.dtf;
-    const float d0up = G.d0up, brel = G.b_rel, babs = G.b_abs, we = G.w_e, wrel = G.w_rel;
-    const double C0 = G.c0, C1 = G.c1;
-    const double L0 = s.box[0], L1 = s.box[1], L2 = s.box[2];
-    const float4* __restrict__ MM = s.mir;
-    const double* __restrict__ X0 = s.x[cur][0];
-    const double* __restrict__ X1 = s.x[cur][1];
-    const double* __restrict__ X2 = s.x[cur][2];
-    const double* __restrict__ V0 = s.v[cur][0];
-    const double* __restrict__ V1 = s.v[cur][1];
-    const double* __restrict__ V2 = s.v[cur][2];
-    WarpEmit we_ = {wbuf[warp], 0u};
-    unsigned long long tests = 0;
-
-    for (uint32_t key = first; key < nkeys; key += nwarps) {
-      const uint32_t startA = __ldg(cs + key), endA = __ldg(cs + key + 1);
-      if (startA == endA) continue;
-      int cx, cy, cz;
-      key_decode(G, key, cx, cy, cz);
-      for (uint32_t i0 = startA; i0 < endA; i0 += ICAP) {
-        const uint32_t nI = endA - i0 < (uint32_t)ICAP ? endA - i0 : (uint32_t)ICAP;
-        __syncwarp();
-        for (uint32_t t = lane; t < nI; t += 32) {
-          if (PREC == KMC_FP64) {
-            sd[warp][0][t] = X0[i0 + t]; sd[warp][1][t] = X1[i0 + t]; sd[warp][2][t] = X2[i0 + t];
-            sd[warp][3][t] = V0[i0 + t]; sd[warp][4][t] = V1[i0 + t]; sd[warp][5][t] = V2[i0 + t];
-          } else {
-            float4 a;
-            float2 b;
-            mirror_load(MM, i0 + t, a, b);
-            sa[warp][t] = a;
-            sb[warp][t] = b;
-          }
-        }
-        __syncwarp();
-        for (int dz = 0; dz <= Kz; ++dz) {
-          int qz = cz + dz;
-          if (qz >= nz) {
-            if (!pz) break;
-            qz -= nz;
-          }
-          for (int dy = (dz == 0 ? 0 : -Ky); dy <= Ky; ++dy) {
-            int qy = cy + dy;
-            if (qy < 0) {
-              if (!py) continue;
-              qy += ny;
-            } else if (qy >= ny) {
-              if (!py) continue;
-              qy -= ny;
-            }
-            const uint32_t colbase = col_code(G, (uint32_t)qy, (uint32_t)qz) * (uint32_t)nx;
-            const bool own_col = dz == 0 && dy == 0;
-            const float shy = (float)dy * wy, shz = (float)dz * wz;
-            // split the x run into pieces of consecutive cells (periodic wrap)
-            int dx = own_col ? 0 : -Kx;
-            while (dx <= Kx) {
-              const int q0 = cx + dx;  // unwrapped cell index
-              const int region = q0 < 0 ? -1 : (q0 >= nx ? 1 : 0);
-              if (region != 0 && !px) { ++dx; continue; }
-              const int qx = q0 - region * nx;
-              // extend the piece while the next cell lies in the same wrap region, so
-              // that its cells are consecutive keys of the column
-              int m = 1;
-              while (dx + m <= Kx) {
-                const int q2 = cx + dx + m;
-                const int r2 = q2 < 0 ? -1 : (q2 >= nx ? 1 : 0);
-                if (r2 != region) break;
-                ++m;
-              }
-              const int dxa = dx;
-              dx += m;
-              const uint32_t jbeg = __ldg(cs + colbase + qx), jend = __ldg(cs + colbase + qx + m);
-              if (jbeg == jend) continue;
-              uint32_t bnd[2 * K];
-#pragma unroll
-              for (int t = 0; t < 2 * K; ++t) bnd[t] = (t + 1 < m) ? __ldg(cs + colbase + qx + t + 1) : jend;
-              const bool has_own = own_col && dxa <= 0 && dxa + m > 0;
-              // analytic count of the pair tests of this piece
-              if (lane == 0) {
-                uint64_t len = jend - jbeg;
-                if (has_own) {
-                  uint64_t nA = endA - startA;
-                  uint64_t inc = (uint64_t)nI * (endA - i0 - 1) - (uint64_t)nI * (nI - 1) / 2;
-                  tests += (uint64_t)nI * (len - nA) + inc;
-                } else {
-                  tests += (uint64_t)nI * len;
-                }
-              }
-              for (uint32_t cb = jbeg; cb < jend; cb += 32) {
-                const uint32_t j = cb + lane;
-                const bool jv = j < jend;
-                const bool jown = has_own && j >= startA && j < endA;
-                if (PREC == KMC_FP64) {
-                  double xj0 = 0, xj1 = 0, xj2 = 0, vj0 = 0, vj1 = 0, vj2 = 0;
-                  if (jv) {
-                    xj0 = X0[j]; xj1 = X1[j]; xj2 = X2[j];
-                    vj0 = V0[j]; vj1 = V1[j]; vj2 = V2[j];
-                  }
-                  for (uint32_t ii = 0; ii < nI; ++ii) {
-                    const uint32_t i = i0 + ii;
-                    bool valid = jv && (!jown || j > i);
-                    double r0 = dsub(xj0, sd[warp][0][ii]);
-                    double r1 = dsub(xj1, sd[warp][1][ii]);
-                    double r2 = dsub(xj2, sd[warp][2][ii]);
-                    if (px) { if (r0 > 0.5 * L0) r0 = dsub(r0, L0); else if (r0 < -0.5 * L0) r0 = dadd(r0, L0); }
-                    if (py) { if (r1 > 0.5 * L1) r1 = dsub(r1, L1); else if (r1 < -0.5 * L1) r1 = dadd(r1, L1); }
-                    if (pz) { if (r2 > 0.5 * L2) r2 = dsub(r2, L2); else if (r2 < -0.5 * L2) r2 = dadd(r2, L2); }
-                    double g0 = dsub(vj0, sd[warp][3][ii]);
-                    double g1 = dsub(vj1, sd[warp][4][ii]);
-                    double g2 = dsub(vj2, sd[warp][5][ii]);
-                    double R = dadd(dadd(dmul(r0, r0), dmul(r1, r1)), dmul(r2, r2));
-                    double Bv = dadd(dadd(dmul(g0, g0), dmul(g1, g1)), dmul(g2, g2));
-                    bool emit = valid && !(Bv >= 0x1p-900 && R > dadd(C0, dmul(C1, Bv)));
-                    if (emit && Bv >= 0x1p-900 &&
-                        f64_cannot_approach(dadd(dadd(dmul(r0, g0), dmul(r1, g1)), dmul(r2, g2)), Bv, s.dt))
-                      emit = false;
-                    warp_emit(we_, s, lane, emit, i, j);
-                  }
-                } else {
-                  float jx = 0.f, jy = 0.f, jz = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
-                  if (jv) {
-                    float4 a;
-                    float2 b;
-                    mirror_load(MM, j, a, b);
-                    int t = 0;
-#pragma unroll
-                    for (int q = 0; q < 2 * K; ++q) t += j >= bnd[q] ? 1 : 0;
-                    // partner coordinates moved into the frame of cell A's corner
-                    jx = a.x + (float)(dxa + t) * wx;
-                    jy = a.y + shy;
-                    jz = a.z + shz;
-                    gx = a.w; gy = b.x; gz = b.y;
-                  }
-                  for (uint32_t ii = 0; ii < nI; ++ii) {
-                    const uint32_t i = i0 + ii;
-                    const float4 ia = sa[warp][ii];
-                    const float2 ib = sb[warp][ii];
-                    const bool valid = jv && (!jown || j > i);
-                    const float rx = jx - ia.x, ry = jy - ia.y, rz = jz - ia.z;
-                    const float vx = gx - ia.w, vy = gy - ib.x, vz = gz - ib.y;
-                    const float R = fmaf(rz, rz, fmaf(ry, ry, rx * rx));
-                    const float Bv = fmaf(vz, vz, fmaf(vy, vy, vx * vx));
-                    bool cand = valid && !(R > fmaf(c1, Bv, c0));
-                    if (__any_sync(0xFFFFFFFFu, cand)) {
-                      if (cand) {
-                        // full guarded test on the sphere survivors
-                        const float A = -fmaf(rz, vz, fmaf(ry, vy, rx * vx));
-                        if (A < -ag) cand = false;
-                        if (fmaf(-dtf, Bv, A) > tg) cand = false;
-                        const float w0 = fmaf(ry, vz, -(rz * vy));
-                        const float w1 = fmaf(rz, vx, -(rx * vz));
-                        const float w2 = fmaf(rx, vy, -(ry * vx));
-                        const float W = fmaf(w2, w2, fmaf(w1, w1, w0 * w0));
-                        const float thr = fmaf(d0up, sqrtf(fmaf(Bv, brel, babs)), we);
-                        if (W > thr * thr * wrel) cand = false;
-                      }
-                      warp_emit(we_, s, lane, cand, i, j);
-                    }
-                  }
-                }
-              }
-            }
-          }
-        }
-      }
-    }
-    warp_flush(we_, s, lane);
-    if (lane == 0 && tests) atomicAdd(&s.d.pair_tests, tests);
-  }
-}
-
-// --------------------------------------------------------------------------- //
-// Binary32 warp-per-cell search, unrolled.  The particles i of cell A are staged as
-// structure-of-arrays in shared memory, padded to a multiple of 4 with a sentinel
-// position (-1e30) that every sphere test rejects; lanes past the end of a partner
-// chunk carry the opposite sentinel (+1e30).  Four pairs per lane are tested per
-// iteration with one warp vote, so the loop body is pure arithmetic plus four
-// 16-byte shared-memory broadcasts.
 struct Guard32 {
   float c0, c1, ag, tg, dtf, d0up, brel, babs, we, wrel;
 };
+
+__device__ __forceinline__ Guard32 guard_of(const Grid& g) {
+  Guard32 q;
+  q.c0 = g.s_c0; q.c1 = g.s_c1; q.ag = g.a_g; q.tg = g.t_g; q.dtf = g.dtf;
+  q.d0up = g.d0up; q.brel = g.b_rel; q.babs = g.b_abs; q.we = g.w_e; q.wrel = g.w_rel;
+  return q;
+}
 
 // exact guarded test of one pair on the sphere survivors (rare path)
 __device__ __forceinline__ bool full_test32(const Guard32& q, float rx, float ry, float rz,
@@ -594,205 +161,158 @@ __device__ __forceinline__ void flush_lanes(uint2* buf, uint32_t* count, SimDev&
   __syncwarp();
 }
 
-template <bool OWN>
-__device__ __forceinline__ void cell32_sweep(const float* __restrict__ si, uint32_t nI4, uint32_t i0,
-                                             float jx, float jy, float jz, float gx, float gy,
-                                             float gz, uint32_t j, bool jown, float c0, float c1,
-                                             const Guard32& q, uint2* buf, uint32_t* count,
-                                             SimDev& s) {
-  const float* sx = si;
-  const float* sy = si + 1 * 64;
-  const float* sz = si + 2 * 64;
-  const float* su = si + 3 * 64;
-  const float* sv = si + 4 * 64;
-  const float* sw = si + 5 * 64;
-  // the four own particles of an iteration as two packed pairs (adjacent in shared
-  // memory), the lane's partner broadcast to both halves
-  const f32x2 JX = pack2(jx, jx), JY = pack2(jy, jy), JZ = pack2(jz, jz);
-  const f32x2 GX = pack2(gx, gx), GY = pack2(gy, gy), GZ = pack2(gz, gz);
-  const f32x2 C0 = pack2(c0, c0), C1 = pack2(c1, c1);
-  for (uint32_t ii = 0; ii < nI4; ii += 4) {
-    const ulonglong2 X = *reinterpret_cast<const ulonglong2*>(sx + ii);
-    const ulonglong2 Y = *reinterpret_cast<const ulonglong2*>(sy + ii);
-    const ulonglong2 Z = *reinterpret_cast<const ulonglong2*>(sz + ii);
-    const ulonglong2 U = *reinterpret_cast<const ulonglong2*>(su + ii);
-    const ulonglong2 V = *reinterpret_cast<const ulonglong2*>(sv + ii);
-    const ulonglong2 W = *reinterpret_cast<const ulonglong2*>(sw + ii);
-    unsigned mask = 0;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const f32x2 rx = sub2(JX, h ? X.y : X.x), ry = sub2(JY, h ? Y.y : Y.x), rz = sub2(JZ, h ? Z.y : Z.x);
-      const f32x2 vx = sub2(GX, h ? U.y : U.x), vy = sub2(GY, h ? V.y : V.x), vz = sub2(GZ, h ? W.y : W.x);
-      const f32x2 R = fma2(rz, rz, fma2(ry, ry, mul2(rx, rx)));
-      const f32x2 Bv = fma2(vz, vz, fma2(vy, vy, mul2(vx, vx)));
-      float R0, R1, T0, T1;
-      unpack2(R, R0, R1);
-      unpack2(fma2(C1, Bv, C0), T0, T1);
-      bool c_0 = R0 <= T0, c_1 = R1 <= T1;
-      if (OWN) {
-        c_0 = c_0 && (!jown || j > i0 + ii + (uint32_t)(2 * h));
-        c_1 = c_1 && (!jown || j > i0 + ii + (uint32_t)(2 * h + 1));
-      }
-      mask |= (c_0 ? (1u << (2 * h)) : 0u) | (c_1 ? (2u << (2 * h)) : 0u);
-    }
-    if (mask) {
-      // rare and divergent: only the lanes with sphere survivors run the full test
-      do {
-        const int u = __ffs(mask) - 1;
-        mask &= mask - 1;
-        const uint32_t t = ii + (uint32_t)u;
-        const float rx = jx - sx[t], ry = jy - sy[t], rz = jz - sz[t];
-        const float vx = gx - su[t], vy = gy - sv[t], vz = gz - sw[t];
-        const float Bv = fmaf(vz, vz, fmaf(vy, vy, vx * vx));
-        if (full_test32(q, rx, ry, rz, vx, vy, vz, Bv)) emit_lane(buf, count, s, i0 + t, j);
-      } while (mask);
-    }
+// --------------------------------------------------------------------------- //
+// Thread per particle: the lane of particle p walks the cells of its forward half
+// stencil.  The search of kmc_params.search_kernel = 1, and of every simulation that has
+// a one-cell periodic axis (fewer than 2K + 1 cells), where each separation needs the
+// minimum image.  Returns the pairs tested.
+template <int PREC, int K>
+__device__ __noinline__ unsigned long long particle_walk(SimDev& s, uint32_t p, uint2* buf,
+                                                         uint32_t* cnt) {
+  const Grid& g = s.d.grid;
+  const int cur = s.d.parity ^ 1;
+  const uint32_t* __restrict__ cs = s.cell_start;
+  const int nx = g.nc[0], ny = g.nc[1], nz = g.nc[2];
+  const int Kx = nx == 1 ? 0 : K, Ky = ny == 1 ? 0 : K, Kz = nz == 1 ? 0 : K;
+  const bool px = s.bc[0] == KMC_PERIODIC, py = s.bc[1] == KMC_PERIODIC,
+             pz = s.bc[2] == KMC_PERIODIC;
+  unsigned long long tests = 0;
+  // the particle's cell, recomputed as the sort computed it
+  const int cx = cell_coord(g, 0, s.x[cur][0][p]), cy = cell_coord(g, 1, s.x[cur][1][p]),
+            cz = cell_coord(g, 2, s.x[cur][2][p]);
+  // own record
+  double xo[3] = {0, 0, 0}, vo[3] = {0, 0, 0};
+  Own32 o32 = {0, 0, 0, 0, 0, 0};
+  const double* __restrict__ X0 = s.x[cur][0];
+  const double* __restrict__ X1 = s.x[cur][1];
+  const double* __restrict__ X2 = s.x[cur][2];
+  const double* __restrict__ V0 = s.v[cur][0];
+  const double* __restrict__ V1 = s.v[cur][1];
+  const double* __restrict__ V2 = s.v[cur][2];
+  const float4* __restrict__ MM = s.mir;
+  if (PREC == KMC_FP64) {
+    xo[0] = X0[p]; xo[1] = X1[p]; xo[2] = X2[p];
+    vo[0] = V0[p]; vo[1] = V1[p]; vo[2] = V2[p];
+  } else {
+    float4 a;
+    float2 b;
+    mirror_load(MM, p, a, b);
+    o32 = {a.x, a.y, a.z, a.w, b.x, b.y};
   }
-}
+  // one-cell periodic axes need the minimum image explicitly
+  const bool cp0 = nx == 1 && px, cp1 = ny == 1 && py, cp2 = nz == 1 && pz;
+  const double L0 = s.box[0], L1 = s.box[1], L2 = s.box[2];
+  const Guard32 q = guard_of(g);
 
-template <int K>
-__global__ void __launch_bounds__(kCellWarps * 32, 3) k_search_cell32(Batch B) {
-  constexpr int ICAP = 64;
-  __shared__ __align__(16) float si[kCellWarps][6 * ICAP];
-  __shared__ uint2 wbuf[kCellWarps][kWarpBuf];
-  __shared__ uint32_t wcount[kCellWarps];
-  __shared__ Guard32 sq;
-  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-  const uint32_t gwarp = blockIdx.x * kCellWarps + warp, nwarps = gridDim.x * kCellWarps;
-
-  // The cells of the batch's simulations are dealt to the warps as one sequence (see
-  // k_search_cell: the dealing decides on launch-fixed fields only).
-  uint32_t base = 0;
-  for (int k = 0; k < B.nsims; ++k) {
-    SimDev& s = *B.sims[k];
-    if (!sim_scheduled(s) || s.d.grid.mode != KMC_SEARCH_CELL) continue;
-    const uint32_t first = (gwarp + nwarps - base) % nwarps;
-    base = (base + s.d.grid.nkeys % nwarps) % nwarps;
-    // every warp is done with the previous simulation's constants; the status word can
-    // change while the search runs, so the block takes one answer
-    if (!__syncthreads_and(sim_active(s))) continue;
-    if (threadIdx.x == 0) {
-      const Grid& G0 = s.d.grid;
-      sq.c0 = G0.s_c0; sq.c1 = G0.s_c1; sq.ag = G0.a_g; sq.tg = G0.t_g; sq.dtf = G0.dtf;
-      sq.d0up = G0.d0up; sq.brel = G0.b_rel; sq.babs = G0.b_abs; sq.we = G0.w_e; sq.wrel = G0.w_rel;
+  // a neighbour reached across a periodic boundary is seen as its image: wrap
+  // flags -1 (below 0) or +1 (at or above the extent) per axis
+  for (int dz = 0; dz <= Kz; ++dz) {
+    int qz = cz + dz, wz = 0;
+    if (qz >= nz) {
+      if (!pz) break;
+      qz -= nz;
+      wz = 1;
     }
-    if (lane == 0) wcount[warp] = 0;
-    __syncthreads();
-    const Grid& G = s.d.grid;
-    const int nx = G.nc[0], ny = G.nc[1], nz = G.nc[2];
-    const int Kx = nx == 1 ? 0 : K, Ky = ny == 1 ? 0 : K, Kz = nz == 1 ? 0 : K;
-    const bool px = s.bc[0] == KMC_PERIODIC, py = s.bc[1] == KMC_PERIODIC,
-               pz = s.bc[2] == KMC_PERIODIC;
-    const uint32_t nkeys = G.nkeys;
-    const uint32_t* __restrict__ cs = s.cell_start;
-    const float Lx = G.Lf[0], Ly = G.Lf[1], Lz = G.Lf[2];
-    const float c0 = G.s_c0, c1 = G.s_c1;
-    const float4* __restrict__ MM = s.mir;
-    float* my = si[warp];
-    uint2* buf = wbuf[warp];
-    uint32_t* cnt = &wcount[warp];
-    unsigned long long tests = 0;
-
-    for (uint32_t key = first; key < nkeys; key += nwarps) {
-      const uint32_t startA = __ldg(cs + key), endA = __ldg(cs + key + 1);
-      if (startA == endA) continue;
-      int cx, cy, cz;
-      key_decode(G, key, cx, cy, cz);
-      for (uint32_t i0 = startA; i0 < endA; i0 += ICAP) {
-        const uint32_t nI = endA - i0 < (uint32_t)ICAP ? endA - i0 : (uint32_t)ICAP;
-        const uint32_t nI4 = (nI + 3u) & ~3u;
-        __syncwarp();
-        for (uint32_t t = lane; t < nI4; t += 32) {
-          if (t < nI) {
+    for (int dy = (dz == 0 ? 0 : -Ky); dy <= Ky; ++dy) {
+      int qy = cy + dy, wy = 0;
+      if (qy < 0) {
+        if (!py) continue;
+        qy += ny;
+        wy = -1;
+      } else if (qy >= ny) {
+        if (!py) continue;
+        qy -= ny;
+        wy = 1;
+      }
+      const uint32_t colbase = col_code(g, (uint32_t)qy, (uint32_t)qz) * (uint32_t)nx;
+      const int dx0 = (dz == 0 && dy == 0) ? 0 : -Kx;
+      for (int dx = dx0; dx <= Kx; ++dx) {
+        int qx = cx + dx, wx = 0;
+        if (qx < 0) {
+          if (!px) continue;
+          qx += nx;
+          wx = -1;
+        } else if (qx >= nx) {
+          if (!px) continue;
+          qx -= nx;
+          wx = 1;
+        }
+        const uint32_t key = colbase + (uint32_t)qx;
+        uint32_t beg = __ldg(cs + key), end = __ldg(cs + key + 1);
+        if (dz == 0 && dy == 0 && dx == 0) beg = p + 1;
+        if (beg >= end) continue;
+        tests += end - beg;
+        if (PREC == KMC_FP64) {
+          for (uint32_t j = beg; j < end; ++j) {
+            double r0 = dsub(__ldg(X0 + j), xo[0]);
+            double r1 = dsub(__ldg(X1 + j), xo[1]);
+            double r2 = dsub(__ldg(X2 + j), xo[2]);
+            if (px) { if (r0 > 0.5 * L0) r0 = dsub(r0, L0); else if (r0 < -0.5 * L0) r0 = dadd(r0, L0); }
+            if (py) { if (r1 > 0.5 * L1) r1 = dsub(r1, L1); else if (r1 < -0.5 * L1) r1 = dadd(r1, L1); }
+            if (pz) { if (r2 > 0.5 * L2) r2 = dsub(r2, L2); else if (r2 < -0.5 * L2) r2 = dadd(r2, L2); }
+            double g0 = dsub(__ldg(V0 + j), vo[0]);
+            double g1 = dsub(__ldg(V1 + j), vo[1]);
+            double g2 = dsub(__ldg(V2 + j), vo[2]);
+            double R = dadd(dadd(dmul(r0, r0), dmul(r1, r1)), dmul(r2, r2));
+            double Bv = dadd(dadd(dmul(g0, g0), dmul(g1, g1)), dmul(g2, g2));
+            if (Bv >= 0x1p-900 && R > dadd(g.c0, dmul(g.c1, Bv))) continue;
+            if (Bv >= 0x1p-900 &&
+                f64_cannot_approach(dadd(dadd(dmul(r0, g0), dmul(r1, g1)), dmul(r2, g2)), Bv, s.dt))
+              continue;
+            emit_lane(buf, cnt, s, p, j);
+          }
+        } else {
+          // own coordinates moved by the image shift (j seen at x_j + w L)
+          const float sx = o32.ox - (float)wx * g.Lf[0];
+          const float sy = o32.oy - (float)wy * g.Lf[1];
+          const float sz = o32.oz - (float)wz * g.Lf[2];
+          for (uint32_t j = beg; j < end; ++j) {
             float4 a;
             float2 b;
-            mirror_load(MM, i0 + t, a, b);
-            my[t] = a.x; my[ICAP + t] = a.y; my[2 * ICAP + t] = a.z;
-            my[3 * ICAP + t] = a.w; my[4 * ICAP + t] = b.x; my[5 * ICAP + t] = b.y;
-          } else {
-            my[t] = -1e30f; my[ICAP + t] = 0.f; my[2 * ICAP + t] = 0.f;
-            my[3 * ICAP + t] = 0.f; my[4 * ICAP + t] = 0.f; my[5 * ICAP + t] = 0.f;
-          }
-        }
-        __syncwarp();
-        for (int dz = 0; dz <= Kz; ++dz) {
-          int qz = cz + dz, wrz = 0;
-          if (qz >= nz) {
-            if (!pz) break;
-            qz -= nz;
-            wrz = 1;
-          }
-          for (int dy = (dz == 0 ? 0 : -Ky); dy <= Ky; ++dy) {
-            int qy = cy + dy, wry = 0;
-            if (qy < 0) {
-              if (!py) continue;
-              qy += ny;
-              wry = -1;
-            } else if (qy >= ny) {
-              if (!py) continue;
-              qy -= ny;
-              wry = 1;
-            }
-            const uint32_t colbase = col_code(G, (uint32_t)qy, (uint32_t)qz) * (uint32_t)nx;
-            const bool own_col = dz == 0 && dy == 0;
-            // image shifts of partners reached across a periodic boundary
-            const float shy = (float)wry * Ly, shz = (float)wrz * Lz;
-            int dx = own_col ? 0 : -Kx;
-            while (dx <= Kx) {
-              const int q0 = cx + dx;
-              const int region = q0 < 0 ? -1 : (q0 >= nx ? 1 : 0);
-              if (region != 0 && !px) { ++dx; continue; }
-              const int qx = q0 - region * nx;
-              int m = 1;
-              while (dx + m <= Kx) {
-                const int q2 = cx + dx + m;
-                const int r2 = q2 < 0 ? -1 : (q2 >= nx ? 1 : 0);
-                if (r2 != region) break;
-                ++m;
-              }
-              const int dxa = dx;
-              dx += m;
-              const uint32_t jbeg = __ldg(cs + colbase + qx), jend = __ldg(cs + colbase + qx + m);
-              if (jbeg == jend) continue;
-              const float shx = (float)region * Lx;
-              const bool has_own = own_col && dxa <= 0 && dxa + m > 0;
-              if (lane == 0) {
-                uint64_t len = jend - jbeg;
-                if (has_own) {
-                  uint64_t nA = endA - startA;
-                  uint64_t inc = (uint64_t)nI * (endA - i0 - 1) - (uint64_t)nI * (nI - 1) / 2;
-                  tests += (uint64_t)nI * (len - nA) + inc;
-                } else {
-                  tests += (uint64_t)nI * len;
-                }
-              }
-              for (uint32_t cb = jbeg; cb < jend; cb += 32) {
-                const uint32_t j = cb + lane;
-                float jx = 1e30f, jy = 0.f, jz = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
-                if (j < jend) {
-                  float4 a;
-                  float2 b;
-                  mirror_load(MM, j, a, b);
-                  jx = a.x + shx;
-                  jy = a.y + shy;
-                  jz = a.z + shz;
-                  gx = a.w; gy = b.x; gz = b.y;
-                }
-                if (has_own) {
-                  const bool jown = j >= startA && j < endA;
-                  cell32_sweep<true>(my, nI4, i0, jx, jy, jz, gx, gy, gz, j, jown, c0, c1, sq, buf, cnt, s);
-                } else {
-                  cell32_sweep<false>(my, nI4, i0, jx, jy, jz, gx, gy, gz, j, false, c0, c1, sq, buf, cnt, s);
-                }
-                __syncwarp();
-                if (*cnt >= (uint32_t)(kWarpBuf / 2)) flush_lanes(buf, cnt, s, lane);
-              }
-            }
+            mirror_load(MM, j, a, b);
+            float rx = a.x - sx, ry = a.y - sy, rz = a.z - sz;
+            bool keep = false;
+            // minimum image on one-cell periodic axes; near the tie the two
+            // images are both possible in binary64: keep the pair unculled
+            if (cp0) min_image_f(rx, g.halfLf[0], g.Lf[0], g.tief[0], keep);
+            if (cp1) min_image_f(ry, g.halfLf[1], g.Lf[1], g.tief[1], keep);
+            if (cp2) min_image_f(rz, g.halfLf[2], g.Lf[2], g.tief[2], keep);
+            const float gx = a.w - o32.vx, gy = b.x - o32.vy, gz = b.y - o32.vz;
+            const float R = fmaf(rz, rz, fmaf(ry, ry, rx * rx));
+            const float Bv = fmaf(gz, gz, fmaf(gy, gy, gx * gx));
+            if (keep || (R <= fmaf(q.c1, Bv, q.c0) && full_test32(q, rx, ry, rz, gx, gy, gz, Bv)))
+              emit_lane(buf, cnt, s, p, j);
           }
         }
       }
     }
-    flush_lanes(buf, cnt, s, lane);
+  }
+  return tests;
+}
+
+template <int PREC, int K>
+__global__ void __launch_bounds__(kTile) k_search(Batch B) {
+  __shared__ uint2 wbuf[kTile / 32][kWarpBuf];
+  __shared__ uint32_t wcount[kTile / 32];
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  if (lane == 0) wcount[warp] = 0;
+  __syncwarp();
+  // grid-stride over tiles of kTile particles (an occupancy-sized grid)
+  const uint32_t ntiles = B.ptile[B.nsims];
+  for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int k = find_sim(B.ptile, B.nsims, tile);
+    SimDev& s = *B.sims[k];
+    if (s.d.grid.mode != MODE_PARTICLE) continue;
+    // the status word can change while the search runs (a full pair buffer): one answer
+    if (!__all_sync(0xFFFFFFFFu, sim_active(s))) continue;
+    const uint32_t p = (tile - B.ptile[k]) * kTile + threadIdx.x;
+    // with the speed split only the slow population (keys below nkeys) is searched here;
+    // particles that left through absorbing walls sit after every cell key
+    const uint32_t nslow = (s.d.grid.split || s.absorb) ? __ldg(s.cell_start + s.d.grid.nkeys) : s.n;
+    unsigned long long tests = 0;
+    if (p < nslow) tests = particle_walk<PREC, K>(s, p, wbuf[warp], &wcount[warp]);
+    flush_lanes(wbuf[warp], &wcount[warp], s, lane);
+    for (int o = 16; o > 0; o >>= 1) tests += __shfl_down_sync(0xFFFFFFFFu, tests, o);
     if (lane == 0 && tests) atomicAdd(&s.d.pair_tests, tests);
   }
 }
@@ -836,7 +356,7 @@ __global__ void __launch_bounds__(kTile, 4) k_search_rows32(Batch B) {
   __shared__ int s_live;            // the current simulation runs this step
   // grid-stride over tiles of kTile particles: the kernel is launched every step on an
   // occupancy-sized grid and exits at once when the step runs another search
-  if (!batch_uses(B, KMC_SEARCH_ROW)) return;
+  if (!batch_uses(B, MODE_ROWS)) return;
   const uint32_t ntiles = B.ptile[B.nsims];
   int kcur = -1;  // simulation whose constants the shared tables hold
   // The warp's pair tests and emitted pairs go to the simulation's counters only when
@@ -864,7 +384,7 @@ __global__ void __launch_bounds__(kTile, 4) k_search_rows32(Batch B) {
     const int k = find_sim(B.ptile, B.nsims, tile);
     SimDev& s = *B.sims[k];
     // launch-fixed fields only: the barriers below depend on it
-    if (!sim_scheduled(s) || s.d.grid.mode != KMC_SEARCH_ROW || (s.bc[0] == KMC_PERIODIC) != PX)
+    if (!sim_scheduled(s) || s.d.grid.mode != MODE_ROWS || (s.bc[0] == KMC_PERIODIC) != PX)
       continue;
     const Grid& g = s.d.grid;
     // The shared constants change only with the simulation (block-uniform: every warp
@@ -874,8 +394,7 @@ __global__ void __launch_bounds__(kTile, 4) k_search_rows32(Batch B) {
       if (kcur >= 0) warp_flush(*B.sims[kcur]);  // staged pairs and counts of the last one
       __syncthreads();  // every warp is done with the previous simulation's constants
       if (threadIdx.x == 0) {
-        sq.c0 = g.s_c0; sq.c1 = g.s_c1; sq.ag = g.a_g; sq.tg = g.t_g; sq.dtf = g.dtf;
-        sq.d0up = g.d0up; sq.brel = g.b_rel; sq.babs = g.b_abs; sq.we = g.w_e; sq.wrel = g.w_rel;
+        sq = guard_of(g);
         // the status word, read once per simulation and block (the search itself can set
         // it: a full pair buffer only stops the stores, which are bounds-checked)
         s_live = sim_active(s) ? 1 : 0;
@@ -1167,6 +686,481 @@ __global__ void __launch_bounds__(kTile, 4) k_search_rows32(Batch B) {
   if (kcur >= 0) warp_flush(*B.sims[kcur]);
 }
 
+// --------------------------------------------------------------------------- //
+// Tiled search of the slow pairs.  A warp takes 32 consecutive particles i (cell order)
+// and all partners that any of them can have: for a run of lanes in one (y, z) column
+// these are one contiguous range of the order per forward column (the cells along x from
+// K below the first lane's to K above the last lane's; in the own column from the first
+// lane's particle on), plus the wrapped part on a periodic x axis.  The ranges are laid
+// end to end and taken 32 partners j at a time, a lane each.  The sphere test of all
+// 32 x 32 pairs is one quadratic form,
+//   |a_i - a_j|^2 - |b_i - b_j|^2 = s_i + s_j - 2 a_i.a_j + 2 b_i.b_j,  s = |a|^2 - |b|^2,
+// a the position and b = dt v, both relative to the run's middle and scaled by a power of
+// two so that |a|, |b| <= 1: an inner product of 16 terms, which eight
+// mma.sync.m16n8k16 (binary16 operands, binary32 sums) form for the whole tile.  Every
+// position is the sum of two binary16 values (22 bits), so are s_i and s_j; the
+// velocities are one.  The sign of (form - threshold) is a bit of a lane's survivor mask,
+// shifted in by one funnel shift per accumulator.  Survivors go to a per-warp queue, and
+// the tests of the precision run on 32 of them at a time with every lane busy: cell
+// offset (each pair at exactly one image), then the binary32 sphere and full guarded
+// tests on the mirror, or the binary64 sphere, approach and time tests on the state.  The
+// filter only saves them work: what it drops they would drop.
+//
+// Error of the filter, in the scaled units.  A candidate has (kmc_grid.cuh)
+// |a_i - a_j|^2 <= c + |b_i - b_j|^2 for the exact binary32 coordinates, with c the
+// scaled constant of the sphere test with 3 er for the separation, since here the
+// coordinates are rounded once more relative to the run's middle.  The rounding of b to
+// 11 bits moves |b_i - b_j|^2 by at most 14 2^-11 b^2 < 2^-7 b^2 (both in tile_c).  The
+// rest, with the four squared extents at most 1 each and u = 2^-24: dropped and rounded
+// low parts 18 u, s and its halves 44 u, the inner product (16 products, exact in
+// binary32, whose partial sums are at most 12, added with truncation) 384 u; 2^-14 =
+// 1024 u is taken.
+//
+// What bounds it: issue slots.  A tile costs 8 mma (2 cycles of the SM's tensor cores
+// each), 32 funnel shifts (half rate), about 75 instructions to pack the 32 partners and
+// about 30 per turn of survivors, so it pays where most of a tile's 1024 pairs are pairs
+// that have to be tested: see kTileOccupancy (kmc_grid.cuh).  Measured, slow pairs of one
+// step: 10^8 particles at 7 per cell 16.0 ms with the row search, 10.5 ms with tiles; an
+// ensemble of 30 boxes and tubes 336 (warp per cell and rows) -> 226 us; binary64 at 2^20
+// 3.11 ms (thread per particle, every pair in binary64) -> 0.167 ms.  Packing the partners
+// once per block or in the sort, 64 partners at a time, and records fetched ahead were no
+// faster: the bookkeeping per run and column, not the packing, fills the issue slots.
+constexpr int kPlane = 36;  // uint4 per plane of packed records: 32 and 4 of padding, so
+                            // that the two planes lie in different shared-memory banks
+constexpr float kFar = 60000.0f;  // form of an absent row or column: above any threshold
+constexpr int kRunCells = 64;     // cells along x that the lanes of a run may span
+
+template <int K>
+struct TileWarp {
+  static constexpr int kCols = 1 + K + K * (2 * K + 1);  // own column + forward columns
+  static constexpr int kPieces = 3 * kCols;              // a range and its two wrapped parts
+  uint4 rec[2 * kPlane];       // packed records: the rows, then 32 partners at a time
+  uint32_t start[kPieces + 1]; // pieces: first slot, first partner, image code
+  uint32_t first[kPieces + 1];
+  uint32_t code[kPieces + 1];
+  uint2 info[32];              // the partners' indices and image codes
+  uint2 queue[64];             // survivors: row particle and partner
+  uint32_t qcode[64];          // and the partner's image code
+  uint2 buf[kWarpBuf];         // emitted pairs
+  uint32_t count;
+};
+
+// image code of a piece: bits 0-1 x, 2-3 y, 4-5 z (1: seen at +L, 2: at -L), bit 6: own
+// column
+constexpr uint32_t kImages = 63u, kOwnColumn = 64u;
+__device__ __forceinline__ float image_shift(uint32_t code, float L) {
+  return (code & 1u) ? L : ((code & 2u) ? -L : 0.0f);
+}
+
+__device__ __forceinline__ uint32_t half_bits(__half2 h) { return *reinterpret_cast<uint32_t*>(&h); }
+__device__ __forceinline__ uint32_t half_pair(float lo, float hi) {
+  return half_bits(__floats2half2_rn(lo, hi));
+}
+
+// The 16 terms as 8 words w0..w7 of two; words c and c + 4 belong to the lanes with
+// lane % 4 == c of the matrix fragments and lie side by side: plane 0 holds
+// (w0, w4, w1, w5), plane 1 (w2, w6, w3, w7).
+//   row:     (-2xh -2xh) (-2yh -2yh) (-2zh -2zh) (1 1)   | (-2xl sh) (-2yl 2bx) (-2zl 2by) (sl 2bz)
+//   partner: (xh xl)     (yh yl)     (zh zl)     (sh sl) | (xh 1)    (yh bx)    (zh by)    (1 bz)
+// with s = |a|^2 - |b|^2 of the rounded b, and the row's s less the threshold.  An absent
+// row or partner is all zero but for its s = kFar and the partner's 1.
+__device__ __forceinline__ void store_row(uint4* rec, uint32_t at, float ax, float ay, float az,
+                                          float bx, float by, float bz, float T, bool in) {
+  const __half2 hb = __floats2half2_rn(bx, by), hz = __floats2half2_rn(bz, 0.0f);
+  bx = __low2float(hb); by = __high2float(hb); bz = __low2float(hz);
+  const float s = in ? fmaf(ax, ax, fmaf(ay, ay, az * az)) - fmaf(bx, bx, fmaf(by, by, bz * bz)) - T
+                     : kFar;
+  const float m = in ? -2.0f : 0.0f;
+  ax *= m; ay *= m; az *= m;
+  bx *= -m; by *= -m; bz *= -m;
+  const __half2 hxy = __floats2half2_rn(ax, ay), hzs = __floats2half2_rn(az, s);
+  uint4 u, w;
+  u.x = half_bits(__low2half2(hxy));
+  u.y = half_pair(ax - __low2float(hxy), s);
+  u.z = half_bits(__high2half2(hxy));
+  u.w = half_pair(ay - __high2float(hxy), bx);
+  w.x = half_bits(__low2half2(hzs));
+  w.y = half_pair(az - __low2float(hzs), by);
+  w.z = in ? 0x3C003C00u : 0u;
+  w.w = half_pair(s - __high2float(hzs), bz);
+  rec[at] = u;
+  rec[kPlane + at] = w;
+}
+__device__ __forceinline__ void store_partner(uint4* rec, uint32_t at, float ax, float ay, float az,
+                                              float bx, float by, float bz, float far) {
+  const __half2 hxy = __floats2half2_rn(ax, ay), hb = __floats2half2_rn(bx, by),
+                hzb = __floats2half2_rn(az, bz);
+  bx = __low2float(hb); by = __high2float(hb); bz = __high2float(hzb);
+  const float s = (fmaf(ax, ax, fmaf(ay, ay, az * az)) + far) - fmaf(bx, bx, fmaf(by, by, bz * bz));
+  const __half2 one = __floats2half2_rn(1.0f, 1.0f);
+  uint4 u, w;
+  u.x = half_pair(ax, ax - __low2float(hxy));
+  u.y = half_bits(__lows2half2(hxy, one));
+  u.z = half_pair(ay, ay - __high2float(hxy));
+  u.w = half_bits(__halves2half2(__high2half(hxy), __low2half(hb)));
+  w.x = half_pair(az, az - __low2float(hzb));
+  w.y = half_bits(__halves2half2(__low2half(hzb), __high2half(hb)));
+  w.z = half_pair(s, s - __half2float(__float2half_rn(s)));
+  w.w = half_bits(__highs2half2(one, hzb));
+  rec[at] = u;
+  rec[kPlane + at] = w;
+}
+
+__device__ __forceinline__ void mma_form(float d[4], const uint32_t a[4], uint2 b) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+      "{%8, %9}, {%10, %10, %10, %10};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y), "f"(0.0f));
+}
+
+// The bits of a lane's mask where the partner comes after the row, in a tile whose partner
+// 0 is the particle after row 0 (the own column: each pair once, no particle with itself).
+// The lane holds rows frag + 8 L (L = 0..3) and partners 8 n + 2 quad + e (n = 0..3, e = 0,
+// 1), bit 31 - (8 n + 2 L + e).
+__device__ __forceinline__ uint32_t later_bits(uint32_t frag, uint32_t quad) {
+  uint32_t bits = 0;
+#pragma unroll
+  for (uint32_t at = 0; at < 32; ++at) {
+    const uint32_t row = frag + 8u * ((at >> 1) & 3u), col = 8u * (at >> 3) + 2u * quad + (at & 1u);
+    if (1u + col > row) bits |= 0x80000000u >> at;
+  }
+  return bits;
+}
+
+// The bits of a lane's mask where row and partner are the same particle, partner 0 of the
+// tile being row `first` of the warp: equal for the one e that makes first + 2 quad + e -
+// frag = 8 k, and there for L = n + k.
+__device__ __forceinline__ uint32_t self_bits(uint32_t first, uint32_t frag, uint32_t quad) {
+  const int u = (int)(first + 2u * quad - frag);
+  const int e = u & 1, k = (u + e) >> 3;
+  if ((u + e) & 7) return 0u;
+  uint32_t bits = 0;
+#pragma unroll
+  for (int n = 0; n < 4; ++n)
+    if (n + k >= 0 && n + k < 4) bits |= 0x80000000u >> (8 * n + 2 * (n + k) + e);
+  return bits;
+}
+
+// binary32 record of a particle (FP64: its state rounded once, as the mirror would hold it)
+template <int PREC>
+__device__ __forceinline__ Own32 record32(const SimDev& s, const float4* __restrict__ M,
+                                          int cur, uint32_t p) {
+  if (PREC == KMC_FP64)
+    return {d2f_rn(__ldg(s.x[cur][0] + p)), d2f_rn(__ldg(s.x[cur][1] + p)),
+            d2f_rn(__ldg(s.x[cur][2] + p)), d2f_rn(__ldg(s.v[cur][0] + p)),
+            d2f_rn(__ldg(s.v[cur][1] + p)), d2f_rn(__ldg(s.v[cur][2] + p))};
+  float4 a;
+  float2 b;
+  mirror_load(M, p, a, b);
+  return {a.x, a.y, a.z, a.w, b.x, b.y};
+}
+
+// the tests of the precision on one survivor: particle i (a row), partner j
+template <int PREC, int K>
+__device__ __noinline__ void test_survivor(SimDev& s, uint2* buf, uint32_t* cnt, uint2 ij,
+                                           uint32_t code) {
+  const Grid& g = s.d.grid;
+  const uint32_t i = ij.x, j = ij.y;
+  const int cur = s.d.parity ^ 1, nx = g.nc[0], Kx = nx == 1 ? 0 : K;
+  const Own32 o = record32<PREC>(s, s.mir, cur, j), q = record32<PREC>(s, s.mir, cur, i);
+  // every pair at exactly one image: the partner's cell, seen through this image, lies in
+  // the row's stencil; in the own column only forward cells and later particles
+  const int d = cell_coord_f(g, 0, o.ox) + ((code & 1u) ? nx : ((code & 2u) ? -nx : 0)) -
+                cell_coord_f(g, 0, q.ox);
+  if (d > Kx || d < -Kx) return;
+  if ((code & kOwnColumn) && (d < 0 || (d == 0 && j <= i))) return;
+  bool emit;
+  if (PREC == KMC_FP64) {
+    double r[3], v[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      r[a] = dsub(__ldg(s.x[cur][a] + j), __ldg(s.x[cur][a] + i));
+      if (s.bc[a] == KMC_PERIODIC) {
+        const double L = s.box[a];
+        if (r[a] > 0.5 * L) r[a] = dsub(r[a], L);
+        else if (r[a] < -0.5 * L) r[a] = dadd(r[a], L);
+      }
+      v[a] = dsub(__ldg(s.v[cur][a] + j), __ldg(s.v[cur][a] + i));
+    }
+    const double R = dadd(dadd(dmul(r[0], r[0]), dmul(r[1], r[1])), dmul(r[2], r[2]));
+    const double Bv = dadd(dadd(dmul(v[0], v[0]), dmul(v[1], v[1])), dmul(v[2], v[2]));
+    emit = !(Bv >= 0x1p-900 && R > dadd(g.c0, dmul(g.c1, Bv)));
+    if (emit && Bv >= 0x1p-900 &&
+        f64_cannot_approach(dadd(dadd(dmul(r[0], v[0]), dmul(r[1], v[1])), dmul(r[2], v[2])), Bv, s.dt))
+      emit = false;
+  } else {
+    // own coordinates moved by the image shift (j seen at x_j + w L)
+    const float rx = o.ox - (q.ox - image_shift(code, g.Lf[0]));
+    const float ry = o.oy - (q.oy - image_shift(code >> 2, g.Lf[1]));
+    const float rz = o.oz - (q.oz - image_shift(code >> 4, g.Lf[2]));
+    const float gx = o.vx - q.vx, gy = o.vy - q.vy, gz = o.vz - q.vz;
+    const float R = fmaf(rz, rz, fmaf(ry, ry, rx * rx));
+    const float Bv = fmaf(gz, gz, fmaf(gy, gy, gx * gx));
+    emit = R <= fmaf(g.s_c1, Bv, g.s_c0) &&
+           full_test32(guard_of(g), rx, ry, rz, gx, gy, gz, Bv);
+  }
+  if (emit) emit_lane(buf, cnt, s, i, j);
+}
+
+template <int PREC, int K>
+__global__ void __launch_bounds__(kTile, 4) k_search_tiles(Batch B) {
+  using TW = TileWarp<K>;
+  constexpr uint32_t kAll = 0xFFFFFFFFu;
+  constexpr int kCols = TW::kCols;
+  __shared__ TW tw[kTile / 32];
+  if (!batch_uses(B, MODE_TILES)) return;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  TW& w = tw[warp];
+  if (lane == 0) w.count = 0;
+  __syncwarp();
+  // The warps of a block never wait for each other.  Survivors, pair counts and emitted
+  // pairs are kept per warp until 32 (survivors) or half a buffer (pairs) are there, the
+  // simulation changes, or the end: per-tile atomics from every warp would serialise in L2.
+  unsigned long long tests = 0;
+  uint32_t queued = 0;
+  int kcur = -1;
+  auto finish = [&](SimDev& f) {
+    if (lane < queued) test_survivor<PREC, K>(f, w.buf, &w.count, w.queue[lane], w.qcode[lane]);
+    queued = 0;
+    flush_lanes(w.buf, &w.count, f, lane);
+    if (lane == 0 && tests) atomicAdd(&f.d.pair_tests, tests);
+    tests = 0;
+  };
+  const uint32_t frag = lane >> 2, quad = lane & 3u, later = later_bits(frag, quad);
+  // this lane's two words of record r: plane quad / 2, half quad % 2
+  const uint2* words = reinterpret_cast<const uint2*>(w.rec + (quad >> 1) * kPlane) + (quad & 1u);
+  const uint32_t ntiles = B.ptile[B.nsims];
+  for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int k = find_sim(B.ptile, B.nsims, tile);
+    SimDev& s = *B.sims[k];
+    if (k != kcur) {
+      if (kcur >= 0) finish(*B.sims[kcur]);
+      kcur = k;
+    }
+    // the status word can change while the search runs (a full pair buffer): one answer
+    if (!__all_sync(kAll, sim_active(s)) || s.d.grid.mode != MODE_TILES) continue;
+    const Grid& g = s.d.grid;
+    const uint32_t* __restrict__ cs = s.cell_start;
+    const uint32_t nslow = (g.split || s.absorb) ? __ldg(cs + g.nkeys) : s.n;
+    const uint32_t p0 = (tile - B.ptile[k]) * kTile + warp * 32u, p = p0 + lane;
+    if (p0 >= nslow) continue;
+    const bool valid = p < nslow;
+    const int nx = g.nc[0], ny = g.nc[1], nz = g.nc[2], cur = s.d.parity ^ 1;
+    const int Kx = nx == 1 ? 0 : K, Ky = ny == 1 ? 0 : K, Kz = nz == 1 ? 0 : K;
+    const bool px = s.bc[0] == KMC_PERIODIC, py = s.bc[1] == KMC_PERIODIC,
+               pz = s.bc[2] == KMC_PERIODIC;
+    if (PREC == KMC_FP64 && ((nx == 1 && px) || (ny == 1 && py) || (nz == 1 && pz))) {
+      // a one-cell periodic axis: the minimum image of every pair (binary32: row search)
+      unsigned long long t = valid ? particle_walk<PREC, K>(s, p, w.buf, &w.count) : 0ull;
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kAll, t, o);
+      tests += t;
+      flush_lanes(w.buf, &w.count, s, lane);
+      continue;
+    }
+    const float4* __restrict__ MM = s.mir;
+    Own32 o = {0, 0, 0, 0, 0, 0};
+    int cx = 0, cy = 0, cz = 0;
+    if (valid) {
+      o = record32<PREC>(s, MM, cur, p);
+      // the particle's cell, recomputed as the sort computed it
+      cx = cell_coord_f(g, 0, o.ox);
+      cy = cell_coord_f(g, 1, o.oy);
+      cz = cell_coord_f(g, 2, o.oz);
+    }
+    // runs of lanes in one column (in cell order: consecutive lanes, cells ascending)
+    unsigned todo = __ballot_sync(kAll, valid);
+    while (todo) {
+      const int lead = __ffs((int)todo) - 1;
+      const int y = __shfl_sync(kAll, cy, lead), z = __shfl_sync(kAll, cz, lead);
+      const int x0 = __shfl_sync(kAll, cx, lead);
+      const unsigned run =
+          todo & __ballot_sync(kAll, valid && cy == y && cz == z && cx - x0 < kRunCells);
+      todo &= ~run;
+      const int x1 = __shfl_sync(kAll, cx, 31 - __clz((int)run));
+
+      // 1. the pieces: lane c takes forward column c
+      uint32_t jb = 0, len = 0, code = 0, jb1 = 0, len1 = 0, jb2 = 0, len2 = 0;
+      if (lane < (uint32_t)kCols) {
+        const int c = (int)lane;
+        const int dz = c <= K ? 0 : 1 + (c - K - 1) / (2 * K + 1);
+        const int dy = c == 0 ? 0 : (c <= K ? c : (c - K - 1) % (2 * K + 1) - K);
+        int qy = y + dy, qz = z + dz;
+        bool ok = dz <= Kz && dy <= Ky && dy >= -Ky;
+        if (qz >= nz) { ok = ok && pz; qz -= nz; code |= 16u; }
+        if (qy < 0) { ok = ok && py; qy += ny; code |= 8u; }
+        else if (qy >= ny) { ok = ok && py; qy -= ny; code |= 4u; }
+        if (c == 0) code |= kOwnColumn;
+        if (ok) {
+          const uint32_t* col = cs + col_code(g, (uint32_t)qy, (uint32_t)qz) * (uint32_t)nx;
+          const int xa = c == 0 ? x0 : x0 - Kx, xb = x1 + Kx;
+          jb = __ldg(col + (xa < 0 ? 0 : xa));
+          const uint32_t je = __ldg(col + (xb >= nx ? nx : xb + 1));
+          if (c == 0) jb = max(jb, p0 + (uint32_t)lead + 1u);
+          len = je > jb ? je - jb : 0u;
+          if (px && xa < 0) {  // cells [xa + nx, nx) seen at -L
+            jb1 = __ldg(col + xa + nx);
+            len1 = __ldg(col + nx) - jb1;
+          }
+          if (px && xb >= nx) {  // cells [0, xb - nx] seen at +L
+            jb2 = __ldg(col);
+            len2 = __ldg(col + xb - nx + 1) - jb2;
+          }
+        } else {
+          code &= ~kImages;
+        }
+      }
+      const uint32_t my_slots = len + len1 + len2;
+      uint32_t slots = my_slots;
+#pragma unroll
+      for (int d = 1; d < kCols; d <<= 1) {
+        const uint32_t u = __shfl_up_sync(kAll, slots, d);
+        if (lane >= (uint32_t)d) slots += u;
+      }
+      const uint32_t total = __shfl_sync(kAll, slots, kCols - 1);
+      if (total == 0u) continue;
+      tests += (unsigned long long)__popc(run) * total;
+      // Plain: no piece is seen through an image.  The five pieces of K = 1 then stay in
+      // registers; otherwise they go to shared memory.
+      const bool plain =
+          K == 1 && !__any_sync(kAll, (code & kImages) != 0u || len1 != 0u || len2 != 0u);
+      uint32_t s1 = 0, s2 = 0, s3 = 0, s4 = 0, o0 = 0, o1 = 0, o2 = 0, o3 = 0, o4 = 0, pieces = 0;
+      if (plain) {
+        const uint32_t first = slots - my_slots, off = jb - first;
+        s1 = __shfl_sync(kAll, first, 1); s2 = __shfl_sync(kAll, first, 2);
+        s3 = __shfl_sync(kAll, first, 3); s4 = __shfl_sync(kAll, first, 4);
+        o0 = __shfl_sync(kAll, off, 0); o1 = __shfl_sync(kAll, off, 1);
+        o2 = __shfl_sync(kAll, off, 2); o3 = __shfl_sync(kAll, off, 3);
+        o4 = __shfl_sync(kAll, off, 4);
+      } else {
+        const uint32_t my_cnt = (len ? 1u : 0u) + (len1 ? 1u : 0u) + (len2 ? 1u : 0u);
+        uint32_t cnt = my_cnt;
+#pragma unroll
+        for (int d = 1; d < kCols; d <<= 1) {
+          const uint32_t u = __shfl_up_sync(kAll, cnt, d);
+          if (lane >= (uint32_t)d) cnt += u;
+        }
+        pieces = __shfl_sync(kAll, cnt, kCols - 1);
+        uint32_t at = cnt - my_cnt, st = slots - my_slots;
+        auto put = [&](uint32_t b, uint32_t n, uint32_t c) {
+          if (!n) return;
+          w.start[at] = st;
+          w.first[at] = b;
+          w.code[at] = c;
+          st += n;
+          ++at;
+        };
+        put(jb, len, code);
+        put(jb1, len1, code | 2u);
+        put(jb2, len2, code | 1u);
+      }
+
+      // 2. the run's frame: origin in its middle, scale the power of two that brings
+      // the extents and dt |v| to at most 1
+      const float wx = g.wf[0], wy = g.wf[1], wz = g.wf[2];
+      const float ox = 0.5f * (float)(x0 + x1 + 1) * wx, oy = ((float)y + 0.5f) * wy,
+                  oz = ((float)z + 0.5f) * wz;
+      const float kv = g.tile_k;
+      const float M = 1.01f * fmaxf(fmaxf((0.5f * (float)(x1 - x0 + 1) + (float)Kx) * wx,
+                                          (0.5f + (float)Ky) * wy),
+                                    fmaxf((0.5f + (float)Kz) * wz, kv * g.s1f));
+      const float sc = __uint_as_float((253u - (__float_as_uint(M) >> 23)) << 23);  // 2^-(e+1)
+      const float T = fmaf(sc * sc, g.tile_c * 1.000001f, 0x1p-14f);
+      const float kb = kv * sc;
+      store_row(w.rec, lane, fmaf(o.ox, sc, -ox * sc), fmaf(o.oy, sc, -oy * sc),
+                fmaf(o.oz, sc, -oz * sc), o.vx * kb, o.vy * kb, o.vz * kb, T, (run >> lane) & 1u);
+      __syncwarp();
+      uint32_t A[2][4];
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        const uint2 lo = words[2 * (16 * t + frag)], hi = words[2 * (16 * t + 8 + frag)];
+        A[t][0] = lo.x; A[t][1] = hi.x; A[t][2] = lo.y; A[t][3] = hi.y;
+      }
+
+      // 3. the tiles
+      uint32_t P = 0;  // piece that holds slot `base`
+      for (uint32_t base = 0; base < total; base += 32) {
+        const uint32_t slot = base + lane;
+        uint32_t j, jc = 0;
+        float qx = -ox * sc, qy = -oy * sc, qz = -oz * sc;
+        if (plain) {
+          uint32_t off = o0;
+          jc = kOwnColumn;
+          if (slot >= s1) { off = o1; jc = 0; }
+          if (slot >= s2) off = o2;
+          if (slot >= s3) off = o3;
+          if (slot >= s4) off = o4;
+          j = slot + off;
+        } else {
+          // pieces starting inside the tile (at most 31, each non-empty, among P + 1 ..
+          // P + 31) mark their first slot in one OR
+          const uint32_t st = P + lane < pieces ? w.start[P + lane] : kNone;
+          const uint32_t bit = (st > base && st - base < 32u) ? 1u << (st - base) : 0u;
+          const uint32_t marks = __reduce_or_sync(kAll, bit);
+          const uint32_t pi = P + __popc(marks & (kAll >> (31u - lane)));
+          j = w.first[pi] + (slot - w.start[pi]);
+          jc = w.code[pi];
+          qx = -(ox - image_shift(jc, g.Lf[0])) * sc;
+          qy = -(oy - image_shift(jc >> 2, g.Lf[1])) * sc;
+          qz = -(oz - image_shift(jc >> 4, g.Lf[2])) * sc;
+          // the next tile starts in lane 31's piece or in the one after it
+          P = __shfl_sync(kAll, pi, 31);
+          if (P + 1u < pieces && w.start[P + 1u] <= base + 32u) ++P;
+        }
+        float ax = 0, ay = 0, az = 0, bx = 0, by = 0, bz = 0, far = kFar;
+        if (slot < total) {
+          const Own32 e = record32<PREC>(s, MM, cur, j);
+          ax = fmaf(e.ox, sc, qx);
+          ay = fmaf(e.oy, sc, qy);
+          az = fmaf(e.oz, sc, qz);
+          bx = e.vx * kb;
+          by = e.vy * kb;
+          bz = e.vz * kb;
+          far = 0.0f;
+        }
+        store_partner(w.rec, lane, ax, ay, az, bx, by, bz, far);
+        w.info[lane] = make_uint2(j, jc);
+        __syncwarp();
+        uint32_t mask = 0;
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+          const uint2 b = words[2 * (8 * n + frag)];
+#pragma unroll
+          for (int t = 0; t < 2; ++t) {
+            float d[4];
+            mma_form(d, A[t], b);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) mask = __funnelshift_l(__float_as_uint(d[e]), mask, 1);
+          }
+        }
+        // in the own column (its first piece) only later partners than the row
+        if (base == 0u) mask &= lead == 0 ? later : ~self_bits((uint32_t)lead + 1u, frag, quad);
+        // survivors to the queue, one per lane and turn; 32 of them are tested at a time
+        for (unsigned any; (any = __ballot_sync(kAll, mask != 0u)) != 0u;) {
+          if (mask) {
+            const uint32_t at = (uint32_t)__clz((int)mask);  // accumulators in order
+            mask &= ~(0x80000000u >> at);
+            const uint32_t row = (at & 4u) * 4u + (at & 2u) * 4u + frag;
+            const uint2 ji = w.info[(at & 24u) + quad * 2u + (at & 1u)];
+            const uint32_t to = queued + __popc(any & ((1u << lane) - 1u));
+            w.queue[to] = make_uint2(p0 + row, ji.x);
+            w.qcode[to] = ji.y;
+          }
+          queued += __popc(any);
+          if (queued >= 32u) {
+            __syncwarp();
+            queued -= 32u;
+            test_survivor<PREC, K>(s, w.buf, &w.count, w.queue[queued + lane], w.qcode[queued + lane]);
+            __syncwarp();
+            if (w.count >= (uint32_t)(kWarpBuf / 2)) flush_lanes(w.buf, &w.count, s, lane);
+          }
+        }
+        __syncwarp();  // fragments and survivors are read before the next tile's records
+      }
+    }
+  }
+  if (kcur >= 0) finish(*B.sims[kcur]);
+}
+
 
 // --------------------------------------------------------------------------- //
 // Fast particles of the speed split: one warp per fast particle p, searching cfast
@@ -1177,8 +1171,7 @@ __global__ void __launch_bounds__(kTile, 4) k_search_rows32(Batch B) {
 // is contiguous in the cell order, so a column costs four loads of the cell table
 // whatever its length.  A warp prefix sum over the lanes' test counts then deals the
 // tests of 32 columns out to the lanes, so every lane tests a pair in every
-// iteration whatever the occupancies.  The pair tests are those of the
-// thread-per-particle search.
+// iteration whatever the occupancies.  The pair tests are those of the other searches.
 template <int PREC>
 __global__ void __launch_bounds__(kCellWarps * 32, 4) k_search_fast(Batch B) {
   __shared__ uint2 wbuf[kCellWarps][kWarpBuf];
@@ -1233,9 +1226,7 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4) k_search_fast(Batch B) {
     const double* __restrict__ V2 = s.v[cur][2];
     const float4* __restrict__ MM = s.mir;
     const double L0 = s.box[0], L1 = s.box[1], L2 = s.box[2];
-    Guard32 q;
-    q.c0 = g.s_c0; q.c1 = g.s_c1; q.ag = g.a_g; q.tg = g.t_g; q.dtf = g.dtf;
-    q.d0up = g.d0up; q.brel = g.b_rel; q.babs = g.b_abs; q.we = g.w_e; q.wrel = g.w_rel;
+    const Guard32 q = guard_of(g);
     const float Lf0 = g.Lf[0], Lf1 = g.Lf[1], Lf2 = g.Lf[2];
     unsigned long long tests = 0;
 
@@ -1453,74 +1444,68 @@ int resident_blocks(F kernel, int threads, size_t smem, int num_sms) {
   }
   return per_sm * num_sms;
 }
+
+template <int PREC, int K>
+void grids_of(int num_sms, uint32_t ptiles, LaunchPlan& L) {
+  auto cap = [&](int blocks) { return (int)std::min<uint32_t>((uint32_t)blocks, std::max(ptiles, 1u)); };
+  L.part_blocks = cap(resident_blocks(k_search<PREC, K>, kTile, 0, num_sms));
+  L.tile_blocks = cap(resident_blocks(k_search_tiles<PREC, K>, kTile, 0, num_sms));
+  L.fast_blocks = cap(resident_blocks(k_search_fast<PREC>, kCellWarps * 32, 0, num_sms));
+  if (PREC != KMC_GUARDED_FP32) return;
+  // the row search keeps its piece lists in dynamic shared memory (above 48 KB for
+  // K = 2); set before any launch or capture
+  cudaFuncSetAttribute(k_search_rows32<K, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)RowLayout<K, true>::kBytes);
+  cudaFuncSetAttribute(k_search_rows32<K, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)RowLayout<K, false>::kBytes);
+  L.row_blocks = cap(resident_blocks(k_search_rows32<K, false>, kTile, RowLayout<K, false>::kBytes, num_sms));
+  L.row_blocks_px = cap(resident_blocks(k_search_rows32<K, true>, kTile, RowLayout<K, true>::kBytes, num_sms));
+}
+
+// Every search that a simulation of the plan may choose for a step; each runs the one its
+// grid selected (the other kernels return at once).
+template <int PREC, int K>
+int launch_slow(const LaunchPlan& L, cudaStream_t st) {
+  int n = 1;
+  k_search_tiles<PREC, K><<<L.tile_blocks, kTile, 0, st>>>(L.b);
+  if (L.particle) {
+    k_search<PREC, K><<<L.part_blocks, kTile, 0, st>>>(L.b);
+    ++n;
+  }
+  if (PREC == KMC_GUARDED_FP32 && L.bounded_x) {
+    k_search_rows32<K, false><<<L.row_blocks, kTile, RowLayout<K, false>::kBytes, st>>>(L.b);
+    ++n;
+  }
+  if (PREC == KMC_GUARDED_FP32 && L.periodic_x) {
+    k_search_rows32<K, true><<<L.row_blocks_px, kTile, RowLayout<K, true>::kBytes, st>>>(L.b);
+    ++n;
+  }
+  return n;
+}
 }  // namespace
 
 void search_grids(int precision, int K, int num_sms, uint32_t ptiles, LaunchPlan& L) {
-  auto cap = [&](int blocks) { return (int)std::min<uint32_t>((uint32_t)blocks, std::max(ptiles, 1u)); };
   if (precision == KMC_FP64) {
-    L.cell_blocks = K == 2 ? resident_blocks(k_search_cell<KMC_FP64, 2>, kCellWarps * 32, 0, num_sms)
-                           : resident_blocks(k_search_cell<KMC_FP64, 1>, kCellWarps * 32, 0, num_sms);
-    L.part_blocks = cap(K == 2 ? resident_blocks(k_search<KMC_FP64, 2>, kTile, 0, num_sms)
-                               : resident_blocks(k_search<KMC_FP64, 1>, kTile, 0, num_sms));
-    L.row_blocks = 0;
-    L.row_blocks_px = 0;
-    L.fast_blocks = cap(resident_blocks(k_search_fast<KMC_FP64>, kCellWarps * 32, 0, num_sms));
-    return;
-  }
-  // the row search keeps its piece lists in dynamic shared memory (above 48 KB for
-  // K = 2); set before any launch or capture
-  if (K == 2) {
-    cudaFuncSetAttribute(k_search_rows32<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)RowLayout<2, true>::kBytes);
-    cudaFuncSetAttribute(k_search_rows32<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)RowLayout<2, false>::kBytes);
-    L.cell_blocks = resident_blocks(k_search_cell32<2>, kCellWarps * 32, 0, num_sms);
-    L.part_blocks = cap(resident_blocks(k_search<KMC_GUARDED_FP32, 2>, kTile, 0, num_sms));
-    L.row_blocks = cap(resident_blocks(k_search_rows32<2, false>, kTile, RowLayout<2, false>::kBytes, num_sms));
-    L.row_blocks_px = cap(resident_blocks(k_search_rows32<2, true>, kTile, RowLayout<2, true>::kBytes, num_sms));
+    if (K == 2) grids_of<KMC_FP64, 2>(num_sms, ptiles, L);
+    else grids_of<KMC_FP64, 1>(num_sms, ptiles, L);
   } else {
-    cudaFuncSetAttribute(k_search_rows32<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)RowLayout<1, true>::kBytes);
-    cudaFuncSetAttribute(k_search_rows32<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)RowLayout<1, false>::kBytes);
-    L.cell_blocks = resident_blocks(k_search_cell32<1>, kCellWarps * 32, 0, num_sms);
-    L.part_blocks = cap(resident_blocks(k_search<KMC_GUARDED_FP32, 1>, kTile, 0, num_sms));
-    L.row_blocks = cap(resident_blocks(k_search_rows32<1, false>, kTile, RowLayout<1, false>::kBytes, num_sms));
-    L.row_blocks_px = cap(resident_blocks(k_search_rows32<1, true>, kTile, RowLayout<1, true>::kBytes, num_sms));
+    if (K == 2) grids_of<KMC_GUARDED_FP32, 2>(num_sms, ptiles, L);
+    else grids_of<KMC_GUARDED_FP32, 1>(num_sms, ptiles, L);
   }
-  L.fast_blocks = cap(resident_blocks(k_search_fast<KMC_GUARDED_FP32>, kCellWarps * 32, 0, num_sms));
 }
 
 int launch_search(const LaunchPlan& L, int precision, int K, cudaStream_t st, cudaEvent_t* ev_slow) {
-  // every search kernel is launched; each simulation runs in the one its grid selected
-  // (the others return at once)
-  const int cb = L.cell_blocks;
+  int n = 0;
   if (ev_slow) cudaEventRecord(ev_slow[0], st);
   if (precision == KMC_FP64) {
-    if (K == 2) {
-      k_search<KMC_FP64, 2><<<L.part_blocks, kTile, 0, st>>>(L.b);
-      k_search_cell<KMC_FP64, 2><<<cb, kCellWarps * 32, 0, st>>>(L.b);
-    } else {
-      k_search<KMC_FP64, 1><<<L.part_blocks, kTile, 0, st>>>(L.b);
-      k_search_cell<KMC_FP64, 1><<<cb, kCellWarps * 32, 0, st>>>(L.b);
-    }
+    n = K == 2 ? launch_slow<KMC_FP64, 2>(L, st) : launch_slow<KMC_FP64, 1>(L, st);
   } else {
-    if (K == 2) {
-      k_search<KMC_GUARDED_FP32, 2><<<L.part_blocks, kTile, 0, st>>>(L.b);
-      k_search_cell32<2><<<cb, kCellWarps * 32, 0, st>>>(L.b);
-      k_search_rows32<2, false><<<L.row_blocks, kTile, RowLayout<2, false>::kBytes, st>>>(L.b);
-      k_search_rows32<2, true><<<L.row_blocks_px, kTile, RowLayout<2, true>::kBytes, st>>>(L.b);
-    } else {
-      k_search<KMC_GUARDED_FP32, 1><<<L.part_blocks, kTile, 0, st>>>(L.b);
-      k_search_cell32<1><<<cb, kCellWarps * 32, 0, st>>>(L.b);
-      k_search_rows32<1, false><<<L.row_blocks, kTile, RowLayout<1, false>::kBytes, st>>>(L.b);
-      k_search_rows32<1, true><<<L.row_blocks_px, kTile, RowLayout<1, true>::kBytes, st>>>(L.b);
-    }
+    n = K == 2 ? launch_slow<KMC_GUARDED_FP32, 2>(L, st) : launch_slow<KMC_GUARDED_FP32, 1>(L, st);
   }
   if (ev_slow) cudaEventRecord(ev_slow[1], st);
   if (precision == KMC_FP64) k_search_fast<KMC_FP64><<<L.fast_blocks, kCellWarps * 32, 0, st>>>(L.b);
   else k_search_fast<KMC_GUARDED_FP32><<<L.fast_blocks, kCellWarps * 32, 0, st>>>(L.b);
-  return precision == KMC_FP64 ? 3 : 5;
+  return n + 1;
 }
 
 }  // namespace kmc

@@ -20,7 +20,7 @@ from .sim import Simulation, params_from_setup
 
 DEFAULT_CANDIDATES = [
     # (search_kernel, stencil, cell_scale, split_min_occ): kernels 0 auto, 1 particle,
-    # 2 cell, 3 row; split_min_occ = smallest mean slow-cell occupancy a speed split
+    # 2 tiles, 3 row; split_min_occ = smallest mean slow-cell occupancy a speed split
     # may leave (0: no floor, 1e9: no split)
     (0, 1, 1.0, 0.0), (0, 1, 1.0, 2.0), (0, 1, 1.0, 4.0), (0, 1, 1.0, 8.0),
     (0, 1, 1.0, 1e9), (2, 1, 1.0, 1e9), (2, 1, 1.0, 16.0), (2, 1, 1.0, 8.0),
