@@ -78,8 +78,10 @@ struct kmc_sim {
   // group's issued-step count then, so that a sync can tell how many of the group's
   // steps this member missed after an overflow
   uint64_t sync_step = 0, issued_base = 0;
-  // a decomposition into x slabs (sim_create_domains): the steps run on its domains
+  // a decomposition into x slabs (sim_create_domains): the steps run on its domains,
+  // which match over per-particle candidate lists
   struct Domains* dom = nullptr;
+  bool lists = false;
   std::string err;
 };
 
@@ -142,9 +144,8 @@ Sizes sizes_of(const kmc_params& p) {
 }
 
 size_t edge_bytes(uint32_t cap) {
-  // pairs, keys, slots; candidate lists (2 per pair) and the two round work lists
-  return (size_t)cap * (sizeof(uint2) + 2 * sizeof(double) + sizeof(uint2)) +
-         (size_t)2 * cap * (sizeof(uint2) + 2 * sizeof(uint32_t));
+  // pairs, keys, candidate marks, the two lists of open pairs
+  return (size_t)cap * (sizeof(uint2) + 2 * sizeof(double) + sizeof(uint2) + 2 * sizeof(uint32_t));
 }
 
 size_t bytes_for(const Sizes& z) {
@@ -155,9 +156,8 @@ size_t bytes_for(const Sizes& z) {
   b += 3 * n * sizeof(uint32_t) + n;                                  // key, rank, src, speed class
   b += n + 4096;                                                      // mixture species (if any)
   b += 2 * ((size_t)z.cell_cap + 2) * sizeof(uint32_t);               // cell count / start
-  b += n * sizeof(uint32_t) + (n + 1) * sizeof(uint32_t);             // deg, list starts
-  b += 4 * n * sizeof(uint32_t);                                      // best, best_e, partner, medge
-  b += (n / 2 + 1) * sizeof(uint32_t);                                // pair list
+  b += 3 * n * sizeof(uint32_t);                                      // best, best_e, partner
+  b += (n / 2 + 1) * sizeof(uint32_t);                                // matched pairs
   b += edge_bytes(z.edge_cap);
   b += (size_t)z.hist_cap * sizeof(kmc_step_counts);
   if (z.bins) b += (size_t)z.prof_cap * z.bins * kProfQ * sizeof(long long) + z.prof_cap * sizeof(uint64_t);
@@ -235,9 +235,9 @@ int alloc_edges(kmc_sim* s, uint32_t cap) {
   if ((rc = dalloc(s, &h.e_d2, cap))) return rc;
   if ((rc = dalloc(s, &h.e_t, cap))) return rc;
   if ((rc = dalloc(s, &h.e_slot, cap))) return rc;
-  if ((rc = dalloc(s, &h.adj, 2 * (size_t)cap))) return rc;
-  if ((rc = dalloc(s, &h.wl[0], 2 * (size_t)cap))) return rc;
-  if ((rc = dalloc(s, &h.wl[1], 2 * (size_t)cap))) return rc;
+  if (s->lists && (rc = dalloc(s, &h.adj, 2 * (size_t)cap))) return rc;
+  if ((rc = dalloc(s, &h.wl[0], (s->lists ? 2 : 1) * (size_t)cap))) return rc;
+  if ((rc = dalloc(s, &h.wl[1], cap))) return rc;
   h.edge_cap = cap;
   return KMC_OK;
 }
@@ -276,14 +276,15 @@ int build_plan(Plan& P, const std::vector<kmc_sim*>& sims, cudaStream_t st, std:
     P.max_rounds = std::max(P.max_rounds, h.max_rounds);
     if (h.profile_bins > 0) P.has_profiles = true;
     if (h.absorb) P.L.absorb = true;
+    if (sims[k]->lists) P.L.lists = true;
     if (h.mix) P.L.mix = true;
     if (h.search_kernel == KMC_SEARCH_PARTICLE) P.L.particle = true;
     (h.bc[0] == KMC_PERIODIC ? P.L.periodic_x : P.L.bounded_x) = true;
   }
-  // prefixes (3 (m + 1) words, padded to an even count), the scan's two control
-  // words, then one 64-bit status word per scan tile
+  // prefixes (3 (m + 1) words, padded to an even count), the scan's and the rounds' two
+  // control words each, then one 64-bit status word per scan tile
   const size_t head = (3 * (size_t)(m + 1) + 1) & ~(size_t)1;
-  size_t words = head + 2 + 2 * ((size_t)sc[m] + 1);
+  size_t words = head + 4 + 2 * ((size_t)sc[m] + 1);
   if (cudaMalloc(&P.d_table, sizeof(SimDev*) * m) != cudaSuccess ||
       cudaMalloc(&P.d_pre, words * sizeof(uint32_t)) != cudaSuccess) {
     cudaGetLastError();
@@ -306,11 +307,15 @@ int build_plan(Plan& P, const std::vector<kmc_sim*>& sims, cudaStream_t st, std:
   L.b.stile_c = P.d_pre + (m + 1);
   L.b.prtile = P.d_pre + 2 * (m + 1);
   L.b.scan_ctl = P.d_pre + head;
-  L.b.tile_status = reinterpret_cast<unsigned long long*>(P.d_pre + head + 2);
+  L.b.round_ctl = P.d_pre + head + 2;
+  L.b.tile_status = reinterpret_cast<unsigned long long*>(P.d_pre + head + 4);
   L.ptiles = pt[m];
   L.stiles_c = sc[m];
   L.prtiles = pr[m];
   L.edge_blocks = 8 * num_sms();
+  // a block of the later rounds per 2^16 particles (their lists hold about one pair in a
+  // thousand particles); one per SM at most, so that all of them run at once
+  L.round_blocks = (int)std::min<uint32_t>(std::max(pt[m] / 256u, 1u), (uint32_t)num_sms());
   search_grids(P.precision, P.K, num_sms(), L.ptiles, L);
   return KMC_OK;
 }
@@ -563,7 +568,8 @@ int validate_mixture(const kmc_params* p, const Mixture* m, std::string& err) {
 // shared body of sim_create (src: six state arrays), sim_create_init (init) and
 // sim_create_mixture (mix)
 int create_impl(const kmc_params* p, const double* const* src6, const uint32_t* last,
-                const kmc_init* init, const Mixture* mix, void* stream, kmc_sim** out) {
+                const kmc_init* init, const Mixture* mix, void* stream, kmc_sim** out,
+                bool lists = false) {
   if (out) *out = nullptr;
   g_create_error.clear();
   int rc = validate(p, g_create_error);
@@ -577,6 +583,7 @@ int create_impl(const kmc_params* p, const double* const* src6, const uint32_t* 
   kmc_sim* s = new (std::nothrow) kmc_sim();
   if (!s) { g_create_error = "out of host memory"; return KMC_ENOMEM; }
   s->p = *p;
+  s->lists = lists;
   if (stream) {
     s->stream = (cudaStream_t)stream;
   } else {
@@ -649,12 +656,14 @@ int create_impl(const kmc_params* p, const double* const* src6, const uint32_t* 
   // cell keys (at most cell_cap), the absorbed particles' key, the total
   if ((rc = dalloc(s, &h.cell_count, (size_t)zs.cell_cap + 2))) return fail(rc);
   if ((rc = dalloc(s, &h.cell_start, (size_t)zs.cell_cap + 2))) return fail(rc);
-  if ((rc = dalloc(s, &h.deg, n))) return fail(rc);
-  if ((rc = dalloc(s, &h.off, n + 1))) return fail(rc);
   if ((rc = dalloc(s, &h.best, n))) return fail(rc);
   if ((rc = dalloc(s, &h.best_e, n))) return fail(rc);
   if ((rc = dalloc(s, &h.partner, n))) return fail(rc);
-  if ((rc = dalloc(s, &h.medge, n))) return fail(rc);
+  if (lists) {
+    if ((rc = dalloc(s, &h.deg, n))) return fail(rc);
+    if ((rc = dalloc(s, &h.off, n + 1))) return fail(rc);
+    if ((rc = dalloc(s, &h.medge, n))) return fail(rc);
+  }
   if ((rc = dalloc(s, &h.pairs, n / 2 + 1))) return fail(rc);
   if ((rc = alloc_edges(s, zs.edge_cap))) return fail(rc);
   if ((rc = dalloc(s, &h.hist, zs.hist_cap))) return fail(rc);
@@ -837,7 +846,7 @@ int dom_create(const kmc_params* p, uint32_t ndom, const double* const* src6, co
   const double* mem6[6] = {h.x[0], h.x[1], h.x[2], h.v[0], h.v[1], h.v[2]};
   for (uint32_t k = 0; k < ndom; ++k) {
     kmc_sim* m = nullptr;
-    rc = create_impl(&q, mem6, h.last, nullptr, nullptr, st, &m);
+    rc = create_impl(&q, mem6, h.last, nullptr, nullptr, st, &m, true);
     if (rc) {
       s->err = g_create_error;
       return fail(rc);

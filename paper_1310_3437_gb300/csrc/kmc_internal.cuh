@@ -87,10 +87,10 @@ struct Dyn {
   uint32_t n_raw;       // pairs emitted by the search (may exceed edge_cap)
   uint32_t n_edges;     // candidate pairs after the exact test
   uint32_t round_pairs[4];
-  uint32_t n_pairs;     // entries of the pair list
-  uint32_t adj_used;    // candidate-list entries handed out this step
-  uint32_t wl_len[5];   // particles on the work list of matching round r (0: all with
-                        // candidates; r + 1 is filled by round r)
+  uint32_t n_pairs;     // entries of pairs
+  uint32_t adj_used;    // domains: candidate-list entries handed out this step
+  uint32_t wl_len[5];   // open pairs before matching round r >= 1, filled by round r - 1
+                        // (domains: [0] particles with candidates)
   unsigned long long pair_tests;
   unsigned long long fast_tests;  // the part of pair_tests done by the fast-particle search
   uint32_t last_raw;    // n_raw of the last completed step (its pair buffer is kept)
@@ -131,20 +131,21 @@ struct SimDev {
   uint32_t* src;        // pre-sort position of the particle at each sorted position
   uint32_t* cell_count; // nkeys counters, all zero between steps
   uint32_t* cell_start; // nkeys + 1
-  uint32_t* deg;        // candidate pairs per particle
-  uint32_t* off;        // start of each particle's candidate list in adj (set for deg > 0)
+  uint32_t* deg;        // domains: candidate pairs per particle
+  uint32_t* off;        // domains: start of each particle's candidate list in adj
   uint2* edge;          // emitted pairs (sorted indices, owner first)
   double* e_d2;         // binary64 key of each pair
   double* e_t;
-  uint2* e_slot;        // slot of the pair in each endpoint's list, x = kNone if rejected
-  uint2* adj;           // candidate lists, each particle's contiguous: (other end, pair)
-  uint32_t* wl[2];      // work lists of the matching rounds (unmatched particles that
-                        // still had an unmatched candidate), used alternately
-  uint32_t* best;       // best unmatched candidate (sorted index) in the current round
-  uint32_t* best_e;
+  uint2* e_slot;        // x = kNone if the pair is no candidate (domains: its slot in each
+                        // endpoint's list)
+  uint2* adj;           // domains: candidate lists, each particle's contiguous: (other end, pair)
+  uint32_t* wl[2];      // open pairs of the matching rounds, used alternately (domains: [0]
+                        // the particles with candidates)
+  uint32_t* best;       // chosen pair of each particle in odd rounds (domains: chosen partner)
+  uint32_t* best_e;     // chosen pair in even rounds (domains: of the chosen partner)
   uint32_t* partner;    // partner (sorted index) this step, kNone if none
-  uint32_t* medge;      // pair index of the collision
-  uint32_t* pairs;      // colliding pairs of the step, by their smaller-id member
+  uint32_t* medge;      // domains: pair index of the collision
+  uint32_t* pairs;      // the step's matched pairs (domains: their smaller-id members)
   kmc_step_counts* hist;
   long long* prof_acc;  // prof_cap x bins x kProfQ fixed-point counters
   uint64_t* prof_step;
@@ -172,6 +173,7 @@ struct Batch {
   // value), and the control words [0] next tile to hand out, [1] current epoch
   unsigned long long* tile_status;
   uint32_t* scan_ctl;
+  uint32_t* round_ctl;     // grid barrier of the later matching rounds: arrivals, generation
 };
 
 __device__ __forceinline__ int find_sim(const uint32_t* prefix, int nsims, uint32_t tile) {
@@ -481,6 +483,8 @@ struct LaunchPlan {
   Batch b;
   uint32_t ptiles, stiles_c, prtiles;
   int edge_blocks;
+  int round_blocks;        // cooperative grid of the later matching rounds
+  bool lists = false;      // domains: the rounds work on per-particle candidate lists
   int part_blocks;  // grid-stride grids of the particle, tiled, row and fast searches
   int tile_blocks;
   int row_blocks;     // row search, no periodic x axis

@@ -11,76 +11,73 @@
 //             r = x_j - x_i (minimum image on periodic axes), v = v_j - v_i,
 //             t* = -(r.v)/|v|^2, d_min^2 = |r x v|^2/|v|^2; candidate iff |v| != 0,
 //             0 <= t* < dt, d_min^2 < d0^2, and the pair is not the pair that last
-//             collided for both of its members.  Survivors take a slot in each
-//             endpoint's candidate list.
-//   k_alloc   each particle with candidates gets a contiguous list (one warp-
-//             aggregated atomic per warp) and a place on the first round's work list;
-//             only the particles with candidates are touched, no pass over all n.
-//   k_fill    the lists: (other end, pair) per slot.
-//   k_best    per round, over the round's work list: every unmatched particle picks
-//             its unmatched candidate of least key (d_min^2, t*, partner id) -- a
-//             total order, so the choice does not depend on the order of the list.
-//   k_mutual  per round, over the same list: pairs that picked each other are
-//             matched (warp-aggregated appends); a particle left unmatched that still
-//             had an unmatched candidate goes on the next round's list, so later
-//             rounds only visit the few particles they can still match.
-//   k_collide isotropic centre-of-mass scatter at the time of closest approach.
-#include <algorithm>
-
+//             collided for both of its members.  Candidates propose themselves to both
+//             members, which keep the one of least key.
+//   k_settle  pairs that both members chose are matched; pairs with both members left
+//             unmatched go to the next round.
+//   k_rounds  the further rounds, in one launch: propose, settle.
+//   k_collide isotropic centre-of-mass scatter of the matched pairs at the time of closest
+//             approach.
+// A domain decomposition exchanges choices between its domains inside every round, by
+// particle: there k_refine hands out slots, k_alloc and k_fill build each particle's
+// candidate list (only particles with candidates are touched), and kmc_domain.cu runs the
+// rounds over them.
 #include "kmc_internal.cuh"
 #include "kmc_rng.cuh"
 
 namespace kmc {
 
-// Point on the unit sphere by Marsaglia's method (Ann. Math. Stat. 43, 1972):
-// u1, u2 uniform in [-1, 1) from 32-bit words, s = u1^2 + u2^2 accepted if
-// 0 < s < 1, n = (2 u1 sqrt(1-s), 2 u2 sqrt(1-s), 1 - 2 s).  Counter (id, step lo,
-// k, step hi), key (seed lo, seed hi); two attempts per Philox call.
-__device__ bool sphere_point(uint64_t seed, uint64_t step, uint32_t id, double nv[3]) {
+// The point (u1, u2) of the unit disk from 32-bit words, u = w 2^-31 - 1 uniform in
+// [-1, 1): accepted if 0 < s < 1 with s = fl(fl(u1^2) + fl(u2^2)).  Counter (id, step lo, k,
+// step hi), key (seed lo, seed hi); two attempts per Philox call, both evaluated and the
+// first accepted one kept, so that lanes whose first attempt fails do not split the warp.
+// The acceptance is decided on integers (the binary64 pipe has two lanes per SM): with
+// a = |w - 2^31|, s 2^62 is a1^2 + a2^2 within three roundings of 2^9 each, so outside
+// 2^11 of 2^62 the exact sum decides alike, and inside the binary64 sum is formed.
+__device__ __forceinline__ bool in_disk(uint32_t w1, uint32_t w2) {
+  const uint32_t a1 = w1 >= 0x80000000u ? w1 - 0x80000000u : 0x80000000u - w1;
+  const uint32_t a2 = w2 >= 0x80000000u ? w2 - 0x80000000u : 0x80000000u - w2;
+  const unsigned long long q = (unsigned long long)a1 * a1 + (unsigned long long)a2 * a2;
+  constexpr unsigned long long one = 1ull << 62, zone = 1ull << 11;
+  if (q < one - zone) return q != 0ull;
+  if (q > one + zone) return false;
+  const double u1 = word_uniform(w1), u2 = word_uniform(w2);
+  return dadd(dmul(u1, u1), dmul(u2, u2)) < 1.0;
+}
+
+__device__ __forceinline__ bool disk_point(uint64_t seed, uint64_t step, uint32_t id, double& u1,
+                                           double& u2) {
   for (uint32_t k = 0; k < 64; ++k) {
     uint32_t c[4] = {id, (uint32_t)step, k, (uint32_t)(step >> 32)};
     philox4x32_10(c, (uint32_t)seed, (uint32_t)(seed >> 32));
-    // both attempts of the call are evaluated and the first accepted one is kept, so
-    // that lanes whose first attempt fails do not split the warp
-    const double u1a = word_uniform(c[0]), u2a = word_uniform(c[1]);
-    const double u1b = word_uniform(c[2]), u2b = word_uniform(c[3]);
-    const double sa = dadd(dmul(u1a, u1a), dmul(u2a, u2a));
-    const double sb = dadd(dmul(u1b, u1b), dmul(u2b, u2b));
-    const bool oka = sa > 0.0 && sa < 1.0, okb = sb > 0.0 && sb < 1.0;
+    const bool oka = in_disk(c[0], c[1]), okb = in_disk(c[2], c[3]);
     if (oka || okb) {
-      const double u1 = oka ? u1a : u1b, u2 = oka ? u2a : u2b, s = oka ? sa : sb;
-      const double q = dsqrt(dsub(1.0, s));
-      nv[0] = dmul(dadd(u1, u1), q);
-      nv[1] = dmul(dadd(u2, u2), q);
-      nv[2] = dsub(1.0, dadd(s, s));
+      u1 = word_uniform(oka ? c[0] : c[2]);
+      u2 = word_uniform(oka ? c[1] : c[3]);
       return true;
     }
   }
   return false;
 }
 
-// Planar mode: a direction uniform on the unit circle from the same counters.  A point
-// (u1, u2) uniform in the unit disk (the same rejection) has a uniform polar angle;
-// the vector at twice that angle, ((u1^2 - u2^2)/s, (2 u1 u2)/s), is uniform on the
-// circle (von Neumann's method, no trigonometric function).
-__device__ bool circle_point(uint64_t seed, uint64_t step, uint32_t id, double nv[3]) {
-  for (uint32_t k = 0; k < 64; ++k) {
-    uint32_t c[4] = {id, (uint32_t)step, k, (uint32_t)(step >> 32)};
-    philox4x32_10(c, (uint32_t)seed, (uint32_t)(seed >> 32));
-    const double u1a = word_uniform(c[0]), u2a = word_uniform(c[1]);
-    const double u1b = word_uniform(c[2]), u2b = word_uniform(c[3]);
-    const double sa = dadd(dmul(u1a, u1a), dmul(u2a, u2a));
-    const double sb = dadd(dmul(u1b, u1b), dmul(u2b, u2b));
-    const bool oka = sa > 0.0 && sa < 1.0, okb = sb > 0.0 && sb < 1.0;
-    if (oka || okb) {
-      const double u1 = oka ? u1a : u1b, u2 = oka ? u2a : u2b, s = oka ? sa : sb;
-      nv[0] = ddiv(dsub(dmul(u1, u1), dmul(u2, u2)), s);
-      nv[1] = ddiv(dmul(dadd(u1, u1), u2), s);
-      nv[2] = 0.0;
-      return true;
-    }
-  }
-  return false;
+// Point on the unit sphere by Marsaglia's method (Ann. Math. Stat. 43, 1972):
+// n = (2 u1 sqrt(1-s), 2 u2 sqrt(1-s), 1 - 2 s).
+__device__ __forceinline__ void sphere_point(double u1, double u2, double nv[3]) {
+  const double s = dadd(dmul(u1, u1), dmul(u2, u2));
+  const double q = dsqrt(dsub(1.0, s));
+  nv[0] = dmul(dadd(u1, u1), q);
+  nv[1] = dmul(dadd(u2, u2), q);
+  nv[2] = dsub(1.0, dadd(s, s));
+}
+
+// Planar mode: a direction uniform on the unit circle from the same point, whose polar
+// angle is uniform: the vector at twice that angle, ((u1^2 - u2^2)/s, (2 u1 u2)/s) (von
+// Neumann's method, no trigonometric function).
+__device__ __forceinline__ void circle_point(double u1, double u2, double nv[3]) {
+  const double q1 = dmul(u1, u1), q2 = dmul(u2, u2), s = dadd(q1, q2);
+  nv[0] = ddiv(dsub(q1, q2), s);
+  nv[1] = ddiv(dmul(dadd(u1, u1), u2), s);
+  nv[2] = 0.0;
 }
 
 __device__ __forceinline__ double min_image(double r, double L) {
@@ -98,17 +95,36 @@ __device__ __forceinline__ double min_image(double r, double L) {
 // of up to kEdgeBlock members at once, one thread each (walked one member after
 // another, the counts were a chain of dependent loads of about a microsecond per
 // member and kernel), places the members by a block-wide scan of the blocks each one
-// spans, and visits only the members it holds items of.  count(s) gives member s's
-// items from fields that stay fixed during the launch, so every block deals alike; the
-// status word is read once per member and block.  body(s, first, trips) does the
-// block's share: items first, first + stride, ..., trips of them per thread, the same
-// trips for every thread of the block (the last may lie past the end), so body may use
-// block-wide appends.  Blocks of kEdgeBlock threads.
+// spans, and visits only the members it holds items of.  A lone simulation skips all
+// that, and when its items are fewer than the grid's threads they are dealt 32 at a time,
+// to warp 0 of every block, then to warp 1: the 2500 collisions of a 50 k tube sat on ten
+// SMs, whose binary64 pipes (two lanes each) they kept busy; spread over 78 they take 15 us
+// instead of 19.  (For more items, and for the members of a group, whole blocks are better: 1.54
+// against 1.71 ms for the collisions of 10^8 particles, 27 against 49 us for the exact
+// tests of a 30-member ensemble, whose blocks would visit more members each.)  count(s)
+// gives member s's items from fields that stay fixed during the launch, so every block
+// deals alike; the status word is read once per member and block.  body(s, first, trips)
+// does the block's share: items first, first + stride, ..., trips of them per thread,
+// stride = gridDim.x * kEdgeBlock, the same trips for every thread of the block (the last
+// may lie past the end), so body may use block-wide appends.  Blocks of kEdgeBlock
+// threads.
 template <class Count, class Body>
 __device__ __forceinline__ void for_dealt(const Batch& B, Count count, Body body) {
   __shared__ uint32_t s_first[kEdgeBlock], s_trips[kEdgeBlock], s_wsum[kEdgeBlock / 32];
   const uint32_t nb = gridDim.x, stride = nb * (uint32_t)kEdgeBlock;
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  if (B.nsims == 1) {
+    SimDev& s = *B.sims[0];
+    const uint32_t c = count(s);
+    // one answer for the block (the status word can change during the launch)
+    if (!__syncthreads_and(s.d.status == 0)) return;
+    const bool spread = c <= stride;
+    const uint32_t at = blockIdx.x * (spread ? 32u : (uint32_t)kEdgeBlock);
+    if (c > at)
+      body(s, spread ? at + warp * nb * 32u + lane : at + threadIdx.x,
+           spread ? 1u : (uint32_t)(((uint64_t)(c - at) + stride - 1) / stride));
+    return;
+  }
   uint32_t base = 0;  // the block where the chunk's first member starts
   for (int k0 = 0; k0 < B.nsims; k0 += kEdgeBlock) {
     const int k = k0 + (int)threadIdx.x;
@@ -157,14 +173,168 @@ __device__ __forceinline__ uint32_t raw_pairs(const SimDev& s) {
   return s.d.n_raw < s.edge_cap ? s.d.n_raw : s.edge_cap;
 }
 
-// ---- k_refine ------------------------------------------------------------ //
-// MIX: the plan has a mixture (per-pair contact distance, mass-weighted scatter)
+// ---- collision update ------------------------------------------------------ //
+// For the pair (a, b) with a the smaller id: stream both to t*, scatter
+//   g = v_a - v_b, V = (v_a + v_b) * 0.5, G = |g|,  v_a' = V + (G/2) n,  v_b' = V - (G/2) n,
+// then stream the rest of the step:  x' = (x + v t*) + v' (dt - t*).
+// (i the smaller id's position, j the other's.)  Everything is loaded before the first
+// store: a load after one would have to wait for it (the compiler cannot know that the
+// arrays do not overlap).
 template <bool MIX>
+__device__ __forceinline__ void collide_pair(SimDev& s, int cur, uint32_t i, uint32_t j,
+                                             uint32_t ida, uint32_t idb, double t) {
+  double* const px[3] = {s.x[cur][0], s.x[cur][1], s.x[cur][2]};
+  double* const pv[3] = {s.v[cur][0], s.v[cur][1], s.v[cur][2]};
+  const double dt = s.dt;
+  double xa[3], xb[3], va[3], vb[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    va[c] = pv[c][i];
+    vb[c] = pv[c][j];
+    xa[c] = px[c][i];
+    xb[c] = px[c][j];
+  }
+  // equal masses: V = (v_a + v_b)/2 and both get half the relative speed; a mixture:
+  // V = (m_a v_a + m_b v_b)/M, v_a' = V + (m_b/M) G n, v_b' = V - (m_a/M) G n
+  const bool mixed = MIX && s.mix;
+  double ma = 1.0, mb = 1.0;
+  if (mixed) {
+    ma = s.sp_mass[s.species[ida]];
+    mb = s.sp_mass[s.species[idb]];
+  }
+  double u1, u2, nv[3];
+  if (!disk_point(s.seed, s.d.step, ida, u1, u2)) {
+    atomicOr(&s.d.status, ST_RANDOM);
+    return;
+  }
+  if (s.planar) circle_point(u1, u2, nv);
+  else sphere_point(u1, u2, nv);
+  double g[3], V[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) g[c] = dsub(va[c], vb[c]);
+  double fa = 0.5, fb = 0.5;
+  if (mixed) {
+    const double M = dadd(ma, mb);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) V[c] = ddiv(dadd(dmul(ma, va[c]), dmul(mb, vb[c])), M);
+    fa = ddiv(mb, M);
+    fb = ddiv(ma, M);
+  } else {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) V[c] = dmul(dadd(va[c], vb[c]), 0.5);
+  }
+  double G = dsqrt(dadd(dadd(dmul(g[0], g[0]), dmul(g[1], g[1])), dmul(g[2], g[2])));
+  const double hGa = dmul(fa, G);
+  const double hGb = dmul(fb, G);
+  double rest = dsub(dt, t);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    double na = dadd(V[c], dmul(hGa, nv[c]));
+    double nb = dsub(V[c], dmul(hGb, nv[c]));
+    px[c][i] = dadd(dadd(xa[c], dmul(va[c], t)), dmul(na, rest));
+    px[c][j] = dadd(dadd(xb[c], dmul(vb[c], t)), dmul(nb, rest));
+    pv[c][i] = na;
+    pv[c][j] = nb;
+  }
+}
+
+// ---- matching by pairs ------------------------------------------------------ //
+// best[round & 1][i] is the pair that particle i chose in the round: the one of least key
+// (d_min^2, t*, partner id) among its pairs with both members unmatched -- a total order,
+// so the choice does not depend on the order in which the pairs come.  Every pair proposes
+// itself to both members (a compare-and-swap each, rarely more: a particle with candidates
+// has 1.1 of them in the tubes); a pair that both members chose is matched.  A pair is
+// still open after the round if neither member is matched in it, which the choices tell
+// without waiting for the matches; the open pairs are the next round's list.  Against
+// candidate lists per particle (built by two more launches, and two launches per round),
+// exact test to last match of a step: 62 -> 27 us at 4096 particles, 403 -> 225 us at 2^24,
+// 2.4 -> 1.2 ms at 10^8.
+__device__ __forceinline__ bool key_less(double d2a, double ta, uint32_t ja, double d2b, double tb,
+                                         uint32_t jb) {
+  if (d2a < d2b) return true;
+  if (d2a > d2b) return false;
+  if (ta < tb) return true;
+  if (ta > tb) return false;
+  return ja < jb;
+}
+
+__device__ __forceinline__ uint32_t* round_best(const SimDev& s, int round) {
+  return (round & 1) ? s.best : s.best_e;
+}
+
+// the other member of pair e
+__device__ __forceinline__ uint32_t other_end(const SimDev& s, uint32_t e, uint32_t i) {
+  const uint2 pr = __ldcg(s.edge + e);
+  return pr.x == i ? pr.y : pr.x;
+}
+
+// Pair e (key d2, t; partner id) proposes itself to particle i.  The keys of the pairs
+// that others put there are read past the L1 (written on other SMs, fenced before their
+// swap).
+__device__ __forceinline__ void propose(const SimDev& s, int cur, uint32_t* best, uint32_t i, uint32_t e,
+                                        double d2, double t, uint32_t partner_id) {
+  uint32_t seen = atomicCAS(best + i, kNone, e);
+  while (seen != kNone) {
+    if (!key_less(d2, t, partner_id, __ldcg(s.e_d2 + seen), __ldcg(s.e_t + seen),
+                  s.id[cur][other_end(s, seen, i)]))
+      return;
+    const uint32_t old = atomicCAS(best + i, seen, e);
+    if (old == seen) return;
+    seen = old;
+  }
+}
+
+// is particle i matched in the round whose choices are in best?
+__device__ __forceinline__ bool matched_by(const SimDev& s, const uint32_t* best, uint32_t i) {
+  const uint32_t e = __ldcg(best + i);
+  return __ldcg(best + other_end(s, e, i)) == e;
+}
+
+// The verdict on pair e (kNone: no pair) after the proposals of a round: 2 if both members
+// chose it, 1 if it is still open, 0 if a member was matched in another pair.
+__device__ __forceinline__ int verdict(const SimDev& s, const uint32_t* best, uint32_t e, uint2 pr) {
+  if (e == kNone) return 0;
+  const uint32_t bi = __ldcg(best + pr.x), bj = __ldcg(best + pr.y);
+  if (bi == e && bj == e) return 2;
+  return !matched_by(s, best, pr.x) && !matched_by(s, best, pr.y) ? 1 : 0;
+}
+
+// The second half of a round for the block's turn (every thread calls it): matched pairs
+// go to the list of collisions, open pairs to the next round's list with their members'
+// choices cleared.  (Colliding a pair here, right after its verdict, was slower: 512 us at
+// 2^24 particles where verdict and collisions apart take 300.)
+__device__ __forceinline__ void settle(SimDev& s, int round, uint32_t e, uint2 pr) {
+  const int v = verdict(s, round_best(s, round), e, pr);
+  const uint32_t to = block_append(&s.d.n_pairs, v == 2 ? 1u : 0u, &s.d.round_pairs[round]);
+  if (v == 2) {
+    s.pairs[to] = e;
+    s.partner[pr.x] = pr.y;
+    s.partner[pr.y] = pr.x;
+  }
+  if (round + 1 < s.max_rounds) {
+    const uint32_t at = block_append(&s.d.wl_len[round + 1], v == 1 ? 1u : 0u);
+    if (v == 1) {
+      uint32_t* next = round_best(s, round + 1);
+      s.wl[(round + 1) & 1][at] = e;
+      next[pr.x] = kNone;
+      next[pr.y] = kNone;
+    }
+  }
+}
+
+// ---- k_refine ------------------------------------------------------------ //
+// The exact test of every emitted pair, and round 0's proposals; with LISTS (a domain
+// decomposition, whose rounds exchange choices between the domains) slots in the members'
+// candidate lists instead.
+// MIX: the plan has a mixture (per-pair contact distance, mass-weighted scatter)
+template <bool MIX, bool LISTS>
 __global__ void __launch_bounds__(kEdgeBlock) k_refine(Batch B) {
   for_dealt(B, [](const SimDev& s) { return sim_scheduled(s) ? raw_pairs(s) : 0u; },
             [](SimDev& s, uint32_t first, uint32_t) {
     const int cur = s.d.parity ^ 1;
     const uint32_t nraw = raw_pairs(s);
+    const double* const px[3] = {s.x[cur][0], s.x[cur][1], s.x[cur][2]};
+    const double* const pv[3] = {s.v[cur][0], s.v[cur][1], s.v[cur][2]};
     uint32_t found = 0;
     for (uint32_t e = first; e < nraw; e += gridDim.x * kEdgeBlock) {
       uint2 pr = s.edge[e];
@@ -172,6 +342,13 @@ __global__ void __launch_bounds__(kEdgeBlock) k_refine(Batch B) {
       bool cand = false;
       double d2 = 0.0, t = 0.0;
       uint32_t idi = s.id[cur][i], idj = s.id[cur][j];
+      const uint32_t li = s.last[cur][i], lj = s.last[cur][j];
+      double r[3], v[3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        r[a] = dsub(px[a][j], px[a][i]);
+        v[a] = dsub(pv[a][j], pv[a][i]);
+      }
       // contact distance: d0, or in a mixture the sum of the two effective radii (the
       // search tested against d0, at least every such sum)
       double c2 = s.d0sq;
@@ -179,14 +356,10 @@ __global__ void __launch_bounds__(kEdgeBlock) k_refine(Batch B) {
         const double c = dadd(s.sp_radius[s.species[idi]], s.sp_radius[s.species[idj]]);
         c2 = dmul(c, c);
       }
-      if (!(s.last[cur][i] == idj && s.last[cur][j] == idi)) {
-        double r[3], v[3];
+      if (!(li == idj && lj == idi)) {
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          double dd = dsub(s.x[cur][a][j], s.x[cur][a][i]);
-          r[a] = s.bc[a] == KMC_PERIODIC ? min_image(dd, s.box[a]) : dd;
-          v[a] = dsub(s.v[cur][a][j], s.v[cur][a][i]);
-        }
+        for (int a = 0; a < 3; ++a)
+          if (s.bc[a] == KMC_PERIODIC) r[a] = min_image(r[a], s.box[a]);
         double vv = dadd(dadd(dmul(v[0], v[0]), dmul(v[1], v[1])), dmul(v[2], v[2]));
         if (vv != 0.0) {
           double rv = dadd(dadd(dmul(r[0], v[0]), dmul(r[1], v[1])), dmul(r[2], v[2]));
@@ -201,9 +374,17 @@ __global__ void __launch_bounds__(kEdgeBlock) k_refine(Batch B) {
       if (cand) {
         s.e_d2[e] = d2;
         s.e_t[e] = t;
-        uint32_t si = atomicAdd(&s.deg[i], 1u);
-        uint32_t sj = atomicAdd(&s.deg[j], 1u);
-        s.e_slot[e] = make_uint2(si, sj);
+        if (LISTS) {
+          uint32_t si = atomicAdd(&s.deg[i], 1u);
+          uint32_t sj = atomicAdd(&s.deg[j], 1u);
+          s.e_slot[e] = make_uint2(si, sj);
+        } else {
+          s.e_slot[e] = make_uint2(0u, 0u);
+          __threadfence();  // the key is there before the pair can be seen
+          uint32_t* best = round_best(s, 0);
+          propose(s, cur, best, i, e, d2, t, idj);
+          propose(s, cur, best, j, e, d2, t, idi);
+        }
         ++found;
       } else {
         s.e_slot[e] = make_uint2(kNone, kNone);
@@ -213,7 +394,106 @@ __global__ void __launch_bounds__(kEdgeBlock) k_refine(Batch B) {
   });
 }
 
-// ---- candidate lists -------------------------------------------------------- //
+// round 0's matches and open pairs
+__global__ void __launch_bounds__(kEdgeBlock) k_settle(Batch B) {
+  for_dealt(B, [](const SimDev& s) { return sim_scheduled(s) ? raw_pairs(s) : 0u; },
+            [](SimDev& s, uint32_t first, uint32_t trips) {
+    const uint32_t nraw = raw_pairs(s);
+    // the block's trip count, the same for all its threads: the appends are block-wide
+    uint32_t e = first;
+    for (uint32_t k = 0; k < trips; ++k, e += gridDim.x * kEdgeBlock) {
+      uint32_t pair = kNone;
+      uint2 pr = make_uint2(0u, 0u);
+      if (e < nraw && s.e_slot[e].x != kNone) {
+        pair = e;
+        pr = s.edge[e];
+      }
+      settle(s, 0, pair, pr);
+    }
+  });
+}
+
+// A barrier of all blocks of the launch (launched cooperatively: they all run).  The wait
+// is bounded (about a second); false: it ran out, and every block that notices leaves.
+constexpr int kGridWaitLimit = 1 << 20;  // spins of at least 0.1 us
+__device__ __forceinline__ bool grid_barrier(uint32_t* ctl) {
+  __shared__ int ok;
+  if (gridDim.x == 1) {
+    __threadfence();
+    __syncthreads();
+    return true;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ok = 1;
+    volatile uint32_t* gen = ctl + 1;
+    const uint32_t now = *gen;
+    __threadfence();
+    if (atomicAdd(ctl, 1u) == gridDim.x - 1u) {
+      *(volatile uint32_t*)ctl = 0u;
+      __threadfence();
+      *gen = now + 1u;
+    } else {
+      int spins = 0;
+      while (*gen == now) {
+        if (++spins > kGridWaitLimit) { ok = 0; break; }
+        if (spins > 16) __nanosleep(100);
+      }
+    }
+    __threadfence();
+  }
+  __syncthreads();
+  return ok != 0;
+}
+
+// Rounds 1 and up, all in one launch: their lists hold a few percent of round 0's pairs
+// (2000 of 750 000 in the 2^24 tube), and a launch costs more than their work.  Lists and
+// choices are read past the L1: other blocks wrote them in this launch.
+__device__ __forceinline__ uint32_t open_pairs(const SimDev& s, int round) {
+  return sim_scheduled(s) && round < s.max_rounds ? __ldcg(&s.d.wl_len[round]) : 0u;
+}
+
+__global__ void __launch_bounds__(kEdgeBlock) k_rounds(Batch B, int max_rounds) {
+  for (int round = 1; round < max_rounds; ++round) {
+    for_dealt(B, [round](const SimDev& s) { return open_pairs(s, round); },
+              [round](SimDev& s, uint32_t first, uint32_t) {
+      const int cur = s.d.parity ^ 1;
+      const uint32_t len = __ldcg(&s.d.wl_len[round]);
+      const uint32_t* list = s.wl[round & 1];
+      uint32_t* best = round_best(s, round);
+      for (uint32_t t = first; t < len; t += gridDim.x * kEdgeBlock) {
+        const uint32_t e = __ldcg(list + t);
+        const uint2 pr = s.edge[e];
+        const double d2 = s.e_d2[e], tt = s.e_t[e];
+        propose(s, cur, best, pr.x, e, d2, tt, s.id[cur][pr.y]);
+        propose(s, cur, best, pr.y, e, d2, tt, s.id[cur][pr.x]);
+      }
+    });
+    bool in_time = grid_barrier(B.round_ctl);
+    if (in_time) {
+      for_dealt(B, [round](const SimDev& s) { return open_pairs(s, round); },
+                [round](SimDev& s, uint32_t first, uint32_t trips) {
+        const uint32_t len = __ldcg(&s.d.wl_len[round]);
+        const uint32_t* list = s.wl[round & 1];
+        uint32_t t = first;
+        for (uint32_t k = 0; k < trips; ++k, t += gridDim.x * kEdgeBlock) {
+          const uint32_t e = t < len ? __ldcg(list + t) : kNone;
+          settle(s, round, e, e != kNone ? s.edge[e] : make_uint2(0u, 0u));
+        }
+      });
+      if (round + 1 == max_rounds) return;
+      in_time = grid_barrier(B.round_ctl);
+    }
+    if (!in_time) {
+      for (int k = (int)threadIdx.x; k < B.nsims; k += kEdgeBlock)
+        atomicOr(&B.sims[k]->d.status, ST_SCAN_WAIT);
+      return;
+    }
+    if (B.nsims == 1 && __ldcg(&B.sims[0]->d.wl_len[round + 1]) == 0u) return;  // nothing is open
+  }
+}
+
+// ---- candidate lists (domain decomposition) ---------------------------------- //
 
 // the pair whose slot is 0 at an endpoint opens that endpoint's list
 __global__ void __launch_bounds__(kEdgeBlock) k_alloc(Batch B) {
@@ -255,157 +535,28 @@ __global__ void __launch_bounds__(kEdgeBlock) k_fill(Batch B) {
   });
 }
 
-// ---- matching rounds ------------------------------------------------------ //
-__device__ __forceinline__ bool key_less(double d2a, double ta, uint32_t ja, double d2b, double tb,
-                                         uint32_t jb) {
-  if (d2a < d2b) return true;
-  if (d2a > d2b) return false;
-  if (ta < tb) return true;
-  if (ta > tb) return false;
-  return ja < jb;
-}
-
-// The work list of round r holds every particle that is unmatched after round r - 1
-// and had an unmatched candidate in round r - 1 (round 0: every particle with a
-// candidate).  A particle left off it has no unmatched candidate, so it can neither
-// pick nor be picked: the rounds over the lists match exactly the pairs that rounds
-// over all particles would.
-__device__ __forceinline__ uint32_t round_list(const SimDev& s, int round) {
-  return sim_scheduled(s) && round < s.max_rounds ? s.d.wl_len[round] : 0u;
-}
-
-__global__ void __launch_bounds__(kEdgeBlock) k_best(Batch B, int round) {
-  for_dealt(B, [round](const SimDev& s) { return round_list(s, round); },
-            [round](SimDev& s, uint32_t first, uint32_t) {
-    const int cur = s.d.parity ^ 1;
-    const uint32_t len = s.d.wl_len[round];
-    const uint32_t* __restrict__ list = s.wl[round & 1];
-    for (uint32_t t = first; t < len; t += gridDim.x * kEdgeBlock) {
-      const uint32_t i = list[t];
-      const uint32_t q0 = s.off[i], q1 = q0 + s.deg[i];
-      uint32_t bj = kNone, be = kNone, bid = kNone;
-      double bd2 = 0.0, bt = 0.0;
-      for (uint32_t q = q0; q < q1; ++q) {
-        const uint2 a = s.adj[q];
-        const uint32_t j = a.x;
-        if (s.partner[j] != kNone) continue;
-        const double d2 = s.e_d2[a.y], tt = s.e_t[a.y];
-        const uint32_t idj = s.id[cur][j];
-        if (bj == kNone || key_less(d2, tt, idj, bd2, bt, bid)) {
-          bj = j; be = a.y; bid = idj; bd2 = d2; bt = tt;
-        }
-      }
-      s.best[i] = bj;
-      s.best_e[i] = be;
-    }
-  });
-}
-
-__global__ void __launch_bounds__(kEdgeBlock) k_mutual(Batch B, int round) {
-  for_dealt(B, [round](const SimDev& s) { return round_list(s, round); },
-            [round](SimDev& s, uint32_t first, uint32_t trips) {
-    const int cur = s.d.parity ^ 1;
-    const uint32_t len = s.d.wl_len[round];
-    const uint32_t* __restrict__ list = s.wl[round & 1];
-    uint32_t* __restrict__ next = s.wl[(round + 1) & 1];
-    const uint32_t stride = gridDim.x * kEdgeBlock;
-    // the block's trip count, the same for all its threads: the appends are block-wide
-    uint32_t t = first;
-    for (uint32_t q = 0; q < trips; ++q, t += stride) {
-      bool pair = false, again = false;
-      uint32_t i = kNone;
-      if (t < len) {
-        i = list[t];
-        const uint32_t j = s.best[i];
-        if (j != kNone) {
-          if (s.best[j] == i) {
-            s.partner[i] = j;
-            s.medge[i] = s.best_e[i];
-            pair = s.id[cur][i] < s.id[cur][j];
-          } else {
-            again = true;
-          }
-        }
-      }
-      const uint32_t at = block_append(&s.d.n_pairs, pair ? 1u : 0u, &s.d.round_pairs[round]);
-      if (pair) s.pairs[at] = i;
-      if (round + 1 < s.max_rounds) {
-        const uint32_t w = block_append(&s.d.wl_len[round + 1], again ? 1u : 0u);
-        if (again) next[w] = i;
-      }
-    }
-  });
-}
-
-// ---- collision update ------------------------------------------------------ //
-// For the pair (a, b) with a the smaller id: stream both to t*, scatter
-//   g = v_a - v_b, V = (v_a + v_b) * 0.5, G = |g|,  v_a' = V + (G/2) n,  v_b' = V - (G/2) n,
-// then stream the rest of the step:  x' = (x + v t*) + v' (dt - t*).
-template <bool MIX>
+// the step's collisions: matched pairs (domains: smaller-id members with their partners)
+template <bool MIX, bool LISTS>
 __global__ void __launch_bounds__(kEdgeBlock) k_collide(Batch B) {
   for_dealt(B, [](const SimDev& s) { return sim_scheduled(s) ? s.d.n_pairs : 0u; },
             [](SimDev& s, uint32_t first, uint32_t) {
     const int cur = s.d.parity ^ 1;
     const uint32_t total = s.d.n_pairs;
     for (uint32_t q = first; q < total; q += gridDim.x * kEdgeBlock) {
-      // the pair list holds each colliding pair once, by its smaller-id member
-      const uint32_t i = s.pairs[q];
-      const uint32_t j = s.partner[i];
-      const uint32_t ida = s.id[cur][i];
-      double t = s.e_t[s.medge[i]];
-      double nv[3];
-      if (!(s.planar ? circle_point(s.seed, s.d.step, ida, nv) : sphere_point(s.seed, s.d.step, ida, nv))) {
-        atomicOr(&s.d.status, ST_RANDOM);
-        continue;
-      }
-      // equal masses: V = (v_a + v_b)/2 and both get half the relative speed; a mixture:
-      // V = (m_a v_a + m_b v_b)/M, v_a' = V + (m_b/M) G n, v_b' = V - (m_a/M) G n
-      const bool mixed = MIX && s.mix;
-      double ma = 1.0, mb = 1.0;
-      if (mixed) {
-        ma = s.sp_mass[s.species[ida]];
-        mb = s.sp_mass[s.species[s.id[cur][j]]];
-      }
-      double va[3], vb[3], g[3], V[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        va[c] = s.v[cur][c][i];
-        vb[c] = s.v[cur][c][j];
-        g[c] = dsub(va[c], vb[c]);
-      }
-      double fa = 0.5, fb = 0.5;
-      if (mixed) {
-        const double M = dadd(ma, mb);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) V[c] = ddiv(dadd(dmul(ma, va[c]), dmul(mb, vb[c])), M);
-        fa = ddiv(mb, M);
-        fb = ddiv(ma, M);
-      } else {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) V[c] = dmul(dadd(va[c], vb[c]), 0.5);
-      }
-      double G = dsqrt(dadd(dadd(dmul(g[0], g[0]), dmul(g[1], g[1])), dmul(g[2], g[2])));
-      const double hGa = dmul(fa, G);
-      const double hGb = dmul(fb, G);
-      double rest = dsub(s.dt, t);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        double na = dadd(V[c], dmul(hGa, nv[c]));
-        double nb = dsub(V[c], dmul(hGb, nv[c]));
-        double xa = s.x[cur][c][i], xb = s.x[cur][c][j];
-        s.x[cur][c][i] = dadd(dadd(xa, dmul(va[c], t)), dmul(na, rest));
-        s.x[cur][c][j] = dadd(dadd(xb, dmul(vb[c], t)), dmul(nb, rest));
-        s.v[cur][c][i] = na;
-        s.v[cur][c][j] = nb;
-      }
+      const uint32_t at = s.pairs[q];
+      const uint32_t e = LISTS ? s.medge[at] : at;
+      const uint2 pr = LISTS ? make_uint2(at, s.partner[at]) : s.edge[at];
+      const uint32_t idi = s.id[cur][pr.x], idj = s.id[cur][pr.y];
+      const bool first_is_a = idi < idj;
+      collide_pair<MIX>(s, cur, first_is_a ? pr.x : pr.y, first_is_a ? pr.y : pr.x,
+                        first_is_a ? idi : idj, first_is_a ? idj : idi, s.e_t[e]);
     }
   });
 }
 
 int launch_match_lists(const LaunchPlan& L, cudaStream_t st) {
   const int nb = L.edge_blocks;
-  if (L.mix) k_refine<true><<<nb, kEdgeBlock, 0, st>>>(L.b);
-  else k_refine<false><<<nb, kEdgeBlock, 0, st>>>(L.b);
+  k_refine<false, true><<<nb, kEdgeBlock, 0, st>>>(L.b);  // (domains have no mixtures)
   k_alloc<<<nb, kEdgeBlock, 0, st>>>(L.b);
   k_fill<<<nb, kEdgeBlock, 0, st>>>(L.b);
   return 3;
@@ -413,21 +564,23 @@ int launch_match_lists(const LaunchPlan& L, cudaStream_t st) {
 
 int launch_collide(const LaunchPlan& L, cudaStream_t st) {
   const int nb = L.edge_blocks;
-  if (L.mix) k_collide<true><<<nb, kEdgeBlock, 0, st>>>(L.b);
-  else k_collide<false><<<nb, kEdgeBlock, 0, st>>>(L.b);
+  if (L.mix) k_collide<true, false><<<nb, kEdgeBlock, 0, st>>>(L.b);
+  else if (L.lists) k_collide<false, true><<<nb, kEdgeBlock, 0, st>>>(L.b);
+  else k_collide<false, false><<<nb, kEdgeBlock, 0, st>>>(L.b);
   return 1;
 }
 
 int launch_match(const LaunchPlan& L, int max_rounds, cudaStream_t st) {
   const int nb = L.edge_blocks;
-  int n = launch_match_lists(L, st);
-  for (int r = 0; r < max_rounds; ++r) {
-    // the later rounds' work lists hold a few percent of the first round's: a grid of
-    // one block per SM covers them (grid-stride) without launching idle blocks
-    const int nr = r == 0 ? nb : std::max(1, nb / 8);
-    k_best<<<nr, kEdgeBlock, 0, st>>>(L.b, r);
-    k_mutual<<<nr, kEdgeBlock, 0, st>>>(L.b, r);
-    n += 2;
+  if (L.mix) k_refine<true, false><<<nb, kEdgeBlock, 0, st>>>(L.b);
+  else k_refine<false, false><<<nb, kEdgeBlock, 0, st>>>(L.b);
+  k_settle<<<nb, kEdgeBlock, 0, st>>>(L.b);
+  int n = 2;
+  if (max_rounds > 1) {
+    Batch b = L.b;
+    void* args[] = {&b, &max_rounds};
+    cudaLaunchCooperativeKernel((const void*)k_rounds, dim3(L.round_blocks), dim3(kEdgeBlock), args, 0, st);
+    ++n;
   }
   return n + launch_collide(L, st);
 }

@@ -321,6 +321,8 @@ __global__ void __launch_bounds__(kTile / 2) k_scatter(Batch B) {
     if (pp[h] < s.n) s.src[dst[h]] = pp[h];
 }
 
+// LISTS: a domain decomposition, which counts candidates per particle
+template <bool LISTS>
 __global__ void __launch_bounds__(kTile / 2) k_gather(Batch B) {
   int k = find_sim(B.ptile, B.nsims, blockIdx.x);
   SimDev& s = *B.sims[k];
@@ -354,7 +356,8 @@ __global__ void __launch_bounds__(kTile / 2) k_gather(Batch B) {
     }
     s.id[to][d] = id[h];
     s.last[to][d] = last[h];
-    s.deg[d] = 0;
+    if (LISTS) s.deg[d] = 0;
+    else s.best_e[d] = kNone;  // no choice yet
     s.partner[d] = kNone;
     if (s.precision == KMC_GUARDED_FP32) {
       // box coordinates and velocity, each rounded once to binary32
@@ -376,7 +379,8 @@ int launch_sort(const LaunchPlan& L, cudaStream_t st) {
   else k_count<false><<<L.ptiles, kTile / 2, 0, st>>>(L.b);
   int n = launch_cell_scan(L, st);
   k_scatter<<<L.ptiles, kTile / 2, 0, st>>>(L.b);
-  k_gather<<<L.ptiles, kTile / 2, 0, st>>>(L.b);
+  if (L.lists) k_gather<true><<<L.ptiles, kTile / 2, 0, st>>>(L.b);
+  else k_gather<false><<<L.ptiles, kTile / 2, 0, st>>>(L.b);
   return n + 3;
 }
 
