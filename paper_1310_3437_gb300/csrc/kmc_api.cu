@@ -18,6 +18,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "kmc_internal.cuh"
@@ -32,6 +33,7 @@ struct Plan {
   LaunchPlan L{};
   SimDev** d_table = nullptr;
   uint32_t* d_pre = nullptr;  // one allocation for the four prefix arrays + scratch
+  MemberState* d_states = nullptr;  // (in d_pre) the members' states, read by a group's sync
   cudaGraphExec_t graph = nullptr;
   bool graph_tried = false;
   int precision = 0, K = 1, max_rounds = 4;
@@ -67,6 +69,7 @@ struct kmc_sim {
   Plan solo;
   bool solo_built = false;
   std::vector<void*> allocs;
+  void* edge_slab = nullptr;
   void* stage = nullptr;
   size_t stage_bytes = 0;
   uint64_t hist_read = 0, prof_read = 0;
@@ -143,28 +146,6 @@ Sizes sizes_of(const kmc_params& p) {
   return z;
 }
 
-size_t edge_bytes(uint32_t cap) {
-  // pairs, keys, candidate marks, the two lists of open pairs
-  return (size_t)cap * (sizeof(uint2) + 2 * sizeof(double) + sizeof(uint2) + 2 * sizeof(uint32_t));
-}
-
-size_t bytes_for(const Sizes& z) {
-  size_t n = z.n;
-  size_t b = 0;
-  b += 2 * 6 * n * sizeof(double) + 2 * 2 * n * sizeof(uint32_t);  // state, double-buffered
-  if (z.fp32) b += (n + 1) / 2 * 3 * sizeof(float4);               // binary32 mirror
-  b += 3 * n * sizeof(uint32_t) + n;                                  // key, rank, src, speed class
-  b += n + 4096;                                                      // mixture species (if any)
-  b += 2 * ((size_t)z.cell_cap + 2) * sizeof(uint32_t);               // cell count / start
-  b += 3 * n * sizeof(uint32_t);                                      // best, best_e, partner
-  b += (n / 2 + 1) * sizeof(uint32_t);                                // matched pairs
-  b += edge_bytes(z.edge_cap);
-  b += (size_t)z.hist_cap * sizeof(kmc_step_counts);
-  if (z.bins) b += (size_t)z.prof_cap * z.bins * kProfQ * sizeof(long long) + z.prof_cap * sizeof(uint64_t);
-  b += sizeof(SimDev);
-  return b;
-}
-
 int validate(const kmc_params* p, std::string& err) {
   if (!p) { err = "params is NULL"; return KMC_EINVAL; }
   if (p->n == 0) { err = "n must be >= 1"; return KMC_EINVAL; }
@@ -228,24 +209,107 @@ void dfree(kmc_sim* s, void* ptr) {
   cudaFree(ptr);
 }
 
+// Arrays that share one allocation: add() gives every array its place (256-byte aligned),
+// take() allocates and hands the addresses out.  A simulation of 30 arrays is created and
+// destroyed with two driver calls for them instead of 60: a driver allocation or release
+// takes 10 us and more, and waits for the device.
+class Slab {
+ public:
+  template <typename T>
+  size_t add(T** out, size_t count) {
+    at_.push_back({(void**)out, bytes_});
+    const size_t here = bytes_;
+    bytes_ += (std::max<size_t>(count * sizeof(T), 16) + 255) & ~(size_t)255;
+    return here;
+  }
+  size_t bytes() const { return bytes_; }
+  int take(kmc_sim* s, void** slab) {
+    char* base = nullptr;
+    const int rc = dalloc(s, &base, bytes_);
+    if (rc) return rc;
+    for (const auto& a : at_) *a.first = base + a.second;
+    if (slab) *slab = base;
+    return KMC_OK;
+  }
+
+ private:
+  std::vector<std::pair<void**, size_t>> at_;
+  size_t bytes_ = 0;
+};
+
+// pairs, keys, candidate marks, the two lists of open pairs (domains: and candidate lists)
+void lay_out_edges(Slab& slab, SimDev& h, uint32_t cap, bool lists) {
+  slab.add(&h.edge, cap);
+  slab.add(&h.e_d2, cap);
+  slab.add(&h.e_t, cap);
+  slab.add(&h.e_slot, cap);
+  if (lists) slab.add(&h.adj, 2 * (size_t)cap);
+  slab.add(&h.wl[0], (lists ? 2 : 1) * (size_t)cap);
+  slab.add(&h.wl[1], cap);
+}
+
+// everything else.  key and rank lie between the two state buffers: each buffer (56 bytes
+// per particle) and these two (8) are then one stretch of 64 bytes per particle, where the
+// state is brought into id order by way of the buffer that is not current (k_state_pack).
+void lay_out_arrays(Slab& slab, SimDev& h, const Sizes& z, bool lists, uint32_t nspecies) {
+  const size_t n = z.n;
+  for (int b = 0; b < 2; ++b) {
+    if (b == 1) {
+      slab.add(&h.key, n);
+      slab.add(&h.rank, n);
+    }
+    for (int a = 0; a < 3; ++a) slab.add(&h.x[b][a], n);
+    for (int a = 0; a < 3; ++a) slab.add(&h.v[b][a], n);
+    slab.add(&h.id[b], n);
+    slab.add(&h.last[b], n);
+  }
+  if (z.fp32) slab.add(&h.mir, 3 * ((n + 1) / 2));
+  if (nspecies) {
+    slab.add(&h.species, n);
+    slab.add(&h.sp_mass, nspecies);
+    slab.add(&h.sp_radius, nspecies);
+  }
+  slab.add(&h.src, n);
+  slab.add(&h.vbucket, n);
+  // cell keys (at most cell_cap), the absorbed particles' key, the total
+  slab.add(&h.cell_count, (size_t)z.cell_cap + 2);
+  slab.add(&h.cell_start, (size_t)z.cell_cap + 2);
+  slab.add(&h.best, n);
+  slab.add(&h.best_e, n);
+  slab.add(&h.partner, n);
+  slab.add(&h.pairs, n / 2 + 1);
+  if (lists) {
+    slab.add(&h.deg, n);
+    slab.add(&h.off, n + 1);
+    slab.add(&h.medge, n);
+  }
+  slab.add(&h.hist, z.hist_cap);
+  if (z.bins) {
+    slab.add(&h.prof_acc, (size_t)z.prof_cap * z.bins * kProfQ);
+    slab.add(&h.prof_step, z.prof_cap);
+  }
+}
+
+size_t bytes_for(const Sizes& z) {
+  SimDev h{};
+  Slab arrays, edges;
+  lay_out_arrays(arrays, h, z, false, 256);  // a mixture's arrays included
+  lay_out_edges(edges, h, z.edge_cap, false);
+  return arrays.bytes() + edges.bytes() + sizeof(SimDev);
+}
+
 int alloc_edges(kmc_sim* s, uint32_t cap) {
-  int rc;
-  SimDev& h = s->h;
-  if ((rc = dalloc(s, &h.edge, cap))) return rc;
-  if ((rc = dalloc(s, &h.e_d2, cap))) return rc;
-  if ((rc = dalloc(s, &h.e_t, cap))) return rc;
-  if ((rc = dalloc(s, &h.e_slot, cap))) return rc;
-  if (s->lists && (rc = dalloc(s, &h.adj, 2 * (size_t)cap))) return rc;
-  if ((rc = dalloc(s, &h.wl[0], (s->lists ? 2 : 1) * (size_t)cap))) return rc;
-  if ((rc = dalloc(s, &h.wl[1], cap))) return rc;
-  h.edge_cap = cap;
-  return KMC_OK;
+  Slab slab;
+  lay_out_edges(slab, s->h, cap, s->lists);
+  const int rc = slab.take(s, &s->edge_slab);
+  if (rc == KMC_OK) s->h.edge_cap = cap;
+  return rc;
 }
 
 void free_edges(kmc_sim* s) {
   SimDev& h = s->h;
-  void* ptrs[] = {h.edge, h.e_d2, h.e_t, h.e_slot, h.adj, h.wl[0], h.wl[1]};
-  for (void* q : ptrs) dfree(s, q);
+  dfree(s, s->edge_slab);
+  s->edge_slab = nullptr;
   h.edge = nullptr; h.e_d2 = nullptr; h.e_t = nullptr; h.e_slot = nullptr;
   h.adj = nullptr; h.wl[0] = h.wl[1] = nullptr;
 }
@@ -284,7 +348,8 @@ int build_plan(Plan& P, const std::vector<kmc_sim*>& sims, cudaStream_t st, std:
   // prefixes (3 (m + 1) words, padded to an even count), the scan's and the rounds' two
   // control words each, then one 64-bit status word per scan tile
   const size_t head = (3 * (size_t)(m + 1) + 1) & ~(size_t)1;
-  size_t words = head + 4 + 2 * ((size_t)sc[m] + 1);
+  const size_t states = head + 4 + 2 * ((size_t)sc[m] + 1);  // an even count of words
+  size_t words = states + (sizeof(MemberState) / sizeof(uint32_t)) * (size_t)m;
   if (cudaMalloc(&P.d_table, sizeof(SimDev*) * m) != cudaSuccess ||
       cudaMalloc(&P.d_pre, words * sizeof(uint32_t)) != cudaSuccess) {
     cudaGetLastError();
@@ -301,6 +366,7 @@ int build_plan(Plan& P, const std::vector<kmc_sim*>& sims, cudaStream_t st, std:
   KCHECK(cudaMemcpyAsync(P.d_pre, host.data(), host.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, st), err);
   KCHECK(cudaStreamSynchronize(st), err);
   LaunchPlan& L = P.L;
+  P.d_states = reinterpret_cast<MemberState*>(P.d_pre + states);
   L.b.sims = P.d_table;
   L.b.nsims = m;
   L.b.ptile = P.d_pre;
@@ -633,44 +699,15 @@ int create_impl(const kmc_params* p, const double* const* src6, const uint32_t* 
     s->err = "cudaMalloc failed for the descriptor";
     return fail(KMC_ENOMEM);
   }
-  for (int b = 0; b < 2; ++b) {
-    for (int a = 0; a < 3; ++a) {
-      if ((rc = dalloc(s, &h.x[b][a], n))) return fail(rc);
-      if ((rc = dalloc(s, &h.v[b][a], n))) return fail(rc);
-    }
-    if ((rc = dalloc(s, &h.id[b], n))) return fail(rc);
-    if ((rc = dalloc(s, &h.last[b], n))) return fail(rc);
+  // bad[0]: particles outside the box / non-finite; bad[1]: exhausted init draws
+  uint32_t* bad = nullptr;
+  {
+    Slab slab;
+    lay_out_arrays(slab, h, zs, lists, mix ? mix->nspecies : 0u);
+    slab.add(&bad, 2);
+    if ((rc = slab.take(s, nullptr))) return fail(rc);
   }
-  if (zs.fp32) {
-    if ((rc = dalloc(s, &h.mir, 3 * ((n + 1) / 2)))) return fail(rc);
-  }
-  if (mix) {
-    if ((rc = dalloc(s, &h.species, n))) return fail(rc);
-    if ((rc = dalloc(s, &h.sp_mass, mix->nspecies))) return fail(rc);
-    if ((rc = dalloc(s, &h.sp_radius, mix->nspecies))) return fail(rc);
-  }
-  if ((rc = dalloc(s, &h.key, n))) return fail(rc);
-  if ((rc = dalloc(s, &h.rank, n))) return fail(rc);
-  if ((rc = dalloc(s, &h.src, n))) return fail(rc);
-  if ((rc = dalloc(s, &h.vbucket, n))) return fail(rc);
-  // cell keys (at most cell_cap), the absorbed particles' key, the total
-  if ((rc = dalloc(s, &h.cell_count, (size_t)zs.cell_cap + 2))) return fail(rc);
-  if ((rc = dalloc(s, &h.cell_start, (size_t)zs.cell_cap + 2))) return fail(rc);
-  if ((rc = dalloc(s, &h.best, n))) return fail(rc);
-  if ((rc = dalloc(s, &h.best_e, n))) return fail(rc);
-  if ((rc = dalloc(s, &h.partner, n))) return fail(rc);
-  if (lists) {
-    if ((rc = dalloc(s, &h.deg, n))) return fail(rc);
-    if ((rc = dalloc(s, &h.off, n + 1))) return fail(rc);
-    if ((rc = dalloc(s, &h.medge, n))) return fail(rc);
-  }
-  if ((rc = dalloc(s, &h.pairs, n / 2 + 1))) return fail(rc);
   if ((rc = alloc_edges(s, zs.edge_cap))) return fail(rc);
-  if ((rc = dalloc(s, &h.hist, zs.hist_cap))) return fail(rc);
-  if (zs.bins) {
-    if ((rc = dalloc(s, &h.prof_acc, (size_t)zs.prof_cap * zs.bins * kProfQ))) return fail(rc);
-    if ((rc = dalloc(s, &h.prof_step, zs.prof_cap))) return fail(rc);
-  }
   cudaStream_t st = s->stream;
   auto ck = [&](cudaError_t e) {
     if (e != cudaSuccess) {
@@ -680,9 +717,6 @@ int create_impl(const kmc_params* p, const double* const* src6, const uint32_t* 
     return true;
   };
   bool ok = true;
-  // bad[0]: particles outside the box / non-finite; bad[1]: exhausted init draws
-  uint32_t* bad = nullptr;
-  if ((rc = dalloc(s, &bad, 2))) return fail(rc);
   ok = ck(cudaMemsetAsync(bad, 0, 2 * sizeof(uint32_t), st));
   if (mix) {
     ok = ok && ck(cudaMemcpyAsync(h.species, mix->species, n, cudaMemcpyDefault, st)) &&
@@ -717,9 +751,8 @@ int create_impl(const kmc_params* p, const double* const* src6, const uint32_t* 
       ok = ck(cudaMemcpyAsync(h.x[0][a], src6[a], n * sizeof(double), cudaMemcpyDefault, st)) &&
            ck(cudaMemcpyAsync(h.v[0][a], src6[3 + a], n * sizeof(double), cudaMemcpyDefault, st));
     }
-    std::vector<uint32_t> ids(n);
-    for (size_t i = 0; i < n; ++i) ids[i] = (uint32_t)i;
-    ok = ok && ck(cudaMemcpyAsync(h.id[0], ids.data(), n * sizeof(uint32_t), cudaMemcpyHostToDevice, st));
+    if (ok) launch_ids(h.id[0], p->n, st);
+    ok = ok && ck(cudaGetLastError());
     if (last) ok = ok && ck(cudaMemcpyAsync(h.last[0], last, n * sizeof(uint32_t), cudaMemcpyDefault, st));
     else ok = ok && ck(cudaMemsetAsync(h.last[0], 0xFF, n * sizeof(uint32_t), st));
   }
@@ -741,7 +774,6 @@ int create_impl(const kmc_params* p, const double* const* src6, const uint32_t* 
   if (!ck(cudaMemcpyAsync(nbad, bad, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st)) ||
       !ck(cudaStreamSynchronize(st)))
     return fail(KMC_ECUDA);
-  dfree(s, bad);
   if (nbad[1]) {
     s->err = std::to_string(nbad[1]) + " particle(s) ran out of initialisation draws";
     return fail(KMC_ERANDOM);
@@ -1100,8 +1132,7 @@ int sim_sync(kmc_sim* s) {
   }
   cudaStream_t st = sim_work_stream(s);
   for (int attempt = 0; attempt < 64; ++attempt) {
-    KCHECK(cudaStreamSynchronize(st), s->err);
-    Dyn dy;
+    Dyn dy;  // the read waits for the steps
     int rc = read_dyn(s, &dy, st);
     if (rc) return rc;
     if (dy.status == 0) return KMC_OK;
@@ -1366,19 +1397,37 @@ int64_t sim_group_steps_left(kmc_group* g, kmc_sim* s) {
 int sim_group_sync(kmc_group* g) {
   if (!g) return KMC_EINVAL;
   int worst = KMC_OK;
+  std::vector<MemberState> now;
   for (int attempt = 0; attempt < 64; ++attempt) {
     KCHECK(cudaStreamSynchronize(g->stream), g->err);
+    // the members' step index and status in one read (a group that has not stepped since
+    // its membership changed has no table of its members yet: member by member)
+    now.assign(g->members.size(), MemberState{});
+    if (g->built) {
+      launch_member_states(g->plan.L, g->plan.d_states, g->stream);
+      KCHECK(cudaMemcpyAsync(now.data(), g->plan.d_states, now.size() * sizeof(MemberState),
+                             cudaMemcpyDeviceToHost, g->stream), g->err);
+      KCHECK(cudaStreamSynchronize(g->stream), g->err);
+    } else {
+      for (size_t k = 0; k < now.size(); ++k) {
+        Dyn dy;
+        const int rc = read_dyn(g->members[k], &dy, g->stream);
+        if (rc) return rc;
+        now[k] = {dy.step, dy.status};
+      }
+    }
     bool rerun = false;
     worst = KMC_OK;
-    for (kmc_sim* s : g->members) {
-      Dyn dy;
-      int rc = read_dyn(s, &dy, g->stream);
-      if (rc) return rc;
-      if (dy.status == 0) {
-        s->sync_step = dy.step;
+    for (size_t k = 0; k < now.size(); ++k) {
+      kmc_sim* s = g->members[k];
+      if (now[k].status == 0) {
+        s->sync_step = now[k].step;
         s->issued_base = 0;
         continue;
       }
+      Dyn dy;
+      int rc = read_dyn(s, &dy, g->stream);
+      if (rc) return rc;
       if (dy.status == ST_EDGE_OVERFLOW) {
         rc = recover_overflow(s, dy, g->stream);
         if (rc == KMC_OK) {

@@ -140,6 +140,14 @@ __global__ void __launch_bounds__(256) k_init_state(InitLaunch L) {
   L.last[id] = kNone;
 }
 
+__global__ void k_ids(uint32_t* id, uint32_t n) {
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) id[i] = i;
+}
+void launch_ids(uint32_t* id, uint32_t n, cudaStream_t st) {
+  k_ids<<<(n + 255) / 256, 256, 0, st>>>(id, n);
+}
+
 void launch_init_state(const InitLaunch& L, cudaStream_t st) {
   if (L.n == 0) return;
   k_init_state<<<(L.n + 255) / 256, 256, 0, st>>>(L);

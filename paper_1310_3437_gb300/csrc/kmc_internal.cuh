@@ -522,6 +522,13 @@ void launch_domain_edges(const LaunchPlan& L, DomainDev* D, uint32_t cap, uint2*
                          uint32_t* count, cudaStream_t st);
 void launch_domain_vmax(const DomainDev* D, unsigned long long* acc, double* out, cudaStream_t st);
 
+// a member's step index and status word, for a group's sync
+struct MemberState {
+  uint64_t step;
+  uint64_t status;
+};
+void launch_member_states(const LaunchPlan& L, MemberState* out, cudaStream_t st);
+
 // observe helpers
 void launch_gather_state(SimDev* d, uint32_t n, void* out, cudaStream_t st);
 void launch_gather_partners(SimDev* d, uint32_t n, uint32_t* out, cudaStream_t st);
@@ -551,5 +558,6 @@ struct InitLaunch {
   uint32_t* fails;
 };
 void launch_init_state(const InitLaunch& L, cudaStream_t st);
+void launch_ids(uint32_t* id, uint32_t n, cudaStream_t st);  // id[i] = i
 
 }  // namespace kmc

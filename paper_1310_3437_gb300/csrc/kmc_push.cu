@@ -417,6 +417,14 @@ void launch_add_steps(SimDev* d, uint64_t nsteps, cudaStream_t st) {
   k_add_steps<<<1, 1, 0, st>>>(d, nsteps);
 }
 
+__global__ void k_member_states(Batch B, MemberState* out) {
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < B.nsims; k += gridDim.x * blockDim.x)
+    out[k] = {B.sims[k]->d.step, B.sims[k]->d.status};
+}
+void launch_member_states(const LaunchPlan& L, MemberState* out, cudaStream_t st) {
+  k_member_states<<<(L.b.nsims + 255) / 256, 256, 0, st>>>(L.b, out);
+}
+
 // ---- observables ------------------------------------------------------------ //
 // The state in id order (x, y, z, vx, vy, vz as n binary64 each, then n last
 // partners).  Written as a gather: k_state_where scatters each particle's sorted
