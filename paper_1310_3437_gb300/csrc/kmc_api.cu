@@ -38,7 +38,6 @@ struct Plan {
   bool graph_tried = false;
   int precision = 0, K = 1, max_rounds = 4;
   int launches_per_step = 0;
-  bool has_profiles = false;
 };
 
 int g_num_sms = 0;
@@ -338,7 +337,7 @@ int build_plan(Plan& P, const std::vector<kmc_sim*>& sims, cudaStream_t st, std:
     sc[k + 1] = sc[k] + ceil_div((uint64_t)h.cell_cap + 2, kScanTile);
     pr[k + 1] = pr[k] + ceil_div(h.n, kProfTile);
     P.max_rounds = std::max(P.max_rounds, h.max_rounds);
-    if (h.profile_bins > 0) P.has_profiles = true;
+    if (h.profile_bins > 0 && h.profile_every > 0) P.L.profiles = true;
     if (h.absorb) P.L.absorb = true;
     if (sims[k]->lists) P.L.lists = true;
     if (h.mix) P.L.mix = true;
@@ -368,7 +367,9 @@ int build_plan(Plan& P, const std::vector<kmc_sim*>& sims, cudaStream_t st, std:
   LaunchPlan& L = P.L;
   P.d_states = reinterpret_cast<MemberState*>(P.d_pre + states);
   L.b.sims = P.d_table;
+  L.b.one = m == 1 ? table[0] : nullptr;
   L.b.nsims = m;
+  L.b.ptiles = pt[m];
   L.b.ptile = P.d_pre;
   L.b.stile_c = P.d_pre + (m + 1);
   L.b.prtile = P.d_pre + 2 * (m + 1);
@@ -378,7 +379,9 @@ int build_plan(Plan& P, const std::vector<kmc_sim*>& sims, cudaStream_t st, std:
   L.ptiles = pt[m];
   L.stiles_c = sc[m];
   L.prtiles = pr[m];
-  L.edge_blocks = 8 * num_sms();
+  // a block per tile of particles (one particle in twenty has a candidate pair), as many as
+  // the SMs hold at most: a launch of idle blocks takes 1.1 us, one of a few 0.6
+  L.edge_blocks = (int)std::min<uint32_t>(std::max(pt[m], 1u), 8u * (uint32_t)num_sms());
   // a block of the later rounds per 2^16 particles (their lists hold about one pair in a
   // thousand particles); one per SM at most, so that all of them run at once
   L.round_blocks = (int)std::min<uint32_t>(std::max(pt[m] / 256u, 1u), (uint32_t)num_sms());

@@ -107,8 +107,8 @@ __global__ void k_dom_reach(DomainDev* Dp) {
 __global__ void __launch_bounds__(kTile) k_dom_refresh(Batch B, DomainDev* Dp) {
   DomainDev& D = *Dp;
   const int k = find_sim(B.ptile, B.nsims, blockIdx.x);
-  SimDev& s = *B.sims[k];
-  const uint32_t p = (blockIdx.x - B.ptile[k]) * kTile + threadIdx.x;
+  SimDev& s = B.sim(k);
+  const uint32_t p = (blockIdx.x - B.tile0(B.ptile, k)) * kTile + threadIdx.x;
   bool own = false, ghost = false;
   if (p < s.n) {
     const int par = s.d.parity;
@@ -138,8 +138,8 @@ __global__ void __launch_bounds__(kTile) k_dom_refresh(Batch B, DomainDev* Dp) {
 __global__ void __launch_bounds__(kTile) k_dom_loc(Batch B, DomainDev* Dp) {
   DomainDev& D = *Dp;
   const int k = find_sim(B.ptile, B.nsims, blockIdx.x);
-  SimDev& s = *B.sims[k];
-  const uint32_t p = (blockIdx.x - B.ptile[k]) * kTile + threadIdx.x;
+  SimDev& s = B.sim(k);
+  const uint32_t p = (blockIdx.x - B.tile0(B.ptile, k)) * kTile + threadIdx.x;
   if (p >= s.n || !sim_active(s)) return;
   const int cur = s.d.parity ^ 1;
   D.loc[(size_t)k * D.n + s.id[cur][p]] = p < live_count(s) ? p : kNone;
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(kTile) k_dom_loc(Batch B, DomainDev* Dp) {
 __global__ void __launch_bounds__(kEdgeBlock) k_dom_edges(Batch B, DomainDev* Dp) {
   DomainDev& D = *Dp;
   for (int k = 0; k < B.nsims; ++k) {
-    SimDev& s = *B.sims[k];
+    SimDev& s = B.sim(k);
     if (!sim_active(s)) continue;
     const int cur = s.d.parity ^ 1;
     const uint32_t nraw = s.d.n_raw < s.edge_cap ? s.d.n_raw : s.edge_cap;
@@ -179,7 +179,7 @@ __device__ __forceinline__ bool key_less(double d2a, double ta, uint32_t ja, dou
 
 __global__ void __launch_bounds__(kEdgeBlock) k_dom_best(Batch B) {
   for (int k = 0; k < B.nsims; ++k) {
-    SimDev& s = *B.sims[k];
+    SimDev& s = B.sim(k);
     if (!sim_active(s)) continue;
     const int cur = s.d.parity ^ 1;
     const uint32_t len = s.d.wl_len[0];
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kEdgeBlock) k_dom_publish(Batch B, DomainDev* 
   DomainDev& D = *Dp;
   uint32_t* out = what == 0 ? D.bestG : D.partnerG;
   for (int k = 0; k < B.nsims; ++k) {
-    SimDev& s = *B.sims[k];
+    SimDev& s = B.sim(k);
     if (!sim_active(s)) continue;
     const int cur = s.d.parity ^ 1;
     const uint32_t len = s.d.wl_len[0];
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(kEdgeBlock) k_dom_import(Batch B, DomainDev* D
                                                            int last_round) {
   DomainDev& D = *Dp;
   for (int k = 0; k < B.nsims; ++k) {
-    SimDev& s = *B.sims[k];
+    SimDev& s = B.sim(k);
     if (!sim_active(s)) continue;
     const int cur = s.d.parity ^ 1;
     const uint32_t len = s.d.wl_len[0];
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(kEdgeBlock) k_dom_import(Batch B, DomainDev* D
 __global__ void __launch_bounds__(kEdgeBlock) k_dom_mutual(Batch B, DomainDev* Dp, int round) {
   DomainDev& D = *Dp;
   for (int k = 0; k < B.nsims; ++k) {
-    SimDev& s = *B.sims[k];
+    SimDev& s = B.sim(k);
     if (!sim_active(s)) continue;
     const int cur = s.d.parity ^ 1;
     const uint32_t len = s.d.wl_len[0];
@@ -310,8 +310,8 @@ __global__ void __launch_bounds__(kEdgeBlock) k_dom_mutual(Batch B, DomainDev* D
 __global__ void __launch_bounds__(kTile) k_dom_gather(Batch B, DomainDev* Dp) {
   DomainDev& D = *Dp;
   const int k = find_sim(B.ptile, B.nsims, blockIdx.x);
-  SimDev& s = *B.sims[k];
-  const uint32_t p = (blockIdx.x - B.ptile[k]) * kTile + threadIdx.x;
+  SimDev& s = B.sim(k);
+  const uint32_t p = (blockIdx.x - B.tile0(B.ptile, k)) * kTile + threadIdx.x;
   if (p >= s.n) return;
   const int par = s.d.parity;
   if (s.last[par][p] == KMC_ABSORBED) return;  // absent
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(kTile) k_dom_gather(Batch B, DomainDev* Dp) {
 __global__ void k_dom_record(Batch B, DomainDev* Dp) {
   DomainDev& D = *Dp;
   kmc_step_counts rec = {};
-  const SimDev& s0 = *B.sims[0];
+  const SimDev& s0 = B.sim(0);
   rec.step = s0.d.step - 1;
   uint32_t coll = 0;
   for (int r = 0; r < 4; ++r) {
@@ -340,7 +340,7 @@ __global__ void k_dom_record(Batch B, DomainDev* Dp) {
   rec.collisions = coll;
   rec.edges = D.acc_edges;
   for (int k = 0; k < B.nsims; ++k) {
-    const SimDev& s = *B.sims[k];
+    const SimDev& s = B.sim(k);
     if (s.d.hist_count == 0) continue;
     const kmc_step_counts& h = s.hist[(s.d.hist_count - 1) % s.hist_cap];
     rec.pair_tests += h.pair_tests;
@@ -357,7 +357,7 @@ __global__ void k_dom_record(Batch B, DomainDev* Dp) {
 __global__ void k_dom_gather_edges(Batch B, DomainDev* Dp, uint32_t cap, uint2* out, uint32_t* count) {
   DomainDev& D = *Dp;
   for (int k = 0; k < B.nsims; ++k) {
-    const SimDev& s = *B.sims[k];
+    const SimDev& s = B.sim(k);
     const int par = s.d.parity;
     const uint32_t nraw = s.d.last_raw < s.edge_cap ? s.d.last_raw : s.edge_cap;
     for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < nraw; e += gridDim.x * blockDim.x) {

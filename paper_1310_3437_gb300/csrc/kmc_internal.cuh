@@ -165,7 +165,10 @@ struct SimDev {
 // ---- batch mapping ------------------------------------------------------- //
 struct Batch {
   SimDev* const* sims;     // device table
+  SimDev* one;             // the simulation of a batch of one (else null): its address is a
+                           // kernel parameter, two dependent loads fewer in every kernel
   int nsims;
+  uint32_t ptiles;         // particle tiles of all simulations
   const uint32_t* ptile;   // prefix of ceil(n / kTile) per simulation
   const uint32_t* stile_c; // prefix of ceil((cell_cap + 2) / kScanTile)
   const uint32_t* prtile;  // prefix of ceil(n / kProfTile)
@@ -174,6 +177,12 @@ struct Batch {
   unsigned long long* tile_status;
   uint32_t* scan_ctl;
   uint32_t* round_ctl;     // grid barrier of the later matching rounds: arrivals, generation
+
+  __device__ __forceinline__ SimDev& sim(int k) const { return one ? *one : *sims[k]; }
+  // simulation k's first tile in a tile prefix
+  __device__ __forceinline__ uint32_t tile0(const uint32_t* prefix, int k) const {
+    return one ? 0u : __ldg(prefix + k);
+  }
 };
 
 __device__ __forceinline__ int find_sim(const uint32_t* prefix, int nsims, uint32_t tile) {
@@ -497,6 +506,7 @@ struct LaunchPlan {
   // handle either are launched in their general form only then
   bool absorb = false;
   bool mix = false;
+  bool profiles = false;  // some simulation takes profiles
 };
 
 // each returns the number of kernels it launched

@@ -114,7 +114,7 @@ __device__ __forceinline__ void for_dealt(const Batch& B, Count count, Body body
   const uint32_t nb = gridDim.x, stride = nb * (uint32_t)kEdgeBlock;
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   if (B.nsims == 1) {
-    SimDev& s = *B.sims[0];
+    SimDev& s = B.sim(0);
     const uint32_t c = count(s);
     // one answer for the block (the status word can change during the launch)
     if (!__syncthreads_and(s.d.status == 0)) return;
@@ -131,7 +131,7 @@ __device__ __forceinline__ void for_dealt(const Batch& B, Count count, Body body
     uint32_t c = 0;
     bool live = false;
     if (k < B.nsims) {
-      const SimDev& s = *B.sims[k];
+      const SimDev& s = B.sim(k);
       c = count(s);
       live = s.d.status == 0;
     }
@@ -162,7 +162,7 @@ __device__ __forceinline__ void for_dealt(const Batch& B, Count count, Body body
     const int kn = B.nsims - k0 < kEdgeBlock ? B.nsims - k0 : kEdgeBlock;
     for (int j = 0; j < kn; ++j) {
       const uint32_t trips = s_trips[j];
-      if (trips) body(*B.sims[k0 + j], s_first[j] + threadIdx.x, trips);
+      if (trips) body(B.sim(k0 + j), s_first[j] + threadIdx.x, trips);
     }
     __syncthreads();  // the tables are rewritten for the next chunk
   }
@@ -486,10 +486,10 @@ __global__ void __launch_bounds__(kEdgeBlock) k_rounds(Batch B, int max_rounds) 
     }
     if (!in_time) {
       for (int k = (int)threadIdx.x; k < B.nsims; k += kEdgeBlock)
-        atomicOr(&B.sims[k]->d.status, ST_SCAN_WAIT);
+        atomicOr(&B.sim(k).d.status, ST_SCAN_WAIT);
       return;
     }
-    if (B.nsims == 1 && __ldcg(&B.sims[0]->d.wl_len[round + 1]) == 0u) return;  // nothing is open
+    if (B.nsims == 1 && __ldcg(&B.sim(0).d.wl_len[round + 1]) == 0u) return;  // nothing is open
   }
 }
 

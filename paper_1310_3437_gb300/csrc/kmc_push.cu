@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(kTile) k_push(Batch B) {
   __shared__ uint32_t scnt[kSplitTrials];     // particles above each trial threshold
   __shared__ uint32_t sgone;                  // particles absorbed in this block
   int k = find_sim(B.ptile, B.nsims, blockIdx.x);
-  SimDev& s = *B.sims[k];
+  SimDev& s = B.sim(k);
   if (!sim_active(s)) return;
   const int cur = s.d.parity ^ 1;
   const uint64_t step = s.d.step;
@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kTile) k_push(Batch B) {
   if (threadIdx.x < kSplitTrials) scnt[threadIdx.x] = 0;
   if (ABS && threadIdx.x == 0) sgone = 0;
   __syncthreads();
-  uint32_t p = (blockIdx.x - B.ptile[k]) * kTile + threadIdx.x;
+  uint32_t p = (blockIdx.x - B.tile0(B.ptile, k)) * kTile + threadIdx.x;
   float vm = 0.0f;
   // absorbing walls: particles that left earlier sit at the end of the order and stay
   // as they are (live_count is this step's sort's count of the others)
@@ -198,14 +198,14 @@ template <bool ABS>
 __global__ void __launch_bounds__(kTile) k_profile(Batch B) {
   extern __shared__ long long acc[];
   int k = find_sim(B.prtile, B.nsims, blockIdx.x);
-  SimDev& s = *B.sims[k];
+  SimDev& s = B.sim(k);
   if (!sim_active(s) || !s.d.prof_due) return;
   const int nb = s.profile_bins;
   for (int i = threadIdx.x; i < nb * kProfQ; i += blockDim.x) acc[i] = 0;
   __syncthreads();
   const int cur = s.d.parity ^ 1;
   const double scale = ddiv((double)nb, s.profile_range);
-  uint32_t base = (blockIdx.x - B.prtile[k]) * kProfTile;
+  uint32_t base = (blockIdx.x - B.tile0(B.prtile, k)) * kProfTile;
   for (uint32_t i = threadIdx.x; i < kProfTile; i += blockDim.x) {
     uint32_t p = base + i;
     if (p >= s.n) break;
@@ -262,7 +262,7 @@ __global__ void k_finalize(Batch B) {
   const uint32_t lane = threadIdx.x & 31u;
   const int nwarps = (int)(gridDim.x * blockDim.x / 32u);
   for (int k = (int)((blockIdx.x * blockDim.x + threadIdx.x) / 32u); k < B.nsims; k += nwarps) {
-    SimDev& s = *B.sims[k];
+    SimDev& s = B.sim(k);
     if (!sim_active(s)) continue;
     const uint64_t step = s.d.step, hist_count = s.d.hist_count, steps_left = s.d.steps_left;
     const uint32_t hist_cap = s.hist_cap, was_due = s.d.prof_due, prof_cap = s.prof_cap;
@@ -314,8 +314,8 @@ __global__ void k_finalize(Batch B) {
 template <bool ABS>
 __global__ void __launch_bounds__(kTile) k_vmax(Batch B) {
   int k = find_sim(B.ptile, B.nsims, blockIdx.x);
-  SimDev& s = *B.sims[k];
-  uint32_t p = (blockIdx.x - B.ptile[k]) * kTile + threadIdx.x;
+  SimDev& s = B.sim(k);
+  uint32_t p = (blockIdx.x - B.tile0(B.ptile, k)) * kTile + threadIdx.x;
   float vm = 0.0f;
   if (p < s.n) {
     int par = s.d.parity;
@@ -330,7 +330,7 @@ __global__ void k_init_thresholds(Batch B) {
   const uint32_t lane = threadIdx.x & 31u;
   const int nwarps = (int)(gridDim.x * blockDim.x / 32u);
   for (int k = (int)((blockIdx.x * blockDim.x + threadIdx.x) / 32u); k < B.nsims; k += nwarps) {
-    SimDev& s = *B.sims[k];
+    SimDev& s = B.sim(k);
     const float v2 = __uint_as_float(s.d.vmax2_acc);
     if (lane == 0) s.d.vmax2 = v2;
     set_split_thresholds(s, v2, lane);
@@ -343,11 +343,11 @@ template <bool ABS>
 __global__ void __launch_bounds__(kTile) k_split_count(Batch B) {
   __shared__ uint32_t scnt[kSplitTrials];
   const int k = find_sim(B.ptile, B.nsims, blockIdx.x);
-  SimDev& s = *B.sims[k];
+  SimDev& s = B.sim(k);
   if (!s.split_ok) return;
   if (threadIdx.x < kSplitTrials) scnt[threadIdx.x] = 0;
   __syncthreads();
-  const uint32_t p = (blockIdx.x - B.ptile[k]) * kTile + threadIdx.x;
+  const uint32_t p = (blockIdx.x - B.tile0(B.ptile, k)) * kTile + threadIdx.x;
   const int par = s.d.parity;
   const bool valid = p < s.n && !(ABS && s.absorb && s.last[par][p] == KMC_ABSORBED);
   const float vm = valid ? vmag2_up(s.v[par][0][p], s.v[par][1][p], s.v[par][2][p]) : 0.0f;
@@ -370,7 +370,7 @@ __global__ void k_init_grid(Batch B) {
   const uint32_t lane = threadIdx.x & 31u;
   const int nwarps = (int)(gridDim.x * blockDim.x / 32u);
   for (int k = (int)((blockIdx.x * blockDim.x + threadIdx.x) / 32u); k < B.nsims; k += nwarps) {
-    SimDev& s = *B.sims[k];
+    SimDev& s = B.sim(k);
     if (lane == 0) s.d.have_counts = s.split_ok ? 1u : 0u;  // k_split_count's
     __syncwarp();
     compute_grid(s, s.d.vmax2, s.d.step, lane);
@@ -386,7 +386,7 @@ __global__ void k_init_grid(Batch B) {
 }
 
 __global__ void k_zero_vmax(Batch B) {
-  for (int k = threadIdx.x; k < B.nsims; k += blockDim.x) B.sims[k]->d.vmax2_acc = 0;
+  for (int k = threadIdx.x; k < B.nsims; k += blockDim.x) B.sim(k).d.vmax2_acc = 0;
 }
 
 int launch_init_grid(const LaunchPlan& L, cudaStream_t st) {
@@ -401,15 +401,15 @@ int launch_init_grid(const LaunchPlan& L, cudaStream_t st) {
 }
 
 int launch_push(const LaunchPlan& L, cudaStream_t st) {
-  if (L.absorb) {
-    k_push<true><<<L.ptiles, kTile, 0, st>>>(L.b);
-    k_profile<true><<<L.prtiles, kTile, 256 * kProfQ * sizeof(long long), st>>>(L.b);
-  } else {
-    k_push<false><<<L.ptiles, kTile, 0, st>>>(L.b);
-    k_profile<false><<<L.prtiles, kTile, 256 * kProfQ * sizeof(long long), st>>>(L.b);
+  const size_t smem = 256 * kProfQ * sizeof(long long);
+  if (L.absorb) k_push<true><<<L.ptiles, kTile, 0, st>>>(L.b);
+  else k_push<false><<<L.ptiles, kTile, 0, st>>>(L.b);
+  if (L.profiles) {
+    if (L.absorb) k_profile<true><<<L.prtiles, kTile, smem, st>>>(L.b);
+    else k_profile<false><<<L.prtiles, kTile, smem, st>>>(L.b);
   }
   k_finalize<<<(L.b.nsims + 7) / 8, 256, 0, st>>>(L.b);
-  return 3;
+  return L.profiles ? 3 : 2;
 }
 
 __global__ void k_add_steps(SimDev* d, uint64_t n) { d->d.steps_left += n; }
@@ -419,7 +419,7 @@ void launch_add_steps(SimDev* d, uint64_t nsteps, cudaStream_t st) {
 
 __global__ void k_member_states(Batch B, MemberState* out) {
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < B.nsims; k += gridDim.x * blockDim.x)
-    out[k] = {B.sims[k]->d.step, B.sims[k]->d.status};
+    out[k] = {B.sim(k).d.step, B.sim(k).d.status};
 }
 void launch_member_states(const LaunchPlan& L, MemberState* out, cudaStream_t st) {
   k_member_states<<<(L.b.nsims + 255) / 256, 256, 0, st>>>(L.b, out);

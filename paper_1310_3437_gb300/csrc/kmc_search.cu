@@ -72,7 +72,7 @@ __device__ __forceinline__ void min_image_f(float& r, float halfL, float L, floa
 __device__ __forceinline__ bool batch_uses(const Batch& B, int mode) {
   bool any = false;
   for (int q = threadIdx.x; q < B.nsims; q += blockDim.x) {
-    const SimDev& t = *B.sims[q];
+    const SimDev& t = B.sim(q);
     any = any || (sim_active(t) && (mode < 0 ? t.d.grid.split != 0u : t.d.grid.mode == mode));
   }
   return __syncthreads_or(any) != 0;
@@ -298,14 +298,14 @@ __global__ void __launch_bounds__(kTile) k_search(Batch B) {
   if (lane == 0) wcount[warp] = 0;
   __syncwarp();
   // grid-stride over tiles of kTile particles (an occupancy-sized grid)
-  const uint32_t ntiles = B.ptile[B.nsims];
+  const uint32_t ntiles = B.ptiles;
   for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int k = find_sim(B.ptile, B.nsims, tile);
-    SimDev& s = *B.sims[k];
+    SimDev& s = B.sim(k);
     if (s.d.grid.mode != MODE_PARTICLE) continue;
     // the status word can change while the search runs (a full pair buffer): one answer
     if (!__all_sync(0xFFFFFFFFu, sim_active(s))) continue;
-    const uint32_t p = (tile - B.ptile[k]) * kTile + threadIdx.x;
+    const uint32_t p = (tile - B.tile0(B.ptile, k)) * kTile + threadIdx.x;
     // with the speed split only the slow population (keys below nkeys) is searched here;
     // particles that left through absorbing walls sit after every cell key
     const uint32_t nslow = (s.d.grid.split || s.absorb) ? __ldg(s.cell_start + s.d.grid.nkeys) : s.n;
@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(kTile, 4) k_search_rows32(Batch B) {
   // grid-stride over tiles of kTile particles: the kernel is launched every step on an
   // occupancy-sized grid and exits at once when the step runs another search
   if (!batch_uses(B, MODE_ROWS)) return;
-  const uint32_t ntiles = B.ptile[B.nsims];
+  const uint32_t ntiles = B.ptiles;
   int kcur = -1;  // simulation whose constants the shared tables hold
   // The warp's pair tests and emitted pairs go to the simulation's counters only when
   // the simulation changes, the staging buffer is half full, or at the end: per-tile
@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(kTile, 4) k_search_rows32(Batch B) {
   __syncwarp();
   for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int k = find_sim(B.ptile, B.nsims, tile);
-    SimDev& s = *B.sims[k];
+    SimDev& s = B.sim(k);
     // launch-fixed fields only: the barriers below depend on it
     if (!sim_scheduled(s) || s.d.grid.mode != MODE_ROWS || (s.bc[0] == KMC_PERIODIC) != PX)
       continue;
@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(kTile, 4) k_search_rows32(Batch B) {
     // walks the same tiles), so the warps of a block need not wait for each other at
     // every tile: each runs on to its part of the next tile.
     if (k != kcur) {
-      if (kcur >= 0) warp_flush(*B.sims[kcur]);  // staged pairs and counts of the last one
+      if (kcur >= 0) warp_flush(B.sim(kcur));  // staged pairs and counts of the last one
       __syncthreads();  // every warp is done with the previous simulation's constants
       if (threadIdx.x == 0) {
         sq = guard_of(g);
@@ -412,7 +412,7 @@ __global__ void __launch_bounds__(kTile, 4) k_search_rows32(Batch B) {
     if (!s_live) continue;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const uint32_t nslow = (g.split || s.absorb) ? __ldg(s.cell_start + g.nkeys) : s.n;
-    const uint32_t p = (tile - B.ptile[k]) * kTile + threadIdx.x;
+    const uint32_t p = (tile - B.tile0(B.ptile, k)) * kTile + threadIdx.x;
     if (p - lane >= nslow) continue;  // the whole warp is past the slow population
     uint2* pc = reinterpret_cast<uint2*>(rows_smem) + (size_t)warp * NP * 32;
     uint8_t* cd = rows_smem + RL::kPieceBytes + (size_t)warp * NP * 32;
@@ -683,7 +683,7 @@ __global__ void __launch_bounds__(kTile, 4) k_search_rows32(Batch B) {
     for (int off = 16; off > 0; off >>= 1) tests += __shfl_down_sync(0xFFFFFFFFu, tests, off);
     if (lane == 0) wtests[warp] += tests;
   }
-  if (kcur >= 0) warp_flush(*B.sims[kcur]);
+  if (kcur >= 0) warp_flush(B.sim(kcur));
 }
 
 // --------------------------------------------------------------------------- //
@@ -929,12 +929,12 @@ __global__ void __launch_bounds__(kTile, 4) k_search_tiles(Batch B) {
   const uint32_t frag = lane >> 2, quad = lane & 3u, later = later_bits(frag, quad);
   // this lane's two words of record r: plane quad / 2, half quad % 2
   const uint2* words = reinterpret_cast<const uint2*>(w.rec + (quad >> 1) * kPlane) + (quad & 1u);
-  const uint32_t ntiles = B.ptile[B.nsims];
+  const uint32_t ntiles = B.ptiles;
   for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int k = find_sim(B.ptile, B.nsims, tile);
-    SimDev& s = *B.sims[k];
+    SimDev& s = B.sim(k);
     if (k != kcur) {
-      if (kcur >= 0) finish(*B.sims[kcur]);
+      if (kcur >= 0) finish(B.sim(kcur));
       kcur = k;
     }
     // the status word can change while the search runs (a full pair buffer): one answer
@@ -942,7 +942,7 @@ __global__ void __launch_bounds__(kTile, 4) k_search_tiles(Batch B) {
     const Grid& g = s.d.grid;
     const uint32_t* __restrict__ cs = s.cell_start;
     const uint32_t nslow = (g.split || s.absorb) ? __ldg(cs + g.nkeys) : s.n;
-    const uint32_t p0 = (tile - B.ptile[k]) * kTile + warp * 32u, p = p0 + lane;
+    const uint32_t p0 = (tile - B.tile0(B.ptile, k)) * kTile + warp * 32u, p = p0 + lane;
     if (p0 >= nslow) continue;
     const bool valid = p < nslow;
     const int nx = g.nc[0], ny = g.nc[1], nz = g.nc[2], cur = s.d.parity ^ 1;
@@ -1158,7 +1158,7 @@ __global__ void __launch_bounds__(kTile, 4) k_search_tiles(Batch B) {
       }
     }
   }
-  if (kcur >= 0) finish(*B.sims[kcur]);
+  if (kcur >= 0) finish(B.sim(kcur));
 }
 
 
@@ -1189,10 +1189,10 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4) k_search_fast(Batch B) {
   // grid-stride over tiles (an occupancy-sized grid); the warps of tile t take the
   // fast particles f = 8 (t - first tile) + warp, stepping by 8 tiles per simulation
   if (!batch_uses(B, -1)) return;
-  const uint32_t ntiles = B.ptile[B.nsims];
+  const uint32_t ntiles = B.ptiles;
   for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int k = find_sim(B.ptile, B.nsims, tile);
-    SimDev& s = *B.sims[k];
+    SimDev& s = B.sim(k);
     // launch-fixed fields first; the status word (the search itself can set it) as one
     // answer per warp
     if (!sim_scheduled(s) || !s.d.grid.split) continue;
@@ -1204,10 +1204,10 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4) k_search_fast(Batch B) {
     const uint32_t nslow = __ldg(cs + nk);
     const uint32_t nfast = n - nslow;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const uint32_t blk = tile - B.ptile[k];
+    const uint32_t blk = tile - B.tile0(B.ptile, k);
     // tiles past the fast population have nothing to do (no block-wide barrier below)
     if (blk * kCellWarps >= nfast) continue;
-    const uint32_t wstride = (B.ptile[k + 1] - B.ptile[k]) * kCellWarps;
+    const uint32_t wstride = ((s.n + (uint32_t)kTile - 1u) / (uint32_t)kTile) * kCellWarps;
     uint2* buf = wbuf[warp];
     uint32_t* cnt = &wcount[warp];
     if (lane == 0) *cnt = 0;

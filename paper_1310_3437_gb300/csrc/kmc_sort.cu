@@ -54,10 +54,10 @@ __global__ void __launch_bounds__(kTile / 2) k_count(Batch B) {
     B.scan_ctl[1] += 1u;
   }
   int k = find_sim(B.ptile, B.nsims, blockIdx.x);
-  SimDev& s = *B.sims[k];
+  SimDev& s = B.sim(k);
   if (!sim_active(s)) return;
   const Grid& g = s.d.grid;
-  const uint32_t p0 = (blockIdx.x - B.ptile[k]) * kTile + threadIdx.x;
+  const uint32_t p0 = (blockIdx.x - B.tile0(B.ptile, k)) * kTile + threadIdx.x;
   const uint32_t pp[2] = {p0, p0 + kTile / 2};
   const int par = s.d.parity;
   double xs[2][3];
@@ -139,12 +139,12 @@ __global__ void __launch_bounds__(kTile) k_scan_onepass(Batch B, uint32_t ntiles
   if (tile >= ntiles) return;
   const uint32_t* pre = B.stile_c;
   const int k = find_sim(pre, B.nsims, tile);
-  SimDev& s = *B.sims[k];
+  SimDev& s = B.sim(k);
   // a tile that waited too long sets the status word while the scan runs: the block
   // takes one answer (every thread reaches the barriers below or none does)
   if (!__syncthreads_and(sim_active(s))) return;
   const ScanView v = scan_view(s);
-  const uint32_t first = pre[k];
+  const uint32_t first = B.tile0(pre, k);
   const uint32_t base = (tile - first) * kScanTile;
   if (base > v.len) return;  // past the key space: no later tile of this segment waits
   const uint32_t epoch = *(volatile uint32_t*)&B.scan_ctl[1] & 0x3FFFFFFFu;
@@ -302,9 +302,9 @@ __global__ void __launch_bounds__(kTile) k_scan_onepass(Batch B, uint32_t ntiles
 // dependent load chains (key -> cell start; source -> state) are in flight at once.
 __global__ void __launch_bounds__(kTile / 2) k_scatter(Batch B) {
   int k = find_sim(B.ptile, B.nsims, blockIdx.x);
-  SimDev& s = *B.sims[k];
+  SimDev& s = B.sim(k);
   if (!sim_active(s)) return;
-  const uint32_t p0 = (blockIdx.x - B.ptile[k]) * kTile + threadIdx.x;
+  const uint32_t p0 = (blockIdx.x - B.tile0(B.ptile, k)) * kTile + threadIdx.x;
   const uint32_t pp[2] = {p0, p0 + kTile / 2};
   uint32_t key[2], rank[2];
 #pragma unroll
@@ -325,9 +325,9 @@ __global__ void __launch_bounds__(kTile / 2) k_scatter(Batch B) {
 template <bool LISTS>
 __global__ void __launch_bounds__(kTile / 2) k_gather(Batch B) {
   int k = find_sim(B.ptile, B.nsims, blockIdx.x);
-  SimDev& s = *B.sims[k];
+  SimDev& s = B.sim(k);
   if (!sim_active(s)) return;
-  const uint32_t d0 = (blockIdx.x - B.ptile[k]) * kTile + threadIdx.x;
+  const uint32_t d0 = (blockIdx.x - B.tile0(B.ptile, k)) * kTile + threadIdx.x;
   const uint32_t dd[2] = {d0, d0 + kTile / 2};
   const int from = s.d.parity, to = from ^ 1;
   uint32_t pp[2];
