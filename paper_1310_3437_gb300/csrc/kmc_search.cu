@@ -329,6 +329,8 @@ __global__ void __launch_bounds__(kTile) k_search(Batch B) {
 // warp runs as many iterations as its busiest lane needs.  Rows split only on a
 // periodic x axis (PX); without one the piece lists take half the shared memory,
 // which leaves more of the SM's L1 to cache the partner records.
+// SHARED (few particles, see shift_of): 2^shift warps take the same 32 particles, warp w of
+// them the columns c with c mod 2^shift = w.
 template <int K, bool PX>
 struct RowLayout {
   static constexpr int kCols = 1 + K + K * (2 * K + 1);  // own column + forward columns
@@ -345,8 +347,8 @@ __device__ __forceinline__ uint32_t image_code(int wx, int wy, int wz) {
          ((uint32_t)(wy < 0) << 3) | ((uint32_t)(wz > 0) << 4) | ((uint32_t)(wz < 0) << 5);
 }
 
-template <int K, bool PX>
-__global__ void __launch_bounds__(kTile, 4) k_search_rows32(Batch B) {
+template <int K, bool PX, bool SHARED>
+__global__ void __launch_bounds__(kTile, 4) k_search_rows32(Batch B, uint32_t shift) {
   using RL = RowLayout<K, PX>;
   constexpr int NP = RL::kPieces;
   extern __shared__ __align__(16) unsigned char rows_smem[];
@@ -357,7 +359,7 @@ __global__ void __launch_bounds__(kTile, 4) k_search_rows32(Batch B) {
   // grid-stride over tiles of kTile particles: the kernel is launched every step on an
   // occupancy-sized grid and exits at once when the step runs another search
   if (!batch_uses(B, MODE_ROWS)) return;
-  const uint32_t ntiles = B.ptiles;
+  const uint32_t parts = SHARED ? 1u << shift : 1u, units = B.ptiles * parts;
   int kcur = -1;  // simulation whose constants the shared tables hold
   // The warp's pair tests and emitted pairs go to the simulation's counters only when
   // the simulation changes, the staging buffer is half full, or at the end: per-tile
@@ -380,7 +382,8 @@ __global__ void __launch_bounds__(kTile, 4) k_search_rows32(Batch B) {
     wtests[threadIdx.x >> 5] = 0;
   }
   __syncwarp();
-  for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+  for (uint32_t unit = blockIdx.x; unit < units; unit += gridDim.x) {
+    const uint32_t tile = SHARED ? unit >> shift : unit;
     const int k = find_sim(B.ptile, B.nsims, tile);
     SimDev& s = B.sim(k);
     // launch-fixed fields only: the barriers below depend on it
@@ -412,7 +415,9 @@ __global__ void __launch_bounds__(kTile, 4) k_search_rows32(Batch B) {
     if (!s_live) continue;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const uint32_t nslow = (g.split || s.absorb) ? __ldg(s.cell_start + g.nkeys) : s.n;
-    const uint32_t p = (tile - B.tile0(B.ptile, k)) * kTile + threadIdx.x;
+    const uint32_t part = SHARED ? warp & (parts - 1u) : 0u;
+    uint32_t p = (tile - B.tile0(B.ptile, k)) * kTile + threadIdx.x;
+    if (SHARED) p = p - warp * 32u + (unit & (parts - 1u)) * (kTile >> shift) + (warp >> shift) * 32u;
     if (p - lane >= nslow) continue;  // the whole warp is past the slow population
     uint2* pc = reinterpret_cast<uint2*>(rows_smem) + (size_t)warp * NP * 32;
     uint8_t* cd = rows_smem + RL::kPieceBytes + (size_t)warp * NP * 32;
@@ -488,6 +493,7 @@ __global__ void __launch_bounds__(kTile, 4) k_search_rows32(Batch B) {
       const float wyf = g.wf[1], wzf = g.wf[2], ivx = g.inv_wf[0];
 #pragma unroll
       for (int c = 0; c < RL::kCols; ++c) {
+        if (SHARED && ((uint32_t)c & (parts - 1u)) != part) continue;
         const int dz = c <= K ? 0 : 1 + (c - K - 1) / (2 * K + 1);
         const int dy = c == 0 ? 0 : (c <= K ? c : (c - K - 1) % (2 * K + 1) - K);
         // the column's key base and image flags (warp table, or this lane's own)
@@ -716,6 +722,9 @@ __global__ void __launch_bounds__(kTile, 4) k_search_rows32(Batch B) {
 // binary32, whose partial sums are at most 12, added with truncation) 384 u; 2^-14 =
 // 1024 u is taken.
 //
+// SHARED (few particles, see shift_of): 2^shift warps take the same 32 particles, warp w of
+// them the tiles w, w + 2^shift, ... of every run.
+//
 // What bounds it: issue slots.  A tile costs 8 mma (2 cycles of the SM's tensor cores
 // each), 32 funnel shifts (half rate), about 75 instructions to pack the 32 partners and
 // about 30 per turn of survivors, so it pays where most of a tile's 1024 pairs are pairs
@@ -902,8 +911,8 @@ __device__ __noinline__ void test_survivor(SimDev& s, uint2* buf, uint32_t* cnt,
   if (emit) emit_lane(buf, cnt, s, i, j);
 }
 
-template <int PREC, int K>
-__global__ void __launch_bounds__(kTile, 4) k_search_tiles(Batch B) {
+template <int PREC, int K, bool SHARED>
+__global__ void __launch_bounds__(kTile, 4) k_search_tiles(Batch B, uint32_t shift) {
   using TW = TileWarp<K>;
   constexpr uint32_t kAll = 0xFFFFFFFFu;
   constexpr int kCols = TW::kCols;
@@ -929,8 +938,12 @@ __global__ void __launch_bounds__(kTile, 4) k_search_tiles(Batch B) {
   const uint32_t frag = lane >> 2, quad = lane & 3u, later = later_bits(frag, quad);
   // this lane's two words of record r: plane quad / 2, half quad % 2
   const uint2* words = reinterpret_cast<const uint2*>(w.rec + (quad >> 1) * kPlane) + (quad & 1u);
-  const uint32_t ntiles = B.ptiles;
-  for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+  constexpr uint32_t kWarps = kTile / 32;
+  const uint32_t parts = SHARED ? 1u << shift : 1u, step = gridDim.x * kWarps;
+  const uint32_t units = B.ptiles * kWarps * parts;
+  for (uint32_t unit = SHARED ? blockIdx.x + gridDim.x * warp : blockIdx.x * kWarps + warp;
+       unit < units; unit += step) {
+    const uint32_t part = unit & (parts - 1u), rows = SHARED ? unit >> shift : unit, tile = rows / kWarps;
     const int k = find_sim(B.ptile, B.nsims, tile);
     SimDev& s = B.sim(k);
     if (k != kcur) {
@@ -942,7 +955,7 @@ __global__ void __launch_bounds__(kTile, 4) k_search_tiles(Batch B) {
     const Grid& g = s.d.grid;
     const uint32_t* __restrict__ cs = s.cell_start;
     const uint32_t nslow = (g.split || s.absorb) ? __ldg(cs + g.nkeys) : s.n;
-    const uint32_t p0 = (tile - B.tile0(B.ptile, k)) * kTile + warp * 32u, p = p0 + lane;
+    const uint32_t p0 = (rows - B.tile0(B.ptile, k) * kWarps) * 32u, p = p0 + lane;
     if (p0 >= nslow) continue;
     const bool valid = p < nslow;
     const int nx = g.nc[0], ny = g.nc[1], nz = g.nc[2], cur = s.d.parity ^ 1;
@@ -951,6 +964,7 @@ __global__ void __launch_bounds__(kTile, 4) k_search_tiles(Batch B) {
                pz = s.bc[2] == KMC_PERIODIC;
     if (PREC == KMC_FP64 && ((nx == 1 && px) || (ny == 1 && py) || (nz == 1 && pz))) {
       // a one-cell periodic axis: the minimum image of every pair (binary32: row search)
+      if (part != 0u) continue;
       unsigned long long t = valid ? particle_walk<PREC, K>(s, p, w.buf, &w.count) : 0ull;
       for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kAll, t, o);
       tests += t;
@@ -1017,8 +1031,8 @@ __global__ void __launch_bounds__(kTile, 4) k_search_tiles(Batch B) {
         if (lane >= (uint32_t)d) slots += u;
       }
       const uint32_t total = __shfl_sync(kAll, slots, kCols - 1);
-      if (total == 0u) continue;
-      tests += (unsigned long long)__popc(run) * total;
+      if (total <= 32u * part) continue;
+      if (part == 0u) tests += (unsigned long long)__popc(run) * total;
       // Plain: no piece is seen through an image.  The five pieces of K = 1 then stay in
       // registers; otherwise they go to shared memory.
       const bool plain =
@@ -1077,8 +1091,7 @@ __global__ void __launch_bounds__(kTile, 4) k_search_tiles(Batch B) {
       }
 
       // 3. the tiles
-      uint32_t P = 0;  // piece that holds slot `base`
-      for (uint32_t base = 0; base < total; base += 32) {
+      for (uint32_t base = 32u * part; base < total; base += 32u * parts) {
         const uint32_t slot = base + lane;
         uint32_t j, jc = 0;
         float qx = -ox * sc, qy = -oy * sc, qz = -oz * sc;
@@ -1091,8 +1104,13 @@ __global__ void __launch_bounds__(kTile, 4) k_search_tiles(Batch B) {
           if (slot >= s4) off = o4;
           j = slot + off;
         } else {
-          // pieces starting inside the tile (at most 31, each non-empty, among P + 1 ..
-          // P + 31) mark their first slot in one OR
+          // P is the piece that holds slot `base`; the pieces starting inside the tile (at
+          // most 31, each non-empty, among P + 1 .. P + 31) mark their first slot in one OR
+          uint32_t P = 0;
+#pragma unroll
+          for (uint32_t q = 0; q < (uint32_t)TW::kPieces; q += 32)
+            P += __popc(__ballot_sync(kAll, q + lane < pieces && w.start[q + lane] <= base));
+          --P;
           const uint32_t st = P + lane < pieces ? w.start[P + lane] : kNone;
           const uint32_t bit = (st > base && st - base < 32u) ? 1u << (st - base) : 0u;
           const uint32_t marks = __reduce_or_sync(kAll, bit);
@@ -1102,9 +1120,6 @@ __global__ void __launch_bounds__(kTile, 4) k_search_tiles(Batch B) {
           qx = -(ox - image_shift(jc, g.Lf[0])) * sc;
           qy = -(oy - image_shift(jc >> 2, g.Lf[1])) * sc;
           qz = -(oz - image_shift(jc >> 4, g.Lf[2])) * sc;
-          // the next tile starts in lane 31's piece or in the one after it
-          P = __shfl_sync(kAll, pi, 31);
-          if (P + 1u < pieces && w.start[P + 1u] <= base + 32u) ++P;
         }
         float ax = 0, ay = 0, az = 0, bx = 0, by = 0, bz = 0, far = kFar;
         if (slot < total) {
@@ -1172,6 +1187,17 @@ __global__ void __launch_bounds__(kTile, 4) k_search_tiles(Batch B) {
 // whatever its length.  A warp prefix sum over the lanes' test counts then deals the
 // tests of 32 columns out to the lanes, so every lane tests a pair in every
 // iteration whatever the occupancies.  The pair tests are those of the other searches.
+// The particles are dealt to the grid by for_dealt, a warp each: few of them go to as many
+// SMs as there are (one block per 256 particles of the gas put the fast ones of 4096
+// binary64 particles on 16 SMs: 18.3 -> 13.1 us), and the members of a group follow one
+// another (an ensemble of 30: 103 -> 82 us; 2^24 tube 262 -> 216, 10^8 gas 1.79 -> 1.50 ms).
+// fast particles of a simulation's step (fields that stay fixed during the search)
+__device__ __forceinline__ uint32_t fast_count(const SimDev& s) {
+  if (!sim_scheduled(s) || !s.d.grid.split) return 0u;
+  const uint32_t nk = s.d.grid.nkeys;
+  return __ldg(s.cell_start + 2 * nk) - __ldg(s.cell_start + nk);
+}
+
 template <int PREC>
 __global__ void __launch_bounds__(kCellWarps * 32, 4) k_search_fast(Batch B) {
   __shared__ uint2 wbuf[kCellWarps][kWarpBuf];
@@ -1186,17 +1212,8 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4) k_search_fast(Batch B) {
   // image flags
   __shared__ uint32_t fst[kCellWarps][kFastPieces * 32], fjb[kCellWarps][kFastPieces * 32];
   __shared__ uint8_t fcd[kCellWarps][kFastPieces * 32];
-  // grid-stride over tiles (an occupancy-sized grid); the warps of tile t take the
-  // fast particles f = 8 (t - first tile) + warp, stepping by 8 tiles per simulation
-  if (!batch_uses(B, -1)) return;
-  const uint32_t ntiles = B.ptiles;
-  for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int k = find_sim(B.ptile, B.nsims, tile);
-    SimDev& s = B.sim(k);
-    // launch-fixed fields first; the status word (the search itself can set it) as one
-    // answer per warp
-    if (!sim_scheduled(s) || !s.d.grid.split) continue;
-    if (!__all_sync(0xFFFFFFFFu, sim_active(s))) continue;
+  for_dealt<kCellWarps>(B, [](const SimDev& s) { return fast_count(s); },
+                        [&](SimDev& s, uint32_t first, uint32_t) {
     const Grid& g = s.d.grid;
     const uint32_t* __restrict__ cs = s.cell_start;
     const uint32_t nk = g.nkeys;
@@ -1204,10 +1221,7 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4) k_search_fast(Batch B) {
     const uint32_t nslow = __ldg(cs + nk);
     const uint32_t nfast = n - nslow;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const uint32_t blk = tile - B.tile0(B.ptile, k);
-    // tiles past the fast population have nothing to do (no block-wide barrier below)
-    if (blk * kCellWarps >= nfast) continue;
-    const uint32_t wstride = ((s.n + (uint32_t)kTile - 1u) / (uint32_t)kTile) * kCellWarps;
+    if (first >= nfast) return;
     uint2* buf = wbuf[warp];
     uint32_t* cnt = &wcount[warp];
     if (lane == 0) *cnt = 0;
@@ -1230,7 +1244,7 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4) k_search_fast(Batch B) {
     const float Lf0 = g.Lf[0], Lf1 = g.Lf[1], Lf2 = g.Lf[2];
     unsigned long long tests = 0;
 
-    for (uint32_t f = blk * kCellWarps + warp; f < nfast; f += wstride) {
+    for (uint32_t f = first; f < nfast; f += gridDim.x * kCellWarps) {
       const uint32_t p = nslow + f;
       // the particle's cell, recomputed as the sort computed it
       const int cx = cell_coord(g, 0, X0[p]), cy = cell_coord(g, 1, X1[p]), cz = cell_coord(g, 2, X2[p]);
@@ -1429,7 +1443,7 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4) k_search_fast(Batch B) {
       atomicAdd(&s.d.pair_tests, tests);
       atomicAdd(&s.d.fast_tests, tests);
     }
-  }
+  });
 }
 
 namespace {
@@ -1445,21 +1459,47 @@ int resident_blocks(F kernel, int threads, size_t smem, int num_sms) {
   return per_sm * num_sms;
 }
 
+// Warps that share the partners of 32 particles in the tiled and the row search: as many as
+// leave every one of them resident at once (at most eight, a block of them).  A warp with
+// 32 particles for itself runs 10 to 20 us whatever the rest of the chip does, a chain of
+// loads, so with fewer of them than the SMs hold the step waits for one chain; shared by 8, 8
+// and 2 warps the searches of boxes of 4096 particles (binary32, binary64) and of a 50 k tube
+// take 9.0, 17.0 and 12.9 us instead of 17.6, 33.0 and 17.3.  Past that the repeated set-up
+// costs more than the shorter chains give: 262 k particles 38.5 us alone, 41.6 and 55.9 with
+// two and four warps, the tiled search of a 2^20 binary64 tube 172 and 204 with one and four.
+int shift_of(int blocks, uint32_t ptiles) {
+  int shift = 0;
+  while (shift < 3 && ((uint64_t)ptiles << (shift + 1)) <= (uint64_t)blocks) ++shift;
+  return shift;
+}
+
 template <int PREC, int K>
 void grids_of(int num_sms, uint32_t ptiles, LaunchPlan& L) {
-  auto cap = [&](int blocks) { return (int)std::min<uint32_t>((uint32_t)blocks, std::max(ptiles, 1u)); };
-  L.part_blocks = cap(resident_blocks(k_search<PREC, K>, kTile, 0, num_sms));
-  L.tile_blocks = cap(resident_blocks(k_search_tiles<PREC, K>, kTile, 0, num_sms));
-  L.fast_blocks = cap(resident_blocks(k_search_fast<PREC>, kCellWarps * 32, 0, num_sms));
+  auto cap = [&](int blocks, int shift) {
+    return (int)std::min<uint64_t>((uint64_t)blocks, (uint64_t)std::max(ptiles, 1u) << shift);
+  };
+  L.part_blocks = cap(resident_blocks(k_search<PREC, K>, kTile, 0, num_sms), 0);
+  int blocks = resident_blocks(k_search_tiles<PREC, K, false>, kTile, 0, num_sms);
+  L.tile_shift = shift_of(blocks, ptiles);
+  // shared units go to the blocks one warp each: at least a block per SM
+  L.tile_blocks = cap(blocks, L.tile_shift);
+  if (L.tile_shift) L.tile_blocks = std::max(L.tile_blocks, num_sms);
+  L.fast_blocks = std::min(resident_blocks(k_search_fast<PREC>, kCellWarps * 32, 0, num_sms),
+                           (int)std::max(ptiles, (uint32_t)num_sms));
   if (PREC != KMC_GUARDED_FP32) return;
   // the row search keeps its piece lists in dynamic shared memory (above 48 KB for
   // K = 2); set before any launch or capture
-  cudaFuncSetAttribute(k_search_rows32<K, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)RowLayout<K, true>::kBytes);
-  cudaFuncSetAttribute(k_search_rows32<K, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)RowLayout<K, false>::kBytes);
-  L.row_blocks = cap(resident_blocks(k_search_rows32<K, false>, kTile, RowLayout<K, false>::kBytes, num_sms));
-  L.row_blocks_px = cap(resident_blocks(k_search_rows32<K, true>, kTile, RowLayout<K, true>::kBytes, num_sms));
+  auto rows = [&](auto alone, auto shared, size_t bytes, int& grid, int& shift) {
+    cudaFuncSetAttribute(alone, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaFuncSetAttribute(shared, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    const int n = resident_blocks(alone, kTile, bytes, num_sms);
+    shift = shift_of(n, ptiles);
+    grid = cap(n, shift);
+  };
+  rows(k_search_rows32<K, false, false>, k_search_rows32<K, false, true>, RowLayout<K, false>::kBytes,
+       L.row_blocks, L.row_shift);
+  rows(k_search_rows32<K, true, false>, k_search_rows32<K, true, true>, RowLayout<K, true>::kBytes,
+       L.row_blocks_px, L.row_shift_px);
 }
 
 // Every search that a simulation of the plan may choose for a step; each runs the one its
@@ -1467,19 +1507,23 @@ void grids_of(int num_sms, uint32_t ptiles, LaunchPlan& L) {
 template <int PREC, int K>
 int launch_slow(const LaunchPlan& L, cudaStream_t st) {
   int n = 1;
-  k_search_tiles<PREC, K><<<L.tile_blocks, kTile, 0, st>>>(L.b);
+  if (L.tile_shift) k_search_tiles<PREC, K, true><<<L.tile_blocks, kTile, 0, st>>>(L.b, L.tile_shift);
+  else k_search_tiles<PREC, K, false><<<L.tile_blocks, kTile, 0, st>>>(L.b, 0);
   if (L.particle) {
     k_search<PREC, K><<<L.part_blocks, kTile, 0, st>>>(L.b);
     ++n;
   }
-  if (PREC == KMC_GUARDED_FP32 && L.bounded_x) {
-    k_search_rows32<K, false><<<L.row_blocks, kTile, RowLayout<K, false>::kBytes, st>>>(L.b);
+  auto rows = [&](auto alone, auto shared, size_t bytes, int grid, int shift) {
+    if (shift) shared<<<grid, kTile, bytes, st>>>(L.b, shift);
+    else alone<<<grid, kTile, bytes, st>>>(L.b, 0);
     ++n;
-  }
-  if (PREC == KMC_GUARDED_FP32 && L.periodic_x) {
-    k_search_rows32<K, true><<<L.row_blocks_px, kTile, RowLayout<K, true>::kBytes, st>>>(L.b);
-    ++n;
-  }
+  };
+  if (PREC == KMC_GUARDED_FP32 && L.bounded_x)
+    rows(k_search_rows32<K, false, false>, k_search_rows32<K, false, true>, RowLayout<K, false>::kBytes,
+         L.row_blocks, L.row_shift);
+  if (PREC == KMC_GUARDED_FP32 && L.periodic_x)
+    rows(k_search_rows32<K, true, false>, k_search_rows32<K, true, true>, RowLayout<K, true>::kBytes,
+         L.row_blocks_px, L.row_shift_px);
   return n;
 }
 }  // namespace
