@@ -1,5 +1,5 @@
 // kmc_grid.cuh -- per-step search grid and the guard bands of the binary32
-// pre-tests, computed on the device by one thread per simulation.
+// pre-tests, computed on the device by a few warps per simulation.
 //
 // Cell size.  A candidate pair has |r| <= d_min + |v| t* < d0 + |v_i - v_j| dt
 // <= d0 + (s_i + s_j) dt with s = |v| (Sec. 2: the partner must reach its distance
@@ -34,8 +34,9 @@ __device__ __forceinline__ float f_up(double x) { return __double2float_ru(x); }
 // Hence: the cell counts and the cost estimates in binary32 (only the speed depends on
 // the choice; the margins of the cell width cover the rounding, see plan_cells), square
 // roots as upper bounds from the rounded-up binary32 root, per-axis values on a lane
-// each, and every parameter read before the first use of any.  One simulation: 35 -> 10 us
-// at 4096 particles, 47 -> 12 us at 2^20.
+// each, every parameter read before the first use of any, and the guard bands, which the
+// count does not need, left to the scan (compute_guards).  One simulation, record and grid:
+// 35 -> 4.8 us at 4096 particles, 47 -> 5.3 us at 2^20.
 struct CellPlan {
   int nc[3];
   float m;
@@ -125,6 +126,14 @@ __device__ inline float fast_cost(float nfast, float rho, float rf_cells, float 
   return nfast * (2.0f * tests + 15.0f * ncol);
 }
 
+// extent along x: the box, or the upper wall at the start of the step (particles are below it)
+__device__ __forceinline__ double extent_x(int bc, double box, double x0, double up, double dt,
+                                           uint64_t step) {
+  if (bc != KMC_REFLECT) return box;
+  const double X = x0 - up * ((double)step * dt);
+  return X > 0.0 ? X : box;
+}
+
 // Trial thresholds of the speed split, fractions of the bound V of max |v| (squares
 // rounded down), with their particle counts cleared for the next count: lane t the
 // threshold t.
@@ -138,19 +147,19 @@ __device__ inline void set_split_thresholds(SimDev& s, float vmax2_bound, uint32
 // Called by all 32 lanes of a warp: lane t < kSplitTrials estimates the cost of
 // trial threshold t, all lanes choose alike, lanes 0..2 take one axis each and lane 0
 // writes the rest of the grid.
-__device__ inline void compute_grid(SimDev& s, float vmax2_bound, uint64_t step, uint32_t lane) {
+__device__ inline void compute_grid(SimDev& s, float vmax2_bound, uint64_t step, bool have_counts,
+                                    uint32_t lane) {
   constexpr uint32_t kAll = 0xFFFFFFFFu;
-  const double u32 = 0x1p-24, u64 = 0x1p-53;
   // ---- parameters, all loads in flight together --------------------------------
   const int K = s.K, search_kernel = s.search_kernel, split_ok = s.split_ok;
   const uint32_t n = s.n, cell_cap = s.cell_cap;
   const bool fp32 = s.precision == KMC_GUARDED_FP32;
-  const double d0 = s.d0, dt = s.dt, d0sq = s.d0sq, cell_scale = s.cell_scale;
+  const double d0 = s.d0, dt = s.dt, cell_scale = s.cell_scale;
   const float min_occ = (float)s.split_min_occ;
   const double box0 = s.box[0], box1 = s.box[1], box2 = s.box[2];
   const int bc0 = s.bc[0], bc1 = s.bc[1], bc2 = s.bc[2];
   const double x0 = s.piston_x0, up = s.piston_u;
-  const bool can_split = split_ok && s.d.have_counts;
+  const bool can_split = split_ok && have_counts;
   const uint32_t my_trial = lane < (uint32_t)kSplitTrials ? lane : 0u;
   const float my_thr = s.d.split_thr[my_trial];
   const float my_nfast = (float)s.d.split_cnt[my_trial];
@@ -158,12 +167,7 @@ __device__ inline void compute_grid(SimDev& s, float vmax2_bound, uint64_t step,
   const double scale = cell_scale > 1.0 ? cell_scale : 1.0;
   const double V = sqrt_up(vmax2_bound);  // upper bound of max |v|
   const double Rfull = d0 + 2.0 * V * dt;
-  double ext0 = box0;
-  if (bc0 == KMC_REFLECT) {
-    // upper x wall at the start of this step (particles are below it)
-    const double X = x0 - up * ((double)step * dt);
-    ext0 = X > 0.0 ? X : box0;
-  }
+  const double ext0 = extent_x(bc0, box0, x0, up, dt, step);
   const float extf[3] = {(float)ext0, (float)box1, (float)box2};
   const bool per[3] = {bc0 == KMC_PERIODIC, bc1 == KMC_PERIODIC, bc2 == KMC_PERIODIC};
   const float Rf = f_up(Rfull);
@@ -266,58 +270,23 @@ __device__ inline void compute_grid(SimDev& s, float vmax2_bound, uint64_t step,
       kx = 2 * K;
     }
   }
-  const double m = (double)p.m;
-
-  // ---- per axis (lanes 0..2; the other lanes repeat lane 2) ---------------------
-  // Error of the binary32 separation against the binary64 one, per component (the
-  // binary32 mirror holds box coordinates and velocities, each rounded once):
-  //   multi-cell axis: both coordinates (u32 L each), a periodic image shifts one
-  //     side by the rounded box length (u32 L) and that sum is rounded (u32 L); the
-  //     difference itself rounds with u32 |r|: 4 u32 L + u32 rb, plus 8 u64 L for the
-  //     binary64 separation's own rounding;
-  //   one-cell axis (minimum image in binary32): u32 * 6.1 * extent + 8 u64 L.
-  // Velocity difference: 4.1 u32 V.  Component bounds: |r_k| <= rb_k, |v_k| <= 2V.
+  // per axis (lanes 0..2; the other lanes repeat lane 2)
   const int ax = lane < 2u ? (int)lane : 2;
   const int my_nc = ax == 0 ? p.nc[0] : ax == 1 ? p.nc[1] : p.nc[2];
-  const double my_ext = ax == 0 ? ext0 : ax == 1 ? box1 : box2;
-  const double my_box = ax == 0 ? box0 : ax == 1 ? box1 : box2;
-  const bool my_per = ax == 0 ? per[0] : ax == 1 ? per[1] : per[2];
+  const float my_iw = (float)my_nc / (ax == 0 ? extf[0] : ax == 1 ? extf[1] : extf[2]);
   const int Ka = ax == 0 ? kx : K;
-  const double my_w = my_nc == 1 ? my_ext : my_ext / (double)my_nc;
-  const float my_iw = (float)my_nc / (float)my_ext;
   int my_cfast = 0;
   if (split && my_nc != 1) {
     // at least Rfull (1 + m) / w cells: the product is within 4 u32 of it
     my_cfast = (int)ceilf(Rf * (1.0f + p.m) * my_iw * (1.0f + 1e-6f));
     if (my_cfast < Ka) my_cfast = Ka;
   }
-  const double L = my_box > my_ext ? my_box : my_ext;
-  const int Ke = my_cfast > Ka ? my_cfast : Ka;
-  double my_e, my_rb;
-  if (my_nc == 1) {
-    my_e = 6.1 * u32 * L + 8.0 * u64 * L;
-    my_rb = my_per ? 0.5 * L * (1.0 + 8.0 * u32) + 2.0 * my_e : L;
-  } else {
-    my_rb = (Ke + 1.0 + 2.0 * m) * my_w;
-    my_e = u32 * (4.0 * L + my_rb) * (1.0 + 1e-3) + 8.0 * u64 * L;
-  }
   Grid& g = s.d.grid;
   if (lane < 3u) {
     g.nc[lane] = my_nc;
     g.cfast[lane] = my_cfast;
-    g.w[lane] = my_w;
-    g.wf[lane] = (float)my_w;
     g.inv_wf[lane] = my_nc == 1 ? 0.0f : my_iw;
-    g.Lf[lane] = (float)my_box;
-    g.halfLf[lane] = (float)(0.5 * my_box);
-    g.tief[lane] = f_up(4.0 * my_e);
   }
-  const double e0 = __shfl_sync(kAll, my_e, 0), e1 = __shfl_sync(kAll, my_e, 1),
-               e2 = __shfl_sync(kAll, my_e, 2);
-  const double b0 = __shfl_sync(kAll, my_rb, 0), b1 = __shfl_sync(kAll, my_rb, 1),
-               b2 = __shfl_sync(kAll, my_rb, 2);
-  const double L0 = __shfl_sync(kAll, L, 0), L1 = __shfl_sync(kAll, L, 1),
-               L2 = __shfl_sync(kAll, L, 2);
   if (lane != 0) return;  // lane 0 writes the rest
   if (!p.ok) s.d.status |= ST_CELL_OVERFLOW;
   g.split = split ? 1u : 0u;
@@ -329,30 +298,68 @@ __device__ inline void compute_grid(SimDev& s, float vmax2_bound, uint64_t step,
   g.col_tz = p.col_tz;
   g.nkeys = p.nkeys;
   g.K = K;
+  g.m = p.m;
+}
 
-  // ---- binary64 sphere pre-test: R > c0 + c1 B  =>  not a candidate ----------
-  // Exactly, |r|^2 |v|^2 = (r.v)^2 + |r x v|^2, so |r|^2 = t*^2 |v|^2 + d_min^2 <
-  // dt^2 |v|^2 + d0^2 for a candidate; with the roundings of the test this holds
-  // with a relative slack below 30 u64, far inside the 2^-40 used here.
+// The guard bands of the step's pre-tests, from the grid that compute_grid chose.  Only the
+// searches need them, so they are worked out while the cells are counted up: in the chain of
+// the grid builder they took 5 us of every step, in a block of their own in the scan nothing
+// that shows (6.1 us at 4096 particles with and without).  All 32 lanes of a warp; part 0
+// sets the sphere tests and the reaches, part 1 the other tests' bands (one warp for both
+// took 6.8 us, longer than the scan of a small simulation).
+__device__ __noinline__ inline void compute_guards(SimDev& s, uint32_t part, uint32_t lane) {
+  constexpr uint32_t kAll = 0xFFFFFFFFu;
+  const double u32 = 0x1p-24, u64 = 0x1p-53;
+  Grid& g = s.d.grid;
+  // ---- per axis (lanes 0..2; the other lanes repeat lane 2) ---------------------
+  // Error of the binary32 separation against the binary64 one, per component (the
+  // binary32 mirror holds box coordinates and velocities, each rounded once):
+  //   multi-cell axis: both coordinates (u32 L each), a periodic image shifts one
+  //     side by the rounded box length (u32 L) and that sum is rounded (u32 L); the
+  //     difference itself rounds with u32 |r|: 4 u32 L + u32 rb, plus 8 u64 L for the
+  //     binary64 separation's own rounding;
+  //   one-cell axis (minimum image in binary32): u32 * 6.1 * extent + 8 u64 L.
+  // Velocity difference: 4.1 u32 V.  Component bounds: |r_k| <= rb_k, |v_k| <= 2V.
+  const int ax = lane < 2u ? (int)lane : 2;
+  const int my_nc = g.nc[ax], my_cfast = g.cfast[ax], Ka = ax == 0 ? g.kx : g.K;
+  const double m = (double)g.m;
+  const double my_box = s.box[ax];
+  const int my_bc = s.bc[ax];
+  const double d0 = s.d0, dt = s.dt, d0sq = s.d0sq, x0 = s.piston_x0, up = s.piston_u;
+  const uint64_t step = s.d.step;
+  const float vmax2_bound = s.d.vmax2, s1sq = g.s1sq;
+  const bool split = g.split != 0u;
+  const double V = sqrt_up(vmax2_bound);  // upper bound of max |v|
+  const double S1 = split ? sqrt_up(s1sq) : V;
+  const double my_ext = ax == 0 ? extent_x(my_bc, my_box, x0, up, dt, step) : my_box;
+  const double my_w = my_nc == 1 ? my_ext : my_ext / (double)my_nc;
+  const double L = my_box > my_ext ? my_box : my_ext;
+  const int Ke = my_cfast > Ka ? my_cfast : Ka;
+  double my_e, my_rb;
+  if (my_nc == 1) {
+    my_e = 6.1 * u32 * L + 8.0 * u64 * L;
+    my_rb = my_bc == KMC_PERIODIC ? 0.5 * L * (1.0 + 8.0 * u32) + 2.0 * my_e : L;
+  } else {
+    my_rb = (Ke + 1.0 + 2.0 * m) * my_w;
+    my_e = u32 * (4.0 * L + my_rb) * (1.0 + 1e-3) + 8.0 * u64 * L;
+  }
+  if (part == 0u && lane < 3u) {
+    g.wf[lane] = (float)my_w;
+    g.Lf[lane] = (float)my_box;
+    g.halfLf[lane] = (float)(0.5 * my_box);
+    g.tief[lane] = f_up(4.0 * my_e);
+  }
+  const double e0 = __shfl_sync(kAll, my_e, 0), e1 = __shfl_sync(kAll, my_e, 1),
+               e2 = __shfl_sync(kAll, my_e, 2);
+  const double b0 = __shfl_sync(kAll, my_rb, 0), b1 = __shfl_sync(kAll, my_rb, 1),
+               b2 = __shfl_sync(kAll, my_rb, 2);
+  const double L0 = __shfl_sync(kAll, L, 0), L1 = __shfl_sync(kAll, L, 1),
+               L2 = __shfl_sync(kAll, L, 2);
+  if (lane != 0) return;  // lane 0 writes the rest
+
   const double dt2 = dt * dt;
-  g.c0 = d0sq * ((1.0 + 0x1p-40) * (1.0 + 0x1p-50));
-  g.c1 = dt2 * ((1.0 + 0x1p-40) * (1.0 + 0x1p-50));
-
-  // ---- binary32 pre-tests ------------------------------------------------------
   const double er = fmax(e0, fmax(e1, e2)), rbmax = fmax(b0, fmax(b1, b2));
   const double Lmax = fmax(L0, fmax(L1, L2));
-  {
-    // row trimming: a slow-slow candidate has |r| < d0 + (|v_i| + |v_j|) dt <= d0 + 2 S1 dt
-    const double S1dt = S1 * dt;
-    const double reach = (d0 + 2.0 * S1dt) * (1.0 + 1e-6);
-    g.row_r2 = f_up(reach * reach * (1.0 + 1e-6));
-    // per particle: (i, j) with j slow has |r| < d0 + (|v_i| + |v_j|) dt <= d0 + S1 dt + |v_i| dt
-    g.row_a = f_up((d0 + S1dt) * (1.0 + 1e-6));
-    g.row_b = f_up(dt * (1.0 + 1e-6));
-    g.fast_a = f_up((d0 + V * dt) * (1.0 + 1e-6));
-    g.row_eps = f_up(16.0 * u32 * Lmax);
-    g.row_pad = f_up(4.0 * u32 * Lmax);
-  }
   const double rn = sqrt_up(f_up((b0 * b0 + b1 * b1) + b2 * b2)) * (1.0 + 1e-6);
   const double V2 = V * V, rnV2 = rn * 2.0 * V;
   const double ev = 4.1 * u32 * V;
@@ -363,17 +370,36 @@ __device__ inline void compute_grid(SimDev& s, float vmax2_bound, uint64_t step,
   const double rel40 = 1.0 + 0x1p-40;
   const double s3 = 1.7320508075688772 * (1.0 + 1e-15);
   const double bslack = 7.0 * ev * V + 3.0 * ev * ev;  // |v|^2 - |v~|^2 slack, absolute
-  // sphere test
-  const double c0 = (rel40 * (d0sq + dt2 * bslack) + 2.0 * s3 * er * rn) * (1.0 + g3);
-  g.s_c0 = f_up(c0 * up2);
-  g.s_c1 = f_up(dt2 * (rel40 * (1.0 + g3) / (1.0 - g3) * up2));
-  // pair filter of the tiled search (kmc_search.cu, "Error of the filter"): the sphere
-  // test's constant with three times the separation error er, and the slack of
-  // velocities rounded to 11 bits, 2^-7 (dt S1)^2
-  g.tile_c = f_up((rel40 * (d0sq + dt2 * bslack) + 8.0 * s3 * er * rn + 27.0 * er * er) *
-                      ((1.0 + g3) * up2) + 0x1p-7 * 1.001 * dt2 * S1 * S1);
-  g.tile_k = sqrtf(g.s_c1);
-  g.s1f = f_up(S1);
+  if (part == 0u) {
+    // ---- binary64 sphere pre-test: R > c0 + c1 B  =>  not a candidate ----------
+    // Exactly, |r|^2 |v|^2 = (r.v)^2 + |r x v|^2, so |r|^2 = t*^2 |v|^2 + d_min^2 <
+    // dt^2 |v|^2 + d0^2 for a candidate; with the roundings of the test this holds
+    // with a relative slack below 30 u64, far inside the 2^-40 used here.
+    g.c0 = d0sq * ((1.0 + 0x1p-40) * (1.0 + 0x1p-50));
+    g.c1 = dt2 * ((1.0 + 0x1p-40) * (1.0 + 0x1p-50));
+    // row trimming: a slow-slow candidate has |r| < d0 + (|v_i| + |v_j|) dt <= d0 + 2 S1 dt
+    const double S1dt = S1 * dt;
+    const double reach = (d0 + 2.0 * S1dt) * (1.0 + 1e-6);
+    g.row_r2 = f_up(reach * reach * (1.0 + 1e-6));
+    // per particle: (i, j) with j slow has |r| < d0 + (|v_i| + |v_j|) dt <= d0 + S1 dt + |v_i| dt
+    g.row_a = f_up((d0 + S1dt) * (1.0 + 1e-6));
+    g.row_b = f_up(dt * (1.0 + 1e-6));
+    g.fast_a = f_up((d0 + V * dt) * (1.0 + 1e-6));
+    g.row_eps = f_up(16.0 * u32 * Lmax);
+    g.row_pad = f_up(4.0 * u32 * Lmax);
+    // sphere test
+    const double c0 = (rel40 * (d0sq + dt2 * bslack) + 2.0 * s3 * er * rn) * (1.0 + g3);
+    g.s_c0 = f_up(c0 * up2);
+    g.s_c1 = f_up(dt2 * (rel40 * (1.0 + g3) / (1.0 - g3) * up2));
+    // pair filter of the tiled search (kmc_search.cu, "Error of the filter"): the sphere
+    // test's constant with three times the separation error er, and the slack of
+    // velocities rounded to 11 bits, 2^-7 (dt S1)^2
+    g.tile_c = f_up((rel40 * (d0sq + dt2 * bslack) + 8.0 * s3 * er * rn + 27.0 * er * er) *
+                        ((1.0 + g3) * up2) + 0x1p-7 * 1.001 * dt2 * S1 * S1);
+    g.tile_k = sqrtf(g.s_c1);
+    g.s1f = f_up(S1);
+    return;
+  }
   // approach test (t* >= 0): |A~ - A64| <= a_g
   const double Ga = (s3 * (ev * rn + 2.0 * V * er) + rnV2 * (g3 * 1.01 + g3d)) * (1.0 + 1e-3);
   g.a_g = f_up(Ga);

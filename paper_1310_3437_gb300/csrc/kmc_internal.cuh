@@ -54,10 +54,11 @@ struct Grid {
   uint32_t col_shift; // log2 of the Morton tile edge T (T <= 8)
   uint32_t col_tz;    // tiles along z
   int32_t kx;         // cells per stencil radius along x (K, or 2K under the row search)
-  double w[3];        // cell widths
-  float wf[3];        // cell widths (binary32)
+  float m;            // relative margin of the cell width
   float inv_wf[3];    // cells per unit length (binary32, cell assignment)
-  // guarded binary32 pre-tests (kmc_search.cu derives them; kmc_push.cu sets them)
+  // from here on set while the step's cells are counted up (compute_guards)
+  float wf[3];        // cell widths (binary32)
+  // guarded binary32 pre-tests (kmc_search.cu derives them)
   float s_c0, s_c1;   // sphere test: drop if R > s_c0 + s_c1 * B
   float a_g;          // approach test: drop if A < -a_g
   float t_g, dtf;     // time test: drop if A - dtf * B > t_g

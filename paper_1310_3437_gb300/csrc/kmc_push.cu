@@ -13,8 +13,8 @@
 //   k_profile   every profile_every steps: per x-bin count, sum v and sum v^2, in
 //               exact fixed point (int64 digits), so the sums do not depend on the
 //               order of the particles.
-//   k_finalize  one thread per simulation: step record, step counter, the next
-//               grid (kmc_grid.cuh) and the per-step counters reset.
+//   k_finalize  two warps per simulation: the next grid (kmc_grid.cuh); step record,
+//               step counter and the per-step counters reset.
 #include "kmc_grid.cuh"
 #include "kmc_internal.cuh"
 
@@ -224,6 +224,8 @@ __global__ void __launch_bounds__(kTile) k_profile(Batch B) {
     if (acc[i]) atomicAdd((unsigned long long*)&out[i], (unsigned long long)acc[i]);
 }
 
+constexpr int kFinalBlock = 256;  // two warps per simulation
+
 // ---- end of step ------------------------------------------------------------ //
 __device__ void reset_step_counters(SimDev& s) {
   s.d.n_raw = 0;
@@ -255,59 +257,61 @@ __device__ __forceinline__ void clear_profile(SimDev& s, uint32_t count, uint32_
   for (int i = (int)lane; i < s.profile_bins * kProfQ; i += 32) out[i] = 0;
 }
 
-// One warp per simulation: lane 0 keeps the books, the warp builds the next grid.  The
-// kernel is one chain of dependent operations, so everything the record needs is read
-// before the first store (the compiler may not move a load of the descriptor across one).
-__global__ void k_finalize(Batch B) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const int nwarps = (int)(gridDim.x * blockDim.x / 32u);
-  for (int k = (int)((blockIdx.x * blockDim.x + threadIdx.x) / 32u); k < B.nsims; k += nwarps) {
-    SimDev& s = B.sim(k);
-    if (!sim_active(s)) continue;
-    const uint64_t step = s.d.step, hist_count = s.d.hist_count, steps_left = s.d.steps_left;
-    const uint32_t hist_cap = s.hist_cap, was_due = s.d.prof_due, prof_cap = s.prof_cap;
-    const uint32_t n_raw = s.d.n_raw, parity = s.d.parity;
-    const uint32_t prof_count = s.d.prof_count + was_due;  // snapshots, this step's included
-    const float vmax2 = __uint_as_float(s.d.vmax2_acc);
-    const uint32_t due = prof_due_at(s, step + 1);
-    if (lane == 0) {
-      kmc_step_counts rec;
-      rec.step = step;
-      uint32_t coll = 0;
-      for (int r = 0; r < 4; ++r) {
-        rec.round_pairs[r] = s.d.round_pairs[r];
-        coll += rec.round_pairs[r];
-      }
-      rec.collisions = coll;
-      rec.edges = s.d.n_edges;
-      rec.survivors = n_raw;
-      rec.cells = s.d.grid.nkeys;
-      rec.pair_tests = s.d.pair_tests;
-      rec.fast_tests = s.d.fast_tests;
-      rec.absorbed = s.d.n_absorbed;
-      rec.live = live_count(s) - rec.absorbed;  // this step's grid, before the next one
-      const uint32_t have = s.split_ok ? 1u : 0u;
-      s.hist[mod_u32(hist_count, hist_cap)] = rec;
-      s.d.hist_count = hist_count + 1;
-      if (was_due) {
-        s.prof_step[(prof_count - 1u) % prof_cap] = step;
-        s.d.prof_count = prof_count;
-      }
-      s.d.last_raw = n_raw;
-      s.d.have_counts = have;
-      s.d.parity = parity ^ 1u;
-      s.d.step = step + 1;
-      s.d.steps_left = steps_left - 1;
-      s.d.vmax2 = vmax2;
-      s.d.prof_due = due;
-    }
-    __syncwarp();
-    compute_grid(s, vmax2, step + 1, lane);
-    __syncwarp();
-    if (lane == 0) reset_step_counters(s);
-    if (due) clear_profile(s, prof_count, lane);
-    __syncwarp();
+// Two warps per simulation: the first builds the next grid, the second keeps the books.
+// Each is one chain of dependent operations, so what both need is read before the barrier
+// that comes before the first store.
+__global__ void __launch_bounds__(kFinalBlock) k_finalize(Batch B) {
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const int k = (int)(blockIdx.x * (kFinalBlock / 64u) + warp / 2u);
+  const bool run = k < B.nsims && sim_active(B.sim(k));
+  SimDev& s = B.sim(run ? k : 0);
+  const uint64_t step = s.d.step;
+  const float vmax2 = __uint_as_float(s.d.vmax2_acc);
+  if (warp % 2u == 0u) {
+    __syncthreads();
+    if (run) compute_grid(s, vmax2, step + 1, s.split_ok != 0, lane);
+    return;
   }
+  const uint64_t hist_count = s.d.hist_count, steps_left = s.d.steps_left;
+  const uint32_t hist_cap = s.hist_cap, was_due = s.d.prof_due, prof_cap = s.prof_cap;
+  const uint32_t n_raw = s.d.n_raw, parity = s.d.parity;
+  const uint32_t prof_count = s.d.prof_count + was_due;  // snapshots, this step's included
+  const uint32_t due = prof_due_at(s, step + 1);
+  kmc_step_counts rec;
+  rec.step = step;
+  uint32_t coll = 0;
+  for (int r = 0; r < 4; ++r) {
+    rec.round_pairs[r] = s.d.round_pairs[r];
+    coll += rec.round_pairs[r];
+  }
+  rec.collisions = coll;
+  rec.edges = s.d.n_edges;
+  rec.survivors = n_raw;
+  rec.cells = s.d.grid.nkeys;
+  rec.pair_tests = s.d.pair_tests;
+  rec.fast_tests = s.d.fast_tests;
+  rec.absorbed = s.d.n_absorbed;
+  rec.live = run ? live_count(s) - rec.absorbed : 0u;  // this step's grid, before the next one
+  const uint32_t have = s.split_ok ? 1u : 0u;
+  __syncthreads();
+  if (!run) return;
+  if (lane == 0) {
+    s.hist[mod_u32(hist_count, hist_cap)] = rec;
+    s.d.hist_count = hist_count + 1;
+    if (was_due) {
+      s.prof_step[(prof_count - 1u) % prof_cap] = step;
+      s.d.prof_count = prof_count;
+    }
+    s.d.last_raw = n_raw;
+    s.d.have_counts = have;
+    s.d.parity = parity ^ 1u;
+    s.d.step = step + 1;
+    s.d.steps_left = steps_left - 1;
+    s.d.vmax2 = vmax2;
+    s.d.prof_due = due;
+    reset_step_counters(s);
+  }
+  if (due) clear_profile(s, prof_count, lane);
 }
 
 // ---- initial grid (creation, resume, after an error is cleared) ------------ //
@@ -365,15 +369,14 @@ __global__ void __launch_bounds__(kTile) k_split_count(Batch B) {
     atomicAdd(&s.d.split_cnt[threadIdx.x], scnt[threadIdx.x]);
 }
 
-// one warp per simulation, as k_finalize
+// one warp per simulation
 __global__ void k_init_grid(Batch B) {
   const uint32_t lane = threadIdx.x & 31u;
   const int nwarps = (int)(gridDim.x * blockDim.x / 32u);
   for (int k = (int)((blockIdx.x * blockDim.x + threadIdx.x) / 32u); k < B.nsims; k += nwarps) {
     SimDev& s = B.sim(k);
     if (lane == 0) s.d.have_counts = s.split_ok ? 1u : 0u;  // k_split_count's
-    __syncwarp();
-    compute_grid(s, s.d.vmax2, s.d.step, lane);
+    compute_grid(s, s.d.vmax2, s.d.step, s.split_ok != 0, lane);
     __syncwarp();
     const uint32_t due = prof_due_at(s, s.d.step);
     if (lane == 0) {
@@ -408,7 +411,7 @@ int launch_push(const LaunchPlan& L, cudaStream_t st) {
     if (L.absorb) k_profile<true><<<L.prtiles, kTile, smem, st>>>(L.b);
     else k_profile<false><<<L.prtiles, kTile, smem, st>>>(L.b);
   }
-  k_finalize<<<(L.b.nsims + 7) / 8, 256, 0, st>>>(L.b);
+  k_finalize<<<(L.b.nsims + 3) / 4, kFinalBlock, 0, st>>>(L.b);
   return L.profiles ? 3 : 2;
 }
 

@@ -6,13 +6,15 @@
 //             atomic increment (a run of equal keys in neighbouring lanes shares one
 //             atomic).
 //   scan      segmented exclusive scan of the counts -> cell_start (one launch,
-//             decoupled look-back); clears the counts for the next step.
+//             decoupled look-back); clears the counts for the next step.  Its first
+//             blocks work out the guard bands of the searches meanwhile.
 //   k_scatter records the source of every position of the new order;
 //   k_gather  permutes the binary64 state into the other buffer, writes the
 //             binary32 mirror (box coordinates and velocity) for the guarded
 //             search and resets the per-particle step arrays.
 // The order inside a cell depends on atomic timing; nothing downstream depends on
 // it (argmin over a total order, integer counters, order-free profile sums).
+#include "kmc_grid.cuh"
 #include "kmc_internal.cuh"
 
 namespace kmc {
@@ -131,8 +133,16 @@ __device__ __forceinline__ unsigned long long scan_word(uint32_t epoch, unsigned
   return ((unsigned long long)epoch << 34) | (state << 32) | (unsigned long long)value;
 }
 
-__global__ void __launch_bounds__(kTile) k_scan_onepass(Batch B, uint32_t ntiles) {
+// The first `guards` blocks have no tile: two warps of them per simulation work out the guard
+// bands of the step's searches.
+__global__ void __launch_bounds__(kTile) k_scan_onepass(Batch B, uint32_t ntiles, uint32_t guards) {
   __shared__ uint32_t s_tile, s_excl;
+  if (blockIdx.x < guards) {
+    const int k = (int)(blockIdx.x * (kTile / 64) + threadIdx.x / 64u);
+    if (k < B.nsims && sim_active(B.sim(k)))
+      compute_guards(B.sim(k), (threadIdx.x >> 5) & 1u, threadIdx.x & 31u);
+    return;
+  }
   if (threadIdx.x == 0) s_tile = atomicAdd(&B.scan_ctl[0], 1u);
   __syncthreads();
   const uint32_t tile = s_tile;
@@ -369,8 +379,8 @@ __global__ void __launch_bounds__(kTile / 2) k_gather(Batch B) {
 
 // --------------------------------------------------------------------------- //
 int launch_cell_scan(const LaunchPlan& L, cudaStream_t st) {
-  const uint32_t nt = L.stiles_c;
-  k_scan_onepass<<<nt, kTile, 0, st>>>(L.b, nt);
+  const uint32_t nt = L.stiles_c, guards = (uint32_t)(L.b.nsims + kTile / 64 - 1) / (kTile / 64);
+  k_scan_onepass<<<guards + nt, kTile, 0, st>>>(L.b, nt, guards);
   return 1;
 }
 
