@@ -1502,18 +1502,59 @@ void grids_of(int num_sms, uint32_t ptiles, LaunchPlan& L) {
        L.row_blocks_px, L.row_shift_px);
 }
 
+// The searches of a step do not depend on each other (they append to one pair buffer by
+// atomics), so in a captured step they become branches that join after the last: next()
+// before each further search puts the capture back to where the first one started.  A step
+// then waits for the longest of them instead of for their sum, and the idle ones cost nothing:
+// ten binary64 steps of 4096 particles 0.96 -> 0.83 ms (17 us of tiles beside 13 of fast
+// particles), four of an ensemble of 30 3.09 -> 2.73 ms, eight of 262 k particles 1.16 -> 1.10.
+// Outside a capture, and after more than kMaxEnds nodes, one follows the other.
+class Branches {
+ public:
+  explicit Branches(cudaStream_t st) : st_(st) { nfirst_ = ends(first_); }
+  void next() {
+    if (nfirst_ == 0) return;
+    nlast_ += ends(last_ + nlast_);
+    cudaStreamUpdateCaptureDependencies(st_, first_, nullptr, nfirst_, cudaStreamSetCaptureDependencies);
+  }
+  void join() {
+    if (nfirst_ == 0) return;
+    nlast_ += ends(last_ + nlast_);
+    cudaStreamUpdateCaptureDependencies(st_, last_, nullptr, nlast_, cudaStreamSetCaptureDependencies);
+  }
+
+ private:
+  static constexpr size_t kMaxEnds = 4, kMaxSearches = 5;
+  // the nodes that the next captured launch would follow (0: no capture, or too many)
+  size_t ends(cudaGraphNode_t* to) const {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    const cudaGraphNode_t* deps = nullptr;
+    size_t n = 0;
+    if (cudaStreamGetCaptureInfo(st_, &status, nullptr, nullptr, &deps, nullptr, &n) != cudaSuccess ||
+        status != cudaStreamCaptureStatusActive || n > kMaxEnds)
+      return 0;
+    std::copy(deps, deps + n, to);
+    return n;
+  }
+  cudaStream_t st_;
+  cudaGraphNode_t first_[kMaxEnds], last_[kMaxEnds * kMaxSearches];
+  size_t nfirst_ = 0, nlast_ = 0;
+};
+
 // Every search that a simulation of the plan may choose for a step; each runs the one its
 // grid selected (the other kernels return at once).
 template <int PREC, int K>
-int launch_slow(const LaunchPlan& L, cudaStream_t st) {
+int launch_slow(const LaunchPlan& L, cudaStream_t st, Branches& b) {
   int n = 1;
   if (L.tile_shift) k_search_tiles<PREC, K, true><<<L.tile_blocks, kTile, 0, st>>>(L.b, L.tile_shift);
   else k_search_tiles<PREC, K, false><<<L.tile_blocks, kTile, 0, st>>>(L.b, 0);
   if (L.particle) {
+    b.next();
     k_search<PREC, K><<<L.part_blocks, kTile, 0, st>>>(L.b);
     ++n;
   }
   auto rows = [&](auto alone, auto shared, size_t bytes, int grid, int shift) {
+    b.next();
     if (shift) shared<<<grid, kTile, bytes, st>>>(L.b, shift);
     else alone<<<grid, kTile, bytes, st>>>(L.b, 0);
     ++n;
@@ -1540,15 +1581,18 @@ void search_grids(int precision, int K, int num_sms, uint32_t ptiles, LaunchPlan
 
 int launch_search(const LaunchPlan& L, int precision, int K, cudaStream_t st, cudaEvent_t* ev_slow) {
   int n = 0;
+  Branches b(st);
   if (ev_slow) cudaEventRecord(ev_slow[0], st);
   if (precision == KMC_FP64) {
-    n = K == 2 ? launch_slow<KMC_FP64, 2>(L, st) : launch_slow<KMC_FP64, 1>(L, st);
+    n = K == 2 ? launch_slow<KMC_FP64, 2>(L, st, b) : launch_slow<KMC_FP64, 1>(L, st, b);
   } else {
-    n = K == 2 ? launch_slow<KMC_GUARDED_FP32, 2>(L, st) : launch_slow<KMC_GUARDED_FP32, 1>(L, st);
+    n = K == 2 ? launch_slow<KMC_GUARDED_FP32, 2>(L, st, b) : launch_slow<KMC_GUARDED_FP32, 1>(L, st, b);
   }
   if (ev_slow) cudaEventRecord(ev_slow[1], st);
+  b.next();
   if (precision == KMC_FP64) k_search_fast<KMC_FP64><<<L.fast_blocks, kCellWarps * 32, 0, st>>>(L.b);
   else k_search_fast<KMC_GUARDED_FP32><<<L.fast_blocks, kCellWarps * 32, 0, st>>>(L.b);
+  b.join();
   return n + 1;
 }
 
