@@ -379,6 +379,7 @@ int build_plan(Plan& P, const std::vector<kmc_sim*>& sims, cudaStream_t st, std:
   L.ptiles = pt[m];
   L.stiles_c = sc[m];
   L.prtiles = pr[m];
+  L.prof_blocks = (int)std::min<uint32_t>(std::max(pr[m], 1u), 4u * (uint32_t)num_sms());
   // a block per tile of particles (one particle in twenty has a candidate pair), as many as
   // the SMs hold at most: a launch of idle blocks takes 1.1 us, one of a few 0.6
   L.edge_blocks = (int)std::min<uint32_t>(std::max(pt[m], 1u), 8u * (uint32_t)num_sms());

@@ -16,7 +16,7 @@ namespace kmc {
 
 constexpr int kTile = 256;          // particles per block in particle kernels
 constexpr int kScanTile = 8192;     // keys per tile of the cell scan
-constexpr int kProfTile = 8192;     // particles per block in the profile kernel
+constexpr int kProfTile = 4096;     // particles per tile of the profile kernel
 constexpr int kEdgeBlock = 256;     // threads per block in edge / adjacency kernels
 constexpr int kSearchBuf = 512;     // per-block shared-memory staging of emitted pairs
 constexpr uint32_t kNone = 0xFFFFFFFFu;
@@ -575,6 +575,7 @@ struct LaunchPlan {
   Batch b;
   uint32_t ptiles, stiles_c, prtiles;
   int edge_blocks;
+  int prof_blocks;         // grid of the profile kernel, each block a range of tiles
   int round_blocks;        // cooperative grid of the later matching rounds
   bool lists = false;      // domains: the rounds work on per-particle candidate lists
   int part_blocks;  // grid-stride grids of the particle, tiled, row and fast searches

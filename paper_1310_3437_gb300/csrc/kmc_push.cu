@@ -194,34 +194,84 @@ __global__ void __launch_bounds__(kTile) k_push(Batch B) {
   if (ABS && s.absorb && threadIdx.x == 0 && sgone) atomicAdd(&s.d.n_absorbed, sgone);
 }
 
-template <bool ABS>
-__global__ void __launch_bounds__(kTile) k_profile(Batch B) {
-  extern __shared__ long long acc[];
-  int k = find_sim(B.prtile, B.nsims, blockIdx.x);
-  SimDev& s = B.sim(k);
-  if (!sim_active(s) || !s.d.prof_due) return;
-  const int nb = s.profile_bins;
-  for (int i = threadIdx.x; i < nb * kProfQ; i += blockDim.x) acc[i] = 0;
-  __syncthreads();
-  const int cur = s.d.parity ^ 1;
-  const double scale = ddiv((double)nb, s.profile_range);
-  uint32_t base = (blockIdx.x - B.tile0(B.prtile, k)) * kProfTile;
-  for (uint32_t i = threadIdx.x; i < kProfTile; i += blockDim.x) {
-    uint32_t p = base + i;
-    if (p >= s.n) break;
-    if (ABS && s.absorb && s.last[cur][p] == KMC_ABSORBED) continue;  // out of the gas
-    double x = s.x[cur][0][p];
-    if (!(x >= 0.0)) continue;
-    double f = dmul(x, scale);
-    if (f >= (double)nb) continue;
-    int b = (int)f;
-    const double v[3] = {s.v[cur][0][p], s.v[cur][1][p], s.v[cur][2][p]};
-    profile_add(acc + b * kProfQ, v);
+// The particles of a block's tiles are summed in shared memory, in 32-bit words of 16-bit
+// digits (an atomic addition of 64 bits in shared memory is a compare-and-swap loop: a
+// profile of 2^20 particles took 240 us, now 50), and the words flushed to the bin's
+// 64-bit counters when the simulation changes or a digit could overflow: up to kProfFlush
+// particles add up to less than 2^31.  A bin is kProfW words, an odd number, so that
+// neighbouring bins lie in different banks: [0] the count, [1 + 6 t + c] digit c of term t
+// (the three v_a, then the three v_a^2), [37] the terms out of range.
+constexpr int kProfW = 39;
+constexpr uint32_t kProfFlush = 1u << 15;
+
+__device__ __forceinline__ void profile_term(int* q, double x, int& bad) {
+  long long d[3];
+  if (!fx_digits(x, d)) {
+    ++bad;
+    return;
   }
-  __syncthreads();
-  long long* out = s.prof_acc + (size_t)(s.d.prof_count % s.prof_cap) * nb * kProfQ;
-  for (int i = threadIdx.x; i < nb * kProfQ; i += blockDim.x)
-    if (acc[i]) atomicAdd((unsigned long long*)&out[i], (unsigned long long)acc[i]);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int m = x < 0.0 ? -1 : 1;
+    const uint32_t w = (uint32_t)(d[c] < 0 ? -d[c] : d[c]);
+    if (w & 0xFFFFu) atomicAdd(q + 2 * c, m * (int)(w & 0xFFFFu));
+    if (w >> 16) atomicAdd(q + 2 * c + 1, m * (int)(w >> 16));
+  }
+}
+
+template <bool ABS>
+__global__ void __launch_bounds__(kTile) k_profile(Batch B, uint32_t ntiles) {
+  extern __shared__ int acc[];
+  const uint32_t per = (ntiles + gridDim.x - 1) / gridDim.x, t0 = blockIdx.x * per;
+  const uint32_t t1 = t0 + per < ntiles ? t0 + per : ntiles;
+  for (uint32_t tile = t0; tile < t1;) {
+    // the block's tiles of one simulation, at most kProfFlush particles
+    const int k = find_sim(B.prtile, B.nsims, tile);
+    const uint32_t first = B.tile0(B.prtile, k);
+    SimDev& s = B.sim(k);
+    const uint32_t all = first + (s.n + kProfTile - 1u) / kProfTile;
+    uint32_t end = t1 < all ? t1 : all;
+    if (!sim_active(s) || !s.d.prof_due) {
+      tile = end;
+      continue;
+    }
+    if (end - tile > kProfFlush / kProfTile) end = tile + kProfFlush / kProfTile;
+    const int nb = s.profile_bins;
+    for (int i = threadIdx.x; i < nb * kProfW; i += blockDim.x) acc[i] = 0;
+    __syncthreads();
+    const int cur = s.d.parity ^ 1;
+    const double scale = ddiv((double)nb, s.profile_range);
+    const uint64_t stop = (uint64_t)(end - first) * kProfTile;
+    const uint32_t pend = stop < s.n ? (uint32_t)stop : s.n;
+    for (uint32_t p = (tile - first) * kProfTile + threadIdx.x; p < pend; p += blockDim.x) {
+      if (ABS && s.absorb && s.last[cur][p] == KMC_ABSORBED) continue;  // out of the gas
+      double x = s.x[cur][0][p];
+      if (!(x >= 0.0)) continue;
+      double f = dmul(x, scale);
+      if (f >= (double)nb) continue;
+      int* q = acc + (int)f * kProfW;
+      int bad = 0;
+      atomicAdd(q, 1);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const double v = s.v[cur][a][p];
+        profile_term(q + 1 + 6 * a, v, bad);
+        profile_term(q + 19 + 6 * a, dmul(v, v), bad);
+      }
+      if (bad) atomicAdd(q + 37, bad);
+    }
+    __syncthreads();
+    long long* out = s.prof_acc + (size_t)(s.d.prof_count % s.prof_cap) * nb * kProfQ;
+    for (int i = threadIdx.x; i < nb * kProfQ; i += blockDim.x) {
+      const int b = i / kProfQ, c = i - b * kProfQ;
+      const int* q = acc + b * kProfW;
+      const long long sum = c == 0 ? q[0] : c == kProfQ - 1 ? q[37]
+                                          : q[2 * c - 1] + 65536ll * q[2 * c];
+      if (sum) atomicAdd((unsigned long long*)&out[i], (unsigned long long)sum);
+    }
+    __syncthreads();
+    tile = end;
+  }
 }
 
 constexpr int kFinalBlock = 256;  // two warps per simulation
@@ -404,12 +454,12 @@ int launch_init_grid(const LaunchPlan& L, cudaStream_t st) {
 }
 
 int launch_push(const LaunchPlan& L, cudaStream_t st) {
-  const size_t smem = 256 * kProfQ * sizeof(long long);
+  const size_t smem = 256 * kProfW * sizeof(int);
   if (L.absorb) k_push<true><<<L.ptiles, kTile, 0, st>>>(L.b);
   else k_push<false><<<L.ptiles, kTile, 0, st>>>(L.b);
   if (L.profiles) {
-    if (L.absorb) k_profile<true><<<L.prtiles, kTile, smem, st>>>(L.b);
-    else k_profile<false><<<L.prtiles, kTile, smem, st>>>(L.b);
+    if (L.absorb) k_profile<true><<<L.prof_blocks, kTile, smem, st>>>(L.b, L.prtiles);
+    else k_profile<false><<<L.prof_blocks, kTile, smem, st>>>(L.b, L.prtiles);
   }
   k_finalize<<<(L.b.nsims + 3) / 4, kFinalBlock, 0, st>>>(L.b);
   return L.profiles ? 3 : 2;
