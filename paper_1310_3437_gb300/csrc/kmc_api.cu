@@ -379,6 +379,7 @@ int build_plan(Plan& P, const std::vector<kmc_sim*>& sims, cudaStream_t st, std:
   L.ptiles = pt[m];
   L.stiles_c = sc[m];
   L.prtiles = pr[m];
+  L.push_blocks = (int)std::min<uint32_t>(std::max(pt[m], 1u), 8u * (uint32_t)num_sms());
   L.prof_blocks = (int)std::min<uint32_t>(std::max(pr[m], 1u), 4u * (uint32_t)num_sms());
   // a block per tile of particles (one particle in twenty has a candidate pair), as many as
   // the SMs hold at most: a launch of idle blocks takes 1.1 us, one of a few 0.6
@@ -667,7 +668,7 @@ int create_impl(const kmc_params* p, const double* const* src6, const uint32_t* 
   Sizes zs = sizes_of(*p);
   SimDev& h = s->h;
   h.n = p->n;
-  for (int a = 0; a < 3; ++a) { h.bc[a] = p->bc[a]; h.box[a] = p->box[a]; }
+  for (int a = 0; a < 3; ++a) { h.bc[a] = p->bc[a]; h.box[a] = p->box[a]; h.half_box[a] = 0.5 * p->box[a]; }
   h.max_rounds = p->max_rounds ? p->max_rounds : 4;
   h.precision = p->precision;
   h.profile_bins = (int32_t)zs.bins;

@@ -324,7 +324,7 @@ __device__ __noinline__ inline void compute_guards(SimDev& s, uint32_t part, uin
   const int my_nc = g.nc[ax], my_cfast = g.cfast[ax], Ka = ax == 0 ? g.kx : g.K;
   const double m = (double)g.m;
   const double my_box = s.box[ax];
-  const int my_bc = s.bc[ax];
+  const int my_bc = s.bc[ax], my_bc0 = s.bc[0];
   const double d0 = s.d0, dt = s.dt, d0sq = s.d0sq, x0 = s.piston_x0, up = s.piston_u;
   const uint64_t step = s.d.step;
   const float vmax2_bound = s.d.vmax2, s1sq = g.s1sq;
@@ -400,6 +400,10 @@ __device__ __noinline__ inline void compute_guards(SimDev& s, uint32_t part, uin
     g.s1f = f_up(S1);
     return;
   }
+  // the upper x wall at the end of the step, for the push (never -0.0)
+  s.d.wall_x = my_bc0 == KMC_PERIODIC
+                   ? 0.0
+                   : __dadd_rn(__dsub_rn(x0, __dmul_rn(up, __dmul_rn((double)(step + 1), dt))), 0.0);
   // approach test (t* >= 0): |A~ - A64| <= a_g
   const double Ga = (s3 * (ev * rn + 2.0 * V * er) + rnV2 * (g3 * 1.01 + g3d)) * (1.0 + 1e-3);
   g.a_g = f_up(Ga);

@@ -92,6 +92,7 @@ struct Dyn {
   uint32_t adj_used;    // domains: candidate-list entries handed out this step
   uint32_t wl_len[5];   // open pairs before matching round r >= 1, filled by round r - 1
                         // (domains: [0] particles with candidates)
+  double wall_x;        // upper x wall at the end of the step (compute_guards)
   unsigned long long pair_tests;
   unsigned long long fast_tests;  // the part of pair_tests done by the fast-particle search
   uint32_t last_raw;    // n_raw of the last completed step (its pair buffer is kept)
@@ -113,6 +114,7 @@ struct SimDev {
   int32_t planar;       // 1: x-y dynamics (vz = 0), scatter directions in the plane
   double split_min_occ; // smallest mean occupancy of the slow grid under a split
   double box[3];
+  double half_box[3];   // box / 2
   double piston_x0, piston_u, d0, dt, d0sq;
   double profile_range, cell_scale;
   uint64_t seed;
@@ -225,6 +227,30 @@ __device__ __forceinline__ double dsub(double a, double b) { return __dsub_rn(a,
 __device__ __forceinline__ double dmul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double ddiv(double a, double b) { return __ddiv_rn(a, b); }
 __device__ __forceinline__ double dsqrt(double a) { return __dsqrt_rn(a); }
+
+// Comparisons of finite doubles on the integer pipes (the binary64 pipe is the
+// scarce one on this part).  For a finite x and a positive finite bound y the order
+// of the values is the order of the bit patterns read as signed integers; negative
+// x (including -0.0) compare below every positive y.
+__device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
+__device__ __forceinline__ bool lt_zero(double x) {  // x < 0.0 (false for -0.0)
+  return (unsigned long long)dbits(x) > 0x8000000000000000ull;
+}
+// x > y of finite doubles, y not -0.0: the patterns of negative values in reverse order
+__device__ __forceinline__ bool gt_bits(double x, double y) {
+  long long a = dbits(x), b = dbits(y);
+  a ^= (long long)((unsigned long long)(a >> 63) >> 1);
+  b ^= (long long)((unsigned long long)(b >> 63) >> 1);
+  return a > b;
+}
+// minimum image on an axis of length L, h = L / 2: r - L if r > h, r + L if r < -h
+__device__ __forceinline__ double min_image(double r, double L, double h) {
+  const uint32_t hi = (uint32_t)__double2hiint(r);
+  const unsigned long long mag =
+      (unsigned long long)(hi & 0x7FFFFFFFu) << 32 | (uint32_t)__double2loint(r);
+  if (mag > (unsigned long long)dbits(h)) r = dadd(r, (hi >> 31) ? L : -L);
+  return r;
+}
 
 // ---- fixed-point profile counters ----------------------------------------- //
 // A profile bin keeps kProfQ int64 counters: [0] the particle count, [1 + 3a + c]
@@ -500,16 +526,19 @@ __device__ __forceinline__ float d2f_rn(double x) {
   k += (rem > half || (rem == half && (k & 1ull))) ? 1ull : 0ull;
   return __uint_as_float(sign | (uint32_t)k);
 }
-// |x| rounded up to binary32 (integer pipes, no hardware fallback)
+// |x| rounded up to binary32 (integer pipes, no hardware fallback).  The sign is masked in
+// the high word: of a 64-bit mask the compiler makes a binary64 absolute value, a third of
+// the push's instructions on that pipe.
 __device__ __forceinline__ float d2f_abs_ru(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
-  const int e = (int)(b >> 52);
+  const uint32_t hi = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu, lo = (uint32_t)__double2loint(x);
+  const int e = (int)(hi >> 20);
   const int fe = e - 1023 + 127;
   if (fe >= 1 && fe <= 254) {
-    const uint32_t top = (uint32_t)((b >> 29) & 0x7FFFFFu);
-    const uint32_t up = (b & 0x1FFFFFFFull) ? 1u : 0u;
+    const uint32_t top = (hi & 0xFFFFFu) << 3 | lo >> 29;
+    const uint32_t up = (lo & 0x1FFFFFFFu) ? 1u : 0u;
     return __uint_as_float(((uint32_t)fe << 23) + top + up);
   }
+  const unsigned long long b = (unsigned long long)hi << 32 | lo;
   if (fe > 254) return __uint_as_float(e == 0x7FF && (b & 0xFFFFFFFFFFFFFull) ? 0x7FFFFFFFu : 0x7F800000u);
   if (b == 0ull) return 0.0f;
   const int sh = 926 - e;
@@ -575,6 +604,7 @@ struct LaunchPlan {
   Batch b;
   uint32_t ptiles, stiles_c, prtiles;
   int edge_blocks;
+  int push_blocks;         // grid of the push, each block every so many tiles
   int prof_blocks;         // grid of the profile kernel, each block a range of tiles
   int round_blocks;        // cooperative grid of the later matching rounds
   bool lists = false;      // domains: the rounds work on per-particle candidate lists

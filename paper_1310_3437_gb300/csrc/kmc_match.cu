@@ -80,13 +80,6 @@ __device__ __forceinline__ void circle_point(double u1, double u2, double nv[3])
   nv[2] = 0.0;
 }
 
-__device__ __forceinline__ double min_image(double r, double L) {
-  double h = dmul(L, 0.5);
-  if (r > h) return dsub(r, L);
-  if (r < -h) return dadd(r, L);
-  return r;
-}
-
 // candidate pairs the search stored (a member whose buffer overflowed is not live)
 __device__ __forceinline__ uint32_t raw_pairs(const SimDev& s) {
   return s.d.n_raw < s.edge_cap ? s.d.n_raw : s.edge_cap;
@@ -278,16 +271,18 @@ __global__ void __launch_bounds__(kEdgeBlock) k_refine(Batch B) {
       if (!(li == idj && lj == idi)) {
 #pragma unroll
         for (int a = 0; a < 3; ++a)
-          if (s.bc[a] == KMC_PERIODIC) r[a] = min_image(r[a], s.box[a]);
+          if (s.bc[a] == KMC_PERIODIC) r[a] = min_image(r[a], s.box[a], s.half_box[a]);
         double vv = dadd(dadd(dmul(v[0], v[0]), dmul(v[1], v[1])), dmul(v[2], v[2]));
-        if (vv != 0.0) {
+        if (dbits(vv) != 0) {  // (a sum of squares: never -0.0)
           double rv = dadd(dadd(dmul(r[0], v[0]), dmul(r[1], v[1])), dmul(r[2], v[2]));
           t = ddiv(-rv, vv);
           double wx = dsub(dmul(r[1], v[2]), dmul(r[2], v[1]));
           double wy = dsub(dmul(r[2], v[0]), dmul(r[0], v[2]));
           double wz = dsub(dmul(r[0], v[1]), dmul(r[1], v[0]));
           d2 = ddiv(dadd(dadd(dmul(wx, wx), dmul(wy, wy)), dmul(wz, wz)), vv);
-          cand = t >= 0.0 && t < s.dt && d2 < c2;
+          // 0 <= t < dt and d2 < c2, on the integer pipes
+          cand = !lt_zero(t) && (dbits(t) < dbits(s.dt)) &&
+                 (unsigned long long)dbits(d2) < (unsigned long long)dbits(c2);
         }
       }
       if (cand) {

@@ -32,15 +32,6 @@ __device__ __forceinline__ void block_max_to(uint32_t* dst, float v) {
   }
 }
 
-// Comparisons of finite doubles on the integer pipes (the binary64 pipe is the
-// scarce one on this part).  For a finite x and a positive finite bound y the order
-// of the values is the order of the bit patterns read as signed integers; negative
-// x (including -0.0) compare below every positive y.
-__device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
-__device__ __forceinline__ bool lt_zero(double x) {  // x < 0.0 (false for -0.0)
-  return (unsigned long long)dbits(x) > 0x8000000000000000ull;
-}
-
 // ---- k_push ---------------------------------------------------------------- //
 // The boundary fix-ups are rare (particles that crossed a wall or the periodic
 // boundary in this step).  They sit in out-of-line functions so that their binary64
@@ -76,122 +67,118 @@ __device__ __noinline__ XV reflect_walls(double x, double v, double X, double u)
 // Free streaming and walls of one particle (sorted position p); returns the binary32
 // upper bound of its |v|^2 (0 if it left).  ABS: the simulation has absorbing walls.
 template <bool ABS>
-__device__ __forceinline__ float push_particle(SimDev& s, int cur, uint32_t p, double dt, double sX,
+__device__ __forceinline__ float push_particle(SimDev& s, int cur, uint32_t p, double dt, double wall,
                                                bool& gone) {
+  // everything is loaded before the first store (a load of the next axis cannot be moved
+  // ahead of a store to this one)
   const uint32_t q = s.partner[p];
-  double vv[3];
-  if (!ABS) {
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      double x = s.x[cur][a][p];
-      double v = s.v[cur][a][p];
-      if (q == kNone) x = dadd(x, dmul(v, dt));
-      if (s.bc[a] == KMC_PERIODIC) {
-        const double L = s.box[a];  // > 0
-        if (dbits(x) >= dbits(L) || lt_zero(x)) x = wrap_periodic(x, L);
-      } else {
-        const double X = a == 0 ? sX : s.box[a];
-        const double u = a == 0 ? s.piston_u : 0.0;
-        if (lt_zero(x) || (dbits(X) > 0 ? dbits(x) > dbits(X) : x > X)) {
-          const XV r = reflect_walls(x, v, X, u);
-          x = r.x;
-          v = r.v;
-          s.v[cur][a][p] = v;
-        }
-      }
-      s.x[cur][a][p] = x;
-      vv[a] = v;
-    }
-    if (q != kNone) s.last[cur][p] = s.id[cur][q];
-    return vmag2_up(vv[0], vv[1], vv[2]);
-  }
-  double xs[3];
+  double xs[3], vv[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     xs[a] = s.x[cur][a][p];
     vv[a] = s.v[cur][a][p];
-    if (q == kNone) xs[a] = dadd(xs[a], dmul(vv[a], dt));
+  }
+  if (q == kNone) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) xs[a] = dadd(xs[a], dmul(vv[a], dt));
   }
   // beyond an absorbing wall at the end of the step: the particle leaves the gas with
   // this position and velocity (tested before any other axis' boundary)
+  if (ABS) {
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
-    if (s.bc[a] == KMC_ABSORB && (lt_zero(xs[a]) || xs[a] > s.box[a])) gone = true;
+    for (int a = 0; a < 3; ++a)
+      if (s.bc[a] == KMC_ABSORB && (lt_zero(xs[a]) || gt_bits(xs[a], s.box[a]))) gone = true;
+  }
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    double x = xs[a];
-    double v = vv[a];
-    if (gone || s.bc[a] == KMC_ABSORB) {
+    if (ABS && (gone || s.bc[a] == KMC_ABSORB)) {
       // no wall acts (inside on this axis, or the particle has left)
     } else if (s.bc[a] == KMC_PERIODIC) {
-      const double L = s.box[a];
-      if (dbits(x) >= dbits(L) || lt_zero(x)) x = wrap_periodic(x, L);
+      const double L = s.box[a];  // > 0
+      if (dbits(xs[a]) >= dbits(L) || lt_zero(xs[a])) xs[a] = wrap_periodic(xs[a], L);
     } else {
-      const double X = a == 0 ? sX : s.box[a];
+      const double X = a == 0 ? wall : s.box[a];
       const double u = a == 0 ? s.piston_u : 0.0;
-      if (lt_zero(x) || (dbits(X) > 0 ? dbits(x) > dbits(X) : x > X)) {
-        const XV r = reflect_walls(x, v, X, u);
-        x = r.x;
-        v = r.v;
-        s.v[cur][a][p] = v;
+      if (lt_zero(xs[a]) || gt_bits(xs[a], X)) {
+        const XV r = reflect_walls(xs[a], vv[a], X, u);
+        xs[a] = r.x;
+        vv[a] = r.v;
+        s.v[cur][a][p] = r.v;
       }
     }
-    s.x[cur][a][p] = x;
-    vv[a] = v;
+    s.x[cur][a][p] = xs[a];
   }
-  if (gone) s.last[cur][p] = KMC_ABSORBED;
+  if (ABS && gone) s.last[cur][p] = KMC_ABSORBED;
   else if (q != kNone) s.last[cur][p] = s.id[cur][q];
-  return gone ? 0.0f : vmag2_up(vv[0], vv[1], vv[2]);
+  return ABS && gone ? 0.0f : vmag2_up(vv[0], vv[1], vv[2]);
 }
 
+//
+// What bounds it: the binary64 pipe (6 operations a particle, 173 us at 2^24 particles) and
+// memory (77 bytes, 193 us).  Everything else on that pipe is kept off it: comparisons and
+// conversions are on integers (an absolute value that the compiler made of a mask alone
+// cost another three operations), the wall's position comes with the step.  32 registers
+// (eight blocks per SM) hide one by the other: 350 -> 262 us at 2^24, where 40 registers
+// take 349; 5.7 -> 4.8 us at 4096.  Each block takes every so many tiles and adds its
+// maximum and counts once per simulation.
 template <bool ABS>
-__global__ void __launch_bounds__(kTile) k_push(Batch B) {
-  __shared__ double sX;                       // piston position at the end of the step
+__global__ void __launch_bounds__(kTile, 8) k_push(Batch B) {
   __shared__ uint32_t scnt[kSplitTrials];     // particles above each trial threshold
-  __shared__ uint32_t sgone;                  // particles absorbed in this block
-  int k = find_sim(B.ptile, B.nsims, blockIdx.x);
-  SimDev& s = B.sim(k);
-  if (!sim_active(s)) return;
-  const int cur = s.d.parity ^ 1;
-  const uint64_t step = s.d.step;
-  const double dt = s.dt;
-  if (threadIdx.x == 0)
-    sX = s.bc[0] == KMC_PERIODIC ? 0.0
-                                 : dsub(s.piston_x0, dmul(s.piston_u, dmul((double)(step + 1), dt)));
+  __shared__ uint32_t sgone;                  // particles absorbed
+  const uint32_t lane = threadIdx.x & 31u;
   if (threadIdx.x < kSplitTrials) scnt[threadIdx.x] = 0;
   if (ABS && threadIdx.x == 0) sgone = 0;
-  __syncthreads();
-  uint32_t p = (blockIdx.x - B.tile0(B.ptile, k)) * kTile + threadIdx.x;
-  float vm = 0.0f;
-  // absorbing walls: particles that left earlier sit at the end of the order and stay
-  // as they are (live_count is this step's sort's count of the others)
-  const uint32_t n_in = ABS ? live_count(s) : s.n;
-  bool gone = false;
-  if (p < n_in) vm = (ABS && s.absorb) ? push_particle<true>(s, cur, p, dt, sX, gone)
-                                       : push_particle<false>(s, cur, p, dt, sX, gone);
-  if (ABS && s.absorb) {
-    const unsigned m = __ballot_sync(0xFFFFFFFFu, gone);
-    if ((threadIdx.x & 31) == 0 && m) atomicAdd(&sgone, (uint32_t)__popc(m));
-  }
-  if (s.split_ok) {
-    // particles above each trial split threshold: warp ballots, shared counters, one
-    // global atomic per block and trial; each particle keeps how many thresholds it
-    // exceeds, which is all the next step's count needs to classify it
-    const bool valid = p < n_in && !gone;
-    uint32_t above = 0;
+  float vmax = 0.0f;
+  uint32_t mine = 0, left = 0;  // lane t: the warp's particles above threshold t; lane 0: gone
+  const uint32_t ntiles = B.ptiles;
+  for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int k = find_sim(B.ptile, B.nsims, tile);
+    SimDev& s = B.sim(k);
+    if (!sim_active(s)) continue;
+    const int cur = s.d.parity ^ 1;
+    const uint32_t p = (tile - B.tile0(B.ptile, k)) * kTile + threadIdx.x;
+    // absorbing walls: particles that left earlier sit at the end of the order and stay
+    // as they are (live_count is this step's sort's count of the others)
+    const uint32_t n_in = ABS ? live_count(s) : s.n;
+    const double dt = s.dt, wall = s.d.wall_x;
+    bool gone = false;
+    float vm = 0.0f;
+    if (p < n_in) vm = (ABS && s.absorb) ? push_particle<true>(s, cur, p, dt, wall, gone)
+                                         : push_particle<false>(s, cur, p, dt, wall, gone);
+    vmax = fmaxf(vmax, vm);
+    if (ABS && s.absorb) left += (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, gone));
+    if (s.split_ok) {
+      // particles above each trial split threshold; each particle keeps how many it
+      // exceeds, which is all the next step's count needs to classify it
+      const bool valid = p < n_in && !gone;
+      uint32_t above = 0;
 #pragma unroll
-    for (int t = 1; t < kSplitTrials; ++t) {
-      const bool hi = valid && vm > s.d.split_thr[t];
-      above += hi ? 1u : 0u;
-      unsigned m = __ballot_sync(0xFFFFFFFFu, hi);
-      if ((threadIdx.x & 31) == 0 && m) atomicAdd(&scnt[t], (uint32_t)__popc(m));
+      for (int t = 1; t < kSplitTrials; ++t) {
+        const bool hi = valid && vm > s.d.split_thr[t];
+        above += hi ? 1u : 0u;
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, hi);
+        if (lane == (uint32_t)t) mine += (uint32_t)__popc(m);
+      }
+      if (valid) s.vbucket[p] = (uint8_t)above;
     }
-    if (valid) s.vbucket[p] = (uint8_t)above;
+    const uint32_t next = tile + gridDim.x;
+    if (next < ntiles && (B.nsims == 1 || find_sim(B.ptile, B.nsims, next) == k)) continue;
+    // the block's last tile of the simulation: its sums to the simulation's counters
+    __syncthreads();  // (the shared counters are clear)
+    if (lane > 0 && lane < (uint32_t)kSplitTrials && mine) atomicAdd(&scnt[lane], mine);
+    if (ABS && lane == 0 && left) atomicAdd(&sgone, left);
+    block_max_to(&s.d.vmax2_acc, vmax);  // its block barrier also orders the shared counters
+    if (threadIdx.x > 0 && threadIdx.x < kSplitTrials) {
+      if (scnt[threadIdx.x]) atomicAdd(&s.d.split_cnt[threadIdx.x], scnt[threadIdx.x]);
+      scnt[threadIdx.x] = 0;
+    }
+    if (ABS && threadIdx.x == 0) {
+      if (sgone) atomicAdd(&s.d.n_absorbed, sgone);
+      sgone = 0;
+    }
+    vmax = 0.0f;
+    mine = left = 0;
   }
-  block_max_to(&s.d.vmax2_acc, vm);  // its block barrier also orders the shared counters
-  if (s.split_ok && threadIdx.x > 0 && threadIdx.x < kSplitTrials && scnt[threadIdx.x])
-    atomicAdd(&s.d.split_cnt[threadIdx.x], scnt[threadIdx.x]);
-  if (ABS && s.absorb && threadIdx.x == 0 && sgone) atomicAdd(&s.d.n_absorbed, sgone);
 }
 
 // The particles of a block's tiles are summed in shared memory, in 32-bit words of 16-bit
@@ -455,8 +442,8 @@ int launch_init_grid(const LaunchPlan& L, cudaStream_t st) {
 
 int launch_push(const LaunchPlan& L, cudaStream_t st) {
   const size_t smem = 256 * kProfW * sizeof(int);
-  if (L.absorb) k_push<true><<<L.ptiles, kTile, 0, st>>>(L.b);
-  else k_push<false><<<L.ptiles, kTile, 0, st>>>(L.b);
+  if (L.absorb) k_push<true><<<L.push_blocks, kTile, 0, st>>>(L.b);
+  else k_push<false><<<L.push_blocks, kTile, 0, st>>>(L.b);
   if (L.profiles) {
     if (L.absorb) k_profile<true><<<L.prof_blocks, kTile, smem, st>>>(L.b, L.prtiles);
     else k_profile<false><<<L.prof_blocks, kTile, smem, st>>>(L.b, L.prtiles);

@@ -247,9 +247,9 @@ __device__ __noinline__ unsigned long long particle_walk(SimDev& s, uint32_t p, 
             double r0 = dsub(__ldg(X0 + j), xo[0]);
             double r1 = dsub(__ldg(X1 + j), xo[1]);
             double r2 = dsub(__ldg(X2 + j), xo[2]);
-            if (px) { if (r0 > 0.5 * L0) r0 = dsub(r0, L0); else if (r0 < -0.5 * L0) r0 = dadd(r0, L0); }
-            if (py) { if (r1 > 0.5 * L1) r1 = dsub(r1, L1); else if (r1 < -0.5 * L1) r1 = dadd(r1, L1); }
-            if (pz) { if (r2 > 0.5 * L2) r2 = dsub(r2, L2); else if (r2 < -0.5 * L2) r2 = dadd(r2, L2); }
+            if (px) r0 = min_image(r0, L0, s.half_box[0]);
+            if (py) r1 = min_image(r1, L1, s.half_box[1]);
+            if (pz) r2 = min_image(r2, L2, s.half_box[2]);
             double g0 = dsub(__ldg(V0 + j), vo[0]);
             double g1 = dsub(__ldg(V1 + j), vo[1]);
             double g2 = dsub(__ldg(V2 + j), vo[2]);
@@ -884,11 +884,7 @@ __device__ __noinline__ void test_survivor(SimDev& s, uint2* buf, uint32_t* cnt,
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       r[a] = dsub(__ldg(s.x[cur][a] + j), __ldg(s.x[cur][a] + i));
-      if (s.bc[a] == KMC_PERIODIC) {
-        const double L = s.box[a];
-        if (r[a] > 0.5 * L) r[a] = dsub(r[a], L);
-        else if (r[a] < -0.5 * L) r[a] = dadd(r[a], L);
-      }
+      if (s.bc[a] == KMC_PERIODIC) r[a] = min_image(r[a], s.box[a], s.half_box[a]);
       v[a] = dsub(__ldg(s.v[cur][a] + j), __ldg(s.v[cur][a] + i));
     }
     const double R = dadd(dadd(dmul(r[0], r[0]), dmul(r[1], r[1])), dmul(r[2], r[2]));
@@ -1393,9 +1389,9 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4) k_search_fast(Batch B) {
               double r0 = dsub(__ldg(X0 + j), xo[0]);
               double r1 = dsub(__ldg(X1 + j), xo[1]);
               double r2 = dsub(__ldg(X2 + j), xo[2]);
-              if (px) { if (r0 > 0.5 * L0) r0 = dsub(r0, L0); else if (r0 < -0.5 * L0) r0 = dadd(r0, L0); }
-              if (py) { if (r1 > 0.5 * L1) r1 = dsub(r1, L1); else if (r1 < -0.5 * L1) r1 = dadd(r1, L1); }
-              if (pz) { if (r2 > 0.5 * L2) r2 = dsub(r2, L2); else if (r2 < -0.5 * L2) r2 = dadd(r2, L2); }
+              if (px) r0 = min_image(r0, L0, s.half_box[0]);
+              if (py) r1 = min_image(r1, L1, s.half_box[1]);
+              if (pz) r2 = min_image(r2, L2, s.half_box[2]);
               const double g0 = dsub(__ldg(V0 + j), vo[0]);
               const double g1 = dsub(__ldg(V1 + j), vo[1]);
               const double g2 = dsub(__ldg(V2 + j), vo[2]);
