@@ -385,8 +385,12 @@ int build_plan(Plan& P, const std::vector<kmc_sim*>& sims, cudaStream_t st, std:
   // the SMs hold at most: a launch of idle blocks takes 1.1 us, one of a few 0.6
   L.edge_blocks = (int)std::min<uint32_t>(std::max(pt[m], 1u), 8u * (uint32_t)num_sms());
   // a block of the later rounds per 2^16 particles (their lists hold about one pair in a
-  // thousand particles); one per SM at most, so that all of them run at once
-  L.round_blocks = (int)std::min<uint32_t>(std::max(pt[m] / 256u, 1u), (uint32_t)num_sms());
+  // thousand particles of a tube), from 2^19 particles on per 2^13 (a blast's lists are
+  // longer: 74 -> 45 us at 2^21; a 2^20 tube 16.5 either way, a box of 2^18 10.7 and 12.1);
+  // one per SM at most, so that all of them run at once
+  L.round_blocks = (int)std::min<uint32_t>(
+      std::max(pt[m] < 2048u ? pt[m] / 256u : pt[m] / 32u, 1u), (uint32_t)num_sms());
+  match_grids(num_sms(), L);
   search_grids(P.precision, P.K, num_sms(), L.ptiles, L);
   return KMC_OK;
 }

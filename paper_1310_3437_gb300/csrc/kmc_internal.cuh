@@ -376,7 +376,8 @@ __device__ __forceinline__ uint32_t block_append(uint32_t* counter, uint32_t wan
 // may lie past the end), so body may use block-wide appends.  Blocks of kEdgeBlock
 // threads, kItems items at a time: a thread each, or with kItems = kEdgeBlock / 32 a warp.
 template <uint32_t kItems = kEdgeBlock, class Count, class Body>
-__device__ __forceinline__ void for_dealt(const Batch& B, Count count, Body body) {
+__device__ __forceinline__ void for_dealt(const Batch& B, Count count, Body body,
+                                          uint32_t few = 0xFFFFFFFFu) {
   __shared__ uint32_t s_first[kEdgeBlock], s_trips[kEdgeBlock], s_wsum[kEdgeBlock / 32];
   constexpr uint32_t kThreads = kEdgeBlock / kItems, kWarpItems = kItems / (kEdgeBlock / 32);
   const uint32_t nb = gridDim.x, stride = nb * kItems, own = threadIdx.x / kThreads;
@@ -386,10 +387,13 @@ __device__ __forceinline__ void for_dealt(const Batch& B, Count count, Body body
     const uint32_t c = count(s);
     // one answer for the block (the status word can change during the launch)
     if (!__syncthreads_and(s.d.status == 0)) return;
+    // items that the first `few` blocks can take in one go are spread over those alone
+    const uint32_t over = few < nb && (uint64_t)c <= (uint64_t)few * kItems ? few : nb;
+    if (blockIdx.x >= over) return;
     const bool spread = c <= stride;
     const uint32_t at = blockIdx.x * (spread ? kWarpItems : kItems);
     if (c > at)
-      body(s, spread ? at + warp * (nb - 1u) * kWarpItems + own : at + own,
+      body(s, spread ? at + warp * (over - 1u) * kWarpItems + own : at + own,
            spread ? 1u : (uint32_t)(((uint64_t)(c - at) + stride - 1) / stride));
     return;
   }
@@ -604,6 +608,7 @@ struct LaunchPlan {
   Batch b;
   uint32_t ptiles, stiles_c, prtiles;
   int edge_blocks;
+  int refine_few, collide_few;  // blocks of the exact test and the collision that are resident
   int push_blocks;         // grid of the push, each block every so many tiles
   int prof_blocks;         // grid of the profile kernel, each block a range of tiles
   int round_blocks;        // cooperative grid of the later matching rounds
@@ -634,6 +639,7 @@ int launch_search(const LaunchPlan& L, int precision, int K, cudaStream_t st,
 // attribute); called when a launch plan is built, before any capture
 void search_grids(int precision, int K, int num_sms, uint32_t ptiles, LaunchPlan& L);
 int launch_match(const LaunchPlan& L, int max_rounds, cudaStream_t st);
+void match_grids(int num_sms, LaunchPlan& L);  // with the plan, after its edge_blocks
 // the parts of launch_match around the rounds: exact test and candidate lists; collision
 int launch_match_lists(const LaunchPlan& L, cudaStream_t st);
 int launch_collide(const LaunchPlan& L, cudaStream_t st);

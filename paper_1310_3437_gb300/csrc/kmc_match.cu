@@ -180,12 +180,11 @@ __device__ __forceinline__ uint32_t other_end(const SimDev& s, uint32_t e, uint3
   return pr.x == i ? pr.y : pr.x;
 }
 
-// Pair e (key d2, t; partner id) proposes itself to particle i.  The keys of the pairs
-// that others put there are read past the L1 (written on other SMs, fenced before their
-// swap).
-__device__ __forceinline__ void propose(const SimDev& s, int cur, uint32_t* best, uint32_t i, uint32_t e,
-                                        double d2, double t, uint32_t partner_id) {
-  uint32_t seen = atomicCAS(best + i, kNone, e);
+// Pair e (key d2, t; partner id) competes for particle i with the pair seen there (kNone:
+// it holds the place).  The keys of the pairs that others put there are read past the L1
+// (written on other SMs, fenced before their swap).
+__device__ __forceinline__ void contest(const SimDev& s, int cur, uint32_t* best, uint32_t i, uint32_t e,
+                                        double d2, double t, uint32_t partner_id, uint32_t seen) {
   while (seen != kNone) {
     if (!key_less(d2, t, partner_id, __ldcg(s.e_d2 + seen), __ldcg(s.e_t + seen),
                   s.id[cur][other_end(s, seen, i)]))
@@ -194,6 +193,13 @@ __device__ __forceinline__ void propose(const SimDev& s, int cur, uint32_t* best
     if (old == seen) return;
     seen = old;
   }
+}
+// Pair e proposes itself to both its particles; both first swaps are in flight together.
+__device__ __forceinline__ void propose(const SimDev& s, int cur, uint32_t* best, uint2 pr, uint32_t e,
+                                        double d2, double t, uint32_t idi, uint32_t idj) {
+  const uint32_t si = atomicCAS(best + pr.x, kNone, e), sj = atomicCAS(best + pr.y, kNone, e);
+  contest(s, cur, best, pr.x, e, d2, t, idj, si);
+  contest(s, cur, best, pr.y, e, d2, t, idi, sj);
 }
 
 // is particle i matched in the round whose choices are in best?
@@ -240,7 +246,7 @@ __device__ __forceinline__ void settle(SimDev& s, int round, uint32_t e, uint2 p
 // candidate lists instead.
 // MIX: the plan has a mixture (per-pair contact distance, mass-weighted scatter)
 template <bool MIX, bool LISTS>
-__global__ void __launch_bounds__(kEdgeBlock) k_refine(Batch B) {
+__global__ void __launch_bounds__(kEdgeBlock) k_refine(Batch B, uint32_t few) {
   for_dealt(B, [](const SimDev& s) { return sim_scheduled(s) ? raw_pairs(s) : 0u; },
             [](SimDev& s, uint32_t first, uint32_t) {
     const int cur = s.d.parity ^ 1;
@@ -296,8 +302,7 @@ __global__ void __launch_bounds__(kEdgeBlock) k_refine(Batch B) {
           s.e_slot[e] = make_uint2(0u, 0u);
           __threadfence();  // the key is there before the pair can be seen
           uint32_t* best = round_best(s, 0);
-          propose(s, cur, best, i, e, d2, t, idj);
-          propose(s, cur, best, j, e, d2, t, idi);
+          propose(s, cur, best, pr, e, d2, t, idi, idj);
         }
         ++found;
       } else {
@@ -305,7 +310,7 @@ __global__ void __launch_bounds__(kEdgeBlock) k_refine(Batch B) {
       }
     }
     block_append(&s.d.n_edges, found);  // one atomic per block
-  });
+  }, few);
 }
 
 // round 0's matches and open pairs
@@ -379,8 +384,7 @@ __global__ void __launch_bounds__(kEdgeBlock) k_rounds(Batch B, int max_rounds) 
         const uint32_t e = __ldcg(list + t);
         const uint2 pr = s.edge[e];
         const double d2 = s.e_d2[e], tt = s.e_t[e];
-        propose(s, cur, best, pr.x, e, d2, tt, s.id[cur][pr.y]);
-        propose(s, cur, best, pr.y, e, d2, tt, s.id[cur][pr.x]);
+        propose(s, cur, best, pr, e, d2, tt, s.id[cur][pr.x], s.id[cur][pr.y]);
       }
     });
     bool in_time = grid_barrier(B.round_ctl);
@@ -451,7 +455,7 @@ __global__ void __launch_bounds__(kEdgeBlock) k_fill(Batch B) {
 
 // the step's collisions: matched pairs (domains: smaller-id members with their partners)
 template <bool MIX, bool LISTS>
-__global__ void __launch_bounds__(kEdgeBlock) k_collide(Batch B) {
+__global__ void __launch_bounds__(kEdgeBlock) k_collide(Batch B, uint32_t few) {
   for_dealt(B, [](const SimDev& s) { return sim_scheduled(s) ? s.d.n_pairs : 0u; },
             [](SimDev& s, uint32_t first, uint32_t) {
     const int cur = s.d.parity ^ 1;
@@ -465,29 +469,48 @@ __global__ void __launch_bounds__(kEdgeBlock) k_collide(Batch B) {
       collide_pair<MIX>(s, cur, first_is_a ? pr.x : pr.y, first_is_a ? pr.y : pr.x,
                         first_is_a ? idi : idj, first_is_a ? idj : idi, s.e_t[e]);
     }
-  });
+  }, few);
+}
+
+// The exact test and the collision keep 14 and more binary64 values a pair, so two to four of
+// their blocks fit an SM.  Pairs that those can take in one go are dealt to that many blocks:
+// dealt 32 to a block over a block per 256 particles, the 47 k collisions of a 2^20 tube ran
+// in four waves of two warps per SM (28 -> 18 us, its exact test 25 -> 19).  For more pairs the
+// larger grid is the better one (a 2^21 blast's exact test 61 us, 78 on the resident blocks).
+void match_grids(int num_sms, LaunchPlan& L) {
+  auto few = [&](auto kernel) {
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kEdgeBlock, 0) != cudaSuccess ||
+        per_sm < 1) {
+      cudaGetLastError();
+      per_sm = 2;
+    }
+    return per_sm * num_sms;
+  };
+  L.refine_few = L.mix ? few(k_refine<true, false>) : few(k_refine<false, false>);
+  L.collide_few = L.mix ? few(k_collide<true, false>) : few(k_collide<false, false>);
 }
 
 int launch_match_lists(const LaunchPlan& L, cudaStream_t st) {
   const int nb = L.edge_blocks;
-  k_refine<false, true><<<nb, kEdgeBlock, 0, st>>>(L.b);  // (domains have no mixtures)
+  k_refine<false, true><<<nb, kEdgeBlock, 0, st>>>(L.b, L.refine_few);  // (domains have no mixtures)
   k_alloc<<<nb, kEdgeBlock, 0, st>>>(L.b);
   k_fill<<<nb, kEdgeBlock, 0, st>>>(L.b);
   return 3;
 }
 
 int launch_collide(const LaunchPlan& L, cudaStream_t st) {
-  const int nb = L.edge_blocks;
-  if (L.mix) k_collide<true, false><<<nb, kEdgeBlock, 0, st>>>(L.b);
-  else if (L.lists) k_collide<false, true><<<nb, kEdgeBlock, 0, st>>>(L.b);
-  else k_collide<false, false><<<nb, kEdgeBlock, 0, st>>>(L.b);
+  const int nb = L.edge_blocks, few = L.collide_few;
+  if (L.mix) k_collide<true, false><<<nb, kEdgeBlock, 0, st>>>(L.b, few);
+  else if (L.lists) k_collide<false, true><<<nb, kEdgeBlock, 0, st>>>(L.b, few);
+  else k_collide<false, false><<<nb, kEdgeBlock, 0, st>>>(L.b, few);
   return 1;
 }
 
 int launch_match(const LaunchPlan& L, int max_rounds, cudaStream_t st) {
   const int nb = L.edge_blocks;
-  if (L.mix) k_refine<true, false><<<nb, kEdgeBlock, 0, st>>>(L.b);
-  else k_refine<false, false><<<nb, kEdgeBlock, 0, st>>>(L.b);
+  if (L.mix) k_refine<true, false><<<nb, kEdgeBlock, 0, st>>>(L.b, L.refine_few);
+  else k_refine<false, false><<<nb, kEdgeBlock, 0, st>>>(L.b, L.refine_few);
   k_settle<<<nb, kEdgeBlock, 0, st>>>(L.b);
   int n = 2;
   if (max_rounds > 1) {
