@@ -104,26 +104,22 @@ __device__ inline CellPlan plan_cells(const float ext[3], float h, int K, uint64
 }
 
 // Cost estimates for the choice of the split threshold, in units of one pair test of
-// the row search (measured on GB300 at 2^24 particles; only the ratios matter):
-// a slow particle costs its trimmed half-stencil, about 5 tests per particle per cell
-// (rho = particles per cell of width w), plus its set-up (about 6 tests' time; the
-// warp-per-cell search at high occupancy tests 13.5 rho pairs per particle at about 2.6
-// times the rate, the same cost); a fast particle costs its reach-trimmed stencil
-// (about 1.4 times the sphere of radius R_f, at about 2 tests' time per test) plus 15
-// per (y, z) column it walks.
-__device__ inline float slow_cost(float n, float rho) { return n * (5.0f * rho + 6.0f); }
-// The binary64 path has no row search (thread per particle or warp per cell, whole
-// stencil, binary64 pre-tests): its cost is the half stencil's pair tests, inflated
-// when cells hold fewer particles than a warp's lanes can use; a fast particle costs
-// its whole stencil at 3 units per test.
-__device__ inline float slow_cost_f64(float n, float rho, int K) {
-  const float st = (2 * K + 1.0f) * (2 * K + 1.0f) * (2 * K + 1.0f) * 0.5f;
-  const float eff = rho < 16.0f ? sqrtf(16.0f / fmaxf(rho, 0.25f)) : 1.0f;
-  return n * st * rho * eff;
+// the row search (measured on GB300 at 2^24 particles, 6.6 ps; only the ratios matter).
+// A slow particle in the row search: its trimmed half-stencil, about 5 tests per particle
+// per cell (rho = particles per cell of width w), and its set-up (about 6 tests' time).  In
+// tiles (107 ps at 7 per cell, 262 at about 45): 0.65 rho + 11.5, with binary64 records 23
+// (162 ps at 1.2 per cell).  A fast particle: its reach-trimmed stencil (about 1.4 times the
+// sphere of radius R_f) at 1.4 tests' time per test plus 10 per (y, z) column it walks, three
+// times that with binary64 tests.  (With the row search's cost for well filled cells and the
+// fast search 1.4 times as dear, too many particles were fast: 10 steps of a 2^21 blast 10.4
+// against 9.55 ms, of an ensemble of 30 2.50 against 2.41, 2^24 tube 12.97 against 12.57.)
+__device__ inline float slow_cost(float n, float rho, bool fp32) {
+  if (!fp32) return n * (0.65f * rho + 23.0f);
+  return n * (rho < kTileOccupancy ? 5.0f * rho + 6.0f : 0.65f * rho + 11.5f);
 }
-__device__ inline float fast_cost(float nfast, float rho, float rf_cells, float ncol) {
+__device__ inline float fast_cost(float nfast, float rho, float rf_cells, float ncol, bool fp32) {
   const float tests = rho * 1.4f * 4.18879f * rf_cells * rf_cells * rf_cells;
-  return nfast * (2.0f * tests + 15.0f * ncol);
+  return nfast * (fp32 ? 1.0f : 3.0f) * (1.4f * tests + 10.0f * ncol);
 }
 
 // extent along x: the box, or the upper wall at the start of the step (particles are below it)
@@ -188,14 +184,14 @@ __device__ inline void compute_grid(SimDev& s, float vmax2_bound, uint64_t step,
     if (!p.ok) break;
     const float rho = (float)n / ((float)p.nc[0] * (float)p.nc[1] * (float)p.nc[2]);
     if (t == 0) {
-      my_cost = fp32 ? slow_cost((float)n, rho) : slow_cost_f64((float)n, rho, K);
+      my_cost = slow_cost((float)n, rho, fp32);
       my_feasible = true;
       break;
     }
     if (split_ok == 1 && rho < min_occ) break;
     // fast stencil: c cells on each side per split axis; periodic axes must hold it,
     // and no axis may be a one-cell periodic axis (no minimum-image test there)
-    float ncol = 1.0f, iwmax = 0.0f, fast_cells = 1.0f;
+    float ncol = 1.0f, iwmax = 0.0f;
     bool fits = true;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -210,14 +206,12 @@ __device__ inline void compute_grid(SimDev& s, float vmax2_bound, uint64_t step,
       if (c < K) c = K;
       if (per[a] && p.nc[a] < 2 * c + 2) fits = false;
       if (a > 0) ncol *= (2.0f * c + 1.0f);
-      fast_cells *= (2.0f * c + 1.0f);
     }
     if (!fits) break;
     // a fast particle's reach, its speed taken just above the threshold
     const float rf = (float)(d0 + (1.15 * S1 + V) * dt);
     const float rf_cells = iwmax > 0.0f ? rf * iwmax : 1.0f;
-    my_cost = fp32 ? slow_cost((float)n - my_nfast, rho) + fast_cost(my_nfast, rho, rf_cells, ncol)
-                   : slow_cost_f64((float)n - my_nfast, rho, K) + my_nfast * fast_cells * rho * 3.0f;
+    my_cost = slow_cost((float)n - my_nfast, rho, fp32) + fast_cost(my_nfast, rho, rf_cells, ncol, fp32);
     my_feasible = true;
     } while (false);
   }
@@ -235,7 +229,7 @@ __device__ inline void compute_grid(SimDev& s, float vmax2_bound, uint64_t step,
 #pragma unroll
     for (int t = 1; t < kSplitTrials; ++t) {
       const float ct = __shfl_sync(kAll, my_cost, t);
-      if (((fmask >> t) & 1u) && ct < 0.9f * cost) { best = t; cost = ct; }
+      if (((fmask >> t) & 1u) && ct < 0.95f * cost) { best = t; cost = ct; }
     }
   }
   const bool split = best > 0;
