@@ -46,22 +46,26 @@ __device__ double ln_series(double s) {
   }
   const double f = ddiv(dsub(m, 1.0), dadd(m, 1.0));
   const double z = dmul(f, f);
-  double poly = ddiv(1.0, 23.0);
+  double poly = 1.0 / 23.0;
 #pragma unroll
-  for (int k = 10; k >= 0; --k) poly = dadd(dmul(poly, z), ddiv(1.0, (double)(2 * k + 1)));
+  for (int k = 10; k >= 0; --k) poly = dadd(dmul(poly, z), 1.0 / (double)(2 * k + 1));
   const double lnm = dmul(dadd(f, f), poly);
   return dadd(dmul((double)e, 0x1.62e42fefa39efp-1), lnm);
 }
 
 __device__ __forceinline__ double u53(uint32_t w0, uint32_t w1) {
-  // (w0 >> 5) 2^26 + (w1 >> 6) < 2^53: every step is exact
-  return dmul(dadd(dmul((double)(w0 >> 5), 67108864.0), (double)(w1 >> 6)), 0x1p-53);
+  // ((w0 >> 5) 2^26 + (w1 >> 6)) 2^-53, exact, put together on the integer pipes
+  const unsigned long long M = (unsigned long long)(w0 >> 5) << 26 | (w1 >> 6);
+  if (M == 0ull) return 0.0;
+  const int top = 63 - __clzll((long long)M);  // M in [2^top, 2^(top + 1)), top <= 52
+  return __longlong_as_double((long long)(((M << (52 - top)) & 0xFFFFFFFFFFFFFull) |
+                                          (unsigned long long)(top - 53 + 1023) << 52));
 }
 
 __device__ __forceinline__ double scale_into(double u, double L) {
   const double x = dmul(u, L);
   // the largest double below a positive normal L
-  return x < L ? x : __longlong_as_double(__double_as_longlong(L) - 1);
+  return dbits(x) < dbits(L) ? x : __longlong_as_double(__double_as_longlong(L) - 1);
 }
 
 __device__ __forceinline__ void init_block(uint32_t id, uint32_t k, uint64_t seed, uint32_t w[4]) {
@@ -97,31 +101,45 @@ __global__ void __launch_bounds__(256) k_init_state(InitLaunch L) {
   const int want = (L.kind == KMC_INIT_EQUAL_SPEED || L.planar) ? 1 : 2;
   int got = 0;
   double g[4] = {0.0, 0.0, 0.0, 0.0};
+  // The kept attempts' words first: with the logarithms inside the loop, a warp went
+  // through them as often as the attempts of its last lane, most lanes idle (2^21 blast:
+  // 1.43 ms, now 0.60).
+  uint32_t k1[2] = {0u, 0u}, k2[2] = {0u, 0u};
   for (uint32_t j = 0; j < 64 && got < want; ++j) {
     uint32_t w[4];
     init_block(id, 128 + j, L.seed, w);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      if (got >= want) break;
-      const double u1 = word_uniform(w[2 * h]), u2 = word_uniform(w[2 * h + 1]);
-      const double s = dadd(dmul(u1, u1), dmul(u2, u2));
-      if (!(s > 0.0 && s < 1.0)) continue;
-      if (L.kind == KMC_INIT_EQUAL_SPEED) {
-        if (L.planar) {
-          v[0] = dmul(L.speed, ddiv(dsub(dmul(u1, u1), dmul(u2, u2)), s));
-          v[1] = dmul(L.speed, ddiv(dmul(dadd(u1, u1), u2), s));
-        } else {
-          const double q = dsqrt(dsub(1.0, s));
-          v[0] = dmul(L.speed, dmul(dadd(u1, u1), q));
-          v[1] = dmul(L.speed, dmul(dadd(u2, u2), q));
-          v[2] = dmul(L.speed, dsub(1.0, dadd(s, s)));
-        }
+      if (got >= want || !in_disk(w[2 * h], w[2 * h + 1])) continue;
+      if (got == 0) {
+        k1[0] = w[2 * h];
+        k2[0] = w[2 * h + 1];
       } else {
-        const double f = dsqrt(ddiv(dmul(-2.0, ln_series(s)), s));
-        g[2 * got] = dmul(u1, f);
-        g[2 * got + 1] = dmul(u2, f);
+        k1[1] = w[2 * h];
+        k2[1] = w[2 * h + 1];
       }
       ++got;
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    if (q >= got) break;
+    const double u1 = word_uniform(k1[q]), u2 = word_uniform(k2[q]);
+    const double s = dadd(dmul(u1, u1), dmul(u2, u2));
+    if (L.kind == KMC_INIT_EQUAL_SPEED) {
+      if (L.planar) {
+        v[0] = dmul(L.speed, ddiv(dsub(dmul(u1, u1), dmul(u2, u2)), s));
+        v[1] = dmul(L.speed, ddiv(dmul(dadd(u1, u1), u2), s));
+      } else {
+        const double r = dsqrt(dsub(1.0, s));
+        v[0] = dmul(L.speed, dmul(dadd(u1, u1), r));
+        v[1] = dmul(L.speed, dmul(dadd(u2, u2), r));
+        v[2] = dmul(L.speed, dsub(1.0, dadd(s, s)));
+      }
+    } else {
+      const double f = dsqrt(ddiv(dmul(-2.0, ln_series(s)), s));
+      g[2 * q] = dmul(u1, f);
+      g[2 * q + 1] = dmul(u2, f);
     }
   }
   if (L.kind != KMC_INIT_EQUAL_SPEED) {

@@ -33,4 +33,19 @@ __device__ __forceinline__ double word_uniform(uint32_t w) {
   return __longlong_as_double((long long)((neg << 63) | ((unsigned long long)(1023 + e - 31) << 52) | mant));
 }
 
+// Is the point (u1, u2) of two words in the unit disk without its centre, 0 < s < 1 with
+// s = fl(fl(u1^2) + fl(u2^2))?  Decided on integers (the binary64 pipe has two lanes per
+// SM): with a = |w - 2^31|, s 2^62 is a1^2 + a2^2 within three roundings of 2^9 each, so
+// outside 2^11 of 2^62 the exact sum decides alike, and inside the binary64 sum is formed.
+__device__ __forceinline__ bool in_disk(uint32_t w1, uint32_t w2) {
+  const uint32_t a1 = w1 >= 0x80000000u ? w1 - 0x80000000u : 0x80000000u - w1;
+  const uint32_t a2 = w2 >= 0x80000000u ? w2 - 0x80000000u : 0x80000000u - w2;
+  const unsigned long long q = (unsigned long long)a1 * a1 + (unsigned long long)a2 * a2;
+  constexpr unsigned long long one = 1ull << 62, zone = 1ull << 11;
+  if (q < one - zone) return q != 0ull;
+  if (q > one + zone) return false;
+  const double u1 = word_uniform(w1), u2 = word_uniform(w2);
+  return dadd(dmul(u1, u1), dmul(u2, u2)) < 1.0;
+}
+
 }  // namespace kmc
