@@ -464,14 +464,6 @@ __device__ __forceinline__ void mirror_store(float4* M, uint32_t j, float x, flo
 }
 
 // ---- Morton column code --------------------------------------------------- //
-__device__ __forceinline__ uint32_t dilate16(uint32_t x) {
-  x &= 0xFFFFu;
-  x = (x | (x << 8)) & 0x00FF00FFu;
-  x = (x | (x << 4)) & 0x0F0F0F0Fu;
-  x = (x | (x << 2)) & 0x33333333u;
-  x = (x | (x << 1)) & 0x55555555u;
-  return x;
-}
 __device__ __forceinline__ uint32_t compact16(uint32_t x) {
   x &= 0x55555555u;
   x = (x | (x >> 1)) & 0x33333333u;
@@ -486,7 +478,11 @@ __device__ __forceinline__ uint32_t compact16(uint32_t x) {
 __device__ __forceinline__ uint32_t col_code(const Grid& g, uint32_t cy, uint32_t cz) {
   const uint32_t t = g.col_shift, mask = (1u << t) - 1u;
   const uint32_t tile = (cy >> t) * g.col_tz + (cz >> t);
-  return (tile << (2 * t)) | dilate16(cy & mask) | (dilate16(cz & mask) << 1);
+  // both offsets in the tile (at most 3 bits: t <= 3) spread out in one word
+  uint32_t d = (cy & mask) | (cz & mask) << 16;
+  d = (d | d << 2) & 0x00130013u;
+  d = (d | d << 1) & 0x00150015u;
+  return (tile << (2 * t)) | ((d | d >> 15) & 0x3Fu);
 }
 __device__ __forceinline__ void key_decode(const Grid& g, uint32_t key, int& cx, int& cy, int& cz) {
   const uint32_t nx = (uint32_t)g.nc[0];
@@ -508,16 +504,17 @@ __device__ __forceinline__ void key_decode(const Grid& g, uint32_t key, int& cx,
 // range are k 2^-149 with k = M 2^(e-926) rounded (M the 53-bit significand);
 // overflow gives infinity and NaN a quiet NaN.
 __device__ __forceinline__ float d2f_rn(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const uint32_t sign = (uint32_t)(b >> 63) << 31;
-  const int e = (int)((b >> 52) & 0x7FF);
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t sign = hi & 0x80000000u;
+  const int e = (int)((hi >> 20) & 0x7FFu);
   const int fe = e - 1023 + 127;
-  if (fe >= 1 && fe <= 254) {
-    const uint32_t top = (uint32_t)((b >> 29) & 0x7FFFFFu);
-    const uint32_t rest = (uint32_t)(b & 0x1FFFFFFFu);
-    const uint32_t up = (rest > 0x10000000u || (rest == 0x10000000u && (top & 1u))) ? 1u : 0u;
-    return __uint_as_float(sign | (((uint32_t)fe << 23) + top + up));  // carry may reach inf
+  if ((uint32_t)(fe - 1) < 254u) {
+    // bits 29 to 60, the exponent's bias 1023 changed to 127 (896 2^23 modulo 2^32)
+    const uint32_t m = __funnelshift_l(lo, hi, 3) - 0xC0000000u;
+    const uint32_t up = (lo & 0x1FFFFFFFu) > 0x10000000u - (m & 1u) ? 1u : 0u;
+    return __uint_as_float(sign | (m + up));  // carry may reach inf
   }
+  const unsigned long long b = (unsigned long long)hi << 32 | lo;
   if (fe > 254) {
     const bool nan = e == 0x7FF && (b & 0xFFFFFFFFFFFFFull) != 0ull;
     return __uint_as_float(nan ? 0x7FFFFFFFu : (sign | 0x7F800000u));
@@ -537,10 +534,9 @@ __device__ __forceinline__ float d2f_abs_ru(double x) {
   const uint32_t hi = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu, lo = (uint32_t)__double2loint(x);
   const int e = (int)(hi >> 20);
   const int fe = e - 1023 + 127;
-  if (fe >= 1 && fe <= 254) {
-    const uint32_t top = (hi & 0xFFFFFu) << 3 | lo >> 29;
+  if ((uint32_t)(fe - 1) < 254u) {
     const uint32_t up = (lo & 0x1FFFFFFFu) ? 1u : 0u;
-    return __uint_as_float(((uint32_t)fe << 23) + top + up);
+    return __uint_as_float(__funnelshift_l(lo, hi, 3) - 0xC0000000u + up);
   }
   const unsigned long long b = (unsigned long long)hi << 32 | lo;
   if (fe > 254) return __uint_as_float(e == 0x7FF && (b & 0xFFFFFFFFFFFFFull) ? 0x7FFFFFFFu : 0x7F800000u);
