@@ -1509,14 +1509,14 @@ class Branches {
  public:
   explicit Branches(cudaStream_t st) : st_(st) { nfirst_ = ends(first_); }
   void next() {
-    if (nfirst_ == 0) return;
-    nlast_ += ends(last_ + nlast_);
+    const size_t n = nfirst_ ? ends(last_ + nlast_) : 0;
+    if (n == 0) return;
+    nlast_ += n;
     cudaStreamUpdateCaptureDependencies(st_, first_, nullptr, nfirst_, cudaStreamSetCaptureDependencies);
   }
-  void join() {
-    if (nfirst_ == 0) return;
-    nlast_ += ends(last_ + nlast_);
-    cudaStreamUpdateCaptureDependencies(st_, last_, nullptr, nlast_, cudaStreamSetCaptureDependencies);
+  void join() {  // what follows comes after the earlier branches too
+    if (nlast_ == 0) return;
+    cudaStreamUpdateCaptureDependencies(st_, last_, nullptr, nlast_, cudaStreamAddCaptureDependencies);
   }
 
  private:
