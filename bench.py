@@ -776,12 +776,12 @@ def run_gpu(args):
         return
 
     pk, pk_kind = peaks()
-    # dominant kernel: the slow-population search (the row search at this workload),
+    # dominant kernel: the slow-population search (tiles or rows, as the grid builder chose),
     # timed alone with CUDA events on the simulation's stream
     achieved_tflops = slow_tests * FLOPS_PER_PAIR_TEST / (slow_ms / 1e3) / 1e12 if slow_ms > 0 else 0.0
     traffic = ncu_traffic("kmc_search.cu")
     roofline = {
-        "kernel": "k_search_rows32 (slow-population search, guarded binary32)",
+        "kernel": "k_search_tiles / k_search_rows32 (slow-population search, guarded binary32)",
         "bound": "alu",
         "achieved": achieved_tflops,
         "peak": ALU_FP32_PEAK_TFLOPS,
