@@ -167,11 +167,13 @@ __device__ __forceinline__ uint32_t other_end(const SimDev& s, uint32_t e, uint3
 }
 
 // Pair e (key d2, t; partner id) competes for particle i with the pair seen there (kNone:
-// it holds the place).  The keys of the pairs that others put there are read past the L1
-// (written on other SMs, fenced before their swap).
+// it holds the place).  The keys of the pairs that others put there are read past the L1,
+// and ordered after the swap that showed the pair as their writes are before theirs: a fence
+// on either side.
 __device__ __forceinline__ void contest(const SimDev& s, int cur, uint32_t* best, uint32_t i, uint32_t e,
                                         double d2, double t, uint32_t partner_id, uint32_t seen) {
   while (seen != kNone) {
+    __threadfence();
     if (!key_less(d2, t, partner_id, __ldcg(s.e_d2 + seen), __ldcg(s.e_t + seen),
                   s.id[cur][other_end(s, seen, i)]))
       return;
