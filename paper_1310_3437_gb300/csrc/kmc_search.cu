@@ -1085,6 +1085,7 @@ __global__ void __launch_bounds__(kTile, 4) k_search_tiles(Batch B, uint32_t shi
         const uint2 lo = words[2 * (16 * t + frag)], hi = words[2 * (16 * t + 8 + frag)];
         A[t][0] = lo.x; A[t][1] = hi.x; A[t][2] = lo.y; A[t][3] = hi.y;
       }
+      __syncwarp();  // the rows are read before the first partners take their place
 
       // 3. the tiles
       for (uint32_t base = 32u * part; base < total; base += 32u * parts) {
