@@ -57,6 +57,12 @@ __device__ __forceinline__ double sqrt_up(float x) {
   return (double)__fsqrt_ru(x) * (1.0 + 0x1p-20);
 }
 
+// x 2^e for a positive x, e in the place of a high word's exponent; 0 below the normal range
+__device__ __forceinline__ double times_2(double x, int e) {
+  const int hi = __double2hiint(x) + e;
+  return hi < 0x00100000 ? 0.0 : __hiloint2double(hi, __double2loint(x));
+}
+
 // cells for search radius h (before the stencil split); key space capped by max_keys.
 // Along x the radius is split into K * kxm cells (kxm = 2: narrow cells along the rows
 // of the row search), along y and z into K.  In binary32: the quotient is within 4 u32
@@ -331,6 +337,9 @@ __device__ __noinline__ inline void compute_guards(SimDev& s, uint32_t part, uin
   const double my_w = my_nc == 1 ? my_ext : my_ext / (double)my_nc;
   const double L = my_box > my_ext ? my_box : my_ext;
   const int Ke = my_cfast > Ka ? my_cfast : Ka;
+  // half extent of a tile's frame along the axis, for a run in one cell (kmc_search.cu): the
+  // high word, which orders positive values
+  const int my_fr = __double2hiint((my_nc == 1 ? 0.5 : g.K == 1 ? 1.5 : 2.5) * my_w);
   double my_e, my_rb;
   if (my_nc == 1) {
     my_e = 6.1 * u32 * L + 8.0 * u64 * L;
@@ -351,12 +360,24 @@ __device__ __noinline__ inline void compute_guards(SimDev& s, uint32_t part, uin
                b2 = __shfl_sync(kAll, my_rb, 2);
   const double L0 = __shfl_sync(kAll, L, 0), L1 = __shfl_sync(kAll, L, 1),
                L2 = __shfl_sync(kAll, L, 2);
+  const int f0 = __shfl_sync(kAll, my_fr, 0), f1 = __shfl_sync(kAll, my_fr, 1),
+            f2 = __shfl_sync(kAll, my_fr, 2);
   if (lane != 0) return;  // lane 0 writes the rest
 
   const double dt2 = dt * dt;
   const double er = fmax(e0, fmax(e1, e2)), rbmax = fmax(b0, fmax(b1, b2));
   const double Lmax = fmax(L0, fmax(L1, L2));
-  const double rn = sqrt_up(f_up((b0 * b0 + b1 * b1) + b2 * b2)) * (1.0 + 1e-6);
+  // The power of two at or below the smallest frame of the tiled search (the largest of the
+  // three half extents and of S1 dt) is the unit in which squares of lengths are brought to
+  // binary32, so that they stay inside its range in whatever unit the caller measures lengths.
+  // (On exponents, the bits from 20 of the high word: the binary64 pipe has two lanes.)
+  const int frame = max(max(f0, f1), max(f2, __double2hiint(S1 * dt)));
+  const bool sane = frame >= 0x3A500000 && frame < 0x45900000;  // 2^-90 to 2^90
+  const int ue = sane ? (frame & 0x7FF00000) - 0x3FF00000 : 0;
+  const double q0 = times_2(b0, -ue), q1 = times_2(b1, -ue), q2 = times_2(b2, -ue);
+  const double rn = sane ? times_2(sqrt_up(fmaxf(f_up((q0 * q0 + q1 * q1) + q2 * q2), 1e-38f)) *
+                                       (1.0 + 1e-6), ue)
+                         : 1.7320508075688773 * (1.0 + 1e-6) * rbmax;
   const double V2 = V * V, rnV2 = rn * 2.0 * V;
   const double ev = 4.1 * u32 * V;
   const double g3 = 3.0 * u32 / (1.0 - 3.0 * u32);
@@ -389,11 +410,21 @@ __device__ __noinline__ inline void compute_guards(SimDev& s, uint32_t part, uin
     g.s_c1 = f_up(dt2 * (rel40 * (1.0 + g3) / (1.0 - g3) * up2));
     // pair filter of the tiled search (kmc_search.cu, "Error of the filter"): the sphere
     // test's constant with three times the separation error er, and the slack of
-    // velocities rounded to 11 bits, 2^-7 (dt S1)^2
-    g.tile_c = f_up((rel40 * (d0sq + dt2 * bslack) + 8.0 * s3 * er * rn + 27.0 * er * er) *
-                        ((1.0 + g3) * up2) + 0x1p-7 * 1.001 * dt2 * S1 * S1);
-    g.tile_k = sqrtf(g.s_c1);
+    // velocities rounded to 11 bits, 2^-7 (dt S1)^2; in squares of the unit.  tile_k is dt
+    // with at least the root of the sphere test's factor on dt^2.
+    const double c = (rel40 * (d0sq + dt2 * bslack) + 8.0 * s3 * er * rn + 27.0 * er * er) *
+                         ((1.0 + g3) * up2) + 0x1p-7 * 1.001 * dt2 * S1 * S1;
+    g.tile_k = f_up(dt * (rel40 * (1.0 + g3) / (1.0 - g3) * up2));
     g.s1f = f_up(S1);
+    // The filter runs where its operands cannot leave binary16 and binary32: a frame of
+    // ordinary size, a threshold below eight of its squares (not a gas in one cell much smaller
+    // than d0), and dt neither past binary32 nor so much above the frame that scaled
+    // velocities overflow (2^127 and 2^100).
+    const int ce = (__double2hiint(c) >> 20) - 2 * (ue >> 20);  // exponent of c in unit^2
+    const bool filter = sane && ce < 1023 + 3 &&
+                        __double2hiint(dt) < min(0x46300000 + ue, 0x47E00000);
+    g.tile_unit = filter ? __uint_as_float((uint32_t)((ue >> 20) + 127) << 23) : 0.0f;
+    g.tile_c = !filter ? 0.0f : ce < 1023 - 60 ? 0x1p-60f : f_up(times_2(c, -2 * ue));
     return;
   }
   // the upper x wall at the end of the step, for the push (never -0.0)

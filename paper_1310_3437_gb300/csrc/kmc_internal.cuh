@@ -70,9 +70,10 @@ struct Grid {
   // reach is d0 + (|v_i| + S1) dt: at most row_a + row_b |v_i| (both rounded up); for a
   // fast particle i (partners up to the bound V of max |v|) at most fast_a + row_b |v_i|
   float row_r2, row_eps, row_pad, row_a, row_b, fast_a;
-  // pair filter of the tiled search (kmc_search.cu, "Error of the filter"): its constant
-  // before scaling with the slack of the rounded velocities, dt, max slow speed
-  float tile_c, tile_k, s1f;
+  // pair filter of the tiled search (kmc_search.cu, "Error of the filter"): unit of length (0:
+  // it passes every pair), its constant before scaling with the slack of the rounded
+  // velocities in squares of the unit, dt rounded up, max slow speed
+  float tile_unit, tile_c, tile_k, s1f;
   // binary64 sphere pre-test: drop if R > c0 + c1 * B (B >= 2^-900)
   double c0, c1;
 };

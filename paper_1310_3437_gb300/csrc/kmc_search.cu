@@ -710,17 +710,19 @@ __global__ void __launch_bounds__(kTile, 4) k_search_rows32(Batch B, uint32_t sh
 // the tests of the precision run on 32 of them at a time with every lane busy: cell
 // offset (each pair at exactly one image), then the binary32 sphere and full guarded
 // tests on the mirror, or the binary64 sphere, approach and time tests on the state.  The
-// filter only saves them work: what it drops they would drop.
+// filter only saves them work: what it drops they would drop.  In a step whose lengths or
+// threshold are outside what the operands can hold (compute_guards) it passes every pair
+// (binary64: the lanes walk their particles' cells as the thread-per-particle search does).
 //
 // Error of the filter, in the scaled units.  A candidate has (kmc_grid.cuh)
 // |a_i - a_j|^2 <= c + |b_i - b_j|^2 for the exact binary32 coordinates, with c the
 // scaled constant of the sphere test with 3 er for the separation, since here the
 // coordinates are rounded once more relative to the run's middle.  The rounding of b to
 // 11 bits moves |b_i - b_j|^2 by at most 14 2^-11 b^2 < 2^-7 b^2 (both in tile_c).  The
-// rest, with the four squared extents at most 1 each and u = 2^-24: dropped and rounded
-// low parts 18 u, s and its halves 44 u, the inner product (16 products, exact in
-// binary32, whose partial sums are at most 12, added with truncation) 384 u; 2^-14 =
-// 1024 u is taken.
+// rest, with the components of a and |b| at most 1, the threshold at most 2 and u = 2^-24:
+// dropped and rounded low parts 18 u, s and its halves 44 u, the inner product (16 products,
+// exact in binary32, whose partial sums are at most 14, added with truncation) 448 u;
+// 2^-14 = 1024 u is taken.
 //
 // SHARED (few particles, see shift_of): 2^shift warps take the same 32 particles, warp w of
 // them the tiles w, w + 2^shift, ... of every run.
@@ -958,8 +960,10 @@ __global__ void __launch_bounds__(kTile, 4) k_search_tiles(Batch B, uint32_t shi
     const int Kx = nx == 1 ? 0 : K, Ky = ny == 1 ? 0 : K, Kz = nz == 1 ? 0 : K;
     const bool px = s.bc[0] == KMC_PERIODIC, py = s.bc[1] == KMC_PERIODIC,
                pz = s.bc[2] == KMC_PERIODIC;
-    if (PREC == KMC_FP64 && ((nx == 1 && px) || (ny == 1 && py) || (nz == 1 && pz))) {
-      // a one-cell periodic axis: the minimum image of every pair (binary32: row search)
+    if (PREC == KMC_FP64 && (g.tile_unit == 0.0f || (nx == 1 && px) || (ny == 1 && py) ||
+                             (nz == 1 && pz))) {
+      // No filter (lengths may be past binary32), or a one-cell periodic axis: the minimum
+      // image of every pair (binary32: row search)
       if (part != 0u) continue;
       unsigned long long t = valid ? particle_walk<PREC, K>(s, p, w.buf, &w.count) : 0ull;
       for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kAll, t, o);
@@ -1067,15 +1071,19 @@ __global__ void __launch_bounds__(kTile, 4) k_search_tiles(Batch B, uint32_t shi
       // 2. the run's frame: origin in its middle, scale the power of two that brings
       // the extents and dt |v| to at most 1
       const float wx = g.wf[0], wy = g.wf[1], wz = g.wf[2];
-      const float ox = 0.5f * (float)(x0 + x1 + 1) * wx, oy = ((float)y + 0.5f) * wy,
-                  oz = ((float)z + 0.5f) * wz;
+      float ox = 0.5f * (float)(x0 + x1 + 1) * wx, oy = ((float)y + 0.5f) * wy,
+            oz = ((float)z + 0.5f) * wz;
       const float kv = g.tile_k;
       const float M = 1.01f * fmaxf(fmaxf((0.5f * (float)(x1 - x0 + 1) + (float)Kx) * wx,
                                           (0.5f + (float)Ky) * wy),
                                     fmaxf((0.5f + (float)Kz) * wz, kv * g.s1f));
-      const float sc = __uint_as_float((253u - (__float_as_uint(M) >> 23)) << 23);  // 2^-(e+1)
-      const float T = fmaf(sc * sc, g.tile_c * 1.000001f, 0x1p-14f);
-      const float kb = kv * sc;
+      float sc = __uint_as_float((253u - (__float_as_uint(M) >> 23)) << 23);  // 2^-(e+1)
+      const bool filter = PREC == KMC_FP64 || g.tile_unit != 0.0f;
+      if (!filter) sc = ox = oy = oz = 0.0f;  // operands zero, threshold 2^-14: every pair passes
+      // (the unit is at most the frame: the product is a power of two of at most 1/2)
+      const float su = sc * g.tile_unit;
+      const float T = fmaf(su * su, g.tile_c * 1.000001f, 0x1p-14f);
+      const float kb = filter ? kv * sc : 0.0f;
       store_row(w.rec, lane, fmaf(o.ox, sc, -ox * sc), fmaf(o.oy, sc, -oy * sc),
                 fmaf(o.oz, sc, -oz * sc), o.vx * kb, o.vy * kb, o.vz * kb, T, (run >> lane) & 1u);
       __syncwarp();
