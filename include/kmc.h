@@ -62,7 +62,12 @@ extern "C" {
 #define KMC_FP64 0          /* binary64 tests of every pair that the cell geometry and a filter
                               with a proven error bound do not exclude */
 #define KMC_GUARDED_FP32 1  /* binary32 pre-tests with proven guard bands, binary64
-                               re-check of the survivors: identical pair lists */
+                               re-check of the survivors: identical pair lists.  The
+                               pre-tests square lengths, times and their products with
+                               speeds in binary32: choose units in which the reach
+                               d0 + 2 v_max dt, the box, dt and reach * v_max lie between
+                               about 1e-15 and 1e15 (KMC_FP64: lengths within 1e-30 and
+                               1e28 or so, where cells are still told apart) */
 
 /* ---- observables (sim_observe) ------------------------------------------
  * The paper writes its output after the particles are sorted into their bins

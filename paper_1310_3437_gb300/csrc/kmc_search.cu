@@ -1271,10 +1271,13 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4) k_search_fast(Batch B) {
       // so a stencil cell farther than that from p holds no candidate.  |v_p| from the
       // binary32 velocity times 1 + 2e-6 bounds it from above; the distance to a cell is
       // taken from its edges less eps (the binary32 error of a coordinate against a
-      // cell edge), rounded down.
-      const float sp = sqrtf(fmaf(o32.vz, o32.vz, fmaf(o32.vy, o32.vy, o32.vx * o32.vx))) * 1.000002f;
+      // cell edge), rounded down.  Squares are kept normal: the speed's by enlarging it, and
+      // where the reach's is not (units of length beyond about 10^18) nothing is trimmed.
+      const float sv2 = fmaf(o32.vz, o32.vz, fmaf(o32.vy, o32.vy, o32.vx * o32.vx));
+      const float sp = sqrtf(fmaxf(sv2, 1e-36f)) * 1.000002f;
       const float Rp = fmaf(sp, g.row_b, g.fast_a) * 1.000001f;
       const float Rp2 = Rp * Rp * 1.000001f;
+      const bool trim = Rp2 >= 1e-36f && Rp2 <= 1e36f;
       const float teps = g.row_eps;
       const int Wy = 2 * Cy + 1;
       const int ncol = Wy * (2 * Cz + 1);
@@ -1306,7 +1309,7 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4) k_search_fast(Batch B) {
             const float el = fmaxf(e - teps, 0.f);
             d2 = fmaf(el, el, d2);
           }
-          if (d2 * 0.9999995f >= Rp2) ok = false;
+          if (trim && d2 * 0.9999995f >= Rp2) ok = false;
           if (ok) {
             qy -= wy * ny;
             qz -= wz * nz;
@@ -1315,11 +1318,15 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4) k_search_fast(Batch B) {
             // reciprocal square root (3 ulp), widened by 33 ulp and the coordinate error
             int xa = 0, xb = 0;
             if (nx > 1) {
-              const float t2 = fmaxf(Rp2 - d2, 1e-30f);
-              const float ex = fmaf(t2 * rsqrtf(t2), 1.000004f, pad);
-              const int ta = (int)floorf((o32.ox - ex) * ivx), tb = (int)floorf((o32.ox + ex) * ivx);
-              xa = ta > cx - Cx ? ta : cx - Cx;
-              xb = tb < cx + Cx ? tb : cx + Cx;
+              xa = cx - Cx;
+              xb = cx + Cx;
+              if (trim) {
+                const float t2 = fmaxf(Rp2 - d2, 1e-30f);
+                const float ex = fmaf(t2 * rsqrtf(t2), 1.000004f, pad);
+                const int ta = (int)floorf((o32.ox - ex) * ivx), tb = (int)floorf((o32.ox + ex) * ivx);
+                xa = max(ta, xa);
+                xb = min(tb, xb);
+              }
               if (!px) {
                 xa = xa < 0 ? 0 : xa;
                 xb = xb > nx - 1 ? nx - 1 : xb;

@@ -73,6 +73,15 @@ def test_binary64_in_any_unit(kind, kernel):
     compare(*gas(kind), units, kmc.KMC_FP64, kernel, flags=1)
 
 
+@pytest.mark.parametrize("kernel", [0, 1])
+@pytest.mark.parametrize("kind", ["box", "walls"])
+def test_binary64_split_in_any_unit(kind, kernel):
+    """with the speed split whenever it fits (flags 2): the fast particles' reach, too"""
+    units = [(0, 0), (40, -100)] + [(u, 0) for u in UNITS] + [(u, u) for u in UNITS if -75 <= u <= 40]
+    s, arrays = gas(kind)
+    compare(s.with_(d0=0.015, dt=0.002), arrays, units, kmc.KMC_FP64, kernel, flags=2)
+
+
 @pytest.mark.parametrize("flags", [0, 1])
 @pytest.mark.parametrize("kind", ["box", "dense", "walls"])
 def test_binary32_tiles_in_common_units(kind, flags):
