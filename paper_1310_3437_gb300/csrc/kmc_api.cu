@@ -775,6 +775,7 @@ int create_impl(const kmc_params* p, const double* const* src6, const uint32_t* 
   dy.step = p->step0;
   dy.steps_left = 0;
   dy.parity = 0;
+  dy.loose_from = UINT64_MAX;
   if (!ck(cudaMemcpyAsync(s->d, &h, sizeof(SimDev), cudaMemcpyHostToDevice, st))) return fail(KMC_ECUDA);
   if (!ck(cudaMemcpyAsync(&s->d->d, &dy, sizeof(Dyn), cudaMemcpyHostToDevice, st))) return fail(KMC_ECUDA);
   // positions must lie in the box, velocities must be finite

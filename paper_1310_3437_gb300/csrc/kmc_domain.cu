@@ -339,7 +339,10 @@ __global__ void k_dom_record(Batch B, DomainDev* Dp) {
   }
   rec.collisions = coll;
   rec.edges = D.acc_edges;
+  uint64_t loose = s0.d.loose_from;  // a particle outside the box may go to any domain
+  for (int k = 1; k < B.nsims; ++k) loose = min(loose, B.sim(k).d.loose_from);
   for (int k = 0; k < B.nsims; ++k) {
+    B.sim(k).d.loose_from = loose;
     const SimDev& s = B.sim(k);
     if (s.d.hist_count == 0) continue;
     const kmc_step_counts& h = s.hist[(s.d.hist_count - 1) % s.hist_cap];

@@ -303,13 +303,35 @@ __device__ inline void compute_grid(SimDev& s, float vmax2_bound, uint64_t step,
   g.m = p.m;
 }
 
+// A reflecting wall turns a particle back once a step and a periodic axis wraps it once, so one
+// that crosses the whole box within a step can end it outside.  The cell assignment takes it
+// into the nearest cell; the tiled search's frames do not hold it.  From the step after the
+// first in which some particle may have done so (sim_create: from the first step if one starts
+// beyond the wall's position) that search goes without its filter.  No particle moves faster
+// than 1.5 V before the walls act, V the step's bound of max |v|: a collision leaves a speed
+// of at most sqrt(v_a^2 + v_b^2), in a mixture of at most 3 V.
+__device__ inline void watch_box(SimDev& s, uint32_t lane) {
+  const int ax = lane < 2u ? (int)lane : 2;
+  const int bc = s.bc[ax];
+  const double dt = s.dt, up = s.piston_u;
+  const uint64_t step = s.d.step;
+  double room = s.box[ax], go = (s.mix ? 3.01 : 1.5) * sqrt_up(s.d.vmax2) * dt;
+  if (ax == 0 && bc == KMC_REFLECT) {
+    room = s.piston_x0 - up * ((double)step * dt);
+    go += 2.0 * fabs(up) * dt;
+  }
+  const bool out = bc != KMC_ABSORB && !(ax == 2 && s.planar) && !(go <= room);
+  if (__any_sync(0xFFFFFFFFu, out) && lane == 0 && s.d.loose_from > step + 1) s.d.loose_from = step + 1;
+}
+
 // The guard bands of the step's pre-tests, from the grid that compute_grid chose.  Only the
 // searches need them, so they are worked out while the cells are counted up: in the chain of
 // the grid builder they took 5 us of every step, in a block of their own in the scan nothing
 // that shows (6.1 us at 4096 particles with and without).  All 32 lanes of a warp; part 0
 // sets the sphere tests and the reaches, part 1 the other tests' bands (one warp for both
-// took 6.8 us, longer than the scan of a small simulation).
+// took 6.8 us, longer than the scan of a small simulation), part 2 watches the box.
 __device__ __noinline__ inline void compute_guards(SimDev& s, uint32_t part, uint32_t lane) {
+  if (part == 2u) return watch_box(s, lane);
   constexpr uint32_t kAll = 0xFFFFFFFFu;
   const double u32 = 0x1p-24, u64 = 0x1p-53;
   Grid& g = s.d.grid;
@@ -330,6 +352,7 @@ __device__ __noinline__ inline void compute_guards(SimDev& s, uint32_t part, uin
   const double d0 = s.d0, dt = s.dt, d0sq = s.d0sq, x0 = s.piston_x0, up = s.piston_u;
   const uint64_t step = s.d.step;
   const float vmax2_bound = s.d.vmax2, s1sq = g.s1sq;
+  const bool loose = s.d.loose_from <= step;
   const bool split = g.split != 0u;
   const double V = sqrt_up(vmax2_bound);  // upper bound of max |v|
   const double S1 = split ? sqrt_up(s1sq) : V;
@@ -416,12 +439,13 @@ __device__ __noinline__ inline void compute_guards(SimDev& s, uint32_t part, uin
                          ((1.0 + g3) * up2) + 0x1p-7 * 1.001 * dt2 * S1 * S1;
     g.tile_k = f_up(dt * (rel40 * (1.0 + g3) / (1.0 - g3) * up2));
     g.s1f = f_up(S1);
-    // The filter runs where its operands cannot leave binary16 and binary32: a frame of
+    // The filter runs where its operands cannot leave binary16 and binary32: every particle in
+    // its cell (watch_box; the third warp sets it for the steps after this), a frame of
     // ordinary size, a threshold below eight of its squares (not a gas in one cell much smaller
     // than d0), and dt neither past binary32 nor so much above the frame that scaled
     // velocities overflow (2^127 and 2^100).
     const int ce = (__double2hiint(c) >> 20) - 2 * (ue >> 20);  // exponent of c in unit^2
-    const bool filter = sane && ce < 1023 + 3 &&
+    const bool filter = sane && !loose && ce < 1023 + 3 &&
                         __double2hiint(dt) < min(0x46300000 + ue, 0x47E00000);
     g.tile_unit = filter ? __uint_as_float((uint32_t)((ue >> 20) + 127) << 23) : 0.0f;
     g.tile_c = !filter ? 0.0f : ce < 1023 - 60 ? 0x1p-60f : f_up(times_2(c, -2 * ue));

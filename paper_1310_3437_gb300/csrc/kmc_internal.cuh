@@ -104,6 +104,7 @@ struct Dyn {
   uint32_t prof_count;  // snapshots written
   uint64_t hist_count;  // step records written
   uint32_t n_absorbed;  // particles that left through absorbing walls this step
+  uint64_t loose_from;  // from this step on particles may lie outside the box (watch_box)
 };
 
 struct SimDev {

@@ -616,6 +616,10 @@ __global__ void k_validate(SimDev* d, uint32_t* bad) {
   if (s.planar && s.v[s.d.parity][2][p] != 0.0) out = true;
   if (s.mix && s.species[s.id[s.d.parity][p]] >= (uint32_t)s.mix_n) out = true;
   if (out) atomicAdd(bad, 1u);
+  // a wall that has moved below the particle before the first step (watch_box)
+  if (!left && s.bc[0] == KMC_REFLECT &&
+      s.x[s.d.parity][0][p] > dsub(s.piston_x0, dmul(s.piston_u, dmul((double)s.d.step, s.dt))))
+    s.d.loose_from = 0;
 }
 
 void launch_validate(SimDev* d, uint32_t n, uint32_t* bad, cudaStream_t st) {

@@ -134,14 +134,15 @@ __device__ __forceinline__ unsigned long long scan_word(uint32_t epoch, unsigned
   return ((unsigned long long)epoch << 34) | (state << 32) | (unsigned long long)value;
 }
 
-// The first `guards` blocks have no tile: two warps of them per simulation work out the guard
-// bands of the step's searches.
+// The first `guards` blocks have no tile: three warps of them per simulation (of four) work
+// out the guard bands of the step's searches.
 __global__ void __launch_bounds__(kTile) k_scan_onepass(Batch B, uint32_t ntiles, uint32_t guards) {
   __shared__ uint32_t s_tile, s_excl;
   if (blockIdx.x < guards) {
-    const int k = (int)(blockIdx.x * (kTile / 64) + threadIdx.x / 64u);
-    if (k < B.nsims && sim_active(B.sim(k)))
-      compute_guards(B.sim(k), (threadIdx.x >> 5) & 1u, threadIdx.x & 31u);
+    const int k = (int)(blockIdx.x * (kTile / 128) + threadIdx.x / 128u);
+    const uint32_t part = (threadIdx.x >> 5) & 3u;
+    if (k < B.nsims && part < 3u && sim_active(B.sim(k)))
+      compute_guards(B.sim(k), part, threadIdx.x & 31u);
     return;
   }
   if (threadIdx.x == 0) s_tile = atomicAdd(&B.scan_ctl[0], 1u);
@@ -431,7 +432,7 @@ __global__ void __launch_bounds__(kTile / 2) k_gather(Batch B) {
 
 // --------------------------------------------------------------------------- //
 int launch_cell_scan(const LaunchPlan& L, cudaStream_t st) {
-  const uint32_t nt = L.stiles_c, guards = (uint32_t)(L.b.nsims + kTile / 64 - 1) / (kTile / 64);
+  const uint32_t nt = L.stiles_c, guards = (uint32_t)(L.b.nsims + kTile / 128 - 1) / (kTile / 128);
   k_scan_onepass<<<guards + nt, kTile, 0, st>>>(L.b, nt, guards);
   return 1;
 }
