@@ -43,8 +43,10 @@ extern "C" {
 #define KMC_ENOMEM (-2)    /* device allocation failed */
 #define KMC_ECUDA (-3)     /* a CUDA runtime call failed */
 #define KMC_ETIMEOUT (-4)  /* a bounded device-side wait ran out: a tile of the cell
-                              scan waited about a second for its predecessor's sum (the
-                              step's results are void; sim_sync reports it) */
+                              scan waited for its predecessor's sum, or a block of the
+                              matching rounds for the others (2^20 polls, 0.3 s and more; the
+                              step's results are void, sim_sync reports it and
+                              sim_last_error names the wait) */
 #define KMC_EOVERFLOW (-5) /* a buffer capacity was exceeded and could not grow */
 #define KMC_ESTATE (-6)    /* call not allowed in the current state */
 #define KMC_ERANDOM (-7)   /* 128 rejected sphere-point draws (probability ~1e-43) */
@@ -130,6 +132,11 @@ extern "C" {
 #define KMC_FLAG_SCAN_WAIT_TEST 8u /* test of the failure path only: the cell scan's tiles
                                   wait for a status word that is never written, run into
                                   their bounded wait and sim_sync returns KMC_ETIMEOUT */
+#define KMC_FLAG_ROUND_WAIT_TEST 32u /* test of the failure path only: the blocks of the
+                                  matching rounds after the first wait at a barrier that
+                                  never opens, run into their bounded wait and sim_sync
+                                  returns KMC_ETIMEOUT (in a group: for every member that
+                                  runs the step) */
 
 /* ---- search kernels (kmc_params.search_kernel) ----------------------------- */
 #define KMC_SEARCH_AUTO 0      /* per step: tiles in binary64 and when cells are well

@@ -51,6 +51,7 @@ KMC_FLAG_NO_SPLIT = 1
 KMC_FLAG_FORCE_SPLIT = 2
 KMC_FLAG_PLANAR = 4
 KMC_FLAG_SCAN_WAIT_TEST = 8
+KMC_FLAG_ROUND_WAIT_TEST = 32
 
 KMC_INIT_MAXWELL = 1
 KMC_INIT_EQUAL_SPEED = 2

@@ -149,7 +149,7 @@ int validate(const kmc_params* p, std::string& err) {
   if (!p) { err = "params is NULL"; return KMC_EINVAL; }
   if (p->n == 0) { err = "n must be >= 1"; return KMC_EINVAL; }
   if (p->flags & ~(uint32_t)(KMC_FLAG_NO_SPLIT | KMC_FLAG_FORCE_SPLIT | KMC_FLAG_PLANAR |
-                             KMC_FLAG_SCAN_WAIT_TEST)) {
+                             KMC_FLAG_SCAN_WAIT_TEST | KMC_FLAG_ROUND_WAIT_TEST)) {
     err = "unknown flags";
     return KMC_EINVAL;
   }
@@ -343,6 +343,7 @@ int build_plan(Plan& P, const std::vector<kmc_sim*>& sims, cudaStream_t st, std:
     if (h.mix) P.L.mix = true;
     if (h.search_kernel == KMC_SEARCH_PARTICLE) P.L.particle = true;
     (h.bc[0] == KMC_PERIODIC ? P.L.periodic_x : P.L.bounded_x) = true;
+    if (sims[k]->p.flags & KMC_FLAG_ROUND_WAIT_TEST) P.L.round_wait_test = true;
   }
   // prefixes (3 (m + 1) words, padded to an even count), the scan's and the rounds' two
   // control words each, then one 64-bit status word per scan tile
@@ -389,7 +390,8 @@ int build_plan(Plan& P, const std::vector<kmc_sim*>& sims, cudaStream_t st, std:
   // longer: 74 -> 45 us at 2^21; a 2^20 tube 16.5 either way, a box of 2^18 10.7 and 12.1);
   // one per SM at most, so that all of them run at once
   L.round_blocks = (int)std::min<uint32_t>(
-      std::max(pt[m] < 2048u ? pt[m] / 256u : pt[m] / 32u, 1u), (uint32_t)num_sms());
+      std::max(pt[m] < 2048u ? pt[m] / 256u : pt[m] / 32u, L.round_wait_test ? 2u : 1u),
+      (uint32_t)num_sms());
   match_grids(num_sms(), L);
   search_grids(P.precision, P.K, num_sms(), L.ptiles, L);
   return KMC_OK;
@@ -523,6 +525,7 @@ int status_code(uint32_t status, std::string& err) {
   if (status & ST_RANDOM) { err = "128 rejected sphere-point draws"; return KMC_ERANDOM; }
   if (status & ST_CELL_OVERFLOW) { err = "cell grid exceeds capacity"; return KMC_EOVERFLOW; }
   if (status & ST_SCAN_WAIT) { err = "a scan tile's wait for its predecessor ran out"; return KMC_ETIMEOUT; }
+  if (status & ST_ROUND_WAIT) { err = "a wait of the matching rounds' blocks for each other ran out"; return KMC_ETIMEOUT; }
   if (status & ST_EDGE_OVERFLOW) { err = "candidate-pair buffer overflow"; return KMC_EOVERFLOW; }
   return KMC_OK;
 }

@@ -35,6 +35,7 @@ enum : uint32_t {
   ST_RANDOM = 1u << 1,         // 128 rejected sphere-point draws
   ST_CELL_OVERFLOW = 1u << 2,  // grid key space above capacity (cannot happen: coarsened)
   ST_SCAN_WAIT = 1u << 3,      // a scan tile waited too long for its predecessor's sum
+  ST_ROUND_WAIT = 1u << 4,     // a block of the matching rounds waited too long for the others
 };
 
 // how the slow pairs of a step are searched (Grid::mode)
@@ -182,6 +183,7 @@ struct Batch {
   unsigned long long* tile_status;
   uint32_t* scan_ctl;
   uint32_t* round_ctl;     // grid barrier of the later matching rounds: arrivals, generation
+                           // (cleared by every step's count)
 
   __device__ __forceinline__ SimDev& sim(int k) const { return one ? *one : *sims[k]; }
   // simulation k's first tile in a tile prefix
@@ -610,6 +612,7 @@ struct LaunchPlan {
   int push_blocks;         // grid of the push, each block every so many tiles
   int prof_blocks;         // grid of the profile kernel, each block a range of tiles
   int round_blocks;        // cooperative grid of the later matching rounds
+  bool round_wait_test = false;  // KMC_FLAG_ROUND_WAIT_TEST: their barrier never opens
   bool lists = false;      // domains: the rounds work on per-particle candidate lists
   int part_blocks;  // grid-stride grids of the particle, tiled, row and fast searches
   int tile_blocks;

@@ -321,9 +321,10 @@ __global__ void __launch_bounds__(kEdgeBlock) k_settle(Batch B) {
 }
 
 // A barrier of all blocks of the launch (launched cooperatively: they all run).  The wait
-// is bounded (about a second); false: it ran out, and every block that notices leaves.
-constexpr int kGridWaitLimit = 1 << 20;  // spins of at least 0.1 us
-__device__ __forceinline__ bool grid_barrier(uint32_t* ctl) {
+// is bounded; false: it ran out, and every block that notices leaves.  The failure-path
+// test's barrier never opens (closed).
+constexpr int kGridWaitLimit = 1 << 20;  // spins: 0.3 s
+__device__ __forceinline__ bool grid_barrier(uint32_t* ctl, bool closed) {
   __shared__ int ok;
   if (gridDim.x == 1) {
     __threadfence();
@@ -336,7 +337,7 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* ctl) {
     volatile uint32_t* gen = ctl + 1;
     const uint32_t now = *gen;
     __threadfence();
-    if (atomicAdd(ctl, 1u) == gridDim.x - 1u) {
+    if (atomicAdd(ctl, 1u) == gridDim.x - 1u && !closed) {
       *(volatile uint32_t*)ctl = 0u;
       __threadfence();
       *gen = now + 1u;
@@ -360,7 +361,12 @@ __device__ __forceinline__ uint32_t open_pairs(const SimDev& s, int round) {
   return sim_scheduled(s) && round < s.max_rounds ? __ldcg(&s.d.wl_len[round]) : 0u;
 }
 
-__global__ void __launch_bounds__(kEdgeBlock) k_rounds(Batch B, int max_rounds) {
+__global__ void __launch_bounds__(kEdgeBlock) k_rounds(Batch B, int max_rounds, bool closed) {
+  // Steps queued behind a failed one find no member that runs and do not wait again.  (Only
+  // a wait that ran out changes the answer during the launch.)
+  bool any = false;
+  for (int k = (int)threadIdx.x; k < B.nsims; k += kEdgeBlock) any = any || sim_active(B.sim(k));
+  if (!__syncthreads_or(any)) return;
   for (int round = 1; round < max_rounds; ++round) {
     for_dealt(B, [round](const SimDev& s) { return open_pairs(s, round); },
               [round](SimDev& s, uint32_t first, uint32_t) {
@@ -375,7 +381,7 @@ __global__ void __launch_bounds__(kEdgeBlock) k_rounds(Batch B, int max_rounds) 
         propose(s, cur, best, pr, e, d2, tt, s.id[cur][pr.x], s.id[cur][pr.y]);
       }
     });
-    bool in_time = grid_barrier(B.round_ctl);
+    bool in_time = grid_barrier(B.round_ctl, closed);
     if (in_time) {
       for_dealt(B, [round](const SimDev& s) { return open_pairs(s, round); },
                 [round](SimDev& s, uint32_t first, uint32_t trips) {
@@ -388,11 +394,11 @@ __global__ void __launch_bounds__(kEdgeBlock) k_rounds(Batch B, int max_rounds) 
         }
       });
       if (round + 1 == max_rounds) return;
-      in_time = grid_barrier(B.round_ctl);
+      in_time = grid_barrier(B.round_ctl, closed);
     }
     if (!in_time) {
       for (int k = (int)threadIdx.x; k < B.nsims; k += kEdgeBlock)
-        atomicOr(&B.sim(k).d.status, ST_SCAN_WAIT);
+        if (sim_scheduled(B.sim(k))) atomicOr(&B.sim(k).d.status, ST_ROUND_WAIT);
       return;
     }
     if (B.nsims == 1 && __ldcg(&B.sim(0).d.wl_len[round + 1]) == 0u) return;  // nothing is open
@@ -503,7 +509,8 @@ int launch_match(const LaunchPlan& L, int max_rounds, cudaStream_t st) {
   int n = 2;
   if (max_rounds > 1) {
     Batch b = L.b;
-    void* args[] = {&b, &max_rounds};
+    bool closed = L.round_wait_test;
+    void* args[] = {&b, &max_rounds, &closed};
     cudaLaunchCooperativeKernel((const void*)k_rounds, dim3(L.round_blocks), dim3(kEdgeBlock), args, 0, st);
     ++n;
   }

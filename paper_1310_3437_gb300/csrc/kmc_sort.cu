@@ -51,10 +51,12 @@ __device__ __forceinline__ uint32_t run_rank(uint32_t* counts, uint32_t key, boo
 // the key after every cell)
 template <bool ABS>
 __global__ void __launch_bounds__(kTile / 2) k_count(Batch B) {
-  // the scan that follows hands out its tiles from 0 and starts a new epoch
+  // the scan that follows hands out its tiles from 0 and starts a new epoch; the barrier of
+  // the matching rounds starts with no arrivals, whatever an earlier step's wait left there
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     B.scan_ctl[0] = 0u;
     B.scan_ctl[1] += 1u;
+    B.round_ctl[0] = 0u;
   }
   int k = find_sim(B.ptile, B.nsims, blockIdx.x);
   SimDev& s = B.sim(k);
