@@ -40,18 +40,14 @@ struct Plan {
   int launches_per_step = 0;
 };
 
-int g_num_sms = 0;
-
+// SMs of the current device (asked for each plan: a process may use several)
 int num_sms() {
-  if (g_num_sms == 0) {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-      g_num_sms = v;
-    else
-      g_num_sms = 152;
-  }
-  return g_num_sms;
+  int dev = 0, v = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess &&
+      cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
+    return v;
+  cudaGetLastError();
+  return 152;
 }
 
 }  // namespace
@@ -380,29 +376,34 @@ int build_plan(Plan& P, const std::vector<kmc_sim*>& sims, cudaStream_t st, std:
   L.ptiles = pt[m];
   L.stiles_c = sc[m];
   L.prtiles = pr[m];
-  L.push_blocks = (int)std::min<uint32_t>(std::max(pt[m], 1u), 8u * (uint32_t)num_sms());
-  L.prof_blocks = (int)std::min<uint32_t>(std::max(pr[m], 1u), 4u * (uint32_t)num_sms());
+  const uint32_t sms = (uint32_t)num_sms();
+  L.push_blocks = (int)std::min<uint32_t>(std::max(pt[m], 1u), 8u * sms);
+  L.prof_blocks = (int)std::min<uint32_t>(std::max(pr[m], 1u), 4u * sms);
   // a block per tile of particles (one particle in twenty has a candidate pair), as many as
   // the SMs hold at most: a launch of idle blocks takes 1.1 us, one of a few 0.6
-  L.edge_blocks = (int)std::min<uint32_t>(std::max(pt[m], 1u), 8u * (uint32_t)num_sms());
+  L.edge_blocks = (int)std::min<uint32_t>(std::max(pt[m], 1u), 8u * sms);
   // a block of the later rounds per 2^16 particles (their lists hold about one pair in a
   // thousand particles of a tube), from 2^19 particles on per 2^13 (a blast's lists are
   // longer: 74 -> 45 us at 2^21; a 2^20 tube 16.5 either way, a box of 2^18 10.7 and 12.1);
   // one per SM at most, so that all of them run at once
   L.round_blocks = (int)std::min<uint32_t>(
       std::max(pt[m] < 2048u ? pt[m] / 256u : pt[m] / 32u, L.round_wait_test ? 2u : 1u),
-      (uint32_t)num_sms());
-  match_grids(num_sms(), L);
-  search_grids(P.precision, P.K, num_sms(), L.ptiles, L);
+      sms);
+  match_grids((int)sms, L);
+  search_grids(P.precision, P.K, (int)sms, L.ptiles, L);
   return KMC_OK;
 }
 
+constexpr const char* kRefused = "a kernel launch of the step was refused";
+
+// the step's kernels; returns their number, or -1 if a launch was refused (the rest is not
+// launched then)
 int enqueue_step(const Plan& P, cudaStream_t st) {
   int n = launch_sort(P.L, st);
   n += launch_search(P.L, P.precision, P.K, st);
-  n += launch_match(P.L, P.max_rounds, st);
-  n += launch_push(P.L, st);
-  return n;
+  const int m = launch_match(P.L, P.max_rounds, st);
+  if (m < 0) return -1;
+  return n + m + launch_push(P.L, st);
 }
 
 // Diagnostic stepping: phases launched one by one between CUDA events on the
@@ -418,7 +419,15 @@ int run_steps_timed(Plan& P, cudaStream_t st, uint64_t nsteps, kmc_sim* s) {
     cudaEventRecord(ev[1], st);
     n += launch_search(P.L, P.precision, P.K, st, ev + 5);
     cudaEventRecord(ev[2], st);
-    n += launch_match(P.L, P.max_rounds, st);
+    const int m = launch_match(P.L, P.max_rounds, st);
+    if (m < 0) {
+      mark_refused(P.L, st);
+      cudaGetLastError();
+      s->err = std::string("timed step: ") + kRefused;
+      rc = KMC_ECUDA;
+      break;
+    }
+    n += m;
     cudaEventRecord(ev[3], st);
     n += launch_push(P.L, st);
     cudaEventRecord(ev[4], st);
@@ -444,16 +453,19 @@ int run_steps_timed(Plan& P, cudaStream_t st, uint64_t nsteps, kmc_sim* s) {
 }
 
 // Replay the captured step nsteps times (capture on first use; plain launches if
-// the stream cannot be captured).  Returns launches through *launched.
+// the stream cannot be captured, or if a launch was refused meanwhile: a graph without it
+// would run wrong steps).  Returns launches through *launched.
 int run_steps(Plan& P, cudaStream_t st, uint64_t nsteps, std::string& err, uint64_t* launched) {
   if (!P.graph_tried) {
     P.graph_tried = true;
     cudaGraph_t graph = nullptr;
+    cudaGetLastError();
     if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
       P.launches_per_step = enqueue_step(P, st);
-      cudaError_t e = cudaStreamEndCapture(st, &graph);
+      const bool whole = P.launches_per_step >= 0 && cudaGetLastError() == cudaSuccess;
+      const cudaError_t e = cudaStreamEndCapture(st, &graph);
       if (e == cudaSuccess && graph) {
-        if (cudaGraphInstantiate(&P.graph, graph, 0) != cudaSuccess) P.graph = nullptr;
+        if (!whole || cudaGraphInstantiate(&P.graph, graph, 0) != cudaSuccess) P.graph = nullptr;
         cudaGraphDestroy(graph);
       }
     }
@@ -464,7 +476,14 @@ int run_steps(Plan& P, cudaStream_t st, uint64_t nsteps, std::string& err, uint6
       KCHECK(cudaGraphLaunch(P.graph, st), err);
       *launched += P.launches_per_step;
     } else {
-      *launched += enqueue_step(P, st);
+      const int n = enqueue_step(P, st);
+      if (n < 0) {
+        mark_refused(P.L, st);
+        cudaGetLastError();
+        err = kRefused;
+        return KMC_ECUDA;
+      }
+      *launched += n;
     }
   }
   KCHECK(cudaGetLastError(), err);
@@ -526,6 +545,7 @@ int status_code(uint32_t status, std::string& err) {
   if (status & ST_CELL_OVERFLOW) { err = "cell grid exceeds capacity"; return KMC_EOVERFLOW; }
   if (status & ST_SCAN_WAIT) { err = "a scan tile's wait for its predecessor ran out"; return KMC_ETIMEOUT; }
   if (status & ST_ROUND_WAIT) { err = "a wait of the matching rounds' blocks for each other ran out"; return KMC_ETIMEOUT; }
+  if (status & ST_LAUNCH) { err = kRefused; return KMC_ECUDA; }
   if (status & ST_EDGE_OVERFLOW) { err = "candidate-pair buffer overflow"; return KMC_EOVERFLOW; }
   return KMC_OK;
 }
@@ -948,11 +968,13 @@ int dom_step(kmc_sim* s, uint32_t nsteps) {
   if (!D->graph_tried) {
     D->graph_tried = true;
     cudaGraph_t graph = nullptr;
+    cudaGetLastError();
     if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
       D->launches_per_step = dom_enqueue(D, st);
+      const bool whole = cudaGetLastError() == cudaSuccess;
       const cudaError_t e = cudaStreamEndCapture(st, &graph);
       if (e == cudaSuccess && graph) {
-        if (cudaGraphInstantiate(&D->graph, graph, 0) != cudaSuccess) D->graph = nullptr;
+        if (!whole || cudaGraphInstantiate(&D->graph, graph, 0) != cudaSuccess) D->graph = nullptr;
         cudaGraphDestroy(graph);
       }
     }

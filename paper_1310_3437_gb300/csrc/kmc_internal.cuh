@@ -36,6 +36,7 @@ enum : uint32_t {
   ST_CELL_OVERFLOW = 1u << 2,  // grid key space above capacity (cannot happen: coarsened)
   ST_SCAN_WAIT = 1u << 3,      // a scan tile waited too long for its predecessor's sum
   ST_ROUND_WAIT = 1u << 4,     // a block of the matching rounds waited too long for the others
+  ST_LAUNCH = 1u << 5,         // a launch of the step was refused (host: mark_refused)
 };
 
 // how the slow pairs of a step are searched (Grid::mode)
@@ -639,8 +640,10 @@ int launch_search(const LaunchPlan& L, int precision, int K, cudaStream_t st,
 // resident-block grids of the search kernels (and the row search's shared-memory
 // attribute); called when a launch plan is built, before any capture
 void search_grids(int precision, int K, int num_sms, uint32_t ptiles, LaunchPlan& L);
+// (-1: the rounds' cooperative launch was refused, nothing after it was launched)
 int launch_match(const LaunchPlan& L, int max_rounds, cudaStream_t st);
-void match_grids(int num_sms, LaunchPlan& L);  // with the plan, after its edge_blocks
+// with the plan, after its edge_blocks and round_blocks
+void match_grids(int num_sms, LaunchPlan& L);
 // the parts of launch_match around the rounds: exact test and candidate lists; collision
 int launch_match_lists(const LaunchPlan& L, cudaStream_t st);
 int launch_collide(const LaunchPlan& L, cudaStream_t st);
@@ -661,6 +664,8 @@ struct MemberState {
   uint64_t status;
 };
 void launch_member_states(const LaunchPlan& L, MemberState* out, cudaStream_t st);
+// ST_LAUNCH to the members that run the step: it was launched in part
+void mark_refused(const LaunchPlan& L, cudaStream_t st);
 
 // observe helpers
 void launch_gather_state(SimDev* d, uint32_t n, void* out, cudaStream_t st);

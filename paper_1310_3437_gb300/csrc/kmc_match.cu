@@ -22,6 +22,8 @@
 // particle: there k_refine hands out slots, k_alloc and k_fill build each particle's
 // candidate list (only particles with candidates are touched), and kmc_domain.cu runs the
 // rounds over them.
+#include <algorithm>
+
 #include "kmc_internal.cuh"
 #include "kmc_rng.cuh"
 
@@ -483,6 +485,7 @@ void match_grids(int num_sms, LaunchPlan& L) {
   };
   L.refine_few = L.mix ? few(k_refine<true, false>) : few(k_refine<false, false>);
   L.collide_few = L.mix ? few(k_collide<true, false>) : few(k_collide<false, false>);
+  L.round_blocks = std::min(L.round_blocks, few(k_rounds));  // the cooperative grid: all resident
 }
 
 int launch_match_lists(const LaunchPlan& L, cudaStream_t st) {
@@ -511,7 +514,11 @@ int launch_match(const LaunchPlan& L, int max_rounds, cudaStream_t st) {
     Batch b = L.b;
     bool closed = L.round_wait_test;
     void* args[] = {&b, &max_rounds, &closed};
-    cudaLaunchCooperativeKernel((const void*)k_rounds, dim3(L.round_blocks), dim3(kEdgeBlock), args, 0, st);
+    // refused where fewer blocks fit than the device's attributes say (a process that has a
+    // part of its SMs): without the rounds the step must not go on
+    if (cudaLaunchCooperativeKernel((const void*)k_rounds, dim3(L.round_blocks), dim3(kEdgeBlock),
+                                    args, 0, st) != cudaSuccess)
+      return -1;
     ++n;
   }
   return n + launch_collide(L, st);

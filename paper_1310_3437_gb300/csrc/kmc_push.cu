@@ -465,6 +465,14 @@ void launch_member_states(const LaunchPlan& L, MemberState* out, cudaStream_t st
   k_member_states<<<(L.b.nsims + 255) / 256, 256, 0, st>>>(L.b, out);
 }
 
+__global__ void k_mark_refused(Batch B) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < B.nsims && sim_scheduled(B.sim(k))) B.sim(k).d.status |= ST_LAUNCH;
+}
+void mark_refused(const LaunchPlan& L, cudaStream_t st) {
+  k_mark_refused<<<(L.b.nsims + 255) / 256, 256, 0, st>>>(L.b);
+}
+
 // ---- observables ------------------------------------------------------------ //
 // The state in id order (x, y, z, vx, vy, vz as n binary64 each, then n last partners).
 // Ids and positions in the cell order have nothing to do with each other, so one side of
