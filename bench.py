@@ -62,6 +62,16 @@ def sample_setup(box_yz: float = 0.25):
     return s.with_(d0=full.d0, dt=full.dt, name="piston_tube_cross_section")
 
 
+def check_params(setup):
+    """The arm that the timed search is compared with: a thread per particle, every pair of
+    its cells in binary64, no speed split, so that neither the tiles' pair filter nor the
+    row and fast-particle searches are on both sides."""
+    import paper_1310_3437_gb300 as kmc
+
+    return kmc.params_from_setup(setup, precision=kmc.KMC_FP64, search_kernel=kmc.KMC_SEARCH_PARTICLE,
+                                 flags=kmc.KMC_FLAG_NO_SPLIT)
+
+
 def peaks():
     try:
         with open(PEAKS_PATH) as f:
@@ -643,11 +653,12 @@ def run_gpu(args):
         """Guarded binary32 (the timed knobs) and binary64 from the same state, one step
         at a time: sorted candidate-pair lists, partners and step counts compared in
         every step, the whole state after the last (Sec. 2: the criteria and the
-        closest partner fix the list, so the pre-test precision must not change it)."""
+        closest partner fix the list, so the pre-test precision must not change it).
+        The binary64 arm shares no search kernel with the other (check_params)."""
         a = kmc.Simulation(kmc.params_from_setup(setup, precision=kmc.KMC_GUARDED_FP32, **knobs),
                            dev_arrays, stream=stream.cuda_stream)
-        b = kmc.Simulation(kmc.params_from_setup(setup, precision=kmc.KMC_FP64), dev_arrays,
-                           stream=stream.cuda_stream)
+        b = kmc.Simulation(check_params(setup), dev_arrays, stream=stream.cuda_stream)
+        t0 = time.perf_counter()
         res = {"steps": steps, "edges_identical": True, "partners_identical": True,
                "counts_identical": True, "edge_sha256_16": []}
         for _ in range(steps):
@@ -669,6 +680,7 @@ def run_gpu(args):
         torch.cuda.synchronize(dev)
         res["state_identical"] = bool(torch.equal(ba, bb))
         res["candidate_pairs_per_step"] = float(eb.shape[0])
+        res["seconds"] = time.perf_counter() - t0
         a.close()
         b.close()
         del ba, bb
