@@ -99,8 +99,8 @@ extern "C" {
                               sort, search, matching (exact test, lists, rounds,
                               scatter) and push phases while timing was on, the number
                               of timed steps, then the milliseconds of the main search
-                              kernel alone (the one that searches the slow population:
-                              row, cell or particle search), part of the search phase */
+                              kernels alone (tiles, rows or thread per particle),
+                              part of the search phase */
 #define KMC_OBS_VMAX 9     /* one binary64: the largest particle speed of the current
                               state, sqrt(max ((vx*vx + vy*vy) + vz*vz)) over the particles
                               in the gas, each operation correctly rounded (0 for an
@@ -190,7 +190,12 @@ typedef struct kmc_step_counts {
   uint32_t round_pairs[4];  /* pairs matched in rounds 1..4 */
   uint32_t survivors;       /* pairs that passed the search pre-tests */
   uint32_t cells;           /* cells of the search grid */
-  uint64_t pair_tests;      /* pair tests done by the search */
+  uint64_t pair_tests;      /* pairs that the searches looked at.  Rows, fast particles and
+                               thread per particle: pairs tested one by one.  Tiles: every
+                               pair of a row and a partner of its tiles, most of which only
+                               the pair filter sees (pairs outside the row's own cells and
+                               the own column's earlier ones included).  The number depends
+                               on the search, a rate of it compares like with like only */
   uint64_t fast_tests;      /* the part of pair_tests done for the fast particles of the
                                speed split (the rest is the slow-population search) */
   uint32_t absorbed;        /* particles that left through absorbing walls this step */
