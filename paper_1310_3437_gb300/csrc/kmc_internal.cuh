@@ -18,7 +18,6 @@ constexpr int kTile = 256;          // particles per block in particle kernels
 constexpr int kScanTile = 8192;     // keys per tile of the cell scan
 constexpr int kProfTile = 4096;     // particles per tile of the profile kernel
 constexpr int kEdgeBlock = 256;     // threads per block in edge / adjacency kernels
-constexpr int kSearchBuf = 512;     // per-block shared-memory staging of emitted pairs
 constexpr uint32_t kNone = 0xFFFFFFFFu;
 constexpr int kProfQ = 20;          // int64 counters per profile bin (see profile_add below)
 constexpr int kMaxGroup = 4096;     // simulations per batch
@@ -469,14 +468,6 @@ __device__ __forceinline__ void mirror_store(float4* M, uint32_t j, float x, flo
 }
 
 // ---- Morton column code --------------------------------------------------- //
-__device__ __forceinline__ uint32_t compact16(uint32_t x) {
-  x &= 0x55555555u;
-  x = (x | (x >> 1)) & 0x33333333u;
-  x = (x | (x >> 2)) & 0x0F0F0F0Fu;
-  x = (x | (x >> 4)) & 0x00FF00FFu;
-  x = (x | (x >> 8)) & 0x0000FFFFu;
-  return x;
-}
 // Column order: the (y, z) plane is cut into T x T tiles (T = 2^col_shift <= 8)
 // walked row by row; inside a tile the columns follow the Z-order (Morton) curve.
 // Padding is below T per axis.
@@ -488,17 +479,6 @@ __device__ __forceinline__ uint32_t col_code(const Grid& g, uint32_t cy, uint32_
   d = (d | d << 2) & 0x00130013u;
   d = (d | d << 1) & 0x00150015u;
   return (tile << (2 * t)) | ((d | d >> 15) & 0x3Fu);
-}
-__device__ __forceinline__ void key_decode(const Grid& g, uint32_t key, int& cx, int& cy, int& cz) {
-  const uint32_t nx = (uint32_t)g.nc[0];
-  const uint32_t col = key / nx;
-  cx = (int)(key - col * nx);
-  const uint32_t t = g.col_shift;
-  const uint32_t tile = col >> (2 * t);
-  const uint32_t in = col & ((1u << (2 * t)) - 1u);
-  const uint32_t by = tile / g.col_tz, bz = tile - by * g.col_tz;
-  cy = (int)((by << t) | compact16(in));
-  cz = (int)((bz << t) | compact16(in >> 1));
 }
 
 // binary64 -> binary32 conversions on the integer pipes (on this part the hardware

@@ -13,7 +13,7 @@
 // The scratch array holds kStaticBins x 20 int64 fixed-point counters (40,960
 // bytes): per bin the count, three 32-bit digits of each velocity sum and of each
 // sum of squares, and the number of terms out of the digits' range (profile_add in
-// kmc_internal.cuh; the profile kernel of the simulations uses the same helpers).
+// kmc_internal.cuh; the profile kernel of the simulations adds up the same digits).
 // Every GPU that loads the library keeps its own copy until the process exits.
 // All calls on a device share it and it keeps the last call's contents; each call
 // clears the counters it uses before accumulating.  Two calls whose work overlaps
