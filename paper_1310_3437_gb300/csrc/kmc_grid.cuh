@@ -44,12 +44,17 @@ struct CellPlan {
   bool ok;
 };
 
-// Mean particles per cell from which the binary32 path searches with tiles.  The row search's
-// time hardly depends on the filling (its rows are trimmed to the particle's reach), the
-// tiled one's on the cells, so in fuller cells, with fewer fast particles, tiles gain.  With
-// the line at 2.5, 3.5, 5, 7 and 10 per cell: four steps of the 2^24 tube 12.1, 12.1, 12.4,
-// 12.9 and 13.4 ms, of 10^7 particles in the plane 5.87, 5.84, 5.87, 5.95 and 6.03; smaller
-// runs are the same within 1 %.
+// Mean particles per cell from which the binary32 path searches with tiles.  On the same grid
+// the two are close: slow pairs of a step at 2^21 particles, rows against tiles, tube at 1 per
+// cell 165 and 175 us, at 4.8 180 and 198; plane at 2.5 102 and 117; box at 4.1 226 and 212, at
+// 8.4 268 and 250; blast at 5.8 319 and 249, at 13 393 and 308.  But the line also sets the
+// grid: the row search's time hardly depends on the filling (its rows are trimmed to the
+// particle's reach), the tiled one's on the cells, so with tiles the speed split takes fuller
+// cells and fewer fast particles.  Whole passes with the line at 2.5, 3.5, 5, 7 and 10: four
+// steps of the 2^24 tube 13.11, 13.12, 13.10, 13.52 and 14.39 ms, of 10^7 particles in the
+// plane 5.83, 5.83, 5.84, 6.04 and 6.35, eight of a box of 262 k 1.033, 1.045, 1.058, 1.083 and
+// 1.041 (which search takes how much of it changes from line to line); a request of 50 k, a
+// 2^20 job, an ensemble of 30 and a 2^21 blast are the same within 1 %.
 constexpr float kTileOccupancy = 3.5f;
 
 // an upper bound of sqrt(x) for x >= 0, within 2^-19 of it
