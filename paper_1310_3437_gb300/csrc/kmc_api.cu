@@ -803,7 +803,14 @@ int create_impl(const kmc_params* p, const double* const* src6, const uint32_t* 
   if (!ck(cudaMemcpyAsync(&s->d->d, &dy, sizeof(Dyn), cudaMemcpyHostToDevice, st))) return fail(KMC_ECUDA);
   // positions must lie in the box, velocities must be finite
   uint32_t nbad[2] = {0, 0};
-  launch_validate(s->d, p->n, bad, st);
+  // particles beyond a wall that has moved since step 0 (the frames of the tiled search hold
+  // what lies a 10^-9th beyond it)
+  double wall = INFINITY;
+  if (p->bc[0] == KMC_REFLECT && p->step0 != 0) {
+    wall = h.piston_x0 - h.piston_u * ((double)p->step0 * h.dt);
+    wall = wall > 0.0 ? wall * (1.0 + 1e-9) : 0.0;
+  }
+  launch_validate(s->d, p->n, bad, wall, st);
   if (!ck(cudaMemcpyAsync(nbad, bad, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st)) ||
       !ck(cudaStreamSynchronize(st)))
     return fail(KMC_ECUDA);

@@ -654,7 +654,7 @@ void launch_gather_edges(SimDev* d, uint32_t cap, uint2* out, uint32_t* count, c
 void launch_profile_convert(SimDev* d, uint32_t first, uint32_t count, uint32_t bins,
                             double* out, cudaStream_t st);
 void launch_add_steps(SimDev* d, uint64_t nsteps, cudaStream_t st);
-void launch_validate(SimDev* d, uint32_t n, uint32_t* bad, cudaStream_t st);
+void launch_validate(SimDev* d, uint32_t n, uint32_t* bad, double wall, cudaStream_t st);
 // KMC_OBS_VMAX: acc is 8 bytes of device scratch, out one binary64 (device)
 void launch_vmax_exact(SimDev* d, unsigned long long* acc, double* out, cudaStream_t st);
 

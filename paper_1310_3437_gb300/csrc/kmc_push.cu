@@ -607,7 +607,8 @@ void launch_vmax_exact(SimDev* d, unsigned long long* acc, double* out, cudaStre
 }
 
 // particles outside the box at creation: count them (host reports KMC_EINVAL)
-__global__ void k_validate(SimDev* d, uint32_t* bad) {
+// wall: where the x wall stands before the first step (+inf if it has not moved)
+__global__ void k_validate(SimDev* d, uint32_t* bad, double wall) {
   SimDev& s = *d;
   uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= s.n) return;
@@ -624,14 +625,11 @@ __global__ void k_validate(SimDev* d, uint32_t* bad) {
   if (s.planar && s.v[s.d.parity][2][p] != 0.0) out = true;
   if (s.mix && s.species[s.id[s.d.parity][p]] >= (uint32_t)s.mix_n) out = true;
   if (out) atomicAdd(bad, 1u);
-  // a wall that has moved below the particle before the first step (watch_box)
-  if (!left && s.bc[0] == KMC_REFLECT &&
-      s.x[s.d.parity][0][p] > dsub(s.piston_x0, dmul(s.piston_u, dmul((double)s.d.step, s.dt))))
-    s.d.loose_from = 0;
+  if (!left && gt_bits(s.x[s.d.parity][0][p], wall)) s.d.loose_from = 0;  // see watch_box
 }
 
-void launch_validate(SimDev* d, uint32_t n, uint32_t* bad, cudaStream_t st) {
-  k_validate<<<(n + 255) / 256, 256, 0, st>>>(d, bad);
+void launch_validate(SimDev* d, uint32_t n, uint32_t* bad, double wall, cudaStream_t st) {
+  k_validate<<<(n + 255) / 256, 256, 0, st>>>(d, bad, wall);
 }
 
 void launch_gather_state(SimDev* d, uint32_t n, void* out, cudaStream_t st) {
