@@ -400,7 +400,9 @@ __device__ __noinline__ inline void compute_guards(SimDev& s, uint32_t part, uin
   // binary32, so that they stay inside its range in whatever unit the caller measures lengths.
   // (On exponents, the bits from 20 of the high word: the binary64 pipe has two lanes.)
   const int frame = max(max(f0, f1), max(f2, __double2hiint(S1 * dt)));
-  const bool sane = frame >= 0x3A500000 && frame < 0x45900000;  // 2^-90 to 2^90
+  // (2^-90 to 2^90, and no reach of the fast particles 2^60 times as large)
+  const bool sane = frame >= 0x3A500000 && frame < 0x45900000 &&
+                    __double2hiint(rbmax) < frame + (60 << 20);
   const int ue = sane ? (frame & 0x7FF00000) - 0x3FF00000 : 0;
   const double q0 = times_2(b0, -ue), q1 = times_2(b1, -ue), q2 = times_2(b2, -ue);
   const double rn = sane ? times_2(sqrt_up(fmaxf(f_up((q0 * q0 + q1 * q1) + q2 * q2), 1e-38f)) *
