@@ -1,4 +1,4 @@
-"""A cooperative launch that the driver refuses, faked on the host by a shim in front of the
+"""A cooperative launch that CUDA refuses, faked on the host by a shim in front of the
 runtime's entry point.  Refused once, while the step is captured: the graph without the later
 matching rounds is not used, and the steps equal the oracle's.  Refused always: the call fails
 with KMC_ECUDA, no step is taken, and the simulation stays failed."""
